@@ -54,7 +54,7 @@ ahakv_status launch_score_simt(const Plan& pl, const void* q, const void* k, flo
                                float* final_off, cudaStream_t st);
 // Also streams V and writes nu when the value prior is on (v and nu non-null).
 ahakv_status launch_score_tc(const Plan& pl, const void* q, const void* k, const void* v, float* s_raw, float* nu,
-                             float2* partial, int* counters, int* status, cudaStream_t st);
+                             float* partial, float* off, int* counters, int* status, cudaStream_t st);
 bool score_tc_available();
 void score_tc_test_hooks(long long wait_ns, int withhold);   // see ahakv_test_set_wait
 // The generation phase one token at a time (decode.cu): the score update of one new query per head without

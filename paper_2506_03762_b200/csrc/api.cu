@@ -124,10 +124,10 @@ ahakv_status make_plan(const ahakv_params* p, Plan* pl, const int64_t* obs_pos) 
   size_t off = 0;
   o.off_status = off;  off += 256;
   o.off_sync = off;    off += align_up(units * rb_slots * 2 * sizeof(int), 256);
+  o.off_final = off;   off += align_up(units * rb_slots * (o.use_tc ? 128 : o.R) * sizeof(float2), 256);
   o.off_sraw = off;    off += align_up(units * rb_slots * o.n * sizeof(float), 256);
   o.off_nu = off;      off += align_up(units * o.n * sizeof(float), 256);
   o.off_partial = off; off += align_up(units * rb_slots * o.n_blk * (o.use_tc ? 128 : o.R) * sizeof(float2), 256);
-  o.off_final = off;   off += align_up(units * rb_slots * (o.use_tc ? 128 : o.R) * sizeof(float2), 256);
   o.off_score = off;   off += align_up(units * o.n * sizeof(float), 256);
   o.ws_total = off;
   return AHAKV_OK;
@@ -147,35 +147,29 @@ template <typename T> static T* at(void* ws, size_t off) { return reinterpret_ca
 static ahakv_status queue_raw_score(const Plan& pl, const void* q, const void* k, const void* v, void* ws,
                                     cudaStream_t st, int prof) {
   TraceRange range("ahakv: score");
-  ahakv_status rc = cuda_ok(cudaMemsetAsync(at<char>(ws, pl.off_status), 0, pl.off_sraw - pl.off_status, st));
-  if (rc) return rc;
+  ahakv_status rc;
   profile_mark(prof, 0, st);
   float* s_raw = at<float>(ws, pl.off_sraw);
-  float2* partial = at<float2>(ws, pl.off_partial);
   float* final_off = at<float>(ws, pl.off_final);
   const bool prior = (pl.flags & AHAKV_FLAG_VALUE_PRIOR) != 0;
   float* nu = prior ? at<float>(ws, pl.off_nu) : nullptr;
-  // The tensor-core kernel squares the value rows on its way, as long as its tiles cover all of them: when no
-  // observation row sees the last keys it skips their tiles, their raw score is zero and their value rows are
-  // squared by the streaming kernel.
-  const bool all_keys = pl.n_eff == pl.n;
-  const bool tc_prior = prior && pl.use_tc && all_keys;
-  if (pl.use_tc && !all_keys &&
-      cudaMemsetAsync(s_raw, 0, pl.off_nu - pl.off_sraw, st) != cudaSuccess)
-    return AHAKV_ERR_CUDA;
-  if (pl.use_tc)
-    rc = launch_score_tc(pl, q, k, tc_prior ? v : nullptr, s_raw, nu, partial, at<int>(ws, pl.off_sync),
-                         at<int>(ws, pl.off_status), st);
-  else
-    rc = launch_score_simt(pl, q, k, s_raw, partial, final_off, st);
-  if (rc) return rc;
-  profile_mark(prof, 1, st);
-  if (prior && !tc_prior) {
-    rc = launch_vnorm(pl, v, nu, st);
-    if (rc) return rc;
+  if (pl.use_tc) {
+    // status, counters and row offsets start as all ones: no error, -1, and NaN ("not published yet")
+    if (cudaMemsetAsync(at<char>(ws, pl.off_status), 0xff, pl.off_sraw - pl.off_status, st) != cudaSuccess)
+      return AHAKV_ERR_CUDA;
+    // the kernel skips the tiles that no observation row sees: their raw score is zero
+    if (pl.n_eff != pl.n && cudaMemsetAsync(s_raw, 0, pl.off_nu - pl.off_sraw, st) != cudaSuccess) return AHAKV_ERR_CUDA;
+    rc = launch_score_tc(pl, q, k, prior ? v : nullptr, s_raw, nu, at<float>(ws, pl.off_partial), final_off,
+                         at<int>(ws, pl.off_sync), at<int>(ws, pl.off_status), st);
+    profile_mark(prof, 1, st);
+  } else {
+    if (cudaMemsetAsync(at<char>(ws, pl.off_status), 0, sizeof(int), st) != cudaSuccess) return AHAKV_ERR_CUDA;
+    rc = launch_score_simt(pl, q, k, s_raw, at<float2>(ws, pl.off_partial), final_off, st);
+    profile_mark(prof, 1, st);
+    if (rc == AHAKV_OK && prior) rc = launch_vnorm(pl, v, nu, st);
   }
   profile_mark(prof, 2, st);
-  return AHAKV_OK;
+  return rc;
 }
 
 static int score_slots(const Plan& pl) { return pl.use_tc ? pl.n_rb : 1; }
@@ -452,7 +446,7 @@ ahakv_status ahakv_last_device_status(const void* ws, ahakv_stream_t stream) {
   if (cudaMemcpyAsync(&word, ws, sizeof(int), cudaMemcpyDeviceToHost, (cudaStream_t)stream) != cudaSuccess)
     return AHAKV_ERR_CUDA;
   if (cudaStreamSynchronize((cudaStream_t)stream) != cudaSuccess) return AHAKV_ERR_CUDA;
-  return word == 0 ? AHAKV_OK : AHAKV_ERR_TIMEOUT;
+  return word == (int)AHAKV_ERR_TIMEOUT ? AHAKV_ERR_TIMEOUT : AHAKV_OK;
 }
 
 void ahakv_test_set_wait(int32_t wait_ms, int32_t withhold_first_partial) {
