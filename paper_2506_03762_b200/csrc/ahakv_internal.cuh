@@ -73,12 +73,12 @@ ahakv_status launch_vnorm(const Plan& pl, const void* v, float* nu, cudaStream_t
 // `slots` partial scores per head (row blocks, or query heads when pooling by maximum) are combined here.
 ahakv_status launch_refine(const Plan& pl, const float* s_raw, const float* nu, const float* score_prev,
                            float* score, int slots, cudaStream_t st);
-ahakv_status launch_select(const Plan& pl, const float* score, int32_t* kept_idx, const int32_t* budgets,
-                           cudaStream_t st);
-bool refine_select_fits(const Plan& pl);
+ahakv_status launch_select(const Plan& pl, const float* score, int32_t* kept_idx, cudaStream_t st);
+// Both steps.  Writes the kept tokens' scores to score_out (nullable) itself when a head fits in a cluster; otherwise leaves
+// the refined scores in `score`.  *score_left says which: null, or `score` for the caller to gather from.
 ahakv_status launch_refine_select(const Plan& pl, const float* s_raw, const float* nu, const float* score_prev,
-                                  float* score, int32_t* kept_idx, int slots, const int32_t* budgets,
-                                  cudaStream_t st);
+                                  float* score, float** score_left, float* score_out, int32_t* kept_idx, int slots,
+                                  const int32_t* budgets, cudaStream_t st);
 ahakv_status launch_compact(const Plan& pl, const void* k, const void* v, const float* score,
                             const int32_t* kept_idx, void* k_out, void* v_out, float* score_out,
                             cudaStream_t st);
@@ -88,6 +88,25 @@ int profile_begin_call(cudaStream_t st);             // returns a slot, or -1
 void profile_mark(int slot, int boundary, cudaStream_t st);   // boundary b closes stage b-1, opens stage b
 
 inline ahakv_status cuda_ok(cudaError_t e) { return e == cudaSuccess ? AHAKV_OK : AHAKV_ERR_CUDA; }
+
+// Launches `kernel` so that it may start its prologue while the kernel before it in the stream still runs (programmatic
+// dependent launch; the kernel calls griddep_wait() before it touches anything), as clusters of `cluster` CTAs.
+template <typename... KArgs, typename... Args>
+cudaError_t launch_chained(void (*kernel)(KArgs...), dim3 grid, dim3 block, int cluster, cudaStream_t st, Args&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = cluster;
+  attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = cluster > 1 ? 2 : 1;
+  return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
 
 // ---- device helpers ---------------------------------------------------------
 template <typename T> __device__ __forceinline__ float to_f32(T x);
@@ -126,6 +145,11 @@ template <> struct Vec16<__nv_bfloat16> {
     }
   }
 };
+
+// Programmatic dependent launch: wait for the kernel before this one in the stream (no effect without the launch
+// attribute), and let the one after it start its prologue.
+__device__ __forceinline__ void griddep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void griddep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 __device__ __forceinline__ float fast_exp2(float x) {  // 2 ulp over the whole range; 2^-inf = 0
   float y;

@@ -337,7 +337,7 @@ ahakv_status ahakv_select(const ahakv_params* p, const float* score, int32_t* ke
   if (rc) return rc;
   if (!score || !kept_idx || !aligned16(score) || ((uintptr_t)kept_idx & 3)) return AHAKV_ERR_INVALID_ARG;
   (void)ws; (void)ws_bytes;                    // selection works in shared memory: no scratch is needed
-  return launch_select(pl, score, kept_idx, nullptr, (cudaStream_t)stream);
+  return launch_select(pl, score, kept_idx, (cudaStream_t)stream);
 }
 
 ahakv_status ahakv_compact(const ahakv_params* p, const void* k, const void* v, const float* score,
@@ -373,19 +373,14 @@ static ahakv_status evict_impl(const ahakv_params* p, const int32_t* budgets, co
   float* nu = prior ? at<float>(ws, pl.off_nu) : nullptr;
   float* score = at<float>(ws, pl.off_score);
   nvtxRangePushA("ahakv: refine + select");
-  if (refine_select_fits(pl)) {      // a head's scores fit in one CTA's registers: both steps in one launch
-    rc = launch_refine_select(pl, s_raw, nu, score_prev, score, kept_idx, score_slots(pl), budgets, st);
-    profile_mark(prof, 3, st);
-  } else {
-    rc = launch_refine(pl, s_raw, nu, score_prev, score, score_slots(pl), st);
-    profile_mark(prof, 3, st);
-    if (rc == AHAKV_OK) rc = launch_select(pl, score, kept_idx, budgets, st);
-  }
+  float* score_left = nullptr;
+  rc = launch_refine_select(pl, s_raw, nu, score_prev, score, &score_left, score_out, kept_idx, score_slots(pl), budgets, st);
+  profile_mark(prof, 3, st);
   nvtxRangePop();
   profile_mark(prof, 4, st);
   {
     TraceRange range("ahakv: compact");
-    if (rc == AHAKV_OK) rc = launch_compact(pl, k, v, score_out ? score : nullptr, kept_idx, k_out, v_out, score_out, st);
+    if (rc == AHAKV_OK) rc = launch_compact(pl, k, v, score_left, kept_idx, k_out, v_out, score_left ? score_out : nullptr, st);
   }
   profile_mark(prof, 5, st);
   return rc;

@@ -1,0 +1,74 @@
+"""Refinement and selection at the sizes where a cluster of CTAs per head can go wrong: the edges of a thread's run of
+tokens, of a CTA and of a cluster, rows that do not start on 16-byte boundaries, many heads, ties and scores over many
+octaves.  Selection has no tolerance: the reference is a stable sort of the same float32 scores."""
+import numpy as np
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+
+
+def _expected(s, Br, Bud):
+    n = s.shape[-1]
+    if n <= Bud:
+        return np.arange(n)
+    order = np.argsort(-s[: n - Br], kind="stable")[: Bud - Br]
+    return np.concatenate([np.sort(order), np.arange(n - Br, n)])
+
+
+@pytest.mark.parametrize("H,n,Br,Bud", [
+    (3, 1, 0, 1), (2, 7, 2, 5), (5, 511, 0, 100), (5, 513, 3, 512), (4, 1025, 0, 1), (4, 2049, 64, 300),
+    (3, 4096, 128, 1024), (3, 4097, 0, 4000), (3, 8191, 1, 513), (2, 65535, 7, 3000), (2, 65537, 0, 65536),
+    (1, 131072, 128, 40000), (1, 131073, 128, 40000), (160, 8200, 16, 700), (160, 4098, 0, 2000)])
+@pytest.mark.parametrize("kind", ["spread", "ties", "octaves", "one_bin"])
+def test_selection_equals_a_stable_sort(H, n, Br, Bud, kind):
+    from paper_2506_03762_b200 import binding as ab
+    g = torch.Generator().manual_seed(n * 31 + H)
+    s = torch.rand((1, H, n), generator=g)
+    if kind == "ties":
+        s = torch.round(s * 9) / 9
+    elif kind == "octaves":
+        s = torch.exp2(-60 * s) * torch.where(torch.rand(s.shape, generator=g) < 0.1, -1.0, 1.0)
+    elif kind == "one_bin":
+        s = 1.0 + s * 2.0 ** -9                              # everything in a few bins of the first histogram
+    s = s.cuda()
+    p = ab.Params(1, H, H, 64, n, 1, Br, Bud, dtype=ab.F16, flags=0)
+    idx = torch.full((1, H, min(n, Bud)), -7, dtype=torch.int32, device="cuda")
+    ab.ahakv_select(p, s, idx)
+    sn, got = s.cpu().numpy(), idx.cpu().numpy()
+    for h in range(0, H, max(1, H // 4)):
+        assert np.array_equal(got[0, h], _expected(sn[0, h], Br, Bud))
+
+
+@pytest.mark.parametrize("n", [130, 1027, 4100, 9001, 33001])
+@pytest.mark.parametrize("pool,flags", [(1, 1), (3, 1), (7, 1), (7, 3), (31, 1)])
+def test_refinement_in_the_eviction_call_equals_the_definition(n, pool, flags):
+    """The refined score against Eq. 13-15 in float64 from the same raw scores (value prior off) and the same value rows;
+    both sides round the norms of 64 float16 squares and a handful of products once each, so 1e-5 relative holds."""
+    from paper_2506_03762_b200 import binding as ab
+    B, H, d, r, Br, Bud = 1, 2, 64, 16, 8, 64
+    g = torch.Generator().manual_seed(n + pool)
+    q = torch.randn((B, H, r, d), generator=g).half().cuda()
+    k = torch.randn((B, H, n, d), generator=g).half().cuda()
+    v = (torch.randn((B, H, n, d), generator=g) * (0.2 + torch.rand((B, H, n, 1), generator=g))).half().cuda()
+    prev = (torch.rand((B, H, n), generator=g) * 1e-3).cuda()
+    p = ab.Params(B, H, H, d, n, r, Br, Bud, dtype=ab.F16, flags=flags, pool_kernel=pool)
+    ws = ab.alloc_workspace(p)
+    raw, score = torch.empty((B, H, n), device="cuda"), torch.empty((B, H, n), device="cuda")
+    p.flags = 0
+    ab.ahakv_score(p, q, k, None, None, raw, ws)
+    p.flags = flags
+    ab.ahakv_score(p, q, k, v, prev, score, ws)
+    k_out, v_out, s_out, idx = ab.alloc_outputs(p)
+    ab.ahakv_evict(p, q, k, v, prev, k_out, v_out, s_out, idx, ws)
+    nu = v.double().square().sum(-1)
+    ones = torch.ones((1, 1, pool), dtype=torch.float64, device="cuda")
+    tot = torch.nn.functional.conv1d(nu.view(B * H, 1, n), ones, padding=pool // 2).view(B, H, n)
+    cnt = torch.nn.functional.conv1d(torch.ones_like(nu).view(B * H, 1, n), ones, padding=pool // 2).view(B, H, n)
+    gamma = tot / pool if flags & ab.FLAG_POOL_ZERO_PAD else tot / cnt
+    want = raw.double() * gamma / gamma.amax(-1, keepdim=True) + prev.double()
+    assert torch.allclose(score.double(), want, rtol=1e-5, atol=0)
+    sn = score.cpu().numpy()
+    for h in range(H):
+        assert np.array_equal(idx[0, h].cpu().numpy(), _expected(sn[0, h], Br, Bud))
+    assert torch.equal(s_out, score.gather(-1, idx.long()))
