@@ -50,9 +50,9 @@ ahakv_status make_plan(const ahakv_params* p, Plan* plan, const int64_t* obs_pos
 void count_launch(int n = 1);
 
 // Launchers.  Each returns AHAKV_OK or AHAKV_ERR_CUDA and queues work on `st` only.
-ahakv_status launch_score_simt(const Plan& pl, const void* q, const void* k, float* s_raw, float2* partial,
-                               float* final_off, cudaStream_t st);
-// Also streams V and writes nu when the value prior is on (v and nu non-null).
+// Both also stream V and write nu when the value prior is on (v and nu non-null), and clear the status word.
+ahakv_status launch_score_simt(const Plan& pl, const void* q, const void* k, const void* v, float* s_raw, float* nu, float2* partial,
+                               int* status, cudaStream_t st);
 ahakv_status launch_score_tc(const Plan& pl, const void* q, const void* k, const void* v, float* s_raw, float* nu,
                              float* partial, float* off, int* counters, int* status, cudaStream_t st);
 bool score_tc_available();
@@ -92,10 +92,11 @@ inline ahakv_status cuda_ok(cudaError_t e) { return e == cudaSuccess ? AHAKV_OK 
 // Launches `kernel` so that it may start its prologue while the kernel before it in the stream still runs (programmatic
 // dependent launch; the kernel calls griddep_wait() before it touches anything), as clusters of `cluster` CTAs.
 template <typename... KArgs, typename... Args>
-cudaError_t launch_chained(void (*kernel)(KArgs...), dim3 grid, dim3 block, int cluster, cudaStream_t st, Args&&... args) {
+cudaError_t launch_chained(void (*kernel)(KArgs...), dim3 grid, dim3 block, int cluster, size_t smem, cudaStream_t st, Args&&... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;

@@ -163,10 +163,8 @@ static ahakv_status queue_raw_score(const Plan& pl, const void* q, const void* k
                          at<int>(ws, pl.off_sync), at<int>(ws, pl.off_status), st);
     profile_mark(prof, 1, st);
   } else {
-    if (cudaMemsetAsync(at<char>(ws, pl.off_status), 0, sizeof(int), st) != cudaSuccess) return AHAKV_ERR_CUDA;
-    rc = launch_score_simt(pl, q, k, s_raw, at<float2>(ws, pl.off_partial), final_off, st);
+    rc = launch_score_simt(pl, q, k, v, s_raw, nu, at<float2>(ws, pl.off_partial), at<int>(ws, pl.off_status), st);
     profile_mark(prof, 1, st);
-    if (rc == AHAKV_OK && prior) rc = launch_vnorm(pl, v, nu, st);
   }
   profile_mark(prof, 2, st);
   return rc;

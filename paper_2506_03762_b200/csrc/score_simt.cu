@@ -1,18 +1,29 @@
-// Scoring on the plain FP32 pipes: the path for float32 inputs (where a TF32
+// Scoring on the plain FP pipes: the path for float32 inputs (where a TF32
 // tensor-core product would miss the 1e-5 tolerance) and for 16-bit shapes the
 // tensor-core kernel does not take.
-//
-// One thread owns one key.  Pass 1 gives every observation row its softmax
-// statistics (max and sum of 2^{c w}) per 128-key tile, a small kernel merges the
-// tiles, and pass 2 recomputes the logits and adds the normalised weights of all
-// rows into the key's score (Eq. 1, 5, 9).  Every reduction has a fixed order,
-// so the scores are reproducible bit for bit.
 //
 // float32 inputs are held to 1e-5 on the scores, logits of hundreds included: an FP32
 // logit near 256 is only known to 3e-5, so for them the dot product, the scale and
 // the subtraction of the row's shift run in double (products of two floats are exact
 // there), and only the shifted exponent, a small number, goes back to FP32 for the
 // exponential.  16-bit inputs (1e-3) keep FP32 throughout.
+//
+// Two kernels over 64-key tiles, one CTA a tile of a (sequence, KV head).
+//   simt_row_stats:   every observation row's softmax statistics (max and sum of 2^{c w}) per 128-key block, two CTAs (a
+//                     cluster) a block.
+//   simt_column_sums: merges the blocks' statistics, recomputes the logits and adds the normalised weights of all rows
+//                     into the keys' scores (Eq. 1, 5, 9); squares the tile's value rows on the side.
+// What bounds them: the FP64 units, 64 multiply-adds a cycle and SM, as long as their operands come ready-made and cheaply.
+// Converting FP32 to FP64 runs at a quarter of that rate, so keys and queries are converted once, into shared memory; and
+// shared memory keeps up because the products are mma.sync m8n8k4 in double (the same multiply-adds, one rounding each,
+// at the same rate as the plain instruction, but a warp reads 64 operands for 256 of them).  A thread per key that
+// converted both operands of every multiply-add took 160 us for 8 heads x 3001 tokens x 32 rows x 128 elements; 2 x 4
+// logits a thread with plain multiply-adds 60, and this form 49.  The second kernel starts while the first still runs and forms its first
+// logits before it waits for the statistics.
+//
+// Every reduction has a fixed order, so the scores are reproducible bit for bit.
+#include <cooperative_groups.h>
+
 #include <type_traits>
 
 #include "ahakv_internal.cuh"
@@ -20,32 +31,13 @@
 namespace ahakv {
 namespace {
 
-constexpr int kThreads = 128;
+namespace cg = cooperative_groups;
 
-template <typename T, int D>
-__device__ __forceinline__ void load_q_group(const T* __restrict__ q, const Shape& pl, int b, int h, float* qsm) {
-  // qsm[s][c], s = g * r + i over the G query heads of KV head h
-  constexpr int V = Vec16<T>::N;
-  const int vec_per_row = D / V;
-  for (int t = threadIdx.x; t < pl.R * vec_per_row; t += blockDim.x) {
-    const int s = t / vec_per_row, cv = t % vec_per_row;
-    const int g = s / pl.r, i = s % pl.r;
-    const T* row = q + (long long)b * pl.qs[0] + (long long)(h * pl.G + g) * pl.qs[1] + (long long)i * pl.qs[2];
-    const uint4 u = *reinterpret_cast<const uint4*>(row + cv * V);
-    Vec16<T>::widen(u, qsm + s * D + cv * V);
-  }
-}
-
-template <typename T, int D>
-__device__ __forceinline__ void load_key(const T* __restrict__ k, const Shape& pl, int b, int h, int j, float* kreg) {
-  constexpr int V = Vec16<T>::N;
-  const T* row = k + (long long)b * pl.ks[0] + (long long)h * pl.ks[1] + (long long)j * pl.ks[2];
-#pragma unroll
-  for (int cv = 0; cv < D / V; ++cv) {
-    const uint4 u = *reinterpret_cast<const uint4*>(row + cv * V);
-    Vec16<T>::widen(u, kreg + cv * V);
-  }
-}
+constexpr int kThreads = 256;
+constexpr int kTile = 64;                // keys per CTA
+constexpr int kRows = 32;                // stacked observation rows at a time
+constexpr int kKeyWarps = 4;             // warps along the keys (16 each); two along the rows (16 each)
+static_assert(2 * kTile == kKeyTile, "a cluster of two CTAs is one block of statistics");
 
 // The accumulator type of the logits: double for float32 inputs, float for 16-bit ones.
 template <typename T> using Acc = typename std::conditional<std::is_same<T, float>::value, double, float>::type;
@@ -56,152 +48,345 @@ template <typename A> struct RowScaleOf {
   int last[kMaxRows];
 };
 
-template <int D, typename A>
-__device__ __forceinline__ A dot_row(const float* __restrict__ qrow, const float* kreg) {
-  A a0 = 0, a1 = 0, a2 = 0, a3 = 0;
-#pragma unroll
-  for (int c = 0; c < D; c += 4) {
-    const float4 qv = *reinterpret_cast<const float4*>(qrow + c);
-    a0 = fma((A)qv.x, (A)kreg[c], a0);
-    a1 = fma((A)qv.y, (A)kreg[c + 1], a1);
-    a2 = fma((A)qv.z, (A)kreg[c + 2], a2);
-    a3 = fma((A)qv.w, (A)kreg[c + 3], a3);
-  }
-  return (a0 + a1) + (a2 + a3);
+// Rows of shared memory are padded so that no two lanes of a quarter-warp's 16-byte loads meet on a bank: in double it reads
+// two rows, 64 bytes of each; in float single pieces of up to eight rows.
+template <typename A, int D> constexpr int row_pitch() { return D + (sizeof(A) == 8 ? 8 : 4); }
+
+template <typename A, int D>
+struct Tiles {
+  A k[kTile][row_pitch<A, D>()];
+  A q[kRows][row_pitch<A, D>()];
+  A row_c[kRows];
+  int row_last[kRows];
+  float2 fin[kRows];                                  // shift and 1 / (G sum) of a row
+  float2 stat[kMaxRows][kKeyWarps];                   // simt_row_stats: per row and key warp; simt_column_sums: scratch
+};
+
+// mma.sync m8n8k4 in double: C (8 x 8) += A (8 x 4, lane l has row l / 4, column l % 4) B (4 x 8, row l % 4, column l / 4);
+// lane l has C's row l / 4, columns 2 (l % 4) and + 1.
+__device__ __forceinline__ void mma_884(double& c0, double& c1, double a, double b) {
+  asm volatile("mma.sync.aligned.m8n8k4.row.col.f64.f64.f64.f64 {%0, %1}, {%2}, {%3}, {%0, %1};" : "+d"(c0), "+d"(c1) : "d"(a), "d"(b));
 }
 
-// Pass 1: per (unit, key tile, stacked row) the pair (max of c*w, sum of 2^{c*w - max}).
+// 16 bytes of T into shared memory as accumulator-type values.
+template <typename T, typename A>
+__device__ __forceinline__ void put16(A* dst, const uint4& u) {
+  constexpr int V = Vec16<T>::N;
+  float f[V];
+  Vec16<T>::widen(u, f);
+#pragma unroll
+  for (int e = 0; e < V; ++e) dst[e] = (A)f[e];
+}
+
 template <typename T, int D>
-__global__ void __launch_bounds__(kThreads) simt_row_stats(const T* __restrict__ q, const T* __restrict__ k,
-                                                           float2* __restrict__ partial, const Shape pl,
-                                                           const RowScaleOf<Acc<T>> cs) {
-  using A = Acc<T>;
-  extern __shared__ __align__(16) float smem[];
-  float* qsm = smem;                                            // [R][D]
-  float2* wst = reinterpret_cast<float2*>(smem + pl.R * D);     // [4][R]
-  const int unit = blockIdx.y, b = unit / pl.Hkv, h = unit % pl.Hkv, blk = blockIdx.x;
-  const int j = blk * kKeyTile + threadIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  load_q_group<T, D>(q, pl, b, h, qsm);
-  float kreg[D];
-  const bool valid = j < pl.n;
-  if (valid) load_key<T, D>(k, pl, b, h, j, kreg);
-  else {
+__device__ __forceinline__ void load_keys(Tiles<Acc<T>, D>& sm, const T* __restrict__ k, const Shape& pl, int b, int h, int j0) {
+  constexpr int V = Vec16<T>::N, PER = D / V;
+  const T* base = k + (long long)b * pl.ks[0] + (long long)h * pl.ks[1];
 #pragma unroll
-    for (int c = 0; c < D; ++c) kreg[c] = 0.f;
-  }
-  __syncthreads();
-  for (int s = 0; s < pl.R; ++s) {
-    const int i = s % pl.r;
-    const bool vis = valid && j <= cs.last[i];
-    const A x = vis ? dot_row<D, A>(qsm + s * D, kreg) * cs.c[i] : (A)-INFINITY;
-    float m = (float)x;                                         // the shift is an FP32 number on either path
-#pragma unroll
-    for (int o = 16; o; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-    float z = vis ? fast_exp2((float)(x - (A)m)) : 0.f;
-#pragma unroll
-    for (int o = 16; o; o >>= 1) z += __shfl_xor_sync(0xffffffffu, z, o);
-    if (lane == 0) wst[warp * pl.R + s] = make_float2(m, z);
-  }
-  __syncthreads();
-  for (int s = threadIdx.x; s < pl.R; s += kThreads) {
-    float M = -INFINITY;
-#pragma unroll
-    for (int w = 0; w < kThreads / 32; ++w) M = fmaxf(M, wst[w * pl.R + s].x);
-    float Z = 0.f;
-#pragma unroll
-    for (int w = 0; w < kThreads / 32; ++w) {
-      const float2 p = wst[w * pl.R + s];
-      if (p.y > 0.f) Z += p.y * fast_exp2(p.x - M);
-    }
-    partial[((size_t)unit * pl.n_blk + blk) * pl.R + s] = make_float2(M, Z);
+  for (int t = threadIdx.x; t < kTile * PER; t += kThreads) {
+    const int row = t / PER, cv = t % PER, j = j0 + row;
+    put16<T>(&sm.k[row][cv * V], j < pl.n ? *reinterpret_cast<const uint4*>(base + (long long)j * pl.ks[2] + cv * V) : make_uint4(0, 0, 0, 0));
   }
 }
 
-// Merge the tiles of one unit into (max, 1 / (G * sum)) per stacked row, so that
-// 2^{c w - max} times the second entry is the softmax weight divided by the group size.
-__global__ void simt_merge_stats(const float2* __restrict__ partial, float2* __restrict__ final_st, const Shape pl) {
-  const int unit = blockIdx.x;
-  for (int s = threadIdx.x; s < pl.R; s += blockDim.x) {
-    const float2* p = partial + (size_t)unit * pl.n_blk * pl.R + s;
-    float M = -INFINITY;
-    for (int t = 0; t < pl.n_blk; ++t) M = fmaxf(M, p[(size_t)t * pl.R].x);
-    float Z = 0.f;
-    for (int t = 0; t < pl.n_blk; ++t) {
-      const float2 e = p[(size_t)t * pl.R];
-      if (e.y > 0.f) Z += e.y * fast_exp2(e.x - M);
+// Chunk `ch` of a head's stacked rows (s = g r + i): thirty-two in a row, or, when the query heads are pooled by maximum,
+// thirty-two of one query head.
+struct Chunk {
+  int s0, rows;             // first stacked row, live rows
+  bool head_done;           // the last chunk of its query head (pooling by maximum only)
+};
+__device__ __forceinline__ int n_chunks(const Shape& pl) {
+  return pl.group_max ? pl.G * ((pl.r + kRows - 1) / kRows) : (pl.R + kRows - 1) / kRows;
+}
+__device__ __forceinline__ Chunk chunk_of(const Shape& pl, int ch) {
+  if (!pl.group_max) return {ch * kRows, min(kRows, pl.R - ch * kRows), false};
+  const int per = (pl.r + kRows - 1) / kRows, g = ch / per, i0 = (ch % per) * kRows;
+  return {g * pl.r + i0, min(kRows, pl.r - i0), ch % per == per - 1};
+}
+
+template <typename T, int D>
+__device__ __forceinline__ void load_rows(Tiles<Acc<T>, D>& sm, const T* __restrict__ q, const Shape& pl, const RowScaleOf<Acc<T>>& cs,
+                                          int b, int h, const Chunk& c) {
+  constexpr int V = Vec16<T>::N, PER = D / V;
+  for (int t = threadIdx.x; t < kRows * PER; t += kThreads) {
+    const int row = t / PER, cv = t % PER, s = c.s0 + row, g = s / pl.r, i = s % pl.r;
+    uint4 u = make_uint4(0, 0, 0, 0);
+    if (row < c.rows)
+      u = *reinterpret_cast<const uint4*>(q + (long long)b * pl.qs[0] + (long long)(h * pl.G + g) * pl.qs[1] + (long long)i * pl.qs[2] + cv * V);
+    put16<T>(&sm.q[row][cv * V], u);
+  }
+  if (threadIdx.x < kRows) {
+    const int i = (c.s0 + threadIdx.x) % pl.r;
+    sm.row_c[threadIdx.x] = cs.c[i];
+    sm.row_last[threadIdx.x] = (int)threadIdx.x < c.rows ? cs.last[i] : -1;
+  }
+}
+
+// Dot products of the 16 keys from `key0` with the 16 rows from `row0`, a warp's share; this thread's are acc[x][y], of key
+// key0 + 8 (x / 2) + 2 (lane % 4) + x % 2 and row row0 + 8 y + lane / 4 (the fragment layout of m8n8k4).  Which four elements
+// a step multiplies does not matter as long as both operands agree: a lane takes elements 2 t, 2 t + 1 of eight at a time.
+template <int D>
+__device__ __forceinline__ void dot_16x16(const Tiles<double, D>& sm, int key0, int row0, double (&acc)[4][2]) {
+  const int lane = threadIdx.x & 31, grp = lane >> 2, tig = lane & 3;
+#pragma unroll
+  for (int x = 0; x < 4; ++x) acc[x][0] = acc[x][1] = 0.0;
+#pragma unroll 4
+  for (int d = 0; d < D; d += 8) {
+    double2 kv[2], qv[2];
+#pragma unroll
+    for (int t = 0; t < 2; ++t) {
+      kv[t] = *reinterpret_cast<const double2*>(&sm.k[key0 + 8 * t + grp][d + 2 * tig]);
+      qv[t] = *reinterpret_cast<const double2*>(&sm.q[row0 + 8 * t + grp][d + 2 * tig]);
     }
-    final_st[(size_t)unit * pl.R + s] = make_float2(M, 1.f / (Z * (float)(pl.group_max ? 1 : pl.G)));
+#pragma unroll
+    for (int y = 0; y < 2; ++y)
+#pragma unroll
+      for (int t = 0; t < 2; ++t) {
+        mma_884(acc[2 * t][y], acc[2 * t + 1][y], qv[y].x, kv[t].x);
+        mma_884(acc[2 * t][y], acc[2 * t + 1][y], qv[y].y, kv[t].y);
+      }
+  }
+}
+template <int D>
+__device__ __forceinline__ void dot_16x16(const Tiles<float, D>& sm, int key0, int row0, float (&acc)[4][2]) {
+  const int lane = threadIdx.x & 31, key = key0 + 2 * (lane & 3), row = row0 + (lane >> 2);
+#pragma unroll
+  for (int x = 0; x < 4; ++x) acc[x][0] = acc[x][1] = 0.f;
+#pragma unroll 4
+  for (int d = 0; d < D; d += 4) {
+    float4 kv[4], qv[2];
+#pragma unroll
+    for (int x = 0; x < 4; ++x) kv[x] = *reinterpret_cast<const float4*>(&sm.k[key + 8 * (x >> 1) + (x & 1)][d]);
+#pragma unroll
+    for (int y = 0; y < 2; ++y) qv[y] = *reinterpret_cast<const float4*>(&sm.q[row + 8 * y][d]);
+#pragma unroll
+    for (int x = 0; x < 4; ++x)
+#pragma unroll
+      for (int y = 0; y < 2; ++y)
+        acc[x][y] = fmaf(qv[y].w, kv[x].w, fmaf(qv[y].z, kv[x].z, fmaf(qv[y].y, kv[x].y, fmaf(qv[y].x, kv[x].x, acc[x][y]))));
+  }
+}
+
+// Two (max, sum) pairs of disjoint key sets into one.
+__device__ __forceinline__ float2 merge_pair(float2 a, float2 b) {
+  const float m = fmaxf(a.x, b.x);
+  float z = 0.f;
+  if (a.y > 0.f) z += a.y * fast_exp2(a.x - m);
+  if (b.y > 0.f) z += b.y * fast_exp2(b.x - m);
+  return make_float2(m, z);
+}
+
+// Pass 1: per (unit, 128-key block, stacked row) the pair (max of c*w, sum of 2^{c*w - max}).
+template <typename T, int D>
+__global__ void __launch_bounds__(kThreads, 2) __cluster_dims__(2, 1, 1)
+simt_row_stats(const T* __restrict__ q, const T* __restrict__ k, float2* __restrict__ partial, int* __restrict__ status,
+               const __grid_constant__ Shape pl, const __grid_constant__ RowScaleOf<Acc<T>> cs) {
+  using A = Acc<T>;
+  extern __shared__ __align__(16) char smem_raw[];
+  Tiles<A, D>& sm = *reinterpret_cast<Tiles<A, D>*>(smem_raw);
+  cg::cluster_group cl = cg::this_cluster();
+  const int unit = blockIdx.y, b = unit / pl.Hkv, h = unit % pl.Hkv, j0 = blockIdx.x * kTile, rank = blockIdx.x & 1;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, kw = warp & (kKeyWarps - 1), rw = warp / kKeyWarps;
+  const int row = 16 * rw + (lane >> 2);
+  const auto key = [=](int x) { return 16 * kw + 8 * (x >> 1) + 2 * (lane & 3) + (x & 1); };   // this thread's four keys
+  griddep_wait();
+  griddep_launch();
+  if (unit == 0 && blockIdx.x == 0 && threadIdx.x == 0) *status = 0;
+  load_keys<T, D>(sm, k, pl, b, h, j0);
+  const int chunks = n_chunks(pl);
+  for (int ch = 0; ch < chunks; ++ch) {
+    const Chunk c = chunk_of(pl, ch);
+    if (ch > 0) __syncthreads();
+    load_rows<T, D>(sm, q, pl, cs, b, h, c);
+    __syncthreads();
+    A acc[4][2];
+    dot_16x16<D>(sm, 16 * kw, 16 * rw, acc);
+#pragma unroll
+    for (int y = 0; y < 2; ++y) {
+      const A cc = sm.row_c[row + 8 * y];
+      const int last = sm.row_last[row + 8 * y];
+      float m = -INFINITY;                                      // the shift is an FP32 number on either path
+#pragma unroll
+      for (int x = 0; x < 4; ++x) {
+        acc[x][y] *= cc;
+        if (j0 + key(x) <= last) m = fmaxf(m, (float)acc[x][y]);
+      }
+#pragma unroll
+      for (int o = 2; o; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+      float z = 0.f;
+#pragma unroll
+      for (int x = 0; x < 4; ++x)
+        if (j0 + key(x) <= last) z += fast_exp2((float)(acc[x][y] - (A)m));
+#pragma unroll
+      for (int o = 2; o; o >>= 1) z += __shfl_xor_sync(0xffffffffu, z, o);
+      if ((lane & 3) == 0 && row + 8 * y < c.rows) sm.stat[c.s0 + row + 8 * y][kw] = make_float2(m, z);
+    }
+  }
+  cl.sync();
+  // the two CTAs of a block take a row in turn, its eight warps' pairs in key order
+  const float2* first = &cl.map_shared_rank(&sm, 0)->stat[0][0];
+  const float2* second = &cl.map_shared_rank(&sm, 1)->stat[0][0];
+  for (int s = 2 * threadIdx.x + rank; s < pl.R; s += 2 * kThreads) {
+    float2 p = make_float2(-INFINITY, 0.f);
+#pragma unroll
+    for (int w = 0; w < kKeyWarps; ++w) p = merge_pair(p, first[s * kKeyWarps + w]);
+#pragma unroll
+    for (int w = 0; w < kKeyWarps; ++w) p = merge_pair(p, second[s * kKeyWarps + w]);
+    partial[((size_t)unit * pl.n_blk + blockIdx.x / 2) * pl.R + s] = p;
+  }
+  cl.sync();
+}
+
+// nu_j = |V_j|^2 of the tile's value rows: a warp a row (half a warp where a row is 256 bytes), the pieces' sums folded by a
+// fixed shuffle tree.
+template <typename T, int D>
+__device__ __forceinline__ void tile_norms(const T* __restrict__ v, float* __restrict__ nu, const Shape& pl, int b, int h, int unit,
+                                           int j0) {
+  constexpr int V = Vec16<T>::N, LANES = D / V, ROWS = kThreads / LANES, N = kTile / ROWS > 0 ? kTile / ROWS : 1;
+  const int sub = threadIdx.x % LANES, r0 = threadIdx.x / LANES;
+  const T* base = v + (long long)b * pl.vs[0] + (long long)h * pl.vs[1] + sub * V;
+  uint4 u[N];
+#pragma unroll
+  for (int t = 0; t < N; ++t) {
+    const int j = j0 + r0 + t * ROWS;
+    u[t] = j < pl.n ? __ldcs(reinterpret_cast<const uint4*>(base + (long long)j * pl.vs[2])) : make_uint4(0, 0, 0, 0);
+  }
+#pragma unroll
+  for (int t = 0; t < N; ++t) {
+    float f[V];
+    Vec16<T>::widen(u[t], f);
+    float s = 0.f;
+#pragma unroll
+    for (int e = 0; e < V; ++e) s = fmaf(f[e], f[e], s);
+#pragma unroll
+    for (int o = LANES / 2; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    const int j = j0 + r0 + t * ROWS;
+    if (sub == 0 && j < pl.n) nu[(size_t)unit * pl.n + j] = s;
   }
 }
 
 // Pass 2: S_j = sum over the stacked rows of 2^{c w - max} / (G * sum).
 template <typename T, int D>
-__global__ void __launch_bounds__(kThreads) simt_column_sums(const T* __restrict__ q, const T* __restrict__ k,
-                                                             const float2* __restrict__ final_st,
-                                                             float* __restrict__ s_raw, const Shape pl,
-                                                             const RowScaleOf<Acc<T>> cs) {
+__global__ void __launch_bounds__(kThreads, 2)
+simt_column_sums(const T* __restrict__ q, const T* __restrict__ k, const T* __restrict__ v, const float2* partial,
+                 float* __restrict__ s_raw, float* __restrict__ nu, const __grid_constant__ Shape pl,
+                 const __grid_constant__ RowScaleOf<Acc<T>> cs) {
   using A = Acc<T>;
-  extern __shared__ __align__(16) float smem[];
-  float* qsm = smem;                                            // [R][D]
-  float2* st = reinterpret_cast<float2*>(smem + pl.R * D);      // [R]
-  const int unit = blockIdx.y, b = unit / pl.Hkv, h = unit % pl.Hkv;
-  const int j = blockIdx.x * kKeyTile + threadIdx.x;
-  load_q_group<T, D>(q, pl, b, h, qsm);
-  for (int s = threadIdx.x; s < pl.R; s += kThreads) st[s] = final_st[(size_t)unit * pl.R + s];
-  __syncthreads();
-  if (j >= pl.n) return;
-  float kreg[D];
-  load_key<T, D>(k, pl, b, h, j, kreg);
-  float acc = 0.f, best = 0.f;
-  for (int s = 0; s < pl.R; ++s) {
-    const int i = s % pl.r;
-    if (pl.group_max && i == 0 && s > 0) {        // a query head is complete: keep the largest head's score
-      best = fmaxf(best, acc);
-      acc = 0.f;
+  extern __shared__ __align__(16) char smem_raw[];
+  Tiles<A, D>& sm = *reinterpret_cast<Tiles<A, D>*>(smem_raw);
+  float2 (*part)[kRows] = reinterpret_cast<float2 (*)[kRows]>(&sm.stat[0][0]);       // [8][kRows]
+  float (*col)[kTile] = reinterpret_cast<float (*)[kTile]>(&sm.stat[kMaxRows / 2][0]);   // [2][kTile]
+  const int unit = blockIdx.y, b = unit / pl.Hkv, h = unit % pl.Hkv, j0 = blockIdx.x * kTile;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, kw = warp & (kKeyWarps - 1), rw = warp / kKeyWarps;
+  const int row = 16 * rw + (lane >> 2);
+  const auto key = [=](int x) { return 16 * kw + 8 * (x >> 1) + 2 * (lane & 3) + (x & 1); };   // this thread's four keys
+  // The inputs were there before the statistics kernel began; only its statistics have to be waited for (and nothing
+  // may be written before: the kernel that reads the last call's scores may still run).
+  load_keys<T, D>(sm, k, pl, b, h, j0);
+  const int chunks = n_chunks(pl);
+  float sum[4] = {}, best = 0.f;
+  for (int ch = 0; ch < chunks; ++ch) {
+    const Chunk c = chunk_of(pl, ch);
+    if (ch > 0) __syncthreads();
+    load_rows<T, D>(sm, q, pl, cs, b, h, c);
+    __syncthreads();
+    A acc[4][2];
+    dot_16x16<D>(sm, 16 * kw, 16 * rw, acc);
+    if (ch == 0) {
+      griddep_wait();
+      griddep_launch();
+      if (nu) tile_norms<T, D>(v, nu, pl, b, h, unit, j0);
     }
-    if (j <= cs.last[i])
-      acc = fmaf(fast_exp2((float)fma(dot_row<D, A>(qsm + s * D, kreg), cs.c[i], -(A)st[s].x)), st[s].y, acc);
+    {
+      // eight threads a row, each every eighth block in order, then the eight in order
+      float2 p = make_float2(-INFINITY, 0.f);
+      if (lane < c.rows) {
+        const float2* from = partial + (size_t)unit * pl.n_blk * pl.R + c.s0 + lane;
+#pragma unroll 4
+        for (int t = warp; t < pl.n_blk; t += kThreads / 32) p = merge_pair(p, __ldcg(from + (size_t)t * pl.R));
+      }
+      part[warp][lane] = p;
+      __syncthreads();
+      if (threadIdx.x < kRows) {
+#pragma unroll
+        for (int w = 1; w < kThreads / 32; ++w) p = merge_pair(p, part[w][threadIdx.x]);
+        sm.fin[threadIdx.x] = make_float2(p.x, 1.f / (p.y * (float)(pl.group_max ? 1 : pl.G)));
+      }
+      __syncthreads();
+    }
+#pragma unroll
+    for (int y = 0; y < 2; ++y) {
+      const A cc = sm.row_c[row + 8 * y];
+      const int last = sm.row_last[row + 8 * y];
+      const float2 st = sm.fin[row + 8 * y];
+#pragma unroll
+      for (int x = 0; x < 4; ++x)
+        if (j0 + key(x) <= last) sum[x] = fmaf(fast_exp2((float)fma(acc[x][y], cc, -(A)st.x)), st.y, sum[x]);
+    }
+    if (c.head_done || ch + 1 == chunks) {
+      // the eight row groups of the warp, then the two warps along the rows
+#pragma unroll
+      for (int o = 4; o <= 16; o <<= 1)
+#pragma unroll
+        for (int x = 0; x < 4; ++x) sum[x] += __shfl_xor_sync(0xffffffffu, sum[x], o);
+#pragma unroll
+      for (int x = 0; x < 4; ++x) {
+        if (lane < 4) col[rw][key(x)] = sum[x];
+        sum[x] = 0.f;
+      }
+      __syncthreads();
+      if (threadIdx.x < kTile) best = fmaxf(best, col[0][threadIdx.x] + col[1][threadIdx.x]);
+    }
   }
-  s_raw[(size_t)unit * pl.n + j] = pl.group_max ? fmaxf(best, acc) : acc;
+  if (threadIdx.x < kTile && j0 + (int)threadIdx.x < pl.n) s_raw[(size_t)unit * pl.n + j0 + threadIdx.x] = best;
 }
 
 template <typename T, int D>
-ahakv_status run(const Plan& pl, const void* q, const void* k, float* s_raw, float2* partial, float* final_off,
+ahakv_status run(const Plan& pl, const void* q, const void* k, const void* v, float* s_raw, float* nu, float2* partial, int* status,
                  cudaStream_t st) {
   RowScaleOf<Acc<T>> cs;
   for (int i = 0; i < kMaxRows; ++i) {
     cs.c[i] = i < pl.r ? (Acc<T>)(pl.lambda[i] * 1.4426950408889634) : (Acc<T>)0;
     cs.last[i] = pl.last[i];
   }
-  const size_t smem1 = (size_t)pl.R * D * sizeof(float) + (size_t)(kThreads / 32) * pl.R * sizeof(float2);
-  const size_t smem2 = (size_t)pl.R * D * sizeof(float) + (size_t)pl.R * sizeof(float2);
-  if (cudaFuncSetAttribute(simt_row_stats<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem1) != cudaSuccess ||
-      cudaFuncSetAttribute(simt_column_sums<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem2) != cudaSuccess)
-    return AHAKV_ERR_CUDA;
-  const dim3 grid(pl.n_blk, pl.B * pl.Hkv);
-  simt_row_stats<T, D><<<grid, kThreads, smem1, st>>>((const T*)q, (const T*)k, partial, pl, cs);
-  float2* final_st = reinterpret_cast<float2*>(final_off);
-  simt_merge_stats<<<pl.B * pl.Hkv, 256, 0, st>>>(partial, final_st, pl);
-  simt_column_sums<T, D><<<grid, kThreads, smem2, st>>>((const T*)q, (const T*)k, final_st, s_raw, pl, cs);
-  count_launch(3);
-  return cuda_ok(cudaGetLastError());
+  constexpr size_t smem = sizeof(Tiles<Acc<T>, D>);
+  // leave to use more than 48 KB of shared memory, asked for once per device
+  constexpr int kMaxDevices = 64;
+  static bool configured[kMaxDevices] = {};
+  int dev = -1;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return AHAKV_ERR_CUDA;
+  if (!configured[dev]) {
+    if (cudaFuncSetAttribute(simt_row_stats<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
+        cudaFuncSetAttribute(simt_column_sums<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+      return AHAKV_ERR_CUDA;
+    configured[dev] = true;
+  }
+  const Shape& shape = pl;
+  const int units = pl.B * pl.Hkv;
+  cudaError_t e = launch_chained(simt_row_stats<T, D>, dim3(2 * pl.n_blk, units), dim3(kThreads), 2, smem, st, (const T*)q, (const T*)k,
+                                 partial, status, shape, cs);
+  if (e == cudaSuccess)
+    e = launch_chained(simt_column_sums<T, D>, dim3((pl.n + kTile - 1) / kTile, units), dim3(kThreads), 1, smem, st, (const T*)q,
+                       (const T*)k, (const T*)v, partial, s_raw, nu, shape, cs);
+  count_launch(2);
+  return cuda_ok(e);
 }
 
 }  // namespace
 
-ahakv_status launch_score_simt(const Plan& pl, const void* q, const void* k, float* s_raw, float2* partial,
-                               float* final_off, cudaStream_t st) {
+ahakv_status launch_score_simt(const Plan& pl, const void* q, const void* k, const void* v, float* s_raw, float* nu, float2* partial,
+                               int* status, cudaStream_t st) {
   const bool d64 = pl.d == 64;
   switch (pl.dtype) {
     case AHAKV_F32:
-      return d64 ? run<float, 64>(pl, q, k, s_raw, partial, final_off, st)
-                 : run<float, 128>(pl, q, k, s_raw, partial, final_off, st);
+      return d64 ? run<float, 64>(pl, q, k, v, s_raw, nu, partial, status, st)
+                 : run<float, 128>(pl, q, k, v, s_raw, nu, partial, status, st);
     case AHAKV_F16:
-      return d64 ? run<__half, 64>(pl, q, k, s_raw, partial, final_off, st)
-                 : run<__half, 128>(pl, q, k, s_raw, partial, final_off, st);
+      return d64 ? run<__half, 64>(pl, q, k, v, s_raw, nu, partial, status, st)
+                 : run<__half, 128>(pl, q, k, v, s_raw, nu, partial, status, st);
     default:
-      return d64 ? run<__nv_bfloat16, 64>(pl, q, k, s_raw, partial, final_off, st)
-                 : run<__nv_bfloat16, 128>(pl, q, k, s_raw, partial, final_off, st);
+      return d64 ? run<__nv_bfloat16, 64>(pl, q, k, v, s_raw, nu, partial, status, st)
+                 : run<__nv_bfloat16, 128>(pl, q, k, v, s_raw, nu, partial, status, st);
   }
 }
 

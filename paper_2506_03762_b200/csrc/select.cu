@@ -544,7 +544,7 @@ cudaError_t launch_as(const SelectArgs& a, const Shape& pl, int C, cudaStream_t 
       configured[dev] = true;
     }
   }
-  return launch_chained(refine_select_kernel<kPer, kCluster>, dim3(pl.B * pl.Hkv * C), dim3(kThreads), kCluster ? C : 1, st, a, pl);
+  return launch_chained(refine_select_kernel<kPer, kCluster>, dim3(pl.B * pl.Hkv * C), dim3(kThreads), kCluster ? C : 1, 0, st, a, pl);
 }
 
 // One cluster per head.  False: no cluster holds a head.
@@ -576,7 +576,7 @@ ahakv_status launch_refine(const Plan& pl, const float* s_raw, const float* nu, 
   const Shape& shape = pl;
   cudaError_t e = cudaSuccess;
   if (!nu) {
-    e = launch_chained(combine_kernel, dim3((pl.n + 255) / 256, pl.B * pl.Hkv), dim3(256), 1, st, s_raw, score_prev, score, shape, slots);
+    e = launch_chained(combine_kernel, dim3((pl.n + 255) / 256, pl.B * pl.Hkv), dim3(256), 1, 0, st, s_raw, score_prev, score, shape, slots);
   } else if (!launch_clustered(a, pl, st, &e)) {
     refine_kernel<<<pl.B * pl.Hkv, kWideThreads, 0, st>>>(s_raw, nu, score_prev, score, pl, slots);
     e = cudaGetLastError();

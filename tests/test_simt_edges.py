@@ -1,0 +1,27 @@
+"""The float32 scoring kernels at the edges of their 64-key tiles, 128-key blocks and 32-row chunks, grouped and pooled by
+maximum, against a float64 evaluation of Eq. 1, 5, 9 on the same inputs; 1e-5 relative as for every float32 score (the
+logits and shifts are formed in double; what is left is a few FP32 roundings and ex2's two units in the last place)."""
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("B,Hq,Hkv,d,n,r,flags", [
+    (1, 1, 1, 64, 1, 1, 0), (1, 2, 2, 128, 63, 5, 0), (2, 2, 1, 64, 65, 16, 0), (1, 3, 1, 128, 128, 11, 4),
+    (1, 4, 2, 64, 129, 33, 4), (1, 2, 2, 128, 193, 32, 0), (1, 8, 1, 64, 700, 32, 0), (1, 1, 1, 128, 1025, 256, 0)])
+def test_float32_scores_at_tile_edges(B, Hq, Hkv, d, n, r, flags):
+    from paper_2506_03762_b200 import binding as ab
+    g = torch.Generator().manual_seed(n + r)
+    q = (3 * torch.randn((B, Hq, r, d), generator=g)).cuda()
+    k = torch.randn((B, Hkv, n, d), generator=g).cuda()
+    v = torch.randn((B, Hkv, n, d), generator=g).cuda()
+    p = ab.Params(B, Hq, Hkv, d, n, r, 0, max(1, n // 2), dtype=ab.F32, scale_mode=ab.SCALE_FIXED, scale=0.09, flags=flags)
+    score = torch.empty((B, Hkv, n), device="cuda")
+    ab.ahakv_score(p, q, k, v, None, score, ab.alloc_workspace(p))
+    G = Hq // Hkv
+    w = float(torch.tensor(0.09, dtype=torch.float32)) * q.double() @ k.double().repeat_interleave(G, 1).transpose(-1, -2)
+    seen = torch.arange(n, device="cuda") <= torch.arange(n - r, n, device="cuda").view(r, 1)
+    a = w.masked_fill(~seen, float("-inf")).softmax(-1).sum(2).view(B, Hkv, G, n)
+    want = a.amax(2) if flags & ab.FLAG_GROUP_MAX else a.mean(2)
+    assert torch.allclose(score.double(), want, rtol=1e-5, atol=1e-5 * 1e-3 * r / n)
