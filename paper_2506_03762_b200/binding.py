@@ -67,6 +67,24 @@ class Params:
     k_stride: tuple = field(default=(0, 0, 0))
     v_stride: tuple = field(default=(0, 0, 0))
 
+    # A decode loop makes the same call thousands of times: the C struct and the reference to it that ctypes passes are
+    # built once (3 us) and dropped when a field is set.
+    def __setattr__(self, name, value):
+        self.__dict__[name] = value
+        self.__dict__["_ref"] = None
+
+    def __getstate__(self):
+        return {k: v for k, v in self.__dict__.items() if k != "_ref"}
+
+    def ref(self):
+        """A ctypes reference to the C struct with the present values."""
+        r = self.__dict__.get("_ref")
+        if r is None:
+            r = ctypes.byref(self.c())
+            if type(self.q_stride) is type(self.k_stride) is type(self.v_stride) is tuple:   # a list may change unseen
+                self.__dict__["_ref"] = r
+        return r
+
     def c(self) -> CParams:
         nt = self.n_ctx if self.n_total is None else self.n_total
         return CParams(self.batch, self.n_q_heads, self.n_kv_heads, self.head_dim, self.n_ctx, nt,
@@ -134,15 +152,20 @@ def status_string(status: int) -> str:
 
 
 def _ptr(t):
-    if t is None:
-        return None
-    if isinstance(t, int):
+    if t is None or isinstance(t, int):
         return t
     return t.data_ptr()
 
 
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+_device = getattr(torch._C, "_cuda_getDevice", None)
+
+
 def _stream(stream):
     if stream is None:
+        # the handle alone; torch.cuda.current_stream() builds a Stream object around it (1 us)
+        if _raw_stream is not None and _device is not None and torch.cuda.is_initialized():
+            return _raw_stream(_device())
         return torch.cuda.current_stream().cuda_stream
     if isinstance(stream, int):
         return stream
@@ -155,8 +178,7 @@ def _raise(status: int, where: str):
 
 
 def ahakv_workspace_bytes(p: Params) -> int:
-    cp = p.c()
-    return int(lib().ahakv_workspace_bytes(ctypes.byref(cp)))
+    return int(lib().ahakv_workspace_bytes(p.ref()))
 
 
 def ahakv_lambda(n_total: int, budget: int, head_dim: int) -> float:
@@ -173,9 +195,8 @@ def ahakv_launch_count() -> int:
 
 def ahakv_score(p: Params, q_obs, k, v, score_prev, score, ws, ws_bytes: int | None = None, stream=None,
                 check: bool = True) -> int:
-    cp = p.c()
-    nbytes = ws.numel() * ws.element_size() if ws_bytes is None else ws_bytes
-    st = lib().ahakv_score(ctypes.byref(cp), _ptr(q_obs), _ptr(k), _ptr(v), _ptr(score_prev), _ptr(score),
+    nbytes = ws.nbytes if ws_bytes is None else ws_bytes
+    st = lib().ahakv_score(p.ref(), _ptr(q_obs), _ptr(k), _ptr(v), _ptr(score_prev), _ptr(score),
                            _ptr(ws), nbytes, _stream(stream))
     if check:
         _raise(st, "ahakv_score")
@@ -185,10 +206,9 @@ def ahakv_score(p: Params, q_obs, k, v, score_prev, score, ws, ws_bytes: int | N
 def ahakv_score_rows(p: Params, obs_pos, q_obs, k, v, score_prev, score, ws, ws_bytes: int | None = None,
                      stream=None, check: bool = True) -> int:
     """``ahakv_score`` with the observation rows at the given logical positions (a host sequence of r ints)."""
-    cp = p.c()
     pos = None if obs_pos is None else (ctypes.c_int64 * len(obs_pos))(*[int(x) for x in obs_pos])
-    nbytes = ws.numel() * ws.element_size() if ws_bytes is None else ws_bytes
-    st = lib().ahakv_score_rows(ctypes.byref(cp), pos, _ptr(q_obs), _ptr(k), _ptr(v), _ptr(score_prev),
+    nbytes = ws.nbytes if ws_bytes is None else ws_bytes
+    st = lib().ahakv_score_rows(p.ref(), pos, _ptr(q_obs), _ptr(k), _ptr(v), _ptr(score_prev),
                                 _ptr(score), _ptr(ws), nbytes, _stream(stream))
     if check:
         _raise(st, "ahakv_score_rows")
@@ -198,9 +218,8 @@ def ahakv_score_rows(p: Params, obs_pos, q_obs, k, v, score_prev, score, ws, ws_
 def ahakv_score_full_causal(p: Params, q_all, k, v, score_prev, score, ws, ws_bytes: int | None = None,
                             stream=None, check: bool = True) -> int:
     """Accumulation over all query rows (Eq. 2-3); ``p.obs_window`` rows per pass."""
-    cp = p.c()
-    nbytes = ws.numel() * ws.element_size() if ws_bytes is None else ws_bytes
-    st = lib().ahakv_score_full_causal(ctypes.byref(cp), _ptr(q_all), _ptr(k), _ptr(v), _ptr(score_prev),
+    nbytes = ws.nbytes if ws_bytes is None else ws_bytes
+    st = lib().ahakv_score_full_causal(p.ref(), _ptr(q_all), _ptr(k), _ptr(v), _ptr(score_prev),
                                        _ptr(score), _ptr(ws), nbytes, _stream(stream))
     if check:
         _raise(st, "ahakv_score_full_causal")
@@ -208,24 +227,21 @@ def ahakv_score_full_causal(p: Params, q_all, k, v, score_prev, score, ws, ws_by
 
 
 def ahakv_score_step(p: Params, q_t, k, score_prev, score, stream=None, check: bool = True) -> int:
-    cp = p.c()
-    st = lib().ahakv_score_step(ctypes.byref(cp), _ptr(q_t), _ptr(k), _ptr(score_prev), _ptr(score), _stream(stream))
+    st = lib().ahakv_score_step(p.ref(), _ptr(q_t), _ptr(k), _ptr(score_prev), _ptr(score), _stream(stream))
     if check:
         _raise(st, "ahakv_score_step")
     return st
 
 
 def ahakv_compact_inplace(p: Params, k, v, score, kept_idx, stream=None, check: bool = True) -> int:
-    cp = p.c()
-    st = lib().ahakv_compact_inplace(ctypes.byref(cp), _ptr(k), _ptr(v), _ptr(score), _ptr(kept_idx), _stream(stream))
+    st = lib().ahakv_compact_inplace(p.ref(), _ptr(k), _ptr(v), _ptr(score), _ptr(kept_idx), _stream(stream))
     if check:
         _raise(st, "ahakv_compact_inplace")
     return st
 
 
 def ahakv_step_slots(p: Params, q_t, k_t, v_t, k, v, score, pos, free_slot, stream=None, check: bool = True) -> int:
-    cp = p.c()
-    st = lib().ahakv_step_slots(ctypes.byref(cp), _ptr(q_t), _ptr(k_t), _ptr(v_t), _ptr(k), _ptr(v), _ptr(score),
+    st = lib().ahakv_step_slots(p.ref(), _ptr(q_t), _ptr(k_t), _ptr(v_t), _ptr(k), _ptr(v), _ptr(score),
                                 _ptr(pos), _ptr(free_slot), _stream(stream))
     if check:
         _raise(st, "ahakv_step_slots")
@@ -234,14 +250,13 @@ def ahakv_step_slots(p: Params, q_t, k_t, v_t, k, v, score, pos, free_slot, stre
 
 def ahakv_row_entropy(p: Params, q_obs, k, entropy=None, stream=None):
     """Eq. 6 entropy [B,Hq,r] (float32) of every observation row; allocates its scratch and, if not given, the output."""
-    cp = p.c()
-    nbytes = int(lib().ahakv_entropy_workspace_bytes(ctypes.byref(cp)))
+    nbytes = int(lib().ahakv_entropy_workspace_bytes(p.ref()))
     if nbytes == 0:
         raise AhakvError(ERR_INVALID_ARG, "ahakv_entropy_workspace_bytes")
     ws = torch.empty(nbytes, dtype=torch.uint8, device=k.device)
     if entropy is None:
         entropy = torch.empty((p.batch, p.n_q_heads, p.obs_window), dtype=torch.float32, device=k.device)
-    _raise(lib().ahakv_row_entropy(ctypes.byref(cp), _ptr(q_obs), _ptr(k), _ptr(entropy), _ptr(ws), nbytes,
+    _raise(lib().ahakv_row_entropy(p.ref(), _ptr(q_obs), _ptr(k), _ptr(entropy), _ptr(ws), nbytes,
                                    _stream(stream)), "ahakv_row_entropy")
     return entropy
 
@@ -256,8 +271,7 @@ def ahakv_static_last_device_status(stream=None) -> int:
 
 def ahakv_score_static(p: Params, q_obs, k, v, score_prev, score, stream=None, check: bool = True) -> int:
     """``ahakv_score`` on the library's own fixed scratch array: no workspace argument, no allocation."""
-    cp = p.c()
-    st = lib().ahakv_score_static(ctypes.byref(cp), _ptr(q_obs), _ptr(k), _ptr(v), _ptr(score_prev),
+    st = lib().ahakv_score_static(p.ref(), _ptr(q_obs), _ptr(k), _ptr(v), _ptr(score_prev),
                                   _ptr(score), _stream(stream))
     if check:
         _raise(st, "ahakv_score_static")
@@ -266,9 +280,8 @@ def ahakv_score_static(p: Params, q_obs, k, v, score_prev, score, stream=None, c
 
 def ahakv_select(p: Params, score, kept_idx, ws=None, ws_bytes: int | None = None, stream=None,
                  check: bool = True) -> int:
-    cp = p.c()
-    nbytes = (0 if ws is None else ws.numel() * ws.element_size()) if ws_bytes is None else ws_bytes
-    st = lib().ahakv_select(ctypes.byref(cp), _ptr(score), _ptr(kept_idx), _ptr(ws), nbytes, _stream(stream))
+    nbytes = (0 if ws is None else ws.nbytes) if ws_bytes is None else ws_bytes
+    st = lib().ahakv_select(p.ref(), _ptr(score), _ptr(kept_idx), _ptr(ws), nbytes, _stream(stream))
     if check:
         _raise(st, "ahakv_select")
     return st
@@ -276,8 +289,7 @@ def ahakv_select(p: Params, score, kept_idx, ws=None, ws_bytes: int | None = Non
 
 def ahakv_compact(p: Params, k, v, score, kept_idx, k_out, v_out, score_out, stream=None,
                   check: bool = True) -> int:
-    cp = p.c()
-    st = lib().ahakv_compact(ctypes.byref(cp), _ptr(k), _ptr(v), _ptr(score), _ptr(kept_idx), _ptr(k_out),
+    st = lib().ahakv_compact(p.ref(), _ptr(k), _ptr(v), _ptr(score), _ptr(kept_idx), _ptr(k_out),
                              _ptr(v_out), _ptr(score_out), _stream(stream))
     if check:
         _raise(st, "ahakv_compact")
@@ -286,9 +298,8 @@ def ahakv_compact(p: Params, k, v, score, kept_idx, k_out, v_out, score_out, str
 
 def ahakv_evict(p: Params, q_obs, k, v, score_prev, k_out, v_out, score_out, kept_idx, ws,
                 ws_bytes: int | None = None, stream=None, check: bool = True) -> int:
-    cp = p.c()
-    nbytes = ws.numel() * ws.element_size() if ws_bytes is None else ws_bytes
-    st = lib().ahakv_evict(ctypes.byref(cp), _ptr(q_obs), _ptr(k), _ptr(v), _ptr(score_prev), _ptr(k_out),
+    nbytes = ws.nbytes if ws_bytes is None else ws_bytes
+    st = lib().ahakv_evict(p.ref(), _ptr(q_obs), _ptr(k), _ptr(v), _ptr(score_prev), _ptr(k_out),
                            _ptr(v_out), _ptr(score_out), _ptr(kept_idx), _ptr(ws), nbytes, _stream(stream))
     if check:
         _raise(st, "ahakv_evict")
@@ -298,9 +309,8 @@ def ahakv_evict(p: Params, q_obs, k, v, score_prev, k_out, v_out, score_out, kep
 def ahakv_evict_head_budgets(p: Params, head_budget, q_obs, k, v, score_prev, k_out, v_out, score_out, kept_idx, ws,
                              ws_bytes: int | None = None, stream=None, check: bool = True) -> int:
     """``ahakv_evict`` with ``head_budget`` [B,Hkv] int32 on the device: a budget per (sequence, KV head)."""
-    cp = p.c()
-    nbytes = ws.numel() * ws.element_size() if ws_bytes is None else ws_bytes
-    st = lib().ahakv_evict_head_budgets(ctypes.byref(cp), _ptr(head_budget), _ptr(q_obs), _ptr(k), _ptr(v),
+    nbytes = ws.nbytes if ws_bytes is None else ws_bytes
+    st = lib().ahakv_evict_head_budgets(p.ref(), _ptr(head_budget), _ptr(q_obs), _ptr(k), _ptr(v),
                                         _ptr(score_prev), _ptr(k_out), _ptr(v_out), _ptr(score_out), _ptr(kept_idx),
                                         _ptr(ws), nbytes, _stream(stream))
     if check:
@@ -311,10 +321,9 @@ def ahakv_evict_head_budgets(p: Params, head_budget, q_obs, k, v, score_prev, k_
 def ahakv_evict_ragged(p: Params, seqs, q_obs, k, v, score_prev, k_out, v_out, score_out, kept_idx, ws,
                        ws_bytes: int | None = None, stream=None, check: bool = True) -> int:
     """``seqs``: one (n_ctx, budget, n_total) triple per sequence."""
-    cp = p.c()
     arr = (CSeq * len(seqs))(*[CSeq(int(a), int(b), int(c)) for a, b, c in seqs])
-    nbytes = ws.numel() * ws.element_size() if ws_bytes is None else ws_bytes
-    st = lib().ahakv_evict_ragged(ctypes.byref(cp), arr, _ptr(q_obs), _ptr(k), _ptr(v), _ptr(score_prev), _ptr(k_out),
+    nbytes = ws.nbytes if ws_bytes is None else ws_bytes
+    st = lib().ahakv_evict_ragged(p.ref(), arr, _ptr(q_obs), _ptr(k), _ptr(v), _ptr(score_prev), _ptr(k_out),
                                   _ptr(v_out), _ptr(score_out), _ptr(kept_idx), _ptr(ws), nbytes, _stream(stream))
     if check:
         _raise(st, "ahakv_evict_ragged")

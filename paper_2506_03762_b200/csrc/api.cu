@@ -133,6 +133,25 @@ ahakv_status make_plan(const ahakv_params* p, Plan* pl, const int64_t* obs_pos) 
   return AHAKV_OK;
 }
 
+// The plan of a call.  A thread that repeats a call finds the plan of its last one (comparing 136 bytes instead of 1 us of
+// logarithms and tables); a plan is a pure function of the parameters.
+static ahakv_status plan_for(const ahakv_params* p, const Plan** out) {
+  static thread_local ahakv_params last;
+  static thread_local Plan plan;
+  static thread_local bool valid = false;
+  if (p && valid && std::memcmp(p, &last, sizeof(last)) == 0) {
+    *out = &plan;
+    return AHAKV_OK;
+  }
+  valid = false;
+  const ahakv_status rc = make_plan(p, &plan);
+  if (rc) return rc;
+  std::memcpy(&last, p, sizeof(last));
+  valid = true;
+  *out = &plan;
+  return AHAKV_OK;
+}
+
 static bool aligned16(const void* p) { return ((uintptr_t)p & 15) == 0; }
 
 static ahakv_status check_ws(const Plan& pl, void* ws, size_t ws_bytes) {
@@ -179,9 +198,9 @@ using namespace ahakv;
 extern "C" {
 
 size_t ahakv_workspace_bytes(const ahakv_params* p) {
-  Plan pl;
-  if (make_plan(p, &pl) != AHAKV_OK) return 0;
-  return pl.ws_total;
+  const Plan* plan;
+  if (plan_for(p, &plan) != AHAKV_OK) return 0;
+  return plan->ws_total;
 }
 
 double ahakv_lambda(int64_t n_total, int32_t budget, int32_t head_dim) {
@@ -192,9 +211,11 @@ double ahakv_lambda(int64_t n_total, int32_t budget, int32_t head_dim) {
 static ahakv_status score_impl(const ahakv_params* p, const int64_t* obs_pos, const void* q_obs, const void* k,
                                const void* v, const float* score_prev, float* score, void* ws, size_t ws_bytes,
                                cudaStream_t st) {
-  Plan pl;
-  ahakv_status rc = make_plan(p, &pl, obs_pos);
+  Plan own;
+  const Plan* plan = &own;
+  ahakv_status rc = obs_pos ? make_plan(p, &own, obs_pos) : plan_for(p, &plan);
   if (rc) return rc;
+  const Plan& pl = *plan;
   const bool prior = (pl.flags & AHAKV_FLAG_VALUE_PRIOR) != 0;
   if (!q_obs || !k || !score || (prior && !v)) return AHAKV_ERR_INVALID_ARG;
   if (!aligned16(q_obs) || !aligned16(k) || (v && !aligned16(v)) || !aligned16(score) ||
@@ -274,9 +295,10 @@ ahakv_status ahakv_score_full_causal(const ahakv_params* p, const void* q_all, c
 
 ahakv_status ahakv_score_step(const ahakv_params* p, const void* q_t, const void* k, const float* score_prev,
                               float* score, ahakv_stream_t stream) {
-  Plan pl;
-  ahakv_status rc = make_plan(p, &pl);
+  const Plan* plan;
+  ahakv_status rc = plan_for(p, &plan);
   if (rc) return rc;
+  const Plan& pl = *plan;
   if (pl.r != 1) return AHAKV_ERR_INVALID_ARG;
   if (!q_t || !k || !score || !aligned16(q_t) || !aligned16(k) || !aligned16(score) ||
       (score_prev && !aligned16(score_prev)))
@@ -287,9 +309,10 @@ ahakv_status ahakv_score_step(const ahakv_params* p, const void* q_t, const void
 
 ahakv_status ahakv_step_slots(const ahakv_params* p, const void* q_t, const void* k_t, const void* v_t, void* k, void* v,
                               float* score, int32_t* pos, int32_t* free_slot, ahakv_stream_t stream) {
-  Plan pl;
-  ahakv_status rc = make_plan(p, &pl);
+  const Plan* plan;
+  ahakv_status rc = plan_for(p, &plan);
   if (rc) return rc;
+  const Plan& pl = *plan;
   if (pl.r != 1 || pl.n != pl.Bud + 1) return AHAKV_ERR_INVALID_ARG;
   if (!q_t || !k_t || !v_t || !k || !v || !score || !pos || !free_slot || !aligned16(q_t) || !aligned16(k_t) ||
       !aligned16(v_t) || !aligned16(k) || !aligned16(v) || ((uintptr_t)score & 3) || ((uintptr_t)pos & 3) ||
@@ -302,9 +325,10 @@ ahakv_status ahakv_step_slots(const ahakv_params* p, const void* q_t, const void
 
 ahakv_status ahakv_compact_inplace(const ahakv_params* p, void* k, void* v, float* score, const int32_t* kept_idx,
                                    ahakv_stream_t stream) {
-  Plan pl;
-  ahakv_status rc = make_plan(p, &pl);
+  const Plan* plan;
+  ahakv_status rc = plan_for(p, &plan);
   if (rc) return rc;
+  const Plan& pl = *plan;
   if (!k || !v || !kept_idx || !aligned16(k) || !aligned16(v) || ((uintptr_t)kept_idx & 3) ||
       (score && ((uintptr_t)score & 3)))
     return AHAKV_ERR_INVALID_ARG;
@@ -312,16 +336,17 @@ ahakv_status ahakv_compact_inplace(const ahakv_params* p, void* k, void* v, floa
 }
 
 size_t ahakv_entropy_workspace_bytes(const ahakv_params* p) {
-  Plan pl;
-  if (make_plan(p, &pl) != AHAKV_OK) return 0;
-  return entropy_scratch_bytes(pl);
+  const Plan* plan;
+  if (plan_for(p, &plan) != AHAKV_OK) return 0;
+  return entropy_scratch_bytes(*plan);
 }
 
 ahakv_status ahakv_row_entropy(const ahakv_params* p, const void* q_obs, const void* k, float* entropy, void* ws,
                                size_t ws_bytes, ahakv_stream_t stream) {
-  Plan pl;
-  ahakv_status rc = make_plan(p, &pl);
+  const Plan* plan;
+  ahakv_status rc = plan_for(p, &plan);
   if (rc) return rc;
+  const Plan& pl = *plan;
   if (!q_obs || !k || !entropy || !aligned16(q_obs) || !aligned16(k) || ((uintptr_t)entropy & 3))
     return AHAKV_ERR_INVALID_ARG;
   if (!ws || ((uintptr_t)ws & 255) != 0 || ws_bytes < entropy_scratch_bytes(pl)) return AHAKV_ERR_WORKSPACE;
@@ -330,9 +355,10 @@ ahakv_status ahakv_row_entropy(const ahakv_params* p, const void* q_obs, const v
 
 ahakv_status ahakv_select(const ahakv_params* p, const float* score, int32_t* kept_idx, void* ws,
                           size_t ws_bytes, ahakv_stream_t stream) {
-  Plan pl;
-  ahakv_status rc = make_plan(p, &pl);
+  const Plan* plan;
+  ahakv_status rc = plan_for(p, &plan);
   if (rc) return rc;
+  const Plan& pl = *plan;
   if (!score || !kept_idx || !aligned16(score) || ((uintptr_t)kept_idx & 3)) return AHAKV_ERR_INVALID_ARG;
   (void)ws; (void)ws_bytes;                    // selection works in shared memory: no scratch is needed
   return launch_select(pl, score, kept_idx, (cudaStream_t)stream);
@@ -341,9 +367,10 @@ ahakv_status ahakv_select(const ahakv_params* p, const float* score, int32_t* ke
 ahakv_status ahakv_compact(const ahakv_params* p, const void* k, const void* v, const float* score,
                            const int32_t* kept_idx, void* k_out, void* v_out, float* score_out,
                            ahakv_stream_t stream) {
-  Plan pl;
-  ahakv_status rc = make_plan(p, &pl);
+  const Plan* plan;
+  ahakv_status rc = plan_for(p, &plan);
   if (rc) return rc;
+  const Plan& pl = *plan;
   if (!k || !v || !kept_idx || !k_out || !v_out) return AHAKV_ERR_INVALID_ARG;
   if ((score == nullptr) != (score_out == nullptr)) return AHAKV_ERR_INVALID_ARG;
   if (!aligned16(k) || !aligned16(v) || !aligned16(k_out) || !aligned16(v_out) || ((uintptr_t)kept_idx & 3))
@@ -354,9 +381,10 @@ ahakv_status ahakv_compact(const ahakv_params* p, const void* k, const void* v, 
 static ahakv_status evict_impl(const ahakv_params* p, const int32_t* budgets, const void* q_obs, const void* k,
                                const void* v, const float* score_prev, void* k_out, void* v_out, float* score_out,
                                int32_t* kept_idx, void* ws, size_t ws_bytes, ahakv_stream_t stream) {
-  Plan pl;
-  ahakv_status rc = make_plan(p, &pl);
+  const Plan* plan;
+  ahakv_status rc = plan_for(p, &plan);
   if (rc) return rc;
+  const Plan& pl = *plan;
   if (!q_obs || !k || !v || !k_out || !v_out || !kept_idx) return AHAKV_ERR_INVALID_ARG;
   if (!aligned16(q_obs) || !aligned16(k) || !aligned16(v) || !aligned16(k_out) || !aligned16(v_out) ||
       ((uintptr_t)kept_idx & 3) || (score_prev && !aligned16(score_prev)))
