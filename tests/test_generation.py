@@ -332,3 +332,38 @@ def test_score_step_at_its_largest_size():
     # one more key is one too many
     p2 = ab.Params(B, Hq, Hkv, d, n + 1, 1, 64, 4096, dtype=ab.F16, n_total=50000, flags=0)
     assert ab.ahakv_score_step(p2, q, k, prev, got, check=False) == ab.ERR_UNSUPPORTED
+
+
+@pytest.mark.parametrize("B,Hq,Hkv,d,Bud,Br,dtype_name", [
+    (1, 1, 1, 128, 511, 16, "F16"), (1, 4, 1, 64, 512, 0, "BF16"), (1, 2, 2, 128, 1023, 64, "F16"),   # 1, 2 and 4 CTAs a head
+    (2, 8, 1, 128, 2051, 32, "BF16"), (1, 6, 2, 64, 1030, 8, "F32"), (1, 16, 1, 128, 2100, 5, "F16"),
+    (80, 2, 2, 64, 9, 1, "F16")])                                          # one CTA a head, a handful of keys
+def test_step_and_slots_agree_when_a_head_is_split_over_ctas(B, Hq, Hkv, d, Bud, Br, dtype_name):
+    """The ordered step and the slot step on the same cache (slots in position order) are the same arithmetic on the same
+    split of the keys: equal scores bit for bit, and the slot declared free is the row the ordered step drops."""
+    from paper_2506_03762_b200 import binding as ab
+    dtype, n, N0 = getattr(ab, dtype_name), Bud + 1, 9000
+    g = torch.Generator().manual_seed(Bud)
+    dt = _dt(ab, dtype)
+    q, kt, vt = (torch.randn((B, h, 1, d), generator=g).to(dt).to(DEV) for h in (Hq, Hkv, Hkv))
+    k, v = (torch.randn((B, Hkv, n, d), generator=g).to(dt).to(DEV) for _ in range(2))
+    f = torch.rand((B, Hkv, n), generator=g).to(DEV)
+    f[..., Bud] = 0.0
+    k_ord, v_ord, f_ord = k.clone(), v.clone(), f.clone()
+    k_ord[:, :, Bud], v_ord[:, :, Bud] = kt[:, :, 0], vt[:, :, 0]
+    p = ab.Params(B, Hq, Hkv, d, n, 1, Br, Bud, dtype=dtype, n_total=N0 + n, flags=0)
+    ab.ahakv_score_step(p, q, k_ord, f_ord, f_ord)
+    idx = torch.empty((B, Hkv, Bud), dtype=torch.int32, device=DEV)
+    ab.ahakv_select(p, f_ord, idx)
+    pos = (torch.arange(n, dtype=torch.int32) + N0).expand(B, Hkv, n).contiguous().to(DEV)
+    pos[..., Bud] = -1
+    free = torch.full((B, Hkv), Bud, dtype=torch.int32, device=DEV)
+    ab.ahakv_step_slots(p, q, kt, vt, k, v, f, pos, free)
+    assert torch.equal(f, f_ord) and torch.equal(k, k_ord) and torch.equal(v, v_ord)
+    dropped = torch.ones((B, Hkv, n), dtype=torch.bool, device=DEV).scatter(-1, idx.long(), False).int().argmax(-1)
+    assert torch.equal(dropped.int(), free)
+    assert torch.equal(pos == -1, torch.nn.functional.one_hot(free.long(), n).bool())
+    # moving the rows: the result is the gather
+    want = k_ord.gather(2, idx.long().unsqueeze(-1).expand(-1, -1, -1, d)), f_ord.gather(2, idx.long())
+    ab.ahakv_compact_inplace(p, k_ord, v_ord, f_ord, idx)
+    assert torch.equal(k_ord[:, :, :Bud], want[0]) and torch.equal(f_ord[..., :Bud], want[1])
