@@ -69,6 +69,15 @@ ahakv_status launch_compact_inplace(const Plan& pl, void* k, void* v, float* sco
 // Row entropy of the SG-softmax (entropy.cu): out [B, Hq, r]; `scratch` of entropy_scratch_bytes().
 size_t entropy_scratch_bytes(const Plan& pl);
 ahakv_status launch_entropy(const Plan& pl, const void* q, const void* k, void* scratch, float* out, cudaStream_t st);
+// The same on the tensor cores (score_stream.cu; plans with use_tc).
+size_t entropy_tc_scratch_bytes(const Plan& pl);
+ahakv_status launch_entropy_tc(const Plan& pl, const void* q, const void* k, void* scratch, float* out, cudaStream_t st);
+// Accumulation over every causal row on the tensor cores (score_stream.cu; plans with use_tc).  Leaves *n_slots partial sums
+// per head in *slots (`sums` if there is one: [B * Hkv][n]); `pool` is scratch, 256-byte aligned.
+bool causal_tc_fits(const Plan& pl, size_t pool_bytes);
+ahakv_status launch_causal_tc(const Plan& pl, int scale_mode, double fixed, long long first_cached, const void* q, const long long qs[3],
+                              const void* k, float* pool, size_t pool_bytes, float* sums, const float** slots, int* n_slots,
+                              int* status, cudaStream_t st);
 ahakv_status launch_vnorm(const Plan& pl, const void* v, float* nu, cudaStream_t st);
 // `slots` partial scores per head (row blocks, or query heads when pooling by maximum) are combined here.
 ahakv_status launch_refine(const Plan& pl, const float* s_raw, const float* nu, const float* score_prev,

@@ -126,8 +126,8 @@ ahakv_status make_plan(const ahakv_params* p, Plan* pl, const int64_t* obs_pos) 
   o.off_sync = off;    off += align_up(units * rb_slots * 2 * sizeof(int), 256);
   o.off_final = off;   off += align_up(units * rb_slots * (o.use_tc ? 128 : o.R) * sizeof(float2), 256);
   o.off_sraw = off;    off += align_up(units * rb_slots * o.n * sizeof(float), 256);
-  o.off_nu = off;      off += align_up(units * o.n * sizeof(float), 256);
   o.off_partial = off; off += align_up(units * rb_slots * o.n_blk * (o.use_tc ? 128 : o.R) * sizeof(float2), 256);
+  o.off_nu = off;      off += align_up(units * o.n * sizeof(float), 256);
   o.off_score = off;   off += align_up(units * o.n * sizeof(float), 256);
   o.ws_total = off;
   return AHAKV_OK;
@@ -177,7 +177,7 @@ static ahakv_status queue_raw_score(const Plan& pl, const void* q, const void* k
     if (cudaMemsetAsync(at<char>(ws, pl.off_status), 0xff, pl.off_sraw - pl.off_status, st) != cudaSuccess)
       return AHAKV_ERR_CUDA;
     // the kernel skips the tiles that no observation row sees: their raw score is zero
-    if (pl.n_eff != pl.n && cudaMemsetAsync(s_raw, 0, pl.off_nu - pl.off_sraw, st) != cudaSuccess) return AHAKV_ERR_CUDA;
+    if (pl.n_eff != pl.n && cudaMemsetAsync(s_raw, 0, pl.off_partial - pl.off_sraw, st) != cudaSuccess) return AHAKV_ERR_CUDA;
     rc = launch_score_tc(pl, q, k, prior ? v : nullptr, s_raw, nu, at<float>(ws, pl.off_partial), final_off,
                          at<int>(ws, pl.off_sync), at<int>(ws, pl.off_status), st);
     profile_mark(prof, 1, st);
@@ -266,8 +266,25 @@ ahakv_status ahakv_score_full_causal(const ahakv_params* p, const void* q_all, c
     pc.q_stride[1] = (int64_t)p->n_ctx * p->head_dim;
     pc.q_stride[0] = (int64_t)p->n_q_heads * p->n_ctx * p->head_dim;
   }
-  pc.flags = p->flags & ~(uint32_t)AHAKV_FLAG_VALUE_PRIOR;     // the prior multiplies the finished sum, once
   float* acc = at<float>(ws, full.off_score);                  // running sum over the passes, [B, Hkv, n]
+  float* nu = nullptr;
+  if (prior) {
+    nu = at<float>(ws, full.off_nu);
+    if ((rc = launch_vnorm(full, v, nu, st))) return rc;
+  }
+  const size_t pool = full.off_nu - full.off_final;            // room for row statistics
+  if (full.use_tc && causal_tc_fits(full, pool)) {
+    long long qs[3];
+    if (!resolve_strides(pc.q_stride, qs, full.Hq, full.n, full.d, full.es)) return AHAKV_ERR_INVALID_ARG;
+    const double fixed = p->scale_mode == AHAKV_SCALE_FIXED ? (double)p->scale : eq12((double)p->n_total, (double)p->budget, p->head_dim);
+    const float* slots = nullptr;
+    int n_slots = 1;
+    if ((rc = launch_causal_tc(full, p->scale_mode, fixed, p->n_total - p->n_ctx, q_all, qs, k, at<float>(ws, full.off_final), pool, acc,
+                               &slots, &n_slots, at<int>(ws, full.off_status), st)))
+      return rc;
+    return launch_refine(full, slots, nu, score_prev, score, n_slots, st);
+  }
+  pc.flags = p->flags & ~(uint32_t)AHAKV_FLAG_VALUE_PRIOR;     // the prior multiplies the finished sum, once
   const int R = p->obs_window, n = p->n_ctx;
   const long long first_cached = p->n_total - p->n_ctx;
   int64_t pos[kMaxRows];
@@ -283,14 +300,7 @@ ahakv_status ahakv_score_full_causal(const ahakv_params* p, const void* q_all, c
     if ((rc = launch_refine(pl, at<float>(ws, pl.off_sraw), nullptr, c0 == 0 ? nullptr : acc, acc, score_slots(pl), st)))
       return rc;
   }
-  float* nu = nullptr;
-  if (prior) {
-    nu = at<float>(ws, full.off_nu);
-    if ((rc = launch_vnorm(full, v, nu, st))) return rc;
-  }
-  Plan one = full;
-  one.group_max = 0;
-  return launch_refine(one, acc, nu, score_prev, score, 1, st);
+  return launch_refine(full, acc, nu, score_prev, score, 1, st);
 }
 
 ahakv_status ahakv_score_step(const ahakv_params* p, const void* q_t, const void* k, const float* score_prev,

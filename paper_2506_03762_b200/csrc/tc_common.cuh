@@ -235,6 +235,76 @@ __device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
   return d;
 }
 
+// ---- softmax pieces -------------------------------------------------------------------------------------
+// One 32-key chunk of a row: fold it into the running pair (M, Z) with Z = sum of 2^{c w - M}.
+// M is a shift, not necessarily the maximum: any value within 2^kShiftSlack of the largest logit seen
+// keeps every term finite, so the exponentials of a chunk are taken against the shift the row already
+// has, and their sum tells whether that was sound: below 2^kShiftSlack, no term outran the shift by more
+// than the slack.  Only otherwise (or when the row has no shift yet) is the chunk's maximum looked for and
+// the chunk redone against it.
+constexpr float kAcceptBelow = 18446744073709551616.f;   // 2^64
+
+// Sum of 2^{c v + neg} over 32 values.
+__device__ __forceinline__ float exp_sum32(const float* v, float c, float neg) {
+  const uint64_t c2 = pack2(c, c), neg2 = pack2(neg, neg);
+  uint64_t za = pack2(0.f, 0.f), zb = pack2(0.f, 0.f);
+#pragma unroll
+  for (int t = 0; t < 32; t += 4) {
+    float x0, x1, x2, x3;
+    unpack2(fma2(pack2(v[t], v[t + 1]), c2, neg2), x0, x1);
+    unpack2(fma2(pack2(v[t + 2], v[t + 3]), c2, neg2), x2, x3);
+    za = add2(za, pack2(fast_exp2(x0), fast_exp2(x1)));
+    zb = add2(zb, pack2(fast_exp2(x2), fast_exp2(x3)));
+  }
+  float z0, z1;
+  unpack2(add2(za, zb), z0, z1);
+  return z0 + z1;
+}
+
+__device__ __forceinline__ void fold_chunk(const uint32_t* r, bool full, int j_first, int last, float c, float& M,
+                                           float& Z) {
+  float v[32];
+#pragma unroll
+  for (int t = 0; t < 32; ++t) v[t] = __uint_as_float(r[t]);
+  if (!full) {
+#pragma unroll
+    for (int t = 0; t < 32; ++t)
+      if (j_first + t > last) v[t] = -INFINITY;
+  }
+  if (M > -INFINITY) {
+    const float z = exp_sum32(v, c, -M);
+    if (z < kAcceptBelow) {                          // an overflow or a NaN fails this test too
+      Z += z;
+      return;
+    }
+  }
+  float mx0 = fmaxf(v[0], v[1]), mx1 = fmaxf(v[2], v[3]);
+#pragma unroll
+  for (int t = 4; t < 32; t += 4) {
+    mx0 = fmaxf(mx0, fmaxf(v[t], v[t + 1]));
+    mx1 = fmaxf(mx1, fmaxf(v[t + 2], v[t + 3]));
+  }
+  const float mx = fmaxf(mx0, mx1) * c;
+  if (mx > -INFINITY) {                              // first visible keys of the row, or the shift fell behind
+    Z = (M > -INFINITY ? Z * fast_exp2(M - mx) : 0.f) + exp_sum32(v, c, -mx);
+    M = mx;
+  }
+}
+
+// Several log2 sums into one, in order.
+template <int N>
+__device__ __forceinline__ void merge_logs(const float (&e)[N], float& M, float& Z) {
+  float m = M;
+#pragma unroll
+  for (int t = 0; t < N; ++t) m = fmaxf(m, e[t]);
+  if (m > -INFINITY) {
+    float z = Z > 0.f ? Z * fast_exp2(M - m) : 0.f;
+#pragma unroll
+    for (int t = 0; t < N; ++t) z += fast_exp2(e[t] - m);   // 2^{-inf} = 0 for what is not there
+    Z = z; M = m;
+  }
+}
+
 
 // ---- host: tensor maps ----------------------------------------------------------------------------------
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,

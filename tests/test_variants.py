@@ -147,3 +147,34 @@ def test_full_causal_accumulation_matches_the_oracle(B, Hq, Hkv, d, n, R, dtype_
     if Hq != Hkv:                                                 # pooling by maximum does not split into passes
         pg = ab.Params(B, Hq, Hkv, d, n, R, 16, 100, dtype=dtype, flags=ab.FLAG_GROUP_MAX)
         assert ab.ahakv_score_full_causal(pg, q, k, v, None, score, ws, check=False) == ab.ERR_UNSUPPORTED
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("B,Hq,Hkv,d,n,R,mode", [
+    (1, 1, 1, 64, 128, 128, 1), (1, 2, 2, 128, 129, 1, 0), (1, 16, 2, 64, 257, 32, 1), (1, 8, 1, 128, 640, 16, 2),   # few heads: rows and keys in parts
+    (3, 7, 1, 64, 391, 32, 1), (1, 1, 1, 128, 1500, 256, 1), (2, 12, 4, 128, 1100, 50, 1)])
+def test_full_causal_tiles_and_parts(B, Hq, Hkv, d, n, R, mode):
+    """The tensor-core path at the edges of its 128-row tiles, with query heads in several passes and runs in several parts,
+    against Eq. 2-3 in float64 on the same inputs.  16-bit products are exact, sums FP32: the exponents (up to ~50 in log2
+    units) carry a few 1e-6, ex2 2 ulp, 1e-4 leaves room for both and for the sum over thousands of rows."""
+    from paper_2506_03762_b200 import binding as ab
+    q, k, v = _gpu_case(B, Hq, Hkv, d, n, ab.F16, seed=n + R)
+    p = ab.Params(B, Hq, Hkv, d, n, R, 0, 70, dtype=ab.F16, n_total=n + 300, scale_mode=mode, scale=0.06, flags=0)
+    ws = ab.alloc_workspace(p, "cuda")
+    score = torch.empty((B, Hkv, n), dtype=torch.float32, device="cuda")
+    ab.ahakv_score_full_causal(p, q, k, v, None, score, ws)
+    assert ab.ahakv_last_device_status(ws) == ab.OK
+    G = Hq // Hkv
+    if mode == 0:
+        lam = torch.full((n,), float(torch.tensor(0.06, dtype=torch.float32)), dtype=torch.float64)
+    elif mode == 1:
+        lam = torch.tensor([ab.ahakv_lambda(300 + i + 1, 70, d) for i in range(n)], dtype=torch.float64)
+    else:
+        lam = torch.full((n,), ab.ahakv_lambda(n + 300, 70, d), dtype=torch.float64)
+    w = q.double() @ k.double().repeat_interleave(G, 1).transpose(-1, -2) * lam.cuda().view(n, 1)
+    a = w.masked_fill(~torch.ones((n, n), dtype=torch.bool, device="cuda").tril(), float("-inf")).softmax(-1).sum(2)
+    want = a.view(B, Hkv, G, n).mean(2)
+    assert torch.allclose(score.double(), want, rtol=1e-4, atol=1e-7)
+    first = score.clone()
+    ab.ahakv_score_full_causal(p, q, k, v, None, score, ws)
+    assert torch.equal(first, score)                              # fixed reduction order
