@@ -759,10 +759,12 @@ void score_tc_test_hooks(long long wait_ns, int withhold) {
 
 // How many runs a row block's key tiles are cut into.  A run boundary costs about as much as a tile visit (a Q tile to
 // load, statistics to hand over, constants to pick up), and the runs of all row blocks are dealt to the CTAs in rounds:
-// the number that makes rounds x (tiles of a run + 1) smallest, with runs of at most 8 tiles where the keys of all heads
-// do not fit in half of L2 (what lies between the two passes of a run, two grid rounds, has to), 24 otherwise.
-static int runs_per_row_block(long long units, int n_blk, int slots) {
-  const int longest = units * n_blk > 2048 ? 8 : 24;
+// the number that makes rounds x (tiles of a run + 1) smallest.  Runs have at most 8 tiles where the keys do not stay in
+// L2 (126 MB) as a whole: what lies between the two passes of a run, about two grid rounds, has to.  Where they do (96 MB,
+// with room for what else passes through) they have up to 16: one long request of 70001 tokens x 4 heads 138 -> 88 us a
+// call against 8, a decode round 94 -> 92.5; 12 and 24 are slower or no better.
+static int runs_per_row_block(long long units, int n_blk, int slots, long long key_bytes) {
+  const int longest = key_bytes > (96LL << 20) ? 8 : 16;
   int best = n_blk;
   long long best_cost = -1;
   for (int rpu = (n_blk + longest - 1) / longest; rpu <= n_blk; ++rpu) {
@@ -797,7 +799,7 @@ ahakv_status launch_score_tc(const Plan& pl, const void* q, const void* k, const
   a.D = pl.d;
   for (int i = 0; i < kMaxRows; ++i) a.last[i] = pl.last[i];
   a.min_last = pl.last[0];
-  a.rpu = runs_per_row_block(units, a.n_blk, slots);
+  a.rpu = runs_per_row_block(units, a.n_blk, slots, (long long)pl.B * pl.Hkv * a.n_blk * kKeyTile * pl.d * pl.es);
   a.CH = (a.n_blk + a.rpu - 1) / a.rpu;
   a.rpu = (a.n_blk + a.CH - 1) / a.CH;
   a.n_runs = units * a.rpu;
