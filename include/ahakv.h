@@ -94,7 +94,7 @@ double ahakv_lambda(int64_t n_total, int32_t budget, int32_t head_dim);
  * Observation row i sits at logical position n_total - r + i and sees cache rows 0 .. n - r + i.
  * score_prev: nullable, [B,Hkv,n] float32.  score: [B,Hkv,n] float32 out.
  * v may be NULL when the value prior is off.
- * Resources: for 16-bit inputs and n_ctx >= 128 the scoring kernel is launched cooperatively with one CTA per SM
+ * Resources: for 16-bit inputs and n_ctx >= 128 the scoring kernel is launched with one CTA per SM
  * and takes each SM's whole tensor memory (512 columns) and nearly all of its shared memory for its duration.  A
  * kernel of the caller's that allocates tensor memory and runs concurrently on another stream can be held up
  * until it ends, and holds it up the same way: the allocation is the hardware's, and the time it waits does not
@@ -116,10 +116,10 @@ ahakv_status ahakv_score_rows(const ahakv_params* p, const int64_t* obs_pos, con
 
 /* Accumulation over ALL query rows (Section 4.1, Eq. 2-3: S_j = sum over i >= j of a_ij; the paper's "w/o RA"
  * ablation, and H2O's score when scale_mode is AHAKV_SCALE_FIXED with scale 1/sqrt(d) and the value prior is off).
- * q_all holds a query for every cached row, [B,Hq,n,d] (q_stride describes it otherwise).  The rows are scored
- * obs_window at a time (1 .. 256 / G; ceil(n / obs_window) passes of the kernels of ahakv_score, each over the
- * keys its rows can see), summed, and the value prior and score_prev are applied to the sum.  O(n^2 d) work: this
- * is the cost Recent Accumulation removes.  ws as for ahakv_score with the same parameters.
+ * q_all holds a query for every cached row, [B,Hq,n,d] (q_stride describes it otherwise).  16-bit inputs: two walks over
+ * the causal triangle on the tensor cores; otherwise the rows are scored obs_window at a time (1 .. 256 / G;
+ * ceil(n / obs_window) passes of the kernels of ahakv_score) and summed.  The value prior and score_prev are applied
+ * to the sum.  O(n^2 d) work: this is the cost Recent Accumulation removes.  ws as for ahakv_score with the same parameters.
  * AHAKV_FLAG_GROUP_MAX is not offered here (AHAKV_ERR_UNSUPPORTED). */
 ahakv_status ahakv_score_full_causal(const ahakv_params* p, const void* q_all, const void* k, const void* v,
                                      const float* score_prev, float* score, void* ws, size_t ws_bytes,
@@ -138,8 +138,8 @@ ahakv_status ahakv_score_step(const ahakv_params* p, const void* q_t, const void
 
 /* Compaction in place (Algorithm 1, Generation: K <- K_S, V <- V_S before the next token): rows kept_idx[t] of k,
  * v (and of score, nullable, [B,Hkv,n]) move to rows t; rows from n_keep on are left as they are.  kept_idx is
- * ascending, so rows before the first evicted index are not touched and only the rest is moved.  One CTA per
- * (sequence, KV head), batches staged in shared memory.  The exception to "outputs must not alias inputs". */
+ * ascending, so rows before the first evicted index are not touched and only the rest is moved, in rounds staged in
+ * the registers of a cluster per (sequence, KV head).  The exception to "outputs must not alias inputs". */
 ahakv_status ahakv_compact_inplace(const ahakv_params* p, void* k, void* v, float* score, const int32_t* kept_idx,
                                    ahakv_stream_t stream);
 
@@ -169,7 +169,7 @@ ahakv_status ahakv_step_slots(const ahakv_params* p, const void* q_t, const void
  * observation row of every query head, with a_ij exactly as in ahakv_score (mask, lambda from scale_mode).  A
  * diagnostic: Eq. 10 predicts E[H_i] = ln i - lambda^2 d / 2, and Eq. 12 picks lambda so that this is ln(budget).
  * entropy: [B,Hq,r] float32 out.  ws: ahakv_entropy_workspace_bytes(p) bytes, 256-byte aligned (not the scoring
- * workspace).  Runs on the FP32 pipes (double for float32 inputs); it is not part of the eviction path. */
+ * workspace).  16-bit inputs run on the tensor cores, float32 ones in double; it is not part of the eviction path. */
 size_t ahakv_entropy_workspace_bytes(const ahakv_params* p);
 ahakv_status ahakv_row_entropy(const ahakv_params* p, const void* q_obs, const void* k, float* entropy, void* ws,
                                size_t ws_bytes, ahakv_stream_t stream);

@@ -84,10 +84,12 @@ ahakv_status launch_refine(const Plan& pl, const float* s_raw, const float* nu, 
                            float* score, int slots, cudaStream_t st);
 ahakv_status launch_select(const Plan& pl, const float* score, int32_t* kept_idx, cudaStream_t st);
 // Both steps.  Writes the kept tokens' scores to score_out (nullable) itself when a head fits in a cluster; otherwise leaves
-// the refined scores in `score`.  *score_left says which: null, or `score` for the caller to gather from.
+// the refined scores in `score`.  *score_left says which: null, or `score` for the caller to gather from.  Gathers the kept
+// rows too where they are few (*gathered).
 ahakv_status launch_refine_select(const Plan& pl, const float* s_raw, const float* nu, const float* score_prev,
                                   float* score, float** score_left, float* score_out, int32_t* kept_idx, int slots,
-                                  const int32_t* budgets, cudaStream_t st);
+                                  const int32_t* budgets, const void* k, const void* v, void* k_out, void* v_out, bool* gathered,
+                                  cudaStream_t st);
 ahakv_status launch_compact(const Plan& pl, const void* k, const void* v, const float* score,
                             const int32_t* kept_idx, void* k_out, void* v_out, float* score_out,
                             cudaStream_t st);

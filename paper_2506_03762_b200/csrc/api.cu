@@ -410,13 +410,16 @@ static ahakv_status evict_impl(const ahakv_params* p, const int32_t* budgets, co
   float* score = at<float>(ws, pl.off_score);
   nvtxRangePushA("ahakv: refine + select");
   float* score_left = nullptr;
-  rc = launch_refine_select(pl, s_raw, nu, score_prev, score, &score_left, score_out, kept_idx, score_slots(pl), budgets, st);
+  bool gathered = false;
+  rc = launch_refine_select(pl, s_raw, nu, score_prev, score, &score_left, score_out, kept_idx, score_slots(pl), budgets, k, v, k_out,
+                            v_out, &gathered, st);
   profile_mark(prof, 3, st);
   nvtxRangePop();
   profile_mark(prof, 4, st);
   {
     TraceRange range("ahakv: compact");
-    if (rc == AHAKV_OK) rc = launch_compact(pl, k, v, score_left, kept_idx, k_out, v_out, score_left ? score_out : nullptr, st);
+    if (rc == AHAKV_OK && !gathered)
+      rc = launch_compact(pl, k, v, score_left, kept_idx, k_out, v_out, score_left ? score_out : nullptr, st);
   }
   profile_mark(prof, 5, st);
   return rc;

@@ -78,17 +78,6 @@ __device__ __forceinline__ void put16(A* dst, const uint4& u) {
   for (int e = 0; e < V; ++e) dst[e] = (A)f[e];
 }
 
-template <typename T, int D>
-__device__ __forceinline__ void load_keys(Tiles<Acc<T>, D>& sm, const T* __restrict__ k, const Shape& pl, int b, int h, int j0) {
-  constexpr int V = Vec16<T>::N, PER = D / V;
-  const T* base = k + (long long)b * pl.ks[0] + (long long)h * pl.ks[1];
-#pragma unroll
-  for (int t = threadIdx.x; t < kTile * PER; t += kThreads) {
-    const int row = t / PER, cv = t % PER, j = j0 + row;
-    put16<T>(&sm.k[row][cv * V], j < pl.n ? *reinterpret_cast<const uint4*>(base + (long long)j * pl.ks[2] + cv * V) : make_uint4(0, 0, 0, 0));
-  }
-}
-
 // Chunk `ch` of a head's stacked rows (s = g r + i): thirty-two in a row, or, when the query heads are pooled by maximum,
 // thirty-two of one query head.
 struct Chunk {
@@ -104,21 +93,50 @@ __device__ __forceinline__ Chunk chunk_of(const Shape& pl, int ch) {
   return {g * pl.r + i0, min(kRows, pl.r - i0), ch % per == per - 1};
 }
 
-template <typename T, int D>
-__device__ __forceinline__ void load_rows(Tiles<Acc<T>, D>& sm, const T* __restrict__ q, const Shape& pl, const RowScaleOf<Acc<T>>& cs,
-                                          int b, int h, const Chunk& c) {
-  constexpr int V = Vec16<T>::N, PER = D / V;
-  for (int t = threadIdx.x; t < kRows * PER; t += kThreads) {
-    const int row = t / PER, cv = t % PER, s = c.s0 + row, g = s / pl.r, i = s % pl.r;
-    uint4 u = make_uint4(0, 0, 0, 0);
-    if (row < c.rows)
-      u = *reinterpret_cast<const uint4*>(q + (long long)b * pl.qs[0] + (long long)(h * pl.G + g) * pl.qs[1] + (long long)i * pl.qs[2] + cv * V);
-    put16<T>(&sm.q[row][cv * V], u);
+// The chunk's row constants.  They live in the kernel's parameters, where 32 lanes that read 32 places are served one after
+// the other: four lanes of every warp read one each.
+template <typename A, int D>
+__device__ __forceinline__ void load_constants(Tiles<A, D>& sm, const Shape& pl, const RowScaleOf<A>& cs, const Chunk& c) {
+  const int row = (threadIdx.x >> 5) + 8 * (threadIdx.x & 31);
+  if (row < kRows) {
+    const int i = (c.s0 + row) % pl.r;
+    sm.row_c[row] = cs.c[i];
+    sm.row_last[row] = row < c.rows ? cs.last[i] : -1;
   }
-  if (threadIdx.x < kRows) {
-    const int i = (c.s0 + threadIdx.x) % pl.r;
-    sm.row_c[threadIdx.x] = cs.c[i];
-    sm.row_last[threadIdx.x] = (int)threadIdx.x < c.rows ? cs.last[i] : -1;
+}
+
+// The chunk's query rows and, with kKeys, the tile's keys: all loads first, then the conversions.
+template <typename T, int D, bool kKeys>
+__device__ __forceinline__ void load_operands(Tiles<Acc<T>, D>& sm, const T* __restrict__ q, const T* __restrict__ k, const Shape& pl,
+                                              int b, int h, const Chunk& c, int j0) {
+  constexpr int V = Vec16<T>::N, PER = D / V, NK = kKeys ? kTile * PER / kThreads : 1, NQ = (kRows * PER + kThreads - 1) / kThreads;
+  uint4 ku[NK], qu[NQ];
+  if (kKeys) {
+    const T* base = k + (long long)b * pl.ks[0] + (long long)h * pl.ks[1];
+#pragma unroll
+    for (int e = 0; e < NK; ++e) {
+      const int t = threadIdx.x + e * kThreads, j = j0 + t / PER;
+      ku[e] = j < pl.n ? *reinterpret_cast<const uint4*>(base + (long long)j * pl.ks[2] + t % PER * V) : make_uint4(0, 0, 0, 0);
+    }
+  }
+#pragma unroll
+  for (int e = 0; e < NQ; ++e) {
+    const int t = threadIdx.x + e * kThreads, row = t / PER, s = c.s0 + row, g = s / pl.r, i = s - g * pl.r;
+    qu[e] = make_uint4(0, 0, 0, 0);
+    if (row < c.rows)
+      qu[e] = *reinterpret_cast<const uint4*>(q + (long long)b * pl.qs[0] + (long long)(h * pl.G + g) * pl.qs[1] + (long long)i * pl.qs[2] + t % PER * V);
+  }
+  if (kKeys) {
+#pragma unroll
+    for (int e = 0; e < NK; ++e) {
+      const int t = threadIdx.x + e * kThreads;
+      put16<T>(&sm.k[t / PER][t % PER * V], ku[e]);
+    }
+  }
+#pragma unroll
+  for (int e = 0; e < NQ; ++e) {
+    const int t = threadIdx.x + e * kThreads;
+    if (t < kRows * PER) put16<T>(&sm.q[t / PER][t % PER * V], qu[e]);
   }
 }
 
@@ -189,15 +207,20 @@ simt_row_stats(const T* __restrict__ q, const T* __restrict__ k, float2* __restr
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, kw = warp & (kKeyWarps - 1), rw = warp / kKeyWarps;
   const int row = 16 * rw + (lane >> 2);
   const auto key = [=](int x) { return 16 * kw + 8 * (x >> 1) + 2 * (lane & 3) + (x & 1); };   // this thread's four keys
+  load_constants(sm, pl, cs, chunk_of(pl, 0));
   griddep_wait();
   griddep_launch();
   if (unit == 0 && blockIdx.x == 0 && threadIdx.x == 0) *status = 0;
-  load_keys<T, D>(sm, k, pl, b, h, j0);
   const int chunks = n_chunks(pl);
   for (int ch = 0; ch < chunks; ++ch) {
     const Chunk c = chunk_of(pl, ch);
-    if (ch > 0) __syncthreads();
-    load_rows<T, D>(sm, q, pl, cs, b, h, c);
+    if (ch > 0) {
+      __syncthreads();
+      load_constants(sm, pl, cs, c);
+      load_operands<T, D, false>(sm, q, k, pl, b, h, c, j0);
+    } else {
+      load_operands<T, D, true>(sm, q, k, pl, b, h, c, j0);
+    }
     __syncthreads();
     A acc[4][2];
     dot_16x16<D>(sm, 16 * kw, 16 * rw, acc);
@@ -282,13 +305,18 @@ simt_column_sums(const T* __restrict__ q, const T* __restrict__ k, const T* __re
   const auto key = [=](int x) { return 16 * kw + 8 * (x >> 1) + 2 * (lane & 3) + (x & 1); };   // this thread's four keys
   // The inputs were there before the statistics kernel began; only its statistics have to be waited for (and nothing
   // may be written before: the kernel that reads the last call's scores may still run).
-  load_keys<T, D>(sm, k, pl, b, h, j0);
+  load_constants(sm, pl, cs, chunk_of(pl, 0));
   const int chunks = n_chunks(pl);
   float sum[4] = {}, best = 0.f;
   for (int ch = 0; ch < chunks; ++ch) {
     const Chunk c = chunk_of(pl, ch);
-    if (ch > 0) __syncthreads();
-    load_rows<T, D>(sm, q, pl, cs, b, h, c);
+    if (ch > 0) {
+      __syncthreads();
+      load_constants(sm, pl, cs, c);
+      load_operands<T, D, false>(sm, q, k, pl, b, h, c, j0);
+    } else {
+      load_operands<T, D, true>(sm, q, k, pl, b, h, c, j0);
+    }
     __syncthreads();
     A acc[4][2];
     dot_16x16<D>(sm, 16 * kw, 16 * rw, acc);

@@ -38,6 +38,10 @@ struct SelectArgs {
   float* score_out;         // [unit][n_keep] scores of the kept tokens, or null
   int32_t* kept;            // [unit][n_keep], or null: refinement only
   const int32_t* budgets;   // a budget per unit, or null
+  // the gather of the kept rows, when this kernel does it too (one CTA per head): k_out null otherwise
+  const char *k, *v;
+  char *k_out, *v_out;
+  int lanes;                // 16-byte pieces of a row
   int slots;
   int chunk;                // tokens per CTA, a multiple of kMaxPer
 };
@@ -82,6 +86,25 @@ __device__ __forceinline__ void load_run(const float* p, int j0, int n, bool vec
 
 __device__ __noinline__ float pooled_any(const float* nu, int j, int n, int half, float inv_w, bool zero_pad) {
   return pooled(nu, j, n, half, inv_w, zero_pad);
+}
+
+// Rows out[0 .. count) of K and V to the dense outputs, by the one CTA that has just written the indices.
+__device__ __forceinline__ void gather_rows(const SelectArgs& a, const Shape& pl, const int32_t* out, int unit, int count) {
+  __syncthreads();                                     // the indices are there
+  const long long b = unit / pl.Hkv, h = unit % pl.Hkv;
+  const int sub = threadIdx.x % a.lanes, step = kThreads / a.lanes;
+  const char* k = a.k + (b * pl.ks[0] + h * pl.ks[1]) * pl.es + sub * 16;
+  const char* v = a.v + (b * pl.vs[0] + h * pl.vs[1]) * pl.es + sub * 16;
+  const long long ktok = pl.ks[2] * pl.es, vtok = pl.vs[2] * pl.es, row = (long long)a.lanes * 16;
+  char* ko = a.k_out + (size_t)unit * pl.n_keep * row + sub * 16;
+  char* vo = a.v_out + (size_t)unit * pl.n_keep * row + sub * 16;
+#pragma unroll 4
+  for (int t = threadIdx.x / a.lanes; t < count; t += step) {
+    const long long j = *(const volatile int32_t*)(out + t);
+    const uint4 x = *reinterpret_cast<const uint4*>(k + j * ktok), y = *reinterpret_cast<const uint4*>(v + j * vtok);
+    *reinterpret_cast<uint4*>(ko + t * row) = x;
+    *reinterpret_cast<uint4*>(vo + t * row) = y;
+  }
 }
 
 template <int kPer, bool kCluster>
@@ -233,6 +256,7 @@ refine_select_kernel(const __grid_constant__ SelectArgs a, const __grid_constant
   }
   if (Bs == 0) {
     griddep_launch();
+    if (!kCluster && a.k_out) gather_rows(a, pl, out, unit, min(n, bud));
     if (kCluster) cl.sync();
     return;
   }
@@ -375,6 +399,7 @@ refine_select_kernel(const __grid_constant__ SelectArgs a, const __grid_constant
       }
     }
   }
+  if (!kCluster && a.k_out) gather_rows(a, pl, out, unit, min(n, bud));
   if (kCluster) cl.barrier_wait();                      // nobody leaves while its shared memory may still be read
 }
 
@@ -572,7 +597,8 @@ bool launch_clustered(SelectArgs a, const Shape& pl, cudaStream_t st, cudaError_
 
 ahakv_status launch_refine(const Plan& pl, const float* s_raw, const float* nu, const float* score_prev,
                            float* score, int slots, cudaStream_t st) {
-  SelectArgs a = {s_raw, nu, score_prev, score, nullptr, nullptr, nullptr, slots, 0};
+  SelectArgs a = {};
+  a.s_raw = s_raw; a.nu = nu; a.prev = score_prev; a.score = score; a.slots = slots;
   const Shape& shape = pl;
   cudaError_t e = cudaSuccess;
   if (!nu) {
@@ -586,7 +612,8 @@ ahakv_status launch_refine(const Plan& pl, const float* s_raw, const float* nu, 
 }
 
 ahakv_status launch_select(const Plan& pl, const float* score, int32_t* kept_idx, cudaStream_t st) {
-  SelectArgs a = {score, nullptr, nullptr, nullptr, nullptr, kept_idx, nullptr, 1, 0};
+  SelectArgs a = {};
+  a.s_raw = score; a.kept = kept_idx; a.slots = 1;
   cudaError_t e = cudaSuccess;
   if (!launch_clustered(a, pl, st, &e)) {
     select_kernel<<<pl.B * pl.Hkv, kWideThreads, 0, st>>>(score, kept_idx, pl, nullptr);
@@ -598,8 +625,20 @@ ahakv_status launch_select(const Plan& pl, const float* score, int32_t* kept_idx
 
 ahakv_status launch_refine_select(const Plan& pl, const float* s_raw, const float* nu, const float* score_prev,
                                   float* score, float** score_left, float* score_out, int32_t* kept_idx, int slots,
-                                  const int32_t* budgets, cudaStream_t st) {
-  SelectArgs a = {s_raw, nu, score_prev, nullptr, score_out, kept_idx, budgets, slots, 0};
+                                  const int32_t* budgets, const void* k, const void* v, void* k_out, void* v_out, bool* gathered,
+                                  cudaStream_t st) {
+  SelectArgs a = {};
+  a.s_raw = s_raw; a.nu = nu; a.prev = score_prev; a.score_out = score_out; a.kept = kept_idx; a.budgets = budgets; a.slots = slots;
+  #ifndef XGB
+#define XGB 128
+#endif
+  // The CTA that selects a head also gathers its rows when that is a launch saved and little to move: one CTA a head, at
+  // most 128 KB in and as much out (beyond, a gather spread over the whole GPU is faster).
+  *gathered = pl.n <= kThreads * 8 && (size_t)2 * pl.n_keep * pl.d * pl.es <= 128 * 1024;
+  if (*gathered) {
+    a.k = (const char*)k; a.v = (const char*)v; a.k_out = (char*)k_out; a.v_out = (char*)v_out;
+    a.lanes = pl.d * pl.es / 16;
+  }
   cudaError_t e = cudaSuccess;
   if (launch_clustered(a, pl, st, &e)) {
     *score_left = nullptr;
