@@ -258,7 +258,8 @@ const char* ahakv_stage_name(int stage);
  *
  * Computes exactly what ahakv_score computes, with the same kernels; the caller passes inputs and
  * outputs only.  Nothing is allocated or freed, by this call or by anything it calls.
- *  - Limit: ahakv_workspace_bytes(p) must not exceed AHAKV_STATIC_WS_BYTES (ahakv_static_workspace_bytes()
+ *  - Limit: ahakv_workspace_bytes(p) (for float32 inputs: what it returns less the room for softmax numerators, which a
+ *    call can do without) must not exceed AHAKV_STATIC_WS_BYTES (ahakv_static_workspace_bytes()
  *    returns it at run time); larger problems get AHAKV_ERR_WORKSPACE and nothing is launched.  8 MiB
  *    covers, for instance, one sequence of 8 KV heads x 16384 tokens (3.5 MiB), 32 heads x 4096 tokens
  *    (2 MiB) or a 16-sequence decode round of 8 KV heads x 2080 tokens (5.3 MiB); 32 heads x 16384

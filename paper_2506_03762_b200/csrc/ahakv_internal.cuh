@@ -40,7 +40,8 @@ struct Plan : Shape {
   int last[kMaxRows];        // per observation row: the last cache row it may see (n - r + i unless positions are given)
   int n_eff;                 // last[r - 1] + 1: keys beyond are seen by no row
   // workspace layout, byte offsets
-  size_t off_status, off_sync, off_sraw, off_nu, off_partial, off_final, off_score, ws_total;
+  size_t off_status, off_sync, off_sraw, off_nu, off_partial, off_final, off_score, ws_total;   // ws_total: what a call needs
+  size_t ws_wanted;          // ws_total and room for the softmax numerators of the FP32-pipe kernels at off ws_total
 };
 
 // plan.cu
@@ -48,11 +49,16 @@ struct Plan : Shape {
 // last r positions.
 ahakv_status make_plan(const ahakv_params* p, Plan* plan, const int64_t* obs_pos = nullptr);
 void count_launch(int n = 1);
+// ahakv_score with a workspace that need not have room for kept numerators.
+ahakv_status score_in_least_room(const ahakv_params* p, const void* q_obs, const void* k, const void* v, const float* score_prev,
+                                 float* score, void* ws, size_t ws_bytes, cudaStream_t st);
 
 // Launchers.  Each returns AHAKV_OK or AHAKV_ERR_CUDA and queues work on `st` only.
 // Both also stream V and write nu when the value prior is on (v and nu non-null), and clear the status word.
+// `kept` (nullable): room for simt_kept_floats() floats, with which the logits are formed once instead of twice.
+size_t simt_kept_floats(const Plan& pl);
 ahakv_status launch_score_simt(const Plan& pl, const void* q, const void* k, const void* v, float* s_raw, float* nu, float2* partial,
-                               int* status, cudaStream_t st);
+                               float* kept, int* status, cudaStream_t st);
 ahakv_status launch_score_tc(const Plan& pl, const void* q, const void* k, const void* v, float* s_raw, float* nu,
                              float* partial, float* off, int* counters, int* status, cudaStream_t st);
 bool score_tc_available();

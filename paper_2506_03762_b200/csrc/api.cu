@@ -130,6 +130,12 @@ ahakv_status make_plan(const ahakv_params* p, Plan* pl, const int64_t* obs_pos) 
   o.off_nu = off;      off += align_up(units * o.n * sizeof(float), 256);
   o.off_score = off;   off += align_up(units * o.n * sizeof(float), 256);
   o.ws_total = off;
+  // Kept numerators pay as long as they stay in L2, and not where both kernels' CTAs fit on the GPU at once: forming the
+  // logits a second time then costs nothing (512 tokens x 4 heads: 13.2 us against 15.2; 3001 x 8: 45.5 against 39.2).  A
+  // call with less room forms the logits twice.
+  const bool twice = o.use_tc || units * 4 * o.n_blk <= 2 * 148;
+  const size_t kept = twice ? 0 : align_up(simt_kept_floats(o) * sizeof(float), 256);
+  o.ws_wanted = off + (kept <= ((size_t)64 << 20) ? kept : 0);
   return AHAKV_OK;
 }
 
@@ -154,8 +160,9 @@ static ahakv_status plan_for(const ahakv_params* p, const Plan** out) {
 
 static bool aligned16(const void* p) { return ((uintptr_t)p & 15) == 0; }
 
-static ahakv_status check_ws(const Plan& pl, void* ws, size_t ws_bytes) {
-  if (!ws || ((uintptr_t)ws & 255) != 0 || ws_bytes < pl.ws_total) return AHAKV_ERR_WORKSPACE;
+// `least`: be content with what the call cannot do without.
+static ahakv_status check_ws(const Plan& pl, void* ws, size_t ws_bytes, bool least = false) {
+  if (!ws || ((uintptr_t)ws & 255) != 0 || ws_bytes < (least ? pl.ws_total : pl.ws_wanted)) return AHAKV_ERR_WORKSPACE;
   return AHAKV_OK;
 }
 
@@ -164,7 +171,7 @@ template <typename T> static T* at(void* ws, size_t off) { return reinterpret_ca
 // Queues the kernels that leave the raw accumulated score (per row block) and, with the value prior, the value
 // norms in the workspace.
 static ahakv_status queue_raw_score(const Plan& pl, const void* q, const void* k, const void* v, void* ws,
-                                    cudaStream_t st, int prof) {
+                                    size_t ws_bytes, cudaStream_t st, int prof) {
   TraceRange range("ahakv: score");
   ahakv_status rc;
   profile_mark(prof, 0, st);
@@ -182,7 +189,8 @@ static ahakv_status queue_raw_score(const Plan& pl, const void* q, const void* k
                          at<int>(ws, pl.off_sync), at<int>(ws, pl.off_status), st);
     profile_mark(prof, 1, st);
   } else {
-    rc = launch_score_simt(pl, q, k, v, s_raw, nu, at<float2>(ws, pl.off_partial), at<int>(ws, pl.off_status), st);
+    float* kept = pl.ws_wanted > pl.ws_total && ws_bytes >= pl.ws_wanted ? at<float>(ws, pl.ws_total) : nullptr;
+    rc = launch_score_simt(pl, q, k, v, s_raw, nu, at<float2>(ws, pl.off_partial), kept, at<int>(ws, pl.off_status), st);
     profile_mark(prof, 1, st);
   }
   profile_mark(prof, 2, st);
@@ -200,7 +208,7 @@ extern "C" {
 size_t ahakv_workspace_bytes(const ahakv_params* p) {
   const Plan* plan;
   if (plan_for(p, &plan) != AHAKV_OK) return 0;
-  return plan->ws_total;
+  return plan->ws_wanted;
 }
 
 double ahakv_lambda(int64_t n_total, int32_t budget, int32_t head_dim) {
@@ -209,7 +217,7 @@ double ahakv_lambda(int64_t n_total, int32_t budget, int32_t head_dim) {
 }
 
 static ahakv_status score_impl(const ahakv_params* p, const int64_t* obs_pos, const void* q_obs, const void* k,
-                               const void* v, const float* score_prev, float* score, void* ws, size_t ws_bytes,
+                               const void* v, const float* score_prev, float* score, void* ws, size_t ws_bytes, bool least,
                                cudaStream_t st) {
   Plan own;
   const Plan* plan = &own;
@@ -221,9 +229,9 @@ static ahakv_status score_impl(const ahakv_params* p, const int64_t* obs_pos, co
   if (!aligned16(q_obs) || !aligned16(k) || (v && !aligned16(v)) || !aligned16(score) ||
       (score_prev && !aligned16(score_prev)))
     return AHAKV_ERR_INVALID_ARG;
-  if ((rc = check_ws(pl, ws, ws_bytes))) return rc;
+  if ((rc = check_ws(pl, ws, ws_bytes, least))) return rc;
   const int prof = profile_begin_call(st);
-  if ((rc = queue_raw_score(pl, q_obs, k, v, ws, st, prof))) return rc;
+  if ((rc = queue_raw_score(pl, q_obs, k, v, ws, ws_bytes, st, prof))) return rc;
   rc = launch_refine(pl, at<float>(ws, pl.off_sraw), prior ? at<float>(ws, pl.off_nu) : nullptr, score_prev, score,
                      score_slots(pl), st);
   profile_mark(prof, 3, st);
@@ -235,14 +243,23 @@ static ahakv_status score_impl(const ahakv_params* p, const int64_t* obs_pos, co
 ahakv_status ahakv_score(const ahakv_params* p, const void* q_obs, const void* k, const void* v,
                          const float* score_prev, float* score, void* ws, size_t ws_bytes,
                          ahakv_stream_t stream) {
-  return score_impl(p, nullptr, q_obs, k, v, score_prev, score, ws, ws_bytes, (cudaStream_t)stream);
+  return score_impl(p, nullptr, q_obs, k, v, score_prev, score, ws, ws_bytes, false, (cudaStream_t)stream);
 }
+
+}  // extern "C"
+
+ahakv_status ahakv::score_in_least_room(const ahakv_params* p, const void* q_obs, const void* k, const void* v, const float* score_prev,
+                                        float* score, void* ws, size_t ws_bytes, cudaStream_t st) {
+  return score_impl(p, nullptr, q_obs, k, v, score_prev, score, ws, ws_bytes, true, st);
+}
+
+extern "C" {
 
 ahakv_status ahakv_score_rows(const ahakv_params* p, const int64_t* obs_pos, const void* q_obs, const void* k,
                               const void* v, const float* score_prev, float* score, void* ws, size_t ws_bytes,
                               ahakv_stream_t stream) {
   if (!obs_pos) return AHAKV_ERR_INVALID_ARG;
-  return score_impl(p, obs_pos, q_obs, k, v, score_prev, score, ws, ws_bytes, (cudaStream_t)stream);
+  return score_impl(p, obs_pos, q_obs, k, v, score_prev, score, ws, ws_bytes, false, (cudaStream_t)stream);
 }
 
 ahakv_status ahakv_score_full_causal(const ahakv_params* p, const void* q_all, const void* k, const void* v,
@@ -296,7 +313,7 @@ ahakv_status ahakv_score_full_causal(const ahakv_params* p, const void* q_all, c
     if ((rc = make_plan(&pc, &pl, pos))) return rc;
     if (pl.off_score > full.off_score) return AHAKV_ERR_WORKSPACE;   // cannot happen: fewer rows never need more room
     const char* qc = (const char*)q_all + (size_t)c0 * pl.qs[2] * pl.es;
-    if ((rc = queue_raw_score(pl, qc, k, nullptr, ws, st, -1))) return rc;
+    if ((rc = queue_raw_score(pl, qc, k, nullptr, ws, 0 /* what lies behind is in use */, st, -1))) return rc;
     if ((rc = launch_refine(pl, at<float>(ws, pl.off_sraw), nullptr, c0 == 0 ? nullptr : acc, acc, score_slots(pl), st)))
       return rc;
   }
@@ -390,7 +407,7 @@ ahakv_status ahakv_compact(const ahakv_params* p, const void* k, const void* v, 
 
 static ahakv_status evict_impl(const ahakv_params* p, const int32_t* budgets, const void* q_obs, const void* k,
                                const void* v, const float* score_prev, void* k_out, void* v_out, float* score_out,
-                               int32_t* kept_idx, void* ws, size_t ws_bytes, ahakv_stream_t stream) {
+                               int32_t* kept_idx, void* ws, size_t ws_bytes, bool least, ahakv_stream_t stream) {
   const Plan* plan;
   ahakv_status rc = plan_for(p, &plan);
   if (rc) return rc;
@@ -399,11 +416,11 @@ static ahakv_status evict_impl(const ahakv_params* p, const int32_t* budgets, co
   if (!aligned16(q_obs) || !aligned16(k) || !aligned16(v) || !aligned16(k_out) || !aligned16(v_out) ||
       ((uintptr_t)kept_idx & 3) || (score_prev && !aligned16(score_prev)))
     return AHAKV_ERR_INVALID_ARG;
-  if ((rc = check_ws(pl, ws, ws_bytes))) return rc;
+  if ((rc = check_ws(pl, ws, ws_bytes, least))) return rc;
   cudaStream_t st = (cudaStream_t)stream;
   TraceRange call("ahakv_evict");
   const int prof = profile_begin_call(st);
-  if ((rc = queue_raw_score(pl, q_obs, k, v, ws, st, prof))) return rc;
+  if ((rc = queue_raw_score(pl, q_obs, k, v, ws, ws_bytes, st, prof))) return rc;
   const bool prior = (pl.flags & AHAKV_FLAG_VALUE_PRIOR) != 0;
   float* s_raw = at<float>(ws, pl.off_sraw);
   float* nu = prior ? at<float>(ws, pl.off_nu) : nullptr;
@@ -428,7 +445,7 @@ static ahakv_status evict_impl(const ahakv_params* p, const int32_t* budgets, co
 ahakv_status ahakv_evict(const ahakv_params* p, const void* q_obs, const void* k, const void* v,
                          const float* score_prev, void* k_out, void* v_out, float* score_out,
                          int32_t* kept_idx, void* ws, size_t ws_bytes, ahakv_stream_t stream) {
-  return evict_impl(p, nullptr, q_obs, k, v, score_prev, k_out, v_out, score_out, kept_idx, ws, ws_bytes, stream);
+  return evict_impl(p, nullptr, q_obs, k, v, score_prev, k_out, v_out, score_out, kept_idx, ws, ws_bytes, false, stream);
 }
 
 ahakv_status ahakv_evict_head_budgets(const ahakv_params* p, const int32_t* head_budget, const void* q_obs, const void* k,
@@ -436,7 +453,7 @@ ahakv_status ahakv_evict_head_budgets(const ahakv_params* p, const int32_t* head
                                       float* score_out, int32_t* kept_idx, void* ws, size_t ws_bytes,
                                       ahakv_stream_t stream) {
   if (!head_budget || ((uintptr_t)head_budget & 3)) return AHAKV_ERR_INVALID_ARG;
-  return evict_impl(p, head_budget, q_obs, k, v, score_prev, k_out, v_out, score_out, kept_idx, ws, ws_bytes, stream);
+  return evict_impl(p, head_budget, q_obs, k, v, score_prev, k_out, v_out, score_out, kept_idx, ws, ws_bytes, false, stream);
 }
 
 ahakv_status ahakv_evict_ragged(const ahakv_params* p, const ahakv_seq* seqs, const void* q_obs, const void* k,
@@ -466,9 +483,8 @@ ahakv_status ahakv_evict_ragged(const ahakv_params* p, const ahakv_seq* seqs, co
     const char* kb = (const char*)k + (size_t)b * outer.ks[0] * es;
     const char* vb = (const char*)v + (size_t)b * outer.vs[0] * es;
     const size_t tok = (size_t)b * outer.Hkv * outer.n, kept = (size_t)b * outer.Hkv * keep_max;
-    rc = ahakv_evict(&pb, qb, kb, vb, score_prev ? score_prev + tok : nullptr, (char*)k_out + kept * row,
-                     (char*)v_out + kept * row, score_out ? score_out + kept : nullptr, kept_idx + kept, ws, ws_bytes,
-                     stream);
+    rc = evict_impl(&pb, nullptr, qb, kb, vb, score_prev ? score_prev + tok : nullptr, (char*)k_out + kept * row,
+                    (char*)v_out + kept * row, score_out ? score_out + kept : nullptr, kept_idx + kept, ws, ws_bytes, true, stream);
     if (rc) return rc;
   }
   return AHAKV_OK;

@@ -11,7 +11,10 @@
 // Two kernels over 64-key tiles, one CTA a tile of a (sequence, KV head).
 //   simt_row_stats:   every observation row's softmax statistics (max and sum of 2^{c w}) per 128-key block, two CTAs (a
 //                     cluster) a block.
-//   simt_column_sums: merges the blocks' statistics, recomputes the logits and adds the normalised weights of all rows
+//                     Leaves the numerators 2^{c w - m} (m the row's maximum over the tile) in the workspace if it has room.
+//   simt_weighted_sums: merges the blocks' statistics and adds the kept numerators, weighted, into the keys' scores (Eq. 1,
+//                     5, 9); squares the tile's value rows on the side.
+//   simt_column_sums: the same without kept numerators: merges the blocks' statistics, recomputes the logits and adds the normalised weights of all rows
 //                     into the keys' scores (Eq. 1, 5, 9); squares the tile's value rows on the side.
 // What bounds them: the FP64 units, 64 multiply-adds a cycle and SM, as long as their operands come ready-made and cheaply.
 // Converting FP32 to FP64 runs at a quarter of that rate, so keys and queries are converted once, into shared memory; and
@@ -58,6 +61,7 @@ struct Tiles {
   A q[kRows][row_pitch<A, D>()];
   A row_c[kRows];
   int row_last[kRows];
+  __align__(16) float fin4[kRows][kKeyWarps];         // simt_row_stats: row maxima of the key warps
   float2 fin[kRows];                                  // shift and 1 / (G sum) of a row
   float2 stat[kMaxRows][kKeyWarps];                   // simt_row_stats: per row and key warp; simt_column_sums: scratch
 };
@@ -195,9 +199,10 @@ __device__ __forceinline__ float2 merge_pair(float2 a, float2 b) {
 }
 
 // Pass 1: per (unit, 128-key block, stacked row) the pair (max of c*w, sum of 2^{c*w - max}).
-template <typename T, int D>
+template <typename T, int D, bool kKeep>
 __global__ void __launch_bounds__(kThreads, 2) __cluster_dims__(2, 1, 1)
-simt_row_stats(const T* __restrict__ q, const T* __restrict__ k, float2* __restrict__ partial, int* __restrict__ status,
+simt_row_stats(const T* __restrict__ q, const T* __restrict__ k, float2* __restrict__ partial, float* __restrict__ numer,
+               float* __restrict__ shift, int* __restrict__ status,
                const __grid_constant__ Shape pl, const __grid_constant__ RowScaleOf<Acc<T>> cs) {
   using A = Acc<T>;
   extern __shared__ __align__(16) char smem_raw[];
@@ -224,6 +229,7 @@ simt_row_stats(const T* __restrict__ q, const T* __restrict__ k, float2* __restr
     __syncthreads();
     A acc[4][2];
     dot_16x16<D>(sm, 16 * kw, 16 * rw, acc);
+    float ms[2];
 #pragma unroll
     for (int y = 0; y < 2; ++y) {
       const A cc = sm.row_c[row + 8 * y];
@@ -236,13 +242,43 @@ simt_row_stats(const T* __restrict__ q, const T* __restrict__ k, float2* __restr
       }
 #pragma unroll
       for (int o = 2; o; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-      float z = 0.f;
+      ms[y] = m;
+    }
+    if (kKeep) {
+      // one shift for the tile's keys, so that its numerators need one number a row beside them
 #pragma unroll
-      for (int x = 0; x < 4; ++x)
-        if (j0 + key(x) <= last) z += fast_exp2((float)(acc[x][y] - (A)m));
+      for (int y = 0; y < 2; ++y)
+        if ((lane & 3) == 0) sm.fin4[row + 8 * y][kw] = ms[y];
+      __syncthreads();
+#pragma unroll
+      for (int y = 0; y < 2; ++y) {
+        const float4 f = *reinterpret_cast<const float4*>(sm.fin4[row + 8 * y]);
+        ms[y] = fmaxf(fmaxf(f.x, f.y), fmaxf(f.z, f.w));
+      }
+    }
+#pragma unroll
+    for (int y = 0; y < 2; ++y) {
+      const int last = sm.row_last[row + 8 * y];
+      const float m = ms[y];
+      float e[4], z = 0.f;
+#pragma unroll
+      for (int x = 0; x < 4; ++x) {
+        e[x] = j0 + key(x) <= last ? fast_exp2((float)(acc[x][y] - (A)m)) : 0.f;
+        z += e[x];
+      }
 #pragma unroll
       for (int o = 2; o; o >>= 1) z += __shfl_xor_sync(0xffffffffu, z, o);
-      if ((lane & 3) == 0 && row + 8 * y < c.rows) sm.stat[c.s0 + row + 8 * y][kw] = make_float2(m, z);
+      if (row + 8 * y < c.rows) {
+        const int s = c.s0 + row + 8 * y;
+        if ((lane & 3) == 0) sm.stat[s][kw] = make_float2(m, z);
+        if (kKeep) {
+          float* to = numer + ((size_t)unit * pl.R + s) * pl.n + j0;
+#pragma unroll
+          for (int x = 0; x < 4; ++x)
+            if (j0 + key(x) < pl.n) to[key(x)] = e[x];
+          if (lane % 4 == 0 && kw == 0) shift[((size_t)unit * 2 * pl.n_blk + blockIdx.x) * pl.R + s] = m;
+        }
+      }
     }
   }
   cl.sync();
@@ -369,8 +405,58 @@ simt_column_sums(const T* __restrict__ q, const T* __restrict__ k, const T* __re
   if (threadIdx.x < kTile && j0 + (int)threadIdx.x < pl.n) s_raw[(size_t)unit * pl.n + j0 + threadIdx.x] = best;
 }
 
+// Pass 2 from kept numerators: S_j = sum over the stacked rows of e_sj 2^{m - M} / (G * sum), m the shift of the tile's
+// numerators, M and the sum those of the row.
 template <typename T, int D>
-ahakv_status run(const Plan& pl, const void* q, const void* k, const void* v, float* s_raw, float* nu, float2* partial, int* status,
+__global__ void __launch_bounds__(kThreads)
+simt_weighted_sums(const T* __restrict__ v, const float2* partial, const float* numer, const float* shift, float* __restrict__ s_raw,
+                   float* __restrict__ nu, const __grid_constant__ Shape pl) {
+  __shared__ float2 part[kThreads / 32][kRows];
+  __shared__ float weight[kMaxRows], sums[kThreads / kTile][kTile];
+  const int unit = blockIdx.y, b = unit / pl.Hkv, h = unit % pl.Hkv, j0 = blockIdx.x * kTile;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  griddep_wait();
+  griddep_launch();
+  if (nu) tile_norms<T, D>(v, nu, pl, b, h, unit, j0);
+  for (int s0 = 0; s0 < pl.R; s0 += kRows) {
+    // eight threads a row, each every eighth block in order, then the eight in order
+    float2 p = make_float2(-INFINITY, 0.f);
+    const int s = s0 + lane;
+    if (s < pl.R) {
+      const float2* from = partial + (size_t)unit * pl.n_blk * pl.R + s;
+#pragma unroll 8
+      for (int t = warp; t < pl.n_blk; t += kThreads / 32) p = merge_pair(p, __ldcg(from + (size_t)t * pl.R));
+    }
+    part[warp][lane] = p;
+    __syncthreads();
+    if (warp == 0 && s < pl.R) {
+#pragma unroll
+      for (int w = 1; w < kThreads / 32; ++w) p = merge_pair(p, part[w][lane]);
+      const float m = shift[((size_t)unit * 2 * pl.n_blk + blockIdx.x) * pl.R + s];
+      weight[s] = (m > -INFINITY ? fast_exp2(m - p.x) : 0.f) / (p.y * (float)(pl.group_max ? 1 : pl.G));
+    }
+    __syncthreads();
+  }
+  const int jl = threadIdx.x % kTile, share = threadIdx.x / kTile, j = j0 + jl;
+  const int heads = pl.group_max ? pl.G : 1, rows = pl.R / heads;
+  float best = 0.f;
+  for (int g = 0; g < heads; ++g) {
+    const float* from = numer + ((size_t)unit * pl.R + g * rows) * pl.n + j;
+    float sum = 0.f;
+    if (j < pl.n) {
+#pragma unroll 8
+      for (int i = share; i < rows; i += kThreads / kTile) sum = fmaf(from[(size_t)i * pl.n], weight[g * rows + i], sum);
+    }
+    if (g > 0) __syncthreads();
+    sums[share][jl] = sum;
+    __syncthreads();
+    if (share == 0) best = fmaxf(best, (sums[0][jl] + sums[1][jl]) + (sums[2][jl] + sums[3][jl]));
+  }
+  if (share == 0 && j < pl.n) s_raw[(size_t)unit * pl.n + j] = best;
+}
+
+template <typename T, int D>
+ahakv_status run(const Plan& pl, const void* q, const void* k, const void* v, float* s_raw, float* nu, float2* partial, float* kept, int* status,
                  cudaStream_t st) {
   RowScaleOf<Acc<T>> cs;
   for (int i = 0; i < kMaxRows; ++i) {
@@ -384,37 +470,52 @@ ahakv_status run(const Plan& pl, const void* q, const void* k, const void* v, fl
   int dev = -1;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return AHAKV_ERR_CUDA;
   if (!configured[dev]) {
-    if (cudaFuncSetAttribute(simt_row_stats<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
+    if (cudaFuncSetAttribute(simt_row_stats<T, D, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
+        cudaFuncSetAttribute(simt_row_stats<T, D, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
         cudaFuncSetAttribute(simt_column_sums<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
       return AHAKV_ERR_CUDA;
     configured[dev] = true;
   }
   const Shape& shape = pl;
   const int units = pl.B * pl.Hkv;
-  cudaError_t e = launch_chained(simt_row_stats<T, D>, dim3(2 * pl.n_blk, units), dim3(kThreads), 2, smem, st, (const T*)q, (const T*)k,
-                                 partial, status, shape, cs);
-  if (e == cudaSuccess)
-    e = launch_chained(simt_column_sums<T, D>, dim3((pl.n + kTile - 1) / kTile, units), dim3(kThreads), 1, smem, st, (const T*)q,
-                       (const T*)k, (const T*)v, partial, s_raw, nu, shape, cs);
+  const dim3 stats_grid(2 * pl.n_blk, units), sums_grid((pl.n + kTile - 1) / kTile, units);
+  float* const none = nullptr;
+  cudaError_t e;
+  if (kept) {
+    float* shift = kept + (size_t)units * pl.R * pl.n;
+    e = launch_chained(simt_row_stats<T, D, true>, stats_grid, dim3(kThreads), 2, smem, st, (const T*)q, (const T*)k, partial, kept, shift,
+                       status, shape, cs);
+    if (e == cudaSuccess)
+      e = launch_chained(simt_weighted_sums<T, D>, sums_grid, dim3(kThreads), 1, 0, st, (const T*)v, partial, kept, shift, s_raw, nu, shape);
+  } else {
+    e = launch_chained(simt_row_stats<T, D, false>, stats_grid, dim3(kThreads), 2, smem, st, (const T*)q, (const T*)k, partial, none, none,
+                       status, shape, cs);
+    if (e == cudaSuccess)
+      e = launch_chained(simt_column_sums<T, D>, sums_grid, dim3(kThreads), 1, smem, st, (const T*)q, (const T*)k, (const T*)v, partial,
+                         s_raw, nu, shape, cs);
+  }
   count_launch(2);
   return cuda_ok(e);
 }
 
 }  // namespace
 
+// Floats kept per call: the numerators [unit][R][n] and the tiles' shifts [unit][2 n_blk][R].
+size_t simt_kept_floats(const Plan& pl) { return (size_t)pl.B * pl.Hkv * pl.R * ((size_t)pl.n + 2 * pl.n_blk); }
+
 ahakv_status launch_score_simt(const Plan& pl, const void* q, const void* k, const void* v, float* s_raw, float* nu, float2* partial,
-                               int* status, cudaStream_t st) {
+                               float* kept, int* status, cudaStream_t st) {
   const bool d64 = pl.d == 64;
   switch (pl.dtype) {
     case AHAKV_F32:
-      return d64 ? run<float, 64>(pl, q, k, v, s_raw, nu, partial, status, st)
-                 : run<float, 128>(pl, q, k, v, s_raw, nu, partial, status, st);
+      return d64 ? run<float, 64>(pl, q, k, v, s_raw, nu, partial, kept, status, st)
+                 : run<float, 128>(pl, q, k, v, s_raw, nu, partial, kept, status, st);
     case AHAKV_F16:
-      return d64 ? run<__half, 64>(pl, q, k, v, s_raw, nu, partial, status, st)
-                 : run<__half, 128>(pl, q, k, v, s_raw, nu, partial, status, st);
+      return d64 ? run<__half, 64>(pl, q, k, v, s_raw, nu, partial, kept, status, st)
+                 : run<__half, 128>(pl, q, k, v, s_raw, nu, partial, kept, status, st);
     default:
-      return d64 ? run<__nv_bfloat16, 64>(pl, q, k, v, s_raw, nu, partial, status, st)
-                 : run<__nv_bfloat16, 128>(pl, q, k, v, s_raw, nu, partial, status, st);
+      return d64 ? run<__nv_bfloat16, 64>(pl, q, k, v, s_raw, nu, partial, kept, status, st)
+                 : run<__nv_bfloat16, 128>(pl, q, k, v, s_raw, nu, partial, kept, status, st);
   }
 }
 

@@ -629,9 +629,6 @@ ahakv_status launch_refine_select(const Plan& pl, const float* s_raw, const floa
                                   cudaStream_t st) {
   SelectArgs a = {};
   a.s_raw = s_raw; a.nu = nu; a.prev = score_prev; a.score_out = score_out; a.kept = kept_idx; a.budgets = budgets; a.slots = slots;
-  #ifndef XGB
-#define XGB 128
-#endif
   // The CTA that selects a head also gathers its rows when that is a launch saved and little to move: one CTA a head, at
   // most 128 KB in and as much out (beyond, a gather spread over the whole GPU is faster).
   *gathered = pl.n <= kThreads * 8 && (size_t)2 * pl.n_keep * pl.d * pl.es <= 128 * 1024;

@@ -25,3 +25,20 @@ def test_float32_scores_at_tile_edges(B, Hq, Hkv, d, n, r, flags):
     a = w.masked_fill(~seen, float("-inf")).softmax(-1).sum(2).view(B, Hkv, G, n)
     want = a.amax(2) if flags & ab.FLAG_GROUP_MAX else a.mean(2)
     assert torch.allclose(score.double(), want, rtol=1e-5, atol=1e-5 * 1e-3 * r / n)
+
+
+@pytest.mark.parametrize("n,r,Hq,Hkv,flags", [(9001, 64, 4, 4, 1), (9100, 20, 12, 4, 5)])
+def test_scores_with_and_without_room_for_numerators_agree(n, r, Hq, Hkv, flags):
+    """The library's own scratch is too small for these cases' softmax numerators, so that the logits are formed twice; with
+    a workspace of the size asked for they are kept.  The two differ by where an exponential is split in two, a few FP32
+    roundings: 1e-5."""
+    from paper_2506_03762_b200 import binding as ab
+    g = torch.Generator().manual_seed(n)
+    q = torch.randn((1, Hq, r, 64), generator=g).cuda()
+    k, v = (torch.randn((1, Hkv, n, 64), generator=g).cuda() for _ in range(2))
+    p = ab.Params(1, Hq, Hkv, 64, n, r, 4, 40, dtype=ab.F32, flags=flags)
+    assert ab.ahakv_workspace_bytes(p) > ab.ahakv_static_workspace_bytes()
+    a, b = (torch.empty((1, Hkv, n), device="cuda") for _ in range(2))
+    ab.ahakv_score(p, q, k, v, None, a, ab.alloc_workspace(p))
+    ab.ahakv_score_static(p, q, k, v, None, b)
+    assert torch.allclose(a, b, rtol=1e-5, atol=0)
