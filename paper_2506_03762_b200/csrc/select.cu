@@ -1,7 +1,8 @@
 // Value-prior refinement (Eq. 13-15) and budgeted selection (Algorithm 1).
 //
-// One cluster of C CTAs per (sequence, KV head), each CTA a contiguous piece of its tokens, each thread kPer adjacent ones,
-// whose refined scores stay in registers from the first load to the last store.
+// One cluster of C CTAs per (sequence, KV head), each CTA a contiguous piece of its tokens, each thread kPer of them, in
+// fours that lie beside its neighbours' (loads of whole lines, the filter's window by shuffles), whose refined scores stay in
+// registers from the first load to the last store.
 //   refine: adds the row-block partial scores, smooths nu with the mean filter, normalises by the head-wide maximum,
 //     multiplies, and adds the carried score.
 //   select: the B_s-th largest candidate score by a histogram over the order-preserving integer image of the float: its
@@ -9,11 +10,13 @@
 //     it names the bin the threshold falls into, and the tokens of that bin are ranked against each other from a list;
 //     as long as they are too many for the list, a histogram over the bin's own range comes first (at most three more).
 //     Then every candidate above the threshold plus the lowest-indexed ones equal to it are emitted in ascending index
-//     order (a prefix sum over the cluster), then the recent window; exact, ties lowest index first.
-// What bounds it: for few heads the latency of its steps (about ten block-wide ones; the cluster adds four barriers), for
-// many the instructions.  Adjacent tokens per thread make both cheaper than tokens dealt out in turn: a thread reads its
-// filter window once, straight from L1 (a warp's loads together cover whole lines), and the ordered emission needs one
-// prefix sum over threads instead of a ballot per token.
+//     order, then the recent window; exact, ties lowest index first.
+// What bounds it: for few heads the latency of its steps (about ten block-wide ones, three cluster barriers and a trip to the
+// neighbours' shared memory), for many the instructions and, of a first wave, their way into the instruction cache.  So the
+// CTAs of a cluster send each other what they can before a barrier (maxima, sums over sixteen bins, list entries) and a CTA
+// finds its place in the output from the histograms and the list alone.  Whole CTAs' histograms summed from where they
+// are cost 8000 cycles of a 16-CTA cluster's 36000; the list by atomics of all in one CTA, and the counts exchanged for the
+// output, most of 8000 more.
 #include <cooperative_groups.h>
 
 #include "ahakv_internal.cuh"
@@ -28,6 +31,7 @@ constexpr int kThreads = 512;
 constexpr int kWarps = kThreads / 32;
 constexpr int kBins = 4 * kThreads;
 constexpr int kList = kThreads;          // one list entry per thread
+constexpr int kCoarse = kBins / 16;
 constexpr int kMaxPer = 16, kMaxCluster = 16;
 
 struct SelectArgs {
@@ -69,18 +73,15 @@ __device__ __forceinline__ unsigned block_scan(unsigned x, unsigned* tot, unsign
   return __reduce_add_sync(0xffffffffu, lane < warp ? y : 0u) + inc - x;
 }
 
-// kPer adjacent values from p + j0 (p: a head's row), zero from n on; `vec`: rows start on 16-byte boundaries.
-template <int kPer>
-__device__ __forceinline__ void load_run(const float* p, int j0, int n, bool vec, float (&v)[kPer]) {
-  if (kPer >= 4 && vec && j0 + kPer <= n) {
-#pragma unroll
-    for (int e = 0; e < kPer; e += 4) {
-      const float4 x = *reinterpret_cast<const float4*>(p + j0 + e);
-      v[e] = x.x; v[(e + 1) % kPer] = x.y; v[(e + 2) % kPer] = x.z; v[(e + 3) % kPer] = x.w;
-    }
+// kV adjacent values from p + j0 (p: a head's row), zero from `lim` on; `vec`: rows start on 16-byte boundaries.
+template <int kV>
+__device__ __forceinline__ void load_piece(const float* p, int j0, int lim, bool vec, float* v) {
+  if (kV == 4 && vec && j0 + 4 <= lim) {
+    const float4 x = *reinterpret_cast<const float4*>(p + j0);
+    v[0] = x.x; v[1 % kV] = x.y; v[2 % kV] = x.z; v[3 % kV] = x.w;
   } else {
 #pragma unroll
-    for (int e = 0; e < kPer; ++e) v[e] = j0 + e < n ? p[j0 + e] : 0.f;
+    for (int e = 0; e < kV; ++e) v[e] = j0 + e < lim ? p[j0 + e] : 0.f;
   }
 }
 
@@ -88,8 +89,11 @@ __device__ __noinline__ float pooled_any(const float* nu, int j, int n, int half
   return pooled(nu, j, n, half, inv_w, zero_pad);
 }
 
-// Rows out[0 .. count) of K and V to the dense outputs, by the one CTA that has just written the indices.
-__device__ __forceinline__ void gather_rows(const SelectArgs& a, const Shape& pl, const int32_t* out, int unit, int count) {
+// The kept rows of K and V to the dense outputs, by the one CTA that has just chosen them: row t is token picked[t] below
+// `Bs` and from there on the recent window's.  Four rows of each are in flight per thread (one after the other they cost a
+// trip to memory each: 10800 cycles for 256 rows, now 3000).
+__device__ __forceinline__ void gather_rows(const SelectArgs& a, const Shape& pl, const unsigned short* picked, int unit, int Bs,
+                                            int first_recent, int count) {
   __syncthreads();                                     // the indices are there
   const long long b = unit / pl.Hkv, h = unit % pl.Hkv;
   const int sub = threadIdx.x % a.lanes, step = kThreads / a.lanes;
@@ -98,98 +102,236 @@ __device__ __forceinline__ void gather_rows(const SelectArgs& a, const Shape& pl
   const long long ktok = pl.ks[2] * pl.es, vtok = pl.vs[2] * pl.es, row = (long long)a.lanes * 16;
   char* ko = a.k_out + (size_t)unit * pl.n_keep * row + sub * 16;
   char* vo = a.v_out + (size_t)unit * pl.n_keep * row + sub * 16;
-#pragma unroll 4
-  for (int t = threadIdx.x / a.lanes; t < count; t += step) {
-    const long long j = *(const volatile int32_t*)(out + t);
-    const uint4 x = *reinterpret_cast<const uint4*>(k + j * ktok), y = *reinterpret_cast<const uint4*>(v + j * vtok);
-    *reinterpret_cast<uint4*>(ko + t * row) = x;
-    *reinterpret_cast<uint4*>(vo + t * row) = y;
+  for (int t0 = threadIdx.x / a.lanes; t0 < count; t0 += 4 * step) {
+    uint4 x[4], y[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int t = t0 + i * step;
+      if (t < count) {
+        const long long j = t < Bs ? (int)picked[t] : first_recent + t - Bs;
+        x[i] = *reinterpret_cast<const uint4*>(k + j * ktok);
+        y[i] = *reinterpret_cast<const uint4*>(v + j * vtok);
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int t = t0 + i * step;
+      if (t < count) {
+        *reinterpret_cast<uint4*>(ko + t * row) = x[i];
+        *reinterpret_cast<uint4*>(vo + t * row) = y[i];
+      }
+    }
   }
 }
 
+// What a histogram says: the bin the threshold falls into, how many of its tokens are wanted and how many it holds; and how
+// many tokens above the bin and in it the CTAs before this one have.
+struct Found {
+  unsigned bin, need, in_bin, above_before, in_before;
+};
+
+// ... the histogram of the whole cluster, by one warp.  Each CTA has given every other its sums over 16 bins (coarse); the
+// sixteen bins in question are read from where they are.
+__device__ __forceinline__ Found find_in_cluster(cg::cluster_group& cl, unsigned* hist, const unsigned (*coarse)[kCoarse],
+                                                 unsigned need, int C, int rank) {
+  const int lane = threadIdx.x & 31;
+  // lane l: coarse bins 4 (31 - l) .. + 3, so that sums from the largest bin down are prefix sums
+  uint4 all = make_uint4(0, 0, 0, 0), bef = all;
+  const int c4 = 4 * (31 - lane);
+#pragma unroll 4
+  for (int r = 0; r < C; ++r) {
+    const uint4 x = *reinterpret_cast<const uint4*>(&coarse[r][c4]);
+    all.x += x.x; all.y += x.y; all.z += x.z; all.w += x.w;
+    if (r < rank) { bef.x += x.x; bef.y += x.y; bef.z += x.z; bef.w += x.w; }
+  }
+  const unsigned sum = all.x + all.y + all.z + all.w;
+  unsigned inc = sum;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const unsigned y = __shfl_up_sync(0xffffffffu, inc, o);
+    if (lane >= o) inc += y;
+  }
+  unsigned above = inc - sum, cb = c4 + 3, b = 0, in = all.w;
+  const unsigned owner = __ballot_sync(0xffffffffu, above < need && inc >= need);   // one lane
+  if (above + in < need) {
+    above += in; b += bef.w; in = all.z; --cb;
+    if (above + in < need) {
+      above += in; b += bef.z; in = all.y; --cb;
+      if (above + in < need) { above += in; b += bef.y; --cb; }
+    }
+  }
+  const int src = __ffs(owner) - 1;
+  if (lane < src) b = bef.x + bef.y + bef.z + bef.w;
+  else if (lane > src) b = 0;
+  Found f;
+  f.above_before = __reduce_add_sync(0xffffffffu, b);
+  above = __shfl_sync(0xffffffffu, above, src);
+  cb = __shfl_sync(0xffffffffu, cb, src);
+  // lane 4 r + p: bins 4 p .. + 3 of the sixteen, of CTAs r and r + 8
+  const int r0 = lane >> 2, p = lane & 3, b4 = 16 * (int)cb + 4 * p;
+  const uint4 z = make_uint4(0, 0, 0, 0);
+  const uint4 x = r0 < C ? *reinterpret_cast<const uint4*>(cl.map_shared_rank(hist + b4, r0)) : z;
+  const uint4 y = r0 + 8 < C ? *reinterpret_cast<const uint4*>(cl.map_shared_rank(hist + b4, r0 + 8)) : z;
+  uint4 t = make_uint4(x.x + y.x, x.y + y.y, x.z + y.z, x.w + y.w);
+#pragma unroll
+  for (int o = 4; o < 32; o <<= 1) {
+    t.x += __shfl_xor_sync(0xffffffffu, t.x, o);
+    t.y += __shfl_xor_sync(0xffffffffu, t.y, o);
+    t.z += __shfl_xor_sync(0xffffffffu, t.z, o);
+    t.w += __shfl_xor_sync(0xffffffffu, t.w, o);
+  }
+  const unsigned quad = t.x + t.y + t.z + t.w;
+  unsigned higher = above;                              // in bins above this lane's four
+#pragma unroll
+  for (int o = 1; o < 4; ++o) {
+    const unsigned q = __shfl_sync(0xffffffffu, quad, (lane & ~3) + ((p + o) & 3));
+    if (p + o < 4) higher += q;
+  }
+  unsigned d = b4 + 3;
+  const bool mine = higher < need && higher + quad >= need;
+  in = t.w;
+  if (higher + in < need) {
+    higher += in; in = t.z; --d;
+    if (higher + in < need) {
+      higher += in; in = t.y; --d;
+      if (higher + in < need) { higher += in; in = t.x; --d; }
+    }
+  }
+  const int at = __ffs(__ballot_sync(0xffffffffu, mine)) - 1;
+  f.bin = __shfl_sync(0xffffffffu, d, at);
+  f.need = need - __shfl_sync(0xffffffffu, higher, at);
+  f.in_bin = __shfl_sync(0xffffffffu, in, at);
+  const uint4 o = make_uint4((r0 < rank ? x.x : 0u) + (r0 + 8 < rank ? y.x : 0u), (r0 < rank ? x.y : 0u) + (r0 + 8 < rank ? y.y : 0u),
+                             (r0 < rank ? x.z : 0u) + (r0 + 8 < rank ? y.z : 0u), (r0 < rank ? x.w : 0u) + (r0 + 8 < rank ? y.w : 0u));
+  const int rel = (int)f.bin - b4;                      // 0 .. 3: one of this lane's
+  f.above_before += __reduce_add_sync(0xffffffffu, (rel < 0 ? o.x : 0u) + (rel < 1 ? o.y : 0u) + (rel < 2 ? o.z : 0u) + (rel < 3 ? o.w : 0u));
+  f.in_before = __reduce_add_sync(0xffffffffu, rel == 0 ? o.x : rel == 1 ? o.y : rel == 2 ? o.z : rel == 3 ? o.w : 0u);
+  return f;
+}
+
 template <int kPer, bool kCluster>
-__global__ void __launch_bounds__(kThreads, kPer > 8 ? 1 : 2)
-refine_select_kernel(const __grid_constant__ SelectArgs a, const __grid_constant__ Shape pl) {
+__global__ void __launch_bounds__(kThreads, 2) refine_select_kernel(const __grid_constant__ SelectArgs a, const __grid_constant__ Shape pl) {
+  constexpr int kV = kPer < 4 ? kPer : 4, kPieces = kPer / kV;
   __shared__ __align__(16) unsigned hist[kBins];
+  __shared__ __align__(16) unsigned coarse[kCluster ? kMaxCluster : 1][kCoarse];
   __shared__ __align__(16) unsigned list_key[kList + 4];
-  __shared__ unsigned scan_tot[2][kWarps], cta_count;
-  __shared__ uint2 red[kWarps], cta_max;              // largest filtered norm, largest raw (plus carried) score
-  __shared__ unsigned list_n, sh_bin, sh_need, sh_in_bin, sh_thr, sh_need_eq;
+  __shared__ unsigned scan_tot[2][kWarps], list_tot[kWarps];
+  __shared__ uint2 red[kWarps], cta_max[kMaxCluster];  // largest filtered norm, largest raw (plus carried) score
+  __shared__ unsigned list_n, sh_thr, sh_need_eq;
+  __shared__ Found sh_found;
   cg::cluster_group cl = cg::this_cluster();
   const int C = kCluster ? (int)cl.num_blocks() : 1, rank = kCluster ? (int)cl.block_rank() : 0;
   const int unit = kCluster ? blockIdx.x / C : blockIdx.x, n = pl.n, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int base = rank * a.chunk, end = min(base + a.chunk, n);
-  const int j0 = base + tid * kPer;                    // this thread's tokens: j0 .. j0 + kPer - 1, as far as below `end`
+  // This thread's tokens: kPieces times kV adjacent ones, those of a warp's lanes next to one another, j0 + q kStride + e
+  constexpr int kStride = 32 * kV;
+  const int j0 = base + warp * (32 * kPer) + lane * kV;
   const bool prior = a.nu != nullptr, vec = (n & 3) == 0;
   *reinterpret_cast<uint4*>(&hist[4 * tid]) = make_uint4(0, 0, 0, 0);
   if (tid == 0) list_n = 0;
+  if (kCluster) cl.barrier_arrive();                   // waited for before the first store into another CTA
   griddep_wait();
 
   // ---- this thread's tokens ----
-  float s[kPer], g[kPer], p[kPer];
+  const int bud = head_budget(pl, a.budgets, unit);
+  float s[kPer], g[kPer];
   float top = -INFINITY, m = 0.f;
+  const float* raw = a.s_raw + (size_t)unit * a.slots * n;
 #pragma unroll
-  for (int e = 0; e < kPer; ++e) { s[e] = 0.f; g[e] = 0.f; p[e] = 0.f; }
-  if (j0 < end) {
-    const float* raw = a.s_raw + (size_t)unit * a.slots * n;
-    load_run<kPer>(raw, j0, n, vec, s);
-    if (a.prev) load_run<kPer>(a.prev + (size_t)unit * n, j0, n, vec, p);
-    if (prior) {
-      const float* nu = a.nu + (size_t)unit * n;
-      const int half = pl.pool / 2;
-      const float inv_w = 1.f / (float)pl.pool;
-      const bool zero_pad = (pl.flags & AHAKV_FLAG_POOL_ZERO_PAD) != 0;
-      if (half == 3) {
-        // the usual width: the window's values read once, added in the order of pooled() (the zeros outside the head
-        // change nothing)
-        float w[kPer + 6], own[kPer];
-        load_run<kPer>(nu, j0, n, vec, own);
-        if (vec && kPer >= 4) {
-          const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
-          const float4 l = j0 >= 4 ? *reinterpret_cast<const float4*>(nu + j0 - 4) : z;
-          const float4 r = j0 + kPer + 4 <= n ? *reinterpret_cast<const float4*>(nu + j0 + kPer) : z;
-          w[0] = l.y; w[1] = l.z; w[2] = l.w;
-          w[kPer + 3] = r.x; w[kPer + 4] = r.y; w[kPer + 5] = r.z;
-        } else {
+  for (int q = 0; q < kPieces; ++q) load_piece<kV>(raw, j0 + q * kStride, end, vec, s + q * kV);
 #pragma unroll
-          for (int e = 0; e < 3; ++e) {
-            w[e] = j0 - 3 + e >= 0 ? nu[j0 - 3 + e] : 0.f;
-            w[kPer + 3 + e] = j0 + kPer + e < n ? nu[j0 + kPer + e] : 0.f;
-          }
-        }
+  for (int e = 0; e < kPer; ++e) g[e] = 0.f;
+  if (prior) {
+    const float* nu = a.nu + (size_t)unit * n;
+    const int half = pl.pool / 2;
+    const float inv_w = 1.f / (float)pl.pool;
+    const bool zero_pad = (pl.flags & AHAKV_FLAG_POOL_ZERO_PAD) != 0;
+    if (half == 3) {
+      // the usual width, added in the order of pooled() (the zeros outside the head change nothing).  A piece's neighbours
+      // are in the lanes beside it; only the warp's ends read again.
+      const int lim = min(end + 4, n);
+      float c[kPer];
 #pragma unroll
-        for (int e = 0; e < kPer; ++e) w[3 + e] = own[e];
+      for (int q = 0; q < kPieces; ++q) load_piece<kV>(nu, j0 + q * kStride, lim, vec, c + q * kV);
+      float el[3], er[3];
 #pragma unroll
-        for (int e = 0; e < kPer; ++e)
-          g[e] = (((((w[e] + w[e + 1]) + w[e + 2]) + w[e + 3]) + w[e + 4]) + w[e + 5]) + w[e + 6];
-        if ((j0 >= 3 && j0 + kPer + 3 <= n) || (zero_pad && j0 + kPer <= n)) {
-#pragma unroll
-          for (int e = 0; e < kPer; ++e) g[e] *= inv_w;
-        } else {                                       // near an end: over the taps inside the head
-#pragma unroll
-          for (int e = 0; e < kPer; ++e) {
-            const int taps = 7 - max(3 - j0 - e, 0) - max(j0 + e + 4 - n, 0);
-            g[e] = j0 + e >= n ? 0.f : taps == 7 || zero_pad ? g[e] * inv_w : g[e] / (float)taps;
-          }
-        }
-      } else {
-#pragma unroll
-        for (int e = 0; e < kPer; ++e)
-          if (j0 + e < n) g[e] = pooled_any(nu, j0 + e, n, half, inv_w, zero_pad);
+      for (int t = 0; t < 3; ++t) {
+        // kV < 4: a neighbour's values do not reach far enough, so every lane reads its own
+        const int jl = j0 - 3 + t, jr = j0 + (kPieces - 1) * kStride + kV + t;
+        el[t] = (kV < 4 || lane == 0) && jl >= 0 && jl < lim ? nu[jl] : 0.f;
+        er[t] = (kV < 4 || lane == 31) && jr < lim ? nu[jr] : 0.f;
       }
 #pragma unroll
-      for (int e = 0; e < kPer; ++e) m = fmaxf(m, g[e]);
+      for (int q = 0; q < kPieces; ++q) {
+        float w[kV + 6];
+#pragma unroll
+        for (int e = 0; e < kV; ++e) w[3 + e] = c[q * kV + e];
+#pragma unroll
+        for (int t = 0; t < 3; ++t) {
+          if (kV == 4) {
+            // lane 31's piece before is the left neighbour of lane 0's, lane 0's next one the right neighbour of lane 31's
+            const float l = c[q * kV + (1 + t) % kV], r = c[q * kV + t % kV];
+            const float gl = __shfl_sync(0xffffffffu, q > 0 && lane == 31 ? c[(q > 0 ? q - 1 : 0) * kV + (1 + t) % kV] : l, (lane + 31) & 31);
+            const float gr = __shfl_sync(0xffffffffu, q + 1 < kPieces && lane == 0 ? c[(q + 1 < kPieces ? q + 1 : q) * kV + t % kV] : r,
+                                         (lane + 1) & 31);
+            w[t] = q == 0 && lane == 0 ? el[t] : gl;
+            w[kV + 3 + t] = q == kPieces - 1 && lane == 31 ? er[t] : gr;
+          } else {
+            w[t] = el[t];
+            w[kV + 3 + t] = er[t];
+          }
+        }
+        const int j = j0 + q * kStride;
+        const bool inside = (j >= 3 && j + kV + 3 <= n) || (zero_pad && j + kV <= n);
+#pragma unroll
+        for (int e = 0; e < kV; ++e) {
+          const float x = (((((w[e] + w[e + 1]) + w[e + 2]) + w[e + 3]) + w[e + 4]) + w[e + 5]) + w[e + 6];
+          float y = x * inv_w;
+          if (!inside) {                               // near an end: over the taps inside the head
+            const int taps = 7 - max(3 - j - e, 0) - max(j + e + 4 - n, 0);
+            if (j + e >= n) y = 0.f;
+            else if (taps != 7 && !zero_pad) y = x / (float)taps;
+          }
+          if (j < end) {
+            g[q * kV + e] = y;
+            m = fmaxf(m, y);
+          }
+        }
+      }
+    } else {
+#pragma unroll
+      for (int e = 0; e < kPer; ++e) {
+        const int j = j0 + (e / kV) * kStride + e % kV;
+        if (j < end) g[e] = pooled_any(nu, j, n, half, inv_w, zero_pad);
+        m = fmaxf(m, g[e]);
+      }
     }
+  }
 #pragma unroll 1
-    for (int t = 1; t < a.slots; ++t) {                // in the order of combine_slots()
-      raw += n;
-      float x[kPer];
-      load_run<kPer>(raw, j0, n, vec, x);
+  for (int t = 1; t < a.slots; ++t) {                  // in the order of combine_slots()
+    raw += n;
+    float x[kPer];
 #pragma unroll
-      for (int e = 0; e < kPer; ++e) s[e] = pl.group_max ? fmaxf(s[e], x[e]) : s[e] + x[e];
+    for (int q = 0; q < kPieces; ++q) load_piece<kV>(raw, j0 + q * kStride, end, vec, x + q * kV);
+#pragma unroll
+    for (int e = 0; e < kPer; ++e) s[e] = pl.group_max ? fmaxf(s[e], x[e]) : s[e] + x[e];
+  }
+  // the carried scores: few tokens keep them, many read them again
+  constexpr int kHeld = kPer <= 8 ? kPer : 1;
+  float held[kHeld];
+  if (a.prev) {
+    float p[kPer];
+#pragma unroll
+    for (int q = 0; q < kPieces; ++q) load_piece<kV>(a.prev + (size_t)unit * n, j0 + q * kStride, end, vec, p + q * kV);
+#pragma unroll
+    for (int e = 0; e < kPer; ++e) {
+      if (j0 + (e / kV) * kStride + e % kV < end) top = fmaxf(top, s[e] + p[e]);
+      if (kPer <= 8) held[e % kHeld] = p[e];
     }
+  } else {
 #pragma unroll
-    for (int e = 0; e < kPer; ++e) top = fmaxf(top, s[e] + p[e]);
+    for (int e = 0; e < kPer; ++e)
+      if (j0 + (e / kV) * kStride + e % kV < end) top = fmaxf(top, s[e]);
   }
 
   // ---- head-wide maxima, as integers: the norms are not negative, so that their bits are ordered like they are, and the
@@ -203,72 +345,85 @@ refine_select_kernel(const __grid_constant__ SelectArgs a, const __grid_constant
     ktop = __reduce_max_sync(0xffffffffu, x.y);
   }
   if (kCluster) {
-    if (tid == 0) cta_max = make_uint2(mbits, ktop);
+    cl.barrier_wait();
+    if (warp == 0 && lane < C) *cl.map_shared_rank(&cta_max[rank], lane) = make_uint2(mbits, ktop);
     cl.sync();
-    const uint2 x = *cl.map_shared_rank(&cta_max, lane < C ? lane : 0);
+    const uint2 x = cta_max[lane < C ? lane : 0];
     mbits = __reduce_max_sync(0xffffffffu, x.x);
     ktop = __reduce_max_sync(0xffffffffu, x.y);
   }
 
   uint32_t key[kPer];
-  const float inv_gmax = prior ? __frcp_rn(__uint_as_float(mbits)) : 1.f;
+  if (prior) {
+    const float inv_gmax = __frcp_rn(__uint_as_float(mbits));
 #pragma unroll
-  for (int e = 0; e < kPer; ++e) {
-    if (prior) s[e] = __fmul_rn(__fmul_rn(g[e], inv_gmax), s[e]);
-    if (a.prev) s[e] = __fadd_rn(s[e], p[e]);
-    key[e] = order_key(s[e]);
+    for (int e = 0; e < kPer; ++e) s[e] = __fmul_rn(__fmul_rn(g[e], inv_gmax), s[e]);
   }
-  if (a.score && j0 < end) {
-    float* to = a.score + (size_t)unit * n + j0;
-    if (kPer >= 4 && vec && j0 + kPer <= n) {
+  if (a.prev) {
+    float p[kPer];
+    if (kPer > 8) {
 #pragma unroll
-      for (int e = 0; e < kPer; e += 4)
-        *reinterpret_cast<float4*>(to + e) = make_float4(s[e], s[(e + 1) % kPer], s[(e + 2) % kPer], s[(e + 3) % kPer]);
-    } else {
+      for (int q = 0; q < kPieces; ++q) load_piece<kV>(a.prev + (size_t)unit * n, j0 + q * kStride, end, vec, p + q * kV);
+    }
 #pragma unroll
-      for (int e = 0; e < kPer; ++e)
-        if (j0 + e < n) to[e] = s[e];
+    for (int e = 0; e < kPer; ++e) s[e] = __fadd_rn(s[e], kPer <= 8 ? held[e % kHeld] : p[e]);
+  }
+#pragma unroll
+  for (int e = 0; e < kPer; ++e) key[e] = order_key(s[e]);
+  if (a.score) {
+    float* to = a.score + (size_t)unit * n;
+#pragma unroll
+    for (int q = 0; q < kPieces; ++q) {
+      const int j = j0 + q * kStride;
+      if (kV == 4 && vec && j + 4 <= end) {
+        *reinterpret_cast<float4*>(to + j) = make_float4(s[q * kV], s[q * kV + 1 % kV], s[q * kV + 2 % kV], s[q * kV + 3 % kV]);
+      } else {
+#pragma unroll
+        for (int e = 0; e < kV; ++e)
+          if (j + e < end) to[j + e] = s[q * kV + e];
+      }
     }
   }
   if (a.kept == nullptr) {
     griddep_launch();
-    if (kCluster) cl.sync();
     return;
   }
+  // from here on the key stands for the score
 
   // ---- what is kept whatever the scores ----
   int32_t* out = a.kept + (size_t)unit * pl.n_keep;
   float* so = a.score_out ? a.score_out + (size_t)unit * pl.n_keep : nullptr;
-  const int bud = head_budget(pl, a.budgets, unit);
   if (rank == 0)
     for (int t = min(n, bud) + tid; t < pl.n_keep; t += kThreads) out[t] = -1;   // a head with a budget of its own
   const bool all = n <= bud;                                                   // nothing to evict
   const int n_cand = all ? 0 : n - pl.Br, Bs = all ? 0 : bud - pl.Br;
-  if (j0 < end && j0 + kPer > n_cand) {
+  if (end > n_cand) {
 #pragma unroll
     for (int e = 0; e < kPer; ++e) {
-      const int j = j0 + e;
-      if (j >= n_cand && j < n) {                      // all of them, or the recent window
+      const int j = j0 + (e / kV) * kStride + e % kV;
+      if (j >= n_cand && j < end) {                    // all of them, or the recent window
         out[Bs + j - n_cand] = j;
-        if (so) so[Bs + j - n_cand] = s[e];
+        if (so) so[Bs + j - n_cand] = key_to_float(key[e]);
       }
     }
   }
   if (Bs == 0) {
     griddep_launch();
-    if (!kCluster && a.k_out) gather_rows(a, pl, out, unit, min(n, bud));
-    if (kCluster) cl.sync();
+    if (!kCluster && a.k_out) gather_rows(a, pl, nullptr, unit, 0, n_cand, min(n, bud));
     return;
   }
 
   // ---- threshold ----
-  const int mine = j0 < end ? min(kPer, n_cand - j0) : 0;   // this thread's candidates: its first `mine` tokens
+  const int lim = min(end, n_cand) - j0;               // token (q, e) is a candidate if q kStride + e < lim
   // keys in [lo, hi] are still in question; bin b holds those with (key - lo) >> shift == b, the first histogram's lowest
   // bin everything below it too and its highest everything above
   const unsigned span = (unsigned)kBins << 16;
   unsigned lo = ktop > 0xfffdffffu ? 0xffffffffu - span + 1u : ktop + 0x20000u > span ? ktop + 0x20000u - span : 0u;
   unsigned hi = 0xffffffffu, need = (unsigned)Bs, thr = 0;
   int need_eq = 0, shift = 16;
+  // the CTAs before this one: candidates above the range, the equals that go with them, and how much of the list is theirs
+  unsigned above_before = 0, eq_before = 0, list_before = 0;
+  bool reads_open = kCluster;                          // others may still read this CTA's shared memory
   for (bool wide = true;; wide = false) {
     // `wide`: the first histogram, whose outer bins are open.  Its lowest bin, which may hold nearly everything, is
     // counted in registers: atomics on one address are served one after the other.
@@ -276,7 +431,7 @@ refine_select_kernel(const __grid_constant__ SelectArgs a, const __grid_constant
       unsigned low = 0;
 #pragma unroll
       for (int e = 0; e < kPer; ++e)
-        if (e < mine) {
+        if ((e / kV) * kStride + e % kV < lim) {
           const unsigned d = key[e] > lo ? (key[e] - lo) >> 16 : 0u;
           if (d == 0) ++low;
           else atomicAdd(&hist[min(d, (unsigned)kBins - 1u)], 1u);
@@ -286,32 +441,40 @@ refine_select_kernel(const __grid_constant__ SelectArgs a, const __grid_constant
     } else {
 #pragma unroll
       for (int e = 0; e < kPer; ++e)
-        if (e < mine && key[e] - lo <= hi - lo) atomicAdd(&hist[(key[e] - lo) >> shift], 1u);
-    }
-    if (kCluster) cl.sync(); else __syncthreads();
-    // thread t has bins 4 (511 - t) .. + 3, so that the prefix sum runs from the largest digit down
-    const int b4 = 4 * (kThreads - 1 - tid);
-    uint4 h = *reinterpret_cast<const uint4*>(&hist[b4]);
-    if (kCluster) {
-      for (int r = 1; r < C; ++r) {
-        const int other = rank + r < C ? rank + r : rank + r - C;   // each CTA starts with another neighbour
-        const uint4 x = *reinterpret_cast<const uint4*>(cl.map_shared_rank(&hist[b4], other));
-        h.x += x.x; h.y += x.y; h.z += x.z; h.w += x.w;
-      }
-    }
-    unsigned total;
-    const unsigned sum = h.x + h.y + h.z + h.w, above = block_scan(sum, scan_tot[0], total);
-    if (above < need && above + sum >= need) {          // exactly one thread
-      unsigned higher = above, in = h.w;
-      int d = b4 + 3;
-      if (higher + in < need) { higher += in; in = h.z; --d; }
-      if (higher + in < need && d == b4 + 2) { higher += in; in = h.y; --d; }
-      if (higher + in < need && d == b4 + 1) { higher += in; in = h.x; --d; }
-      sh_bin = (unsigned)d; sh_need = need - higher; sh_in_bin = in;
+        if ((e / kV) * kStride + e % kV < lim && key[e] - lo <= hi - lo) atomicAdd(&hist[(key[e] - lo) >> shift], 1u);
     }
     __syncthreads();
-    const unsigned bin = sh_bin, in_bin = sh_in_bin;
-    need = sh_need;
+    if (kCluster) {
+      // four threads hold sixteen bins; each gives their sum to a quarter of the cluster
+      const uint4 h = *reinterpret_cast<const uint4*>(&hist[4 * tid]);
+      unsigned sum = h.x + h.y + h.z + h.w;
+      sum += __shfl_xor_sync(0xffffffffu, sum, 1);
+      sum += __shfl_xor_sync(0xffffffffu, sum, 2);
+      for (int r = tid & 3; r < C; r += 4) *cl.map_shared_rank(&coarse[rank][tid >> 2], r) = sum;
+      cl.sync();
+      if (warp == 0) {
+        const Found f = find_in_cluster(cl, hist, coarse, need, C, rank);
+        if (lane == 0) sh_found = f;
+      }
+    } else {
+      // thread t has bins 4 (511 - t) .. + 3, so that the prefix sum runs from the largest digit down
+      const int b4 = 4 * (kThreads - 1 - tid);
+      const uint4 h = *reinterpret_cast<const uint4*>(&hist[b4]);
+      unsigned total;
+      const unsigned sum = h.x + h.y + h.z + h.w, above = block_scan(sum, scan_tot[0], total);
+      if (above < need && above + sum >= need) {        // exactly one thread
+        unsigned higher = above, in = h.w;
+        int d = b4 + 3;
+        if (higher + in < need) { higher += in; in = h.z; --d; }
+        if (higher + in < need && d == b4 + 2) { higher += in; in = h.y; --d; }
+        if (higher + in < need && d == b4 + 1) { higher += in; in = h.x; --d; }
+        sh_found = {(unsigned)d, need - higher, in, 0u, 0u};
+      }
+    }
+    __syncthreads();
+    const unsigned bin = sh_found.bin, in_bin = sh_found.in_bin, in_before = sh_found.in_before;
+    need = sh_found.need;
+    above_before += sh_found.above_before;
     {
       const unsigned first_key = lo + (bin << shift), last_key = first_key + ((1u << shift) - 1u);
       if (!(wide && bin == kBins - 1)) hi = min(hi, last_key);
@@ -320,27 +483,30 @@ refine_select_kernel(const __grid_constant__ SelectArgs a, const __grid_constant
     if (lo == hi) {                                     // one key is left
       thr = lo;
       need_eq = (int)need;
+      eq_before = in_before;
       break;
     }
     if (in_bin == need && lo != 0) {                    // the whole bin is kept: everything from its smallest key up
       thr = lo - 1;
+      above_before += in_before;
       break;
     }
     if (in_bin <= (unsigned)kList) {
-      // rank the bin's tokens against each other: the list of the cluster's first CTA, then a copy in every CTA
-      unsigned* ln = kCluster ? cl.map_shared_rank(&list_n, 0) : &list_n;
-      unsigned* lk = kCluster ? cl.map_shared_rank(list_key, 0) : list_key;
+      // rank the bin's tokens against each other: a list in every CTA, the tokens of one CTA behind those of the one before
+      if (tid < 4) list_key[in_bin + tid] = 0u;         // read four at a time; a zero is greater than nothing
 #pragma unroll
       for (int e = 0; e < kPer; ++e)
-        if (e < mine && key[e] - lo <= hi - lo) lk[atomicAdd(ln, 1u)] = key[e];
-      if (kCluster) {
-        cl.sync();
-        if (rank != 0 && tid < (int)in_bin) list_key[tid] = lk[tid];
-      } else {
-        __syncthreads();
-      }
-      if (tid < 4) list_key[in_bin + tid] = 0u;         // read four at a time; a zero is greater than nothing
-      __syncthreads();
+        if ((e / kV) * kStride + e % kV < lim && key[e] - lo <= hi - lo) {
+          const unsigned at = in_before + atomicAdd(&list_n, 1u);
+          if (kCluster) {
+            for (int r = 0; r < C; ++r) *cl.map_shared_rank(&list_key[at], r) = key[e];
+          } else {
+            list_key[at] = key[e];
+          }
+        }
+      if (kCluster) cl.sync(); else __syncthreads();
+      reads_open = false;
+      list_before = in_before;
       if (tid < (int)in_bin) {
         const unsigned k = list_key[tid];
         unsigned greater = 0, equal = 0;
@@ -364,43 +530,62 @@ refine_select_kernel(const __grid_constant__ SelectArgs a, const __grid_constant
     shift = max(0, 32 - __clz(hi - lo) - 11);
     __syncthreads();
   }
+  if (kCluster && reads_open) cl.barrier_arrive();
+  griddep_launch();
 
-  // ---- ordered emission: greater and equal counts of a thread in one word (a CTA has at most 8192 tokens) ----
-  unsigned own = 0;
+  // ---- ordered emission: a warp's tokens follow one another piece by piece, and in a piece lane by lane.  A byte counts a
+  // piece of up to 128 tokens, a half word a warp or a CTA (at most 8192) ----
+  unsigned own_gt = 0, own_eq = 0;
 #pragma unroll
   for (int e = 0; e < kPer; ++e)
-    if (e < mine) own += key[e] > thr ? 1u : key[e] == thr ? 1u << 16 : 0u;
-  unsigned total;
-  const unsigned before = block_scan(own, scan_tot[1], total);
-  int gt = (int)(before & 0xffffu), eq = (int)(before >> 16);
-  if (kCluster) {
-    if (tid == 0) cta_count = total;
-    cl.sync();
-    const unsigned x = lane < rank ? *cl.map_shared_rank(&cta_count, lane) : 0u;
-    gt += __reduce_add_sync(0xffffffffu, (int)(x & 0xffffu));
-    eq += __reduce_add_sync(0xffffffffu, (int)(x >> 16));
-    cl.barrier_arrive();                                // done with the others' shared memory
-  }
-  griddep_launch();
-  if (own != 0) {
-    // this thread's kept tokens follow one another: those above the threshold and the equals still wanted
-    const int at = gt + min(eq, need_eq), eq_end = need_eq - eq;
-    int seen_eq = 0, k = at;
+    if ((e / kV) * kStride + e % kV < lim) {
+      own_gt += key[e] > thr ? 1u << (8 * (e / kV)) : 0u;
+      own_eq += key[e] == thr ? 1u << (8 * (e / kV)) : 0u;
+    }
+  unsigned inc_gt = own_gt, inc_eq = own_eq;
 #pragma unroll
-    for (int e = 0; e < kPer; ++e) {
-      if (e < mine && key[e] >= thr) {
-        const bool keep = key[e] > thr || seen_eq < eq_end;
-        seen_eq += key[e] == thr;
-        if (keep) {
-          out[k] = j0 + e;
-          if (so) so[k] = s[e];
+  for (int o = 1; o < 32; o <<= 1) {
+    const unsigned x = __shfl_up_sync(0xffffffffu, inc_gt, o), y = __shfl_up_sync(0xffffffffu, inc_eq, o);
+    if (lane >= o) { inc_gt += x; inc_eq += y; }
+  }
+  const unsigned tot_gt = __shfl_sync(0xffffffffu, inc_gt, 31), tot_eq = __shfl_sync(0xffffffffu, inc_eq, 31);
+  unsigned listed = 0;                                 // of the list's part that belongs to the CTAs before
+  if (kCluster) {
+    if (tid < (int)list_before) listed = list_key[tid] > thr ? 1u : list_key[tid] == thr ? 1u << 16 : 0u;
+    listed = __reduce_add_sync(0xffffffffu, listed);
+  }
+  if (lane == 0) {
+    scan_tot[1][warp] = __dp4a(tot_gt, 0x01010101u, 0u) + (__dp4a(tot_eq, 0x01010101u, 0u) << 16);
+    list_tot[warp] = listed;
+  }
+  __syncthreads();
+  const unsigned before = __reduce_add_sync(0xffffffffu, (lane < warp ? scan_tot[1][lane & (kWarps - 1)] : 0u) +
+                                                             (kCluster && lane < kWarps ? list_tot[lane & (kWarps - 1)] : 0u));
+  int gt = (int)(above_before + (before & 0xffffu)), eq = (int)(eq_before + (before >> 16));
+#pragma unroll
+  for (int q = 0; q < kPieces; ++q) {
+    const unsigned og = own_gt >> (8 * q) & 0xffu, oe = own_eq >> (8 * q) & 0xffu;
+    if (og + oe) {
+      // the piece's kept tokens follow one another: those above the threshold and the equals still wanted
+      const int eb = eq + (int)(inc_eq >> (8 * q) & 0xffu) - (int)oe;
+      int k = gt + (int)(inc_gt >> (8 * q) & 0xffu) - (int)og + min(eb, need_eq), left = need_eq - eb;
+#pragma unroll
+      for (int e = 0; e < kV; ++e) {
+        const unsigned x = key[q * kV + e];
+        if (q * kStride + e < lim && (x > thr || (x == thr && left-- > 0))) {
+          const int j = j0 + q * kStride + e;
+          out[k] = j;
+          if (so) so[k] = key_to_float(x);
+          if (!kCluster && a.k_out) reinterpret_cast<unsigned short*>(hist)[k] = (unsigned short)j;
           ++k;
         }
       }
     }
+    gt += (int)(tot_gt >> (8 * q) & 0xffu);
+    eq += (int)(tot_eq >> (8 * q) & 0xffu);
   }
-  if (!kCluster && a.k_out) gather_rows(a, pl, out, unit, min(n, bud));
-  if (kCluster) cl.barrier_wait();                      // nobody leaves while its shared memory may still be read
+  if (!kCluster && a.k_out) gather_rows(a, pl, reinterpret_cast<const unsigned short*>(hist), unit, Bs, n_cand, min(n, bud));
+  if (kCluster && reads_open) cl.barrier_wait();        // nobody leaves while its shared memory may still be read
 }
 
 // The accumulated score without value prior: no head-wide maximum, so a plain sweep over all tokens.
@@ -575,8 +760,9 @@ cudaError_t launch_as(const SelectArgs& a, const Shape& pl, int C, cudaStream_t 
 // One cluster per head.  False: no cluster holds a head.
 bool launch_clustered(SelectArgs a, const Shape& pl, cudaStream_t st, cudaError_t* err) {
   if (pl.n > kMaxCluster * kThreads * kMaxPer) return false;   // 131072 tokens
-  // Eight tokens a thread and two CTAs an SM while all heads' clusters fit on the GPU at once; beyond that sixteen, whose
-  // smaller clusters exchange less (256 heads of 32768 tokens: 103 us against 115; 32 of 16384: 19 against 15).
+  // Eight tokens a thread while all heads' clusters fit on the GPU at once, two CTAs an SM; beyond that sixteen, with whose
+  // smaller clusters fewer CTAs go through the same steps (256 heads of 32768 tokens: 72 us against 94, and 106 with one
+  // such CTA an SM; 32 heads of 32768: 19 against 15; 4 of 70001: 21, before 26).
   const long long ctas8 = (long long)pl.B * pl.Hkv * ((pl.n + kThreads * 8 - 1) / (kThreads * 8));
   const int per_cta = kThreads * (ctas8 > 2 * 148 ? 16 : 8);
   int C = (pl.n + per_cta - 1) / per_cta;

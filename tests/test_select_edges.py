@@ -72,3 +72,18 @@ def test_refinement_in_the_eviction_call_equals_the_definition(n, pool, flags):
     for h in range(H):
         assert np.array_equal(idx[0, h].cpu().numpy(), _expected(sn[0, h], Br, Bud))
     assert torch.equal(s_out, score.gather(-1, idx.long()))
+
+
+@pytest.mark.parametrize("d,Bud", [(64, 9), (64, 255), (64, 257), (64, 500), (128, 129), (128, 250)])
+def test_rows_gathered_by_the_selecting_cta_are_the_kept_ones(d, Bud):
+    """Copies: bit for bit, also where a thread's last rows are fewer than it has in flight."""
+    from paper_2506_03762_b200 import binding as ab
+    B, H, n, r, Br = 2, 3, 1500, 16, 8
+    g = torch.Generator().manual_seed(Bud + d)
+    q, k, v = (torch.randn((B, H, m, d), generator=g).half().cuda() for m in (r, n, n))
+    p = ab.Params(B, H, H, d, n, r, Br, Bud, dtype=ab.F16, flags=1)
+    ws = ab.alloc_workspace(p)
+    k_out, v_out, s_out, idx = ab.alloc_outputs(p)
+    ab.ahakv_evict(p, q, k, v, None, k_out, v_out, s_out, idx, ws)
+    at = idx.long().unsqueeze(-1).expand(-1, -1, -1, d)
+    assert torch.equal(k_out, k.gather(2, at)) and torch.equal(v_out, v.gather(2, at))
