@@ -180,11 +180,9 @@ static ahakv_status queue_raw_score(const Plan& pl, const void* q, const void* k
   const bool prior = (pl.flags & AHAKV_FLAG_VALUE_PRIOR) != 0;
   float* nu = prior ? at<float>(ws, pl.off_nu) : nullptr;
   if (pl.use_tc) {
-    // status, counters and row offsets start as all ones: no error, -1, and NaN ("not published yet")
-    if (cudaMemsetAsync(at<char>(ws, pl.off_status), 0xff, pl.off_sraw - pl.off_status, st) != cudaSuccess)
-      return AHAKV_ERR_CUDA;
     // the kernel skips the tiles that no observation row sees: their raw score is zero
     if (pl.n_eff != pl.n && cudaMemsetAsync(s_raw, 0, pl.off_partial - pl.off_sraw, st) != cudaSuccess) return AHAKV_ERR_CUDA;
+    if ((rc = launch_clear(at<char>(ws, pl.off_status), pl.off_sraw - pl.off_status, st))) return rc;
     rc = launch_score_tc(pl, q, k, prior ? v : nullptr, s_raw, nu, at<float>(ws, pl.off_partial), final_off,
                          at<int>(ws, pl.off_sync), at<int>(ws, pl.off_status), st);
     profile_mark(prof, 1, st);

@@ -15,13 +15,14 @@ __global__ void __launch_bounds__(kThreads) compact_kernel(const char* __restric
                                                            const int32_t* __restrict__ kept, char* __restrict__ k_out,
                                                            char* __restrict__ v_out, float* __restrict__ score_out,
                                                            const Shape pl) {
+  griddep_wait();
   const long long total = (long long)pl.B * pl.Hkv * pl.n_keep;
   const long long stride = (long long)gridDim.x * (kThreads / LANES);
   const int lane = threadIdx.x % LANES;
   for (long long row = (long long)blockIdx.x * (kThreads / LANES) + threadIdx.x / LANES; row < total; row += stride) {
     const long long unit = row / pl.n_keep;
     const long long b = unit / pl.Hkv, h = unit % pl.Hkv;
-    const int j = kept[row];
+    const int j = __ldcg(kept + row);
     if (j < 0) continue;                       // a head with a budget of its own keeps fewer rows than the stride
     const long long ksrc = (b * pl.ks[0] + h * pl.ks[1] + (long long)j * pl.ks[2]) * pl.es + lane * 16;
     const long long vsrc = (b * pl.vs[0] + h * pl.vs[1] + (long long)j * pl.vs[2]) * pl.es + lane * 16;
@@ -30,7 +31,7 @@ __global__ void __launch_bounds__(kThreads) compact_kernel(const char* __restric
     const uint4 vv = *reinterpret_cast<const uint4*>(v + vsrc);
     *reinterpret_cast<uint4*>(k_out + dst) = kv;
     *reinterpret_cast<uint4*>(v_out + dst) = vv;
-    if (score_out && lane == 0) score_out[row] = score[unit * pl.n + j];
+    if (score_out && lane == 0) score_out[row] = __ldcg(score + unit * pl.n + j);
   }
 }
 
@@ -42,10 +43,12 @@ ahakv_status run(const Plan& pl, const void* k, const void* v, const float* scor
   long long blocks = (total + rows_per_block - 1) / rows_per_block;
   const long long cap = 148LL * 8 * 8;
   if (blocks > cap) blocks = cap;
-  compact_kernel<LANES><<<(unsigned)blocks, kThreads, 0, st>>>((const char*)k, (const char*)v, score, kept,
-                                                               (char*)k_out, (char*)v_out, score_out, pl);
+  // chained: its CTAs stand ready when the selection ends
+  const Shape& shape = pl;
+  const cudaError_t e = launch_chained(compact_kernel<LANES>, dim3((unsigned)blocks), dim3(kThreads), 1, 0, st, (const char*)k,
+                                       (const char*)v, score, kept, (char*)k_out, (char*)v_out, score_out, shape);
   count_launch();
-  return cuda_ok(cudaGetLastError());
+  return cuda_ok(e);
 }
 
 }  // namespace

@@ -39,8 +39,8 @@
 //
 // Between the passes: the delivery warp stores every run's row statistics as a partial and counts the run on its row
 // block's counter; whoever completes the count merges the partials of the whole row block, always in the order of the
-// runs (the result does not depend on who finished first), and publishes the rows' offsets, which start as NaN (the host
-// fills them before the launch): a reader knows an offset is there when it no longer reads NaN.
+// runs (the result does not depend on who finished first), and publishes the rows' offsets, which start as NaN (see
+// clear.cu): a reader knows an offset is there when it no longer reads NaN.
 //
 // The value rows stream past on the side: seven warps of every CTA read them straight from global memory, square and
 // add, nu_j = |V_j|^2.  They take no part in the schedule.  (Through shared memory the same stream cost the key tiles
@@ -661,6 +661,7 @@ score_tc_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_constant_
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   int p1_first = -1, p2_first = -1;
   if (warp == kSchedWarp && lane == 0) {   // the first two answers of the counters on their way too
+    griddep_wait();
     p1_first = atomicAdd(&a.ctr[0], 1) + 1;
     p2_first = atomicAdd(&a.ctr[1], 1) + 1;
   }
@@ -705,7 +706,7 @@ score_tc_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_constant_
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
   tc_fence_before();
-  __syncthreads();
+  __syncthreads();   // nobody touches memory before the scheduler warp's wait has ended
   tc_fence_after();
   const uint32_t tmem_base = sh->tmem_slot;
 
@@ -828,10 +829,10 @@ ahakv_status launch_score_tc(const Plan& pl, const void* q, const void* k, const
       !make_map(&kmap, k, a.bf16, pl.d, pl.n, pl.Hkv, pl.B, pl.ks, pl.es, kKeyTile, 1))
     return AHAKV_ERR_CUDA;
 
-  if (test) score_tc_kernel<true><<<grid, kThreads, kSmemBytes, st>>>(qmap, kmap, a);
-  else score_tc_kernel<false><<<grid, kThreads, kSmemBytes, st>>>(qmap, kmap, a);
+  const cudaError_t e = launch_chained(test ? score_tc_kernel<true> : score_tc_kernel<false>, dim3(grid), dim3(kThreads), 1, kSmemBytes, st,
+                                       qmap, kmap, a);
   count_launch();
-  return cuda_ok(cudaGetLastError());
+  return cuda_ok(e);
 }
 
 }  // namespace ahakv
