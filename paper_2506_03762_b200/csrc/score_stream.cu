@@ -253,18 +253,27 @@ __device__ __forceinline__ void mma_warp(const StreamArgs& a, Shared* sh, char* 
   });
 }
 
-// Like fold_chunk, with the sum T of 2^{x - M} (x - M) beside Z.  Masked values are finite and huge instead of -inf, so that
-// their terms of T are 0, not NaN.
-constexpr float kMasked = -1e30f;
-__device__ __forceinline__ void exp_sums32(const float* v, float c, float neg, float& z, float& t) {
+// Like fold_chunk, with the sum T of 2^{x - M} (x - M) beside Z.  Masked exponents are finite and huge instead of -inf, so
+// that their terms of T are 0, not NaN; the mask goes over the finished exponent, whatever the scale makes of a logit.
+constexpr float kMaskedExp = -1e30f;
+template <bool kMask>
+__device__ __forceinline__ void exp_sums32(const float* v, float c, float neg, int j_first, int last, float& z, float& t) {
   const uint64_t c2 = pack2(c, c), neg2 = pack2(neg, neg);
   uint64_t za = pack2(0.f, 0.f), zb = za, ta = za, tb = za;
 #pragma unroll
   for (int i = 0; i < 32; i += 4) {
-    const uint64_t xa = fma2(pack2(v[i], v[i + 1]), c2, neg2), xb = fma2(pack2(v[i + 2], v[i + 3]), c2, neg2);
+    uint64_t xa = fma2(pack2(v[i], v[i + 1]), c2, neg2), xb = fma2(pack2(v[i + 2], v[i + 3]), c2, neg2);
     float x0, x1, x2, x3;
     unpack2(xa, x0, x1);
     unpack2(xb, x2, x3);
+    if (kMask) {
+      if (j_first + i > last) x0 = kMaskedExp;
+      if (j_first + i + 1 > last) x1 = kMaskedExp;
+      if (j_first + i + 2 > last) x2 = kMaskedExp;
+      if (j_first + i + 3 > last) x3 = kMaskedExp;
+      xa = pack2(x0, x1);
+      xb = pack2(x2, x3);
+    }
     const uint64_t ea = pack2(fast_exp2(x0), fast_exp2(x1)), eb = pack2(fast_exp2(x2), fast_exp2(x3));
     za = add2(za, ea);
     zb = add2(zb, eb);
@@ -277,40 +286,42 @@ __device__ __forceinline__ void exp_sums32(const float* v, float c, float neg, f
   z = z0 + z1;
   t = t0 + t1;
 }
-__device__ __forceinline__ void fold_chunk_mean(const uint32_t* r, bool full, int j_first, int last, float c, float& M, float& Z,
-                                                float& T) {
-  float v[32];
+// Z and T of a row against its largest logit so far, v_max c.  The shift is the maximum itself and not, as where only Z is
+// wanted, a value near it: the leading term is then 1 exactly, and log2 Z of a row with one key that matters is as small as it
+// should be.  (Found before the exponentials, for 16 three-way maxima a chunk: with a second look only at chunks whose sum
+// says that something exceeded the shift, some row of a warp nearly always does, 135 us a call
+// of 64 heads x 128 rows x 32768 keys against 175.)  Where the shift is so large
+// that rounding it could move an exponential by more than 2^{1/16}, the logits are taken relative to v_max before they are scaled.
+constexpr float kWideShift = 1048576.f;   // 2^20
+template <bool kMask>
+__device__ __forceinline__ void fold_chunk_mean(const uint32_t* r, int j_first, int last, float c, float& v_max, float& Z, float& T) {
+  float v[32], top[4] = {v_max, -INFINITY, -INFINITY, -INFINITY};
 #pragma unroll
-  for (int t = 0; t < 32; ++t) v[t] = __uint_as_float(r[t]);
-  if (!full) {
-#pragma unroll
-    for (int t = 0; t < 32; ++t)
-      if (j_first + t > last) v[t] = kMasked;
+  for (int i = 0; i < 32; ++i) {
+    v[i] = __uint_as_float(r[i]);
+    if (!kMask || j_first + i <= last) top[i & 3] = fmaxf(top[i & 3], v[i]);
   }
-  if (M > -INFINITY) {
-    float z, t;
-    exp_sums32(v, c, -M, z, t);
-    if (z < kAcceptBelow) {
-      Z += z;
-      T += t;
-      return;
-    }
-  }
-  float mx = v[0];
-#pragma unroll
-  for (int t = 1; t < 32; ++t) mx = fmaxf(mx, v[t]);
-  if (mx > 0.1f * kMasked) {                         // first visible keys of the row, or the shift fell behind
-    mx *= c;
-    float z, t;
-    exp_sums32(v, c, -mx, z, t);
+  const float mx = fmaxf(fmaxf(top[0], top[1]), fmaxf(top[2], top[3]));
+  float neg = -mx * c;
+  const bool wide = fabsf(neg) > kWideShift;
+  if (mx > v_max) {
     if (Z > 0.f) {
-      const float s = fast_exp2(M - mx);
-      T = (T + Z * (M - mx)) * s;
+      const float d = wide ? (v_max - mx) * c : v_max * c + neg, s = fast_exp2(d);
+      T = (T + Z * d) * s;
       Z *= s;
     }
+    v_max = mx;
+  }
+  if (mx > -INFINITY) {
+    if (wide) {
+#pragma unroll
+      for (int i = 0; i < 32; ++i) v[i] -= mx;
+      neg = 0.f;
+    }
+    float z, t;
+    exp_sums32<kMask>(v, c, neg, j_first, last, z, t);
     Z += z;
     T += t;
-    M = mx;
   }
 }
 
@@ -380,7 +391,7 @@ __device__ __forceinline__ void softmax_group(const StreamArgs& a, Shared* sh, u
         min_last = w.fix_row;
       }
       const bool live = kMode == kRowStats || quarter * 32 < w.rows;
-      float M = -INFINITY, Z = 0.f, T = 0.f;
+      float M = -INFINITY, Z = 0.f, T = 0.f;         // entropy: M in units of the raw logit until the run is over
       for (int t = g; t < w.cnt; t += kGroups, ++mine) {
         const int acc = (tc0 + t) & 3;
         if (!mbar_wait(&sh->acc_full[g][mine & 3], (mine >> 2) & 1, a.status)) return false;
@@ -397,13 +408,15 @@ __device__ __forceinline__ void softmax_group(const StreamArgs& a, Shared* sh, u
               tc_fence_before();
               mbar_arrive(&sh->acc_empty[acc]);
             }
-            if (kMode == kEntropy) fold_chunk_mean(ra, full, j0 + 32 * ch, last, c, M, Z, T);
-            else fold_chunk(ra, full, j0 + 32 * ch, last, c, M, Z);
+            if (kMode != kEntropy) fold_chunk(ra, full, j0 + 32 * ch, last, c, M, Z);
+            else if (full) fold_chunk_mean<false>(ra, j0 + 32 * ch, last, c, M, Z, T);
+            else fold_chunk_mean<true>(ra, j0 + 32 * ch, last, c, M, Z, T);
           }
         } else {
           mbar_arrive(&sh->acc_empty[acc]);
         }
       }
+      if (kMode == kEntropy) M *= c;
       res = last < 0 ? -INFINITY : Z > 0.f ? M + log2f(Z) : Z == Z ? -INFINITY : Z;   // rows that do not exist weigh nothing
       if (kMode == kEntropy) res2 = Z > 0.f ? M + T / Z : 0.f;
     }

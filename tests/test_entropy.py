@@ -54,3 +54,21 @@ def test_entropy_tracks_eq10_on_gaussian_data():
     p12 = ab.Params(B, H, H, d, n, r, 16, Bud, dtype=ab.F16)                    # Eq. 12 per row
     H12 = float(ab.ahakv_row_entropy(p12, q, k).double().mean())
     assert abs(H12 - np.log(Bud)) < 0.35, (H12, np.log(Bud))
+
+
+@pytest.mark.parametrize("scale", [1e-30, 1e-12, 1e6, 1e9])
+def test_row_entropy_at_the_ends_of_the_scale(scale):
+    """A caller who tunes the scale may try any positive number.  A vanishing one makes every row uniform over the keys it sees
+    (H_i = ln i), a huge one concentrates it on a single key (H_i = 0); masked keys weigh nothing in either."""
+    from paper_2506_03762_b200 import binding as ab
+    d, n, r = 64, 700, 64
+    g = torch.Generator().manual_seed(11)
+    q = torch.randn((1, 2, r, d), generator=g).to(torch.float16).cuda()
+    k = torch.randn((1, 2, n, d), generator=g).to(torch.float16).cuda()
+    p = ab.Params(1, 2, 2, d, n, r, 4, 80, dtype=ab.F16, scale_mode=ab.SCALE_FIXED, scale=scale)
+    H = ab.ahakv_row_entropy(p, q, k).cpu().double()
+    if scale < 1:
+        want = torch.log(torch.arange(n - r + 1, n + 1, dtype=torch.float64)).expand_as(H)
+    else:
+        want = torch.zeros_like(H)
+    assert bool(((H - want).abs() < 1e-5).all()), (H - want).abs().max()
