@@ -1,7 +1,9 @@
 // Two walks over all tiles of a score matrix that, unlike the eviction score, need no second pass inside one kernel:
 //
 //   row statistics   per row of Q the log2 sum of 2^{c w} over the keys it sees, and for the row entropies (Eq. 6) the mean
-//                    of c w under the softmax: H_i = - sum_j a_ij ln a_ij = ln 2 (log2 sum - mean).
+//                    of x = c w - M under the softmax, M the row's largest c w: with Z = sum of 2^x and T = sum of 2^x x,
+//                    H_i = - sum_j a_ij ln a_ij = ln 2 (log2 Z - T / Z).  Parts of a row are kept as (M, Z, T) and merged by
+//                    differences of their M: a row's M may be hundreds, its entropy far below 1, and only differences may meet.
 //   column sums      the score accumulated over every causal row (Eq. 2-3): per key the sum over all later rows of
 //                    2^{c w - L}, L the row's statistic.
 //
@@ -45,7 +47,7 @@ struct StreamArgs {
   int BH, g0, gs, n_pad;
   const float* ctab;               // [n_pad] lambda log2(e) per row, zero past n
   float* stat;                     // row statistics, one float a row: entropy [unit][rpu][128]; causal [rpu][BH * gs][n_pad]
-  float* mean;                     // entropy: the means, like `stat`
+  float *z, *t;                    // entropy: `stat` has the M of every part and row, these its Z and T
   const float* neg_l;              // columns: [BH * gs][n_pad], -L per row, -inf past n
   float* s;                        // columns: [bh][split][n]
   int splits, accumulate;
@@ -57,7 +59,8 @@ struct StreamArgs {
 
 struct Shared {
   float tab_c[4][128], tab_l[4][128];       // columns: constants of the streamed rows, per accumulator
-  float stat[2][kGroups][128], mean[2][kGroups][128];   // by run parity: each group's share of a row's (a key's) result
+  float stat[2][kGroups][128];              // by run parity: each group's share of a row's (a key's) result
+  float z[2][kGroups][128], t[2][kGroups][128];   // entropy: Z and T beside it
   unsigned long long fix_full[2], fix_empty[2];
   unsigned long long str_full[kStages], str_empty[kStages];
   unsigned long long acc_empty[4];          // per accumulator
@@ -354,7 +357,7 @@ __device__ __forceinline__ void softmax_group(const StreamArgs& a, Shared* sh, u
   int tc0 = 0, mine = 0;   // tiles, own tiles so far
   for_each_run<kMode>(a, [&](const Work& w, int k) {
     if (k < 0) return true;
-    float res = 0.f, res2 = 0.f;
+    float res = 0.f, Z = 0.f, T = 0.f;
     if (kMode == kColumns) {
       for (int t = g; t < w.cnt; t += kGroups, ++mine) {
         const int acc = (tc0 + t) & 3;
@@ -391,7 +394,7 @@ __device__ __forceinline__ void softmax_group(const StreamArgs& a, Shared* sh, u
         min_last = w.fix_row;
       }
       const bool live = kMode == kRowStats || quarter * 32 < w.rows;
-      float M = -INFINITY, Z = 0.f, T = 0.f;         // entropy: M in units of the raw logit until the run is over
+      float M = -INFINITY;                           // entropy: M in units of the raw logit until the run is over
       for (int t = g; t < w.cnt; t += kGroups, ++mine) {
         const int acc = (tc0 + t) & 3;
         if (!mbar_wait(&sh->acc_full[g][mine & 3], (mine >> 2) & 1, a.status)) return false;
@@ -416,37 +419,42 @@ __device__ __forceinline__ void softmax_group(const StreamArgs& a, Shared* sh, u
           mbar_arrive(&sh->acc_empty[acc]);
         }
       }
-      if (kMode == kEntropy) M *= c;
-      res = last < 0 ? -INFINITY : Z > 0.f ? M + log2f(Z) : Z == Z ? -INFINITY : Z;   // rows that do not exist weigh nothing
-      if (kMode == kEntropy) res2 = Z > 0.f ? M + T / Z : 0.f;
+      if (kMode == kEntropy) res = last < 0 ? -INFINITY : M * c;
+      else res = last < 0 ? -INFINITY : Z > 0.f ? M + log2f(Z) : Z == Z ? -INFINITY : Z;   // rows that do not exist weigh nothing
     }
     tc0 += w.cnt;
     const int slot = k & 1;
     if (!mbar_wait(&sh->stat_empty[slot], ((k >> 1) & 1) ^ 1, a.status)) return false;
     sh->stat[slot][g][s] = res;
-    if (kMode == kEntropy) sh->mean[slot][g][s] = res2;
+    if (kMode == kEntropy) {
+      sh->z[slot][g][s] = Z;
+      sh->t[slot][g][s] = T;
+    }
     mbar_arrive(&sh->stat_full[slot]);
     return true;
   });
 }
 
-// (L, A) pairs -- log2 sums and means -- into one, in order.
+// (M, Z, T) of disjoint key sets into one, in order.  Nothing (Z = 0) weighs nothing; a NaN stays.
 template <int N>
-__device__ __forceinline__ void merge_means(const float (&l)[N], const float (&m)[N], float& M, float& W, float& S) {
-  float t = M;
+__device__ __forceinline__ void merge_parts(const float (&m)[N], const float (&z)[N], const float (&t)[N], float& M, float& Z, float& T) {
+  float top = M;
 #pragma unroll
-  for (int i = 0; i < N; ++i) t = fmaxf(t, l[i]);
-  if (t > -INFINITY) {
-    const float s = W > 0.f ? fast_exp2(M - t) : 0.f;
-    W *= s;
-    S *= s;
-#pragma unroll
-    for (int i = 0; i < N; ++i) {
-      const float e = fast_exp2(l[i] - t);
-      W += e;
-      S += e * m[i];
+  for (int i = 0; i < N; ++i) top = fmaxf(top, m[i]);
+  if (top > -INFINITY) {
+    if (Z != 0.f) {
+      const float d = M - top, s = fast_exp2(d);
+      T = (T + Z * d) * s;
+      Z *= s;
     }
-    M = t;
+#pragma unroll
+    for (int i = 0; i < N; ++i)
+      if (z[i] != 0.f) {
+        const float d = m[i] - top, s = fast_exp2(d);
+        T += (t[i] + z[i] * d) * s;
+        Z += z[i] * s;
+      }
+    M = top;
   }
 }
 
@@ -455,31 +463,32 @@ template <int kMode>
 __device__ __forceinline__ void delivery(const StreamArgs& a, Shared* sh) {
   const int lane = threadIdx.x & 31;
   for_each_run<kMode>(a, [&](const Work& w, int k) {
-    float v[4], m[4] = {};
+    float v[4], Z[4] = {}, T[4] = {};
     if (k >= 0) {
       const int slot = k & 1;
       if (!mbar_wait(&sh->stat_full[slot], (k >> 1) & 1, a.status)) return false;
 #pragma unroll
       for (int e = 0; e < 4; ++e) {
-        float x[kGroups], y[kGroups];
+        float x[kGroups], z[kGroups], t[kGroups];
 #pragma unroll
         for (int g = 0; g < kGroups; ++g) {
           x[g] = sh->stat[slot][g][4 * lane + e];
-          if (kMode == kEntropy) y[g] = sh->mean[slot][g][4 * lane + e];
+          if (kMode == kEntropy) {
+            z[g] = sh->z[slot][g][4 * lane + e];
+            t[g] = sh->t[slot][g][4 * lane + e];
+          }
         }
         if (kMode == kColumns) {
           v[e] = x[0];
 #pragma unroll
           for (int g = 1; g < kGroups; ++g) v[e] += x[g];
         } else if (kMode == kRowStats) {
-          float M = -INFINITY, Z = 0.f;
-          merge_logs(x, M, Z);
-          v[e] = M + log2f(Z);
+          float M = -INFINITY, sum = 0.f;
+          merge_logs(x, M, sum);
+          v[e] = M + log2f(sum);
         } else {
-          float M = -INFINITY, W = 0.f, S = 0.f;
-          merge_means(x, y, M, W, S);
-          v[e] = M + log2f(W);
-          m[e] = W > 0.f ? S / W : 0.f;
+          v[e] = -INFINITY;
+          merge_parts(x, z, t, v[e], Z[e], T[e]);
         }
       }
       mbar_arrive(&sh->stat_empty[slot]);
@@ -505,7 +514,8 @@ __device__ __forceinline__ void delivery(const StreamArgs& a, Shared* sh) {
     } else {
       const size_t at = ((size_t)w.unit * a.rpu + w.rin) * 128 + 4 * lane;
       *reinterpret_cast<float4*>(a.stat + at) = make_float4(v[0], v[1], v[2], v[3]);
-      *reinterpret_cast<float4*>(a.mean + at) = make_float4(m[0], m[1], m[2], m[3]);
+      *reinterpret_cast<float4*>(a.z + at) = make_float4(Z[0], Z[1], Z[2], Z[3]);
+      *reinterpret_cast<float4*>(a.t + at) = make_float4(T[0], T[1], T[2], T[3]);
     }
     return true;
   });
@@ -582,19 +592,22 @@ __global__ void __launch_bounds__(128) entropy_finish(const __grid_constant__ St
   const Work w = decode<kEntropy>(a, blockIdx.x * a.rpu);
   const int s = threadIdx.x;
   if (s >= w.rows) return;
-  float M = -INFINITY, W = 0.f, S = 0.f;
+  float M = -INFINITY, Z = 0.f, T = 0.f;
   const size_t at = (size_t)w.unit * a.rpu * 128 + s;
   for (int t0 = 0; t0 < a.rpu; t0 += 8) {
-    float l[8], m[8];
+    float m[8], z[8], t[8];
 #pragma unroll
-    for (int t = 0; t < 8; ++t) {
-      l[t] = t0 + t < a.rpu ? a.stat[at + (size_t)(t0 + t) * 128] : -INFINITY;
-      m[t] = t0 + t < a.rpu ? a.mean[at + (size_t)(t0 + t) * 128] : 0.f;
+    for (int i = 0; i < 8; ++i) {
+      const size_t from = at + (size_t)(t0 + i) * 128;
+      const bool there = t0 + i < a.rpu;
+      m[i] = there ? a.stat[from] : -INFINITY;
+      z[i] = there ? a.z[from] : 0.f;
+      t[i] = there ? a.t[from] : 0.f;
     }
-    merge_means(l, m, M, W, S);
+    merge_parts(m, z, t, M, Z, T);
   }
   const int head = a.r <= 128 ? w.fix_head + s / a.r : w.fix_head, i = a.r <= 128 ? s % a.r : w.fix_row + s;
-  out[((size_t)w.b * Hq + head) * a.r + i] = 0.6931471805599453f * (M + log2f(W) - S / W);
+  out[((size_t)w.b * Hq + head) * a.r + i] = 0.6931471805599453f * (log2f(Z) - T / Z);
 }
 
 // The parts of the causal rows' statistics into -L (-inf for rows that do not exist).
@@ -660,7 +673,7 @@ int entropy_parts(const Plan& pl) {
 }  // namespace
 
 size_t entropy_tc_scratch_bytes(const Plan& pl) {
-  return 256 + (size_t)pl.B * pl.Hkv * pl.n_rb * entropy_parts(pl) * 128 * 2 * sizeof(float);
+  return 256 + (size_t)pl.B * pl.Hkv * pl.n_rb * entropy_parts(pl) * 128 * 3 * sizeof(float);
 }
 
 ahakv_status launch_entropy_tc(const Plan& pl, const void* q, const void* k, void* scratch, float* out, cudaStream_t st) {
@@ -673,7 +686,8 @@ ahakv_status launch_entropy_tc(const Plan& pl, const void* q, const void* k, voi
   a.min_last = pl.last[0];
   a.status = (int*)scratch;                 // where a wait that runs out would leave word; nobody reads it
   a.stat = (float*)((char*)scratch + 256);
-  a.mean = a.stat + (size_t)units * a.rpu * 128;
+  a.z = a.stat + (size_t)units * a.rpu * 128;
+  a.t = a.z + (size_t)units * a.rpu * 128;
   for (int i = 0; i < kMaxRows; ++i) { a.c[i] = pl.rows.c[i]; a.last[i] = pl.last[i]; }
   CUtensorMap qmap, kmap;
   const int box_rows = pl.r <= 128 ? pl.r : 128, box_heads = pl.r <= 128 ? pl.heads_per_rb : 1;

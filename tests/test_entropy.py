@@ -72,3 +72,30 @@ def test_row_entropy_at_the_ends_of_the_scale(scale):
     else:
         want = torch.zeros_like(H)
     assert bool(((H - want).abs() < 1e-5).all()), (H - want).abs().max()
+
+
+@pytest.mark.parametrize("B,H,d,n,r,scale,sharp", [(1, 4, 128, 5000, 64, 0.3, 1.0), (1, 4, 64, 9000, 100, 1.0, 1.0), (2, 3, 128, 1100, 17, 1.0, 3.0),
+                                                   (1, 1, 64, 20000, 128, 0.02, 1.0)])
+def test_small_entropies_under_large_logits(B, H, d, n, r, scale, sharp):
+    """Rows whose largest logit is hundreds and whose entropy is far below 1, against a float64 evaluation.  The logits are sums
+    of d exact products in FP32, scaled in FP32: each is off by some ulps of its size, u = 2^-24 x (8 + |x| / ln 2) in the
+    exponent, and an entropy moves by at most the mean |x - E x| of its row, itself of the order of H + its spread, times that;
+    what comes on top is FP32 rounding of terms no larger than max(1, H).  Nothing may depend on the logits' own size beyond."""
+    from paper_2506_03762_b200 import binding as ab
+    g = torch.Generator().manual_seed(n)
+    q = (sharp * torch.randn((B, H, r, d), generator=g)).to(torch.float16).cuda()
+    k = torch.randn((B, H, n, d), generator=g).to(torch.float16).cuda()
+    p = ab.Params(B, H, H, d, n, r, 4, 80, dtype=ab.F16, scale_mode=ab.SCALE_FIXED, scale=scale)
+    got = ab.ahakv_row_entropy(p, q, k).double()
+    x = float(torch.tensor(scale, dtype=torch.float32)) * q.double() @ k.double().transpose(-1, -2)
+    seen = torch.arange(n, device="cuda") <= torch.arange(n - r, n, device="cuda").view(r, 1)
+    x = x.masked_fill(~seen, float("-inf"))
+    lse = x.logsumexp(-1, keepdim=True)
+    a = (x - lse).exp()
+    dev = (x - lse).masked_fill(~seen, 0)
+    want = -(a * dev).sum(-1)
+    spread = (a * (dev + want.unsqueeze(-1)).abs()).sum(-1)
+    size = x.amax(-1).abs() / 0.6931
+    bound = 2.0 ** -24 * (4 * (8 + size) * spread + 16 * want.clamp(min=1.0))
+    assert bool((got >= -2.0 ** -22).all())
+    assert bool(((got - want).abs() <= bound).all()), ((got - want).abs() / bound).max()
