@@ -169,7 +169,8 @@ ahakv_status ahakv_step_slots(const ahakv_params* p, const void* q_t, const void
  * observation row of every query head, with a_ij exactly as in ahakv_score (mask, lambda from scale_mode).  A
  * diagnostic: Eq. 10 predicts E[H_i] = ln i - lambda^2 d / 2, and Eq. 12 picks lambda so that this is ln(budget).
  * entropy: [B,Hq,r] float32 out.  ws: ahakv_entropy_workspace_bytes(p) bytes, 256-byte aligned (not the scoring
- * workspace).  16-bit inputs run on the tensor cores, float32 ones in double; it is not part of the eviction path. */
+ * workspace).  16-bit inputs run on the tensor cores, float32 ones in double; it is not part of the eviction path.
+ * ahakv_last_device_status reads the status word of this scratch too: after AHAKV_ERR_TIMEOUT the entropies are not valid. */
 size_t ahakv_entropy_workspace_bytes(const ahakv_params* p);
 ahakv_status ahakv_row_entropy(const ahakv_params* p, const void* q_obs, const void* k, float* entropy, void* ws,
                                size_t ws_bytes, ahakv_stream_t stream);
@@ -278,13 +279,13 @@ ahakv_status ahakv_static_last_device_status(ahakv_stream_t stream);
 ahakv_status ahakv_score_static(const ahakv_params* p, const void* q_obs, const void* k, const void* v,
                                 const float* score_prev, float* score, ahakv_stream_t stream);
 
-/* For tests of the failure path only (no counterpart in the paper).  Every wait inside the tensor-core scoring
- * kernel on something another thread, the copy engine, the tensor core or another CTA must deliver is bounded
+/* For tests of the failure path only (no counterpart in the paper).  Every wait inside the tensor-core
+ * kernels on something another thread, the copy engine, the tensor core or another CTA must deliver is bounded
  * (1 s); when one runs out the kernel records AHAKV_ERR_TIMEOUT in the workspace's status word and winds down
  * without trapping, so the context stays usable.  wait_ms > 0 shortens that limit for the launches that follow
  * (0 restores 1 s); withhold_first_partial != 0 plants the fault that makes a wait run out: the softmax
  * statistics of the first run of the first row block are never published, so whoever merges that row block waits
- * in vain.  While either is set, launches use a second instantiation of the same kernel code that takes the limit
+ * in vain (row entropies and the accumulation over all rows: one CTA's softmax warps never hand over their first run).  While either is set, launches use a second instantiation of the same kernel code that takes the limit
  * and the fault from its arguments; the instantiation every other call runs has neither.  Process-wide; not for
  * production use. */
 void ahakv_test_set_wait(int32_t wait_ms, int32_t withhold_first_partial);

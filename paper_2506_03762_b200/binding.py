@@ -248,15 +248,21 @@ def ahakv_step_slots(p: Params, q_t, k_t, v_t, k, v, score, pos, free_slot, stre
     return st
 
 
-def ahakv_row_entropy(p: Params, q_obs, k, entropy=None, stream=None):
-    """Eq. 6 entropy [B,Hq,r] (float32) of every observation row; allocates its scratch and, if not given, the output."""
-    nbytes = int(lib().ahakv_entropy_workspace_bytes(p.ref()))
-    if nbytes == 0:
-        raise AhakvError(ERR_INVALID_ARG, "ahakv_entropy_workspace_bytes")
-    ws = torch.empty(nbytes, dtype=torch.uint8, device=k.device)
+def ahakv_entropy_workspace_bytes(p: Params) -> int:
+    return int(lib().ahakv_entropy_workspace_bytes(p.ref()))
+
+
+def ahakv_row_entropy(p: Params, q_obs, k, entropy=None, stream=None, ws=None):
+    """Eq. 6 entropy [B,Hq,r] (float32) of every observation row; allocates the output and its scratch if not given (with a
+    scratch of its own a caller can read ``ahakv_last_device_status`` afterwards)."""
+    if ws is None:
+        nbytes = ahakv_entropy_workspace_bytes(p)
+        if nbytes == 0:
+            raise AhakvError(ERR_INVALID_ARG, "ahakv_entropy_workspace_bytes")
+        ws = torch.empty(nbytes, dtype=torch.uint8, device=k.device)
     if entropy is None:
         entropy = torch.empty((p.batch, p.n_q_heads, p.obs_window), dtype=torch.float32, device=k.device)
-    _raise(lib().ahakv_row_entropy(p.ref(), _ptr(q_obs), _ptr(k), _ptr(entropy), _ptr(ws), nbytes,
+    _raise(lib().ahakv_row_entropy(p.ref(), _ptr(q_obs), _ptr(k), _ptr(entropy), _ptr(ws), ws.nbytes,
                                    _stream(stream)), "ahakv_row_entropy")
     return entropy
 

@@ -62,7 +62,13 @@ ahakv_status launch_score_simt(const Plan& pl, const void* q, const void* k, con
 ahakv_status launch_score_tc(const Plan& pl, const void* q, const void* k, const void* v, float* s_raw, float* nu,
                              float* partial, float* off, int* counters, int* status, cudaStream_t st);
 bool score_tc_available();
-void score_tc_test_hooks(long long wait_ns, int withhold);   // see ahakv_test_set_wait
+// See ahakv_test_set_wait: the limit of the tensor-core kernels' bounded waits (0: their own), and whether a fault is planted.
+struct TestHooks {
+  long long wait_ns;
+  int withhold;
+};
+void set_test_hooks(long long wait_ns, int withhold);
+TestHooks test_hooks();
 // The generation phase one token at a time (decode.cu): the score update of one new query per head without
 // scratch memory, and compaction in place.
 bool step_score_fits(const Plan& pl);

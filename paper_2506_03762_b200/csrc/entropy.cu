@@ -16,6 +16,7 @@ namespace ahakv {
 namespace {
 
 constexpr int kThreads = 128;
+constexpr int kStatusBytes = 256;        // the status word, ahead of the partials
 
 template <typename T> using Acc = typename std::conditional<std::is_same<T, float>::value, double, float>::type;
 template <typename A> struct RowTable {
@@ -93,8 +94,9 @@ __global__ void __launch_bounds__(kThreads) entropy_tiles(const T* __restrict__ 
   }
 }
 
-__global__ void entropy_merge(const float4* __restrict__ partial, float* __restrict__ out, const Shape pl) {
+__global__ void entropy_merge(const float4* __restrict__ partial, float* __restrict__ out, int* __restrict__ status, const Shape pl) {
   const int uq = blockIdx.x;
+  if (uq == 0 && threadIdx.x == 0) *status = 0;                   // no waits on this path
   for (int i = threadIdx.x; i < pl.r; i += blockDim.x) {
     const float4* p = partial + (size_t)uq * pl.n_blk * pl.r + i;
     float M = -INFINITY;
@@ -113,7 +115,9 @@ __global__ void entropy_merge(const float4* __restrict__ partial, float* __restr
 }
 
 template <typename T, int D>
-ahakv_status run(const Plan& pl, const void* q, const void* k, float4* partial, float* out, cudaStream_t st) {
+ahakv_status run(const Plan& pl, const void* q, const void* k, void* scratch, float* out, cudaStream_t st) {
+  int* status = reinterpret_cast<int*>(scratch);
+  float4* partial = reinterpret_cast<float4*>((char*)scratch + kStatusBytes);
   RowTable<Acc<T>> rt;
   for (int i = 0; i < kMaxRows; ++i) {
     rt.c[i] = i < pl.r ? (Acc<T>)(pl.lambda[i] * 1.4426950408889634) : (Acc<T>)0;
@@ -124,7 +128,7 @@ ahakv_status run(const Plan& pl, const void* q, const void* k, float4* partial, 
     return AHAKV_ERR_CUDA;
   const Shape& shape = pl;
   entropy_tiles<T, D><<<dim3(pl.n_blk, pl.B * pl.Hq), kThreads, smem, st>>>((const T*)q, (const T*)k, partial, shape, rt);
-  entropy_merge<<<pl.B * pl.Hq, 256, 0, st>>>(partial, out, shape);
+  entropy_merge<<<pl.B * pl.Hq, 256, 0, st>>>(partial, out, status, shape);
   count_launch(2);
   return cuda_ok(cudaGetLastError());
 }
@@ -132,19 +136,18 @@ ahakv_status run(const Plan& pl, const void* q, const void* k, float4* partial, 
 }  // namespace
 
 size_t entropy_scratch_bytes(const Plan& pl) {
-  const size_t bytes = pl.use_tc ? entropy_tc_scratch_bytes(pl) : (size_t)pl.B * pl.Hq * pl.n_blk * pl.r * sizeof(float4);
+  const size_t bytes = pl.use_tc ? entropy_tc_scratch_bytes(pl) : kStatusBytes + (size_t)pl.B * pl.Hq * pl.n_blk * pl.r * sizeof(float4);
   return (bytes + 255) / 256 * 256;
 }
 
 ahakv_status launch_entropy(const Plan& pl, const void* q, const void* k, void* scratch, float* out, cudaStream_t st) {
   if (pl.use_tc) return launch_entropy_tc(pl, q, k, scratch, out, st);
-  float4* partial = reinterpret_cast<float4*>(scratch);
   const bool d64 = pl.d == 64;
   switch (pl.dtype) {
-    case AHAKV_F32: return d64 ? run<float, 64>(pl, q, k, partial, out, st) : run<float, 128>(pl, q, k, partial, out, st);
-    case AHAKV_F16: return d64 ? run<__half, 64>(pl, q, k, partial, out, st) : run<__half, 128>(pl, q, k, partial, out, st);
-    default: return d64 ? run<__nv_bfloat16, 64>(pl, q, k, partial, out, st)
-                        : run<__nv_bfloat16, 128>(pl, q, k, partial, out, st);
+    case AHAKV_F32: return d64 ? run<float, 64>(pl, q, k, scratch, out, st) : run<float, 128>(pl, q, k, scratch, out, st);
+    case AHAKV_F16: return d64 ? run<__half, 64>(pl, q, k, scratch, out, st) : run<__half, 128>(pl, q, k, scratch, out, st);
+    default: return d64 ? run<__nv_bfloat16, 64>(pl, q, k, scratch, out, st)
+                        : run<__nv_bfloat16, 128>(pl, q, k, scratch, out, st);
   }
 }
 

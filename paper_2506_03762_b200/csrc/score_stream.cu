@@ -52,7 +52,9 @@ struct StreamArgs {
   float* s;                        // columns: [bh][split][n]
   int splits, accumulate;
   float inv_g;
-  int* status;
+  int* status;                     // of the call; entropy: one word a CTA
+  long long test_wait_ns;          // test build of the kernel only: what every bounded wait allows
+  int test_withhold;               // test build only: the softmax warps of CTA 0 never hand their first run over
   float c[kMaxRows];               // entropy: lambda_i log2(e) per observation row
   int last[kMaxRows];              // and the last key it may see
 };
@@ -71,6 +73,16 @@ struct Shared {
   unsigned long long stat_full[2], stat_empty[2];
   uint32_t tmem_slot;
 };
+
+// Every wait is bounded; on expiry a role records AHAKV_ERR_TIMEOUT in the status word and leaves, and the others' own waits
+// run out in turn.  Like the scoring kernel this one exists twice, for the test of that (ahakv_test_set_wait).
+template <bool kTest> __device__ __forceinline__ long long wait_limit(const StreamArgs& a) {
+  return kTest ? a.test_wait_ns : kWaitLimitNs;
+}
+// Row entropies: no kernel runs before this one to clear a status word, so every CTA clears and keeps one of its own, and
+// entropy_finish gathers them into the first word of the scratch.
+constexpr int kStatusBytes = 1024;
+static_assert(kStatusBytes >= (1 + kSms) * (int)sizeof(int), "a word for the call and one for every CTA");
 
 constexpr int kOffFix = 0;
 constexpr int kOffStr = 2 * kTileBytes;
@@ -143,8 +155,8 @@ __device__ __forceinline__ void bulk_load(void* dst, const void* src, int bytes,
 }
 
 // ---- roles --------------------------------------------------------------------------------------------
-template <int kMode>
-__device__ __forceinline__ void producer(const StreamArgs& a, const CUtensorMap* fix, const CUtensorMap* str, Shared* sh, char* tiles) {
+template <int kMode, bool kTest>
+__device__ __forceinline__ void producer(const StreamArgs& a, int* status, const CUtensorMap* fix, const CUtensorMap* str, Shared* sh, char* tiles) {
   const int n_sub = a.D / 64;
   const int fix_bytes = n_sub * 128 * (kMode == kEntropy && a.r <= 128 ? a.hb * a.r : 128), str_bytes = n_sub * kSubTileBytes;
   int tc = 0;
@@ -152,7 +164,7 @@ __device__ __forceinline__ void producer(const StreamArgs& a, const CUtensorMap*
   for_each_run<kMode>(a, [&](const Work& w, int k) {
     if (k < 0) return true;
     const int fb = k & 1;
-    if (!(ok = mbar_wait(&sh->fix_empty[fb], ((k >> 1) & 1) ^ 1, a.status))) return false;
+    if (!(ok = mbar_wait(&sh->fix_empty[fb], ((k >> 1) & 1) ^ 1, status, wait_limit<kTest>(a)))) return false;
     mbar_expect_tx(&sh->fix_full[fb], fix_bytes);
     for (int s = 0; s < n_sub; ++s)
       tma_load_4d(tiles + kOffFix + fb * kTileBytes + s * kSubTileBytes, fix, &sh->fix_full[fb], s * 64, w.fix_row, w.fix_head, w.b);
@@ -167,7 +179,7 @@ __device__ __forceinline__ void producer(const StreamArgs& a, const CUtensorMap*
         head = w.fix_head / a.G;
       }
       const int stage = tc % kStages;
-      if (!(ok = mbar_wait(&sh->str_empty[stage], ((tc / kStages) & 1) ^ 1, a.status))) return false;
+      if (!(ok = mbar_wait(&sh->str_empty[stage], ((tc / kStages) & 1) ^ 1, status, wait_limit<kTest>(a)))) return false;
       mbar_expect_tx(&sh->str_full[stage], str_bytes);
       for (int s = 0; s < n_sub; ++s)
         tma_load_4d(tiles + kOffStr + stage * kTileBytes + s * kSubTileBytes, str, &sh->str_full[stage], s * 64, row, head, w.b);
@@ -189,7 +201,8 @@ __device__ __forceinline__ int take_turn(uint32_t& turns, int g) {
 }
 
 // Columns: the constants of every streamed tile's rows, into the place of the accumulator the tile will use.
-__device__ __forceinline__ void table_loader(const StreamArgs& a, Shared* sh) {
+template <bool kTest>
+__device__ __forceinline__ void table_loader(const StreamArgs& a, int* status, Shared* sh) {
   int tc = 0;
   uint32_t turns = 0;                       // two bits per group: its tiles so far, mod 4
   bool ok = true;
@@ -197,7 +210,7 @@ __device__ __forceinline__ void table_loader(const StreamArgs& a, Shared* sh) {
     if (k < 0) return true;
     for (int t = 0; t < w.cnt; ++t, ++tc) {
       const int acc = tc & 3, g = (w.first + t) / w.per_head, row = w.fix_row + (w.first + t - g * w.per_head) * 128;
-      if (!(ok = mbar_wait(&sh->acc_empty[acc], ((tc >> 2) & 1) ^ 1, a.status))) return false;
+      if (!(ok = mbar_wait(&sh->acc_empty[acc], ((tc >> 2) & 1) ^ 1, status, wait_limit<kTest>(a)))) return false;
       void* full = &sh->tab_full[t % kGroups][take_turn(turns, t % kGroups)];
       mbar_expect_tx(full, 2 * 512);
       bulk_load(sh->tab_c[acc], a.ctab + row, 512, full);
@@ -213,8 +226,8 @@ __device__ __forceinline__ void table_loader(const StreamArgs& a, Shared* sh) {
 
 // D[fixed rows x streamed rows].  The whole warp walks the runs, converged, and one elected lane issues; a tile's barriers
 // are tested while the tile before it is being issued.
-template <int kMode>
-__device__ __forceinline__ void mma_warp(const StreamArgs& a, Shared* sh, char* tiles, uint32_t tmem_base) {
+template <int kMode, bool kTest>
+__device__ __forceinline__ void mma_warp(const StreamArgs& a, int* status, Shared* sh, char* tiles, uint32_t tmem_base) {
   const int nk = a.D / 16;
   const uint32_t idesc = umma_idesc(128, 128, a.bf16);
   int tc = 0;
@@ -222,13 +235,13 @@ __device__ __forceinline__ void mma_warp(const StreamArgs& a, Shared* sh, char* 
   for_each_run<kMode>(a, [&](const Work& w, int k) {
     if (k < 0) return true;
     const int fb = k & 1, cnt = __shfl_sync(0xffffffffu, w.cnt, 0);
-    if (!__all_sync(0xffffffffu, mbar_wait(&sh->fix_full[fb], (k >> 1) & 1, a.status))) return false;
+    if (!__all_sync(0xffffffffu, mbar_wait(&sh->fix_full[fb], (k >> 1) & 1, status, wait_limit<kTest>(a)))) return false;
     const uint32_t a_lo = umma_desc_lo(smem_u32(tiles + kOffFix + fb * kTileBytes));
     bool s_ok = false, a_ok = false;
     for (int t = 0; t < cnt; ++t, ++tc) {
       const int stage = tc % kStages, acc = tc & 3;
-      if (!s_ok && !__all_sync(0xffffffffu, mbar_wait(&sh->str_full[stage], (tc / kStages) & 1, a.status))) return false;
-      if (!a_ok && !__all_sync(0xffffffffu, mbar_wait(&sh->acc_empty[acc], ((tc >> 2) & 1) ^ 1, a.status))) return false;
+      if (!s_ok && !__all_sync(0xffffffffu, mbar_wait(&sh->str_full[stage], (tc / kStages) & 1, status, wait_limit<kTest>(a)))) return false;
+      if (!a_ok && !__all_sync(0xffffffffu, mbar_wait(&sh->acc_empty[acc], ((tc >> 2) & 1) ^ 1, status, wait_limit<kTest>(a)))) return false;
       tc_fence_after();
       const uint32_t d_tmem = tmem_base + (uint32_t)(acc * 128);
       const uint32_t b_lo = umma_desc_lo(smem_u32(tiles + kOffStr + stage * kTileBytes));
@@ -350,8 +363,8 @@ __device__ __forceinline__ void column_chunk(const uint32_t* r, const float* c, 
 }
 
 // Softmax warps: groups of four warps, a thread per TMEM lane; tile t of a run belongs to group t mod kGroups.
-template <int kMode>
-__device__ __forceinline__ void softmax_group(const StreamArgs& a, Shared* sh, uint32_t tmem_base, int g) {
+template <int kMode, bool kTest>
+__device__ __forceinline__ void softmax_group(const StreamArgs& a, int* status, Shared* sh, uint32_t tmem_base, int g) {
   const int s = threadIdx.x & 127, quarter = (threadIdx.x >> 5) & 3;
   const uint32_t lane_base = tmem_base + ((uint32_t)(quarter * 32) << 16);
   int tc0 = 0, mine = 0;   // tiles, own tiles so far
@@ -361,8 +374,8 @@ __device__ __forceinline__ void softmax_group(const StreamArgs& a, Shared* sh, u
     if (kMode == kColumns) {
       for (int t = g; t < w.cnt; t += kGroups, ++mine) {
         const int acc = (tc0 + t) & 3;
-        if (!mbar_wait(&sh->tab_full[g][mine & 3], (mine >> 2) & 1, a.status)) return false;
-        if (!mbar_wait(&sh->acc_full[g][mine & 3], (mine >> 2) & 1, a.status)) return false;
+        if (!mbar_wait(&sh->tab_full[g][mine & 3], (mine >> 2) & 1, status, wait_limit<kTest>(a))) return false;
+        if (!mbar_wait(&sh->acc_full[g][mine & 3], (mine >> 2) & 1, status, wait_limit<kTest>(a))) return false;
         tc_fence_after();
         const bool diagonal = (w.first + t) % w.per_head == 0;
         uint64_t za = pack2(0.f, 0.f), zb = za;
@@ -397,7 +410,7 @@ __device__ __forceinline__ void softmax_group(const StreamArgs& a, Shared* sh, u
       float M = -INFINITY;                           // entropy: M in units of the raw logit until the run is over
       for (int t = g; t < w.cnt; t += kGroups, ++mine) {
         const int acc = (tc0 + t) & 3;
-        if (!mbar_wait(&sh->acc_full[g][mine & 3], (mine >> 2) & 1, a.status)) return false;
+        if (!mbar_wait(&sh->acc_full[g][mine & 3], (mine >> 2) & 1, status, wait_limit<kTest>(a))) return false;
         tc_fence_after();
         const int j0 = (w.first + t) * 128;
         const bool full = j0 + 127 <= min_last && j0 + 128 <= a.n;
@@ -424,13 +437,13 @@ __device__ __forceinline__ void softmax_group(const StreamArgs& a, Shared* sh, u
     }
     tc0 += w.cnt;
     const int slot = k & 1;
-    if (!mbar_wait(&sh->stat_empty[slot], ((k >> 1) & 1) ^ 1, a.status)) return false;
+    if (!mbar_wait(&sh->stat_empty[slot], ((k >> 1) & 1) ^ 1, status, wait_limit<kTest>(a))) return false;
     sh->stat[slot][g][s] = res;
     if (kMode == kEntropy) {
       sh->z[slot][g][s] = Z;
       sh->t[slot][g][s] = T;
     }
-    mbar_arrive(&sh->stat_full[slot]);
+    if (!(kTest && a.test_withhold && blockIdx.x == 0 && k == 0)) mbar_arrive(&sh->stat_full[slot]);
     return true;
   });
 }
@@ -459,14 +472,14 @@ __device__ __forceinline__ void merge_parts(const float (&m)[N], const float (&z
 }
 
 // Delivery warp: the groups' shares of a run, in order, into the run's result; lane l has rows (keys) 4 l .. 4 l + 3.
-template <int kMode>
-__device__ __forceinline__ void delivery(const StreamArgs& a, Shared* sh) {
+template <int kMode, bool kTest>
+__device__ __forceinline__ void delivery(const StreamArgs& a, int* status, Shared* sh) {
   const int lane = threadIdx.x & 31;
   for_each_run<kMode>(a, [&](const Work& w, int k) {
     float v[4], Z[4] = {}, T[4] = {};
     if (k >= 0) {
       const int slot = k & 1;
-      if (!mbar_wait(&sh->stat_full[slot], (k >> 1) & 1, a.status)) return false;
+      if (!mbar_wait(&sh->stat_full[slot], (k >> 1) & 1, status, wait_limit<kTest>(a))) return false;
 #pragma unroll
       for (int e = 0; e < 4; ++e) {
         float x[kGroups], z[kGroups], t[kGroups];
@@ -521,7 +534,7 @@ __device__ __forceinline__ void delivery(const StreamArgs& a, Shared* sh) {
   });
 }
 
-template <int kMode>
+template <int kMode, bool kTest>
 __global__ void __launch_bounds__(kThreads, 1)
 stream_kernel(const __grid_constant__ CUtensorMap fix, const __grid_constant__ CUtensorMap str, const __grid_constant__ StreamArgs a) {
   extern __shared__ char smem_raw[];
@@ -565,16 +578,22 @@ stream_kernel(const __grid_constant__ CUtensorMap fix, const __grid_constant__ C
   const uint32_t tmem_base = sh->tmem_slot;
   griddep_wait();
 
+  int* const status = kMode == kEntropy ? a.status + 1 + blockIdx.x : a.status;
+  if (kMode == kEntropy) {
+    if (threadIdx.x == 0) *status = 0;
+    __syncthreads();
+  }
+
   if (warp == 0) {
-    if (lane == 0) producer<kMode>(a, &fix, &str, sh, tiles);
+    if (lane == 0) producer<kMode, kTest>(a, status, &fix, &str, sh, tiles);
   } else if (warp == 1) {
-    mma_warp<kMode>(a, sh, tiles, __shfl_sync(0xffffffffu, tmem_base, 0));
+    mma_warp<kMode, kTest>(a, status, sh, tiles, __shfl_sync(0xffffffffu, tmem_base, 0));
   } else if (warp == 2) {
-    delivery<kMode>(a, sh);
+    delivery<kMode, kTest>(a, status, sh);
   } else if (warp == 3) {
-    if (kMode == kColumns && lane == 0) table_loader(a, sh);
+    if (kMode == kColumns && lane == 0) table_loader<kTest>(a, status, sh);
   } else {
-    softmax_group<kMode>(a, sh, tmem_base, (warp - 4) >> 2);
+    softmax_group<kMode, kTest>(a, status, sh, tmem_base, (warp - 4) >> 2);
   }
 
   tc_fence_before();
@@ -586,9 +605,15 @@ stream_kernel(const __grid_constant__ CUtensorMap fix, const __grid_constant__ C
   }
 }
 
-// The parts of a row block's statistics into the rows' entropies.
+// The parts of a row block's statistics into the rows' entropies, and the CTAs' status words into the call's.
 __global__ void __launch_bounds__(128) entropy_finish(const __grid_constant__ StreamArgs a, float* __restrict__ out, int Hq) {
   griddep_wait();
+  if (blockIdx.x == 0 && threadIdx.x < 32) {
+    bool expired = false;
+    for (int i = threadIdx.x; i < min(a.n_runs, kSms); i += 32) expired |= a.status[1 + i] == (int)AHAKV_ERR_TIMEOUT;
+    expired = __any_sync(0xffffffffu, expired);
+    if (threadIdx.x == 0) a.status[0] = expired ? (int)AHAKV_ERR_TIMEOUT : 0;
+  }
   const Work w = decode<kEntropy>(a, blockIdx.x * a.rpu);
   const int s = threadIdx.x;
   if (s >= w.rows) return;
@@ -641,7 +666,11 @@ __global__ void __launch_bounds__(256) row_scales(float* ctab, int n, int n_pad,
 
 // ---- host ------------------------------------------------------------------------------------------------
 template <int kMode>
-cudaError_t launch_stream(const CUtensorMap& fix, const CUtensorMap& str, const StreamArgs& a, cudaStream_t st) {
+cudaError_t launch_stream(const CUtensorMap& fix, const CUtensorMap& str, StreamArgs& a, cudaStream_t st) {
+  const TestHooks hooks = test_hooks();
+  const bool test = hooks.wait_ns > 0 || hooks.withhold != 0;
+  a.test_wait_ns = hooks.wait_ns > 0 ? hooks.wait_ns : kWaitLimitNs;
+  a.test_withhold = hooks.withhold;
   // leave to use more than 48 KB of shared memory, asked for once per device
   constexpr int kMaxDevices = 64;
   static bool configured[kMaxDevices] = {};
@@ -649,12 +678,13 @@ cudaError_t launch_stream(const CUtensorMap& fix, const CUtensorMap& str, const 
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess || dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
   if (!configured[dev]) {
-    e = cudaFuncSetAttribute(stream_kernel<kMode>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
+    e = cudaFuncSetAttribute(stream_kernel<kMode, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(stream_kernel<kMode, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
     if (e != cudaSuccess) return e;
     configured[dev] = true;
   }
   count_launch();
-  return launch_chained(stream_kernel<kMode>, dim3(a.n_runs < kSms ? a.n_runs : kSms), dim3(kThreads), 1, kSmemBytes, st, fix, str, a);
+  return launch_chained(test ? stream_kernel<kMode, true> : stream_kernel<kMode, false>, dim3(a.n_runs < kSms ? a.n_runs : kSms), dim3(kThreads), 1, kSmemBytes, st, fix, str, a);
 }
 
 // Parts per row block of the entropy's walk: the number that makes rounds x (tiles of a part + 1) smallest, a run boundary
@@ -673,7 +703,7 @@ int entropy_parts(const Plan& pl) {
 }  // namespace
 
 size_t entropy_tc_scratch_bytes(const Plan& pl) {
-  return 256 + (size_t)pl.B * pl.Hkv * pl.n_rb * entropy_parts(pl) * 128 * 3 * sizeof(float);
+  return kStatusBytes + (size_t)pl.B * pl.Hkv * pl.n_rb * entropy_parts(pl) * 128 * 3 * sizeof(float);
 }
 
 ahakv_status launch_entropy_tc(const Plan& pl, const void* q, const void* k, void* scratch, float* out, cudaStream_t st) {
@@ -684,8 +714,8 @@ ahakv_status launch_entropy_tc(const Plan& pl, const void* q, const void* k, voi
   const int units = pl.B * pl.Hkv * pl.n_rb;
   a.n_runs = units * a.rpu;
   a.min_last = pl.last[0];
-  a.status = (int*)scratch;                 // where a wait that runs out would leave word; nobody reads it
-  a.stat = (float*)((char*)scratch + 256);
+  a.status = (int*)scratch;
+  a.stat = (float*)((char*)scratch + kStatusBytes);
   a.z = a.stat + (size_t)units * a.rpu * 128;
   a.t = a.z + (size_t)units * a.rpu * 128;
   for (int i = 0; i < kMaxRows; ++i) { a.c[i] = pl.rows.c[i]; a.last[i] = pl.last[i]; }

@@ -749,14 +749,15 @@ score_tc_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_constant_
 
 bool score_tc_available() { return encode_fn() != nullptr; }
 
-// Test hooks (see ahakv_test_set_wait): the limit of the kernel's bounded waits, and a planted fault.  While either
-// is set, launches go to the test instantiation of the kernel.
+// Test hooks (see ahakv_test_set_wait): the limit of the bounded waits, and a planted fault.  While either is set, launches go
+// to the test instantiations of the kernels.
 static std::atomic<long long> g_test_wait_ns{0};
 static std::atomic<int> g_test_withhold{0};
-void score_tc_test_hooks(long long wait_ns, int withhold) {
+void set_test_hooks(long long wait_ns, int withhold) {
   g_test_wait_ns.store(wait_ns > 0 ? wait_ns : 0);
   g_test_withhold.store(withhold);
 }
+TestHooks test_hooks() { return {g_test_wait_ns.load(), g_test_withhold.load()}; }
 
 // How many runs a row block's key tiles are cut into.  A run boundary costs about as much as a tile visit (a Q tile to
 // load, statistics to hand over, constants to pick up), and the runs of all row blocks are dealt to the CTAs in rounds:
@@ -818,10 +819,10 @@ ahakv_status launch_score_tc(const Plan& pl, const void* q, const void* k, const
   for (int t = 0; t < 3; ++t) a.vs[t] = pl.vs[t] * pl.es;
   a.ctr = counters;
   a.status = status;
-  a.test_wait_ns = g_test_wait_ns.load();
-  a.test_withhold = g_test_withhold.load();
-  const bool test = a.test_wait_ns > 0 || a.test_withhold != 0;
-  if (a.test_wait_ns <= 0) a.test_wait_ns = kWaitLimitNs;
+  const TestHooks hooks = test_hooks();
+  const bool test = hooks.wait_ns > 0 || hooks.withhold != 0;
+  a.test_wait_ns = hooks.wait_ns > 0 ? hooks.wait_ns : kWaitLimitNs;
+  a.test_withhold = hooks.withhold;
 
   CUtensorMap qmap, kmap;
   const int q_box_rows = pl.r <= 128 ? pl.r : 128, q_box_heads = pl.r <= 128 ? pl.heads_per_rb : 1;

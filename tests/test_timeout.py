@@ -50,3 +50,59 @@ def test_a_wait_that_runs_out_is_reported_and_the_next_call_is_clean():
         ab.ahakv_test_set_wait(0, False)
     for a, b in zip(outs, clean):
         assert torch.equal(a, b)
+
+
+def _entropy_call(ab, dtype, n=9000):
+    g = torch.Generator().manual_seed(3)
+    q = torch.randn((2, 8, 32, 64), generator=g).to(dtype).cuda()
+    k = torch.randn((2, 4, n, 64), generator=g).to(dtype).cuda()
+    p = ab.Params(2, 8, 4, 64, n, 32, 4, 200, dtype=ab.DTYPE_CODE[dtype])
+    ws = torch.full((ab.ahakv_entropy_workspace_bytes(p),), ab.ERR_TIMEOUT, dtype=torch.uint8, device="cuda")
+    ws[1:4] = 0                                               # the status word of scratch that has been something else: 5
+    out = torch.zeros((2, 8, 32), device="cuda")
+    return lambda: (ab.ahakv_row_entropy(p, q, k, out, ws=ws), ab.ahakv_last_device_status(ws)), out
+
+
+def _causal_call(ab):
+    g = torch.Generator().manual_seed(4)
+    n = 3000
+    q = torch.randn((1, 8, n, 128), generator=g).to(torch.bfloat16).cuda()
+    k, v = (torch.randn((1, 4, n, 128), generator=g).to(torch.bfloat16).cuda() for _ in range(2))
+    p = ab.Params(1, 8, 4, 128, n, 64, 4, 200, dtype=ab.BF16)
+    ws = ab.alloc_workspace(p, "cuda")
+    out = torch.zeros((1, 4, n), device="cuda")
+    return lambda: (ab.ahakv_score_full_causal(p, q, k, v, None, out, ws), ab.ahakv_last_device_status(ws)), out
+
+
+def test_a_scratch_of_any_contents_gives_the_status_of_the_last_entropy_call():
+    from paper_2506_03762_b200 import binding as ab
+    for dtype in (torch.float16, torch.float32):
+        call, out = _entropy_call(ab, dtype, 700)
+        assert call()[1] == ab.OK
+        assert bool((out > 0).all())
+
+
+@pytest.mark.parametrize("which", ["entropy", "causal"])
+def test_waits_of_the_streaming_kernel_are_reported_and_the_next_call_is_clean(which):
+    from paper_2506_03762_b200 import binding as ab
+    call, out = _entropy_call(ab, torch.float16) if which == "entropy" else _causal_call(ab)
+    assert call()[1] == ab.OK
+    clean = out.clone()
+    try:
+        ab.ahakv_test_set_wait(20, True)
+        t0, t1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        t0.record()
+        status = call()[1]
+        t1.record()
+        torch.cuda.synchronize()
+        assert status == ab.ERR_TIMEOUT
+        assert t0.elapsed_time(t1) < 2000.0                   # a few wait limits, not a hang
+        ab.ahakv_test_set_wait(50, False)                     # a short limit alone changes nothing
+        out.zero_()
+        assert call()[1] == ab.OK
+        assert torch.equal(out, clean)
+    finally:
+        ab.ahakv_test_set_wait(0, False)
+    out.zero_()
+    assert call()[1] == ab.OK
+    assert torch.equal(out, clean)
