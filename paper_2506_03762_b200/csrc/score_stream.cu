@@ -688,12 +688,13 @@ cudaError_t launch_stream(const CUtensorMap& fix, const CUtensorMap& str, Stream
 }
 
 // Parts per row block of the entropy's walk: the number that makes rounds x (tiles of a part + 1) smallest, a run boundary
-// costing about a tile; at most 64.
+// costing about a tile; at most 64, and at most sixteen rounds of runs.
+constexpr int kMaxParts = 64, kMaxPartRuns = 16 * kSms;
 int entropy_parts(const Plan& pl) {
   const long long units = (long long)pl.B * pl.Hkv * pl.n_rb;
   int best = 1;
   long long best_cost = -1;
-  for (int p = 1; p <= pl.n_blk && p <= 64; ++p) {
+  for (int p = 1; p <= pl.n_blk && p <= kMaxParts && (p == 1 || units * p <= kMaxPartRuns); ++p) {
     const long long cost = (units * p + kSms - 1) / kSms * ((pl.n_blk + p - 1) / p + 1);
     if (best_cost < 0 || cost < best_cost) { best = p; best_cost = cost; }
   }
@@ -702,8 +703,13 @@ int entropy_parts(const Plan& pl) {
 
 }  // namespace
 
+// Room for as many parts as any call with these row blocks and tiles, or fewer, may be cut into: a larger batch or a longer
+// context may want fewer parts, but scratch that was sized for it has to serve the smaller calls too.  One part more than
+// there can be covers what a call with fewer than 128 keys keeps (entropy.cu: 16 bytes a row).
 size_t entropy_tc_scratch_bytes(const Plan& pl) {
-  return kStatusBytes + (size_t)pl.B * pl.Hkv * pl.n_rb * entropy_parts(pl) * 128 * 3 * sizeof(float);
+  const size_t units = (size_t)pl.B * pl.Hkv * pl.n_rb, most = units * (pl.n_blk < kMaxParts ? pl.n_blk : kMaxParts);
+  const size_t runs = most < kMaxPartRuns ? most : units > kMaxPartRuns ? units : kMaxPartRuns;
+  return kStatusBytes + (runs + units) * 128 * 3 * sizeof(float);
 }
 
 ahakv_status launch_entropy_tc(const Plan& pl, const void* q, const void* k, void* scratch, float* out, cudaStream_t st) {

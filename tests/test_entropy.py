@@ -99,3 +99,20 @@ def test_small_entropies_under_large_logits(B, H, d, n, r, scale, sharp):
     bound = 2.0 ** -24 * (4 * (8 + size) * spread + 16 * want.clamp(min=1.0))
     assert bool((got >= -2.0 ** -22).all())
     assert bool(((got - want).abs() <= bound).all()), ((got - want).abs() / bound).max()
+
+
+def test_entropy_scratch_for_a_large_call_serves_the_smaller_ones():
+    """Scratch sized for the largest batch and context a caller has must do for every smaller call."""
+    from paper_2506_03762_b200 import binding as ab
+    def need(B, n, r, dtype, G=4):
+        return ab.ahakv_entropy_workspace_bytes(ab.Params(B, 4 * G, 4, 128, n, r, 0, 64, dtype=dtype))
+    for dtype in (ab.F16, ab.F32):
+        for n in (64, 127, 128, 300, 1000, 4096, 30000):
+            for r in (1, 16, 33, 64):
+                sizes = [need(B, n, r, dtype) for B in range(1, 161)]
+                assert sizes == sorted(sizes), (dtype, n, r)
+        for B in (1, 5, 9, 37, 40, 150):
+            sizes = [need(B, n, 32, dtype) for n in (*range(32, 1200, 31), 3000, 8000, 8192, 20000, 70000)]
+            assert sizes == sorted(sizes), (dtype, B)
+            sizes = [need(B, 5000, r, dtype) for r in range(1, 65)]
+            assert sizes == sorted(sizes), (dtype, B)
