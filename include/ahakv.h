@@ -75,7 +75,9 @@ typedef struct {
   int64_t q_stride[3], k_stride[3], v_stride[3]; /* elements: batch, head, token; all 0 = dense default */
 } ahakv_params;
 
-/* Bytes of scratch the other entry points need for these parameters (0 if they are invalid).
+/* Bytes of scratch the other entry points make use of for these parameters (0 if they are invalid).  Scratch sized for one
+ * call serves every call of no larger batch, context, heads and rows too, also where this function asks for more there:
+ * float32 calls use room for softmax numerators while that is moderate, and form the logits twice without it.
  * The pointer handed in as `ws` must be 256-byte aligned.  The scratch holds no state between
  * calls, but two calls that overlap on the GPU must not share it. */
 size_t ahakv_workspace_bytes(const ahakv_params* p);
@@ -259,8 +261,8 @@ const char* ahakv_stage_name(int stage);
  *
  * Computes exactly what ahakv_score computes, with the same kernels; the caller passes inputs and
  * outputs only.  Nothing is allocated or freed, by this call or by anything it calls.
- *  - Limit: ahakv_workspace_bytes(p) (for float32 inputs: what it returns less the room for softmax numerators, which a
- *    call can do without) must not exceed AHAKV_STATIC_WS_BYTES (ahakv_static_workspace_bytes()
+ *  - Limit: ahakv_workspace_bytes(p) (for float32 inputs: what it returns less the room for softmax numerators, without
+ *    which a call takes longer) must not exceed AHAKV_STATIC_WS_BYTES (ahakv_static_workspace_bytes()
  *    returns it at run time); larger problems get AHAKV_ERR_WORKSPACE and nothing is launched.  8 MiB
  *    covers, for instance, one sequence of 8 KV heads x 16384 tokens (3.5 MiB), 32 heads x 4096 tokens
  *    (2 MiB) or a 16-sequence decode round of 8 KV heads x 2080 tokens (5.3 MiB); 32 heads x 16384

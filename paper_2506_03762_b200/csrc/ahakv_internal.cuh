@@ -49,9 +49,6 @@ struct Plan : Shape {
 // last r positions.
 ahakv_status make_plan(const ahakv_params* p, Plan* plan, const int64_t* obs_pos = nullptr);
 void count_launch(int n = 1);
-// ahakv_score with a workspace that need not have room for kept numerators.
-ahakv_status score_in_least_room(const ahakv_params* p, const void* q_obs, const void* k, const void* v, const float* score_prev,
-                                 float* score, void* ws, size_t ws_bytes, cudaStream_t st);
 
 // Launchers.  Each returns AHAKV_OK or AHAKV_ERR_CUDA and queues work on `st` only.
 // Both also stream V and write nu when the value prior is on (v and nu non-null), and clear the status word.

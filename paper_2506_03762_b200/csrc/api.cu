@@ -160,9 +160,10 @@ static ahakv_status plan_for(const ahakv_params* p, const Plan** out) {
 
 static bool aligned16(const void* p) { return ((uintptr_t)p & 15) == 0; }
 
-// `least`: be content with what the call cannot do without.
-static ahakv_status check_ws(const Plan& pl, void* ws, size_t ws_bytes, bool least = false) {
-  if (!ws || ((uintptr_t)ws & 255) != 0 || ws_bytes < (least ? pl.ws_total : pl.ws_wanted)) return AHAKV_ERR_WORKSPACE;
+// What a call cannot do without; it grows with the batch, the context and the rows, so that scratch sized for a large call serves
+// the smaller ones.  (The room for kept numerators does not, see make_plan, and is used where it is there.)
+static ahakv_status check_ws(const Plan& pl, void* ws, size_t ws_bytes) {
+  if (!ws || ((uintptr_t)ws & 255) != 0 || ws_bytes < pl.ws_total) return AHAKV_ERR_WORKSPACE;
   return AHAKV_OK;
 }
 
@@ -215,8 +216,7 @@ double ahakv_lambda(int64_t n_total, int32_t budget, int32_t head_dim) {
 }
 
 static ahakv_status score_impl(const ahakv_params* p, const int64_t* obs_pos, const void* q_obs, const void* k,
-                               const void* v, const float* score_prev, float* score, void* ws, size_t ws_bytes, bool least,
-                               cudaStream_t st) {
+                               const void* v, const float* score_prev, float* score, void* ws, size_t ws_bytes, cudaStream_t st) {
   Plan own;
   const Plan* plan = &own;
   ahakv_status rc = obs_pos ? make_plan(p, &own, obs_pos) : plan_for(p, &plan);
@@ -227,7 +227,7 @@ static ahakv_status score_impl(const ahakv_params* p, const int64_t* obs_pos, co
   if (!aligned16(q_obs) || !aligned16(k) || (v && !aligned16(v)) || !aligned16(score) ||
       (score_prev && !aligned16(score_prev)))
     return AHAKV_ERR_INVALID_ARG;
-  if ((rc = check_ws(pl, ws, ws_bytes, least))) return rc;
+  if ((rc = check_ws(pl, ws, ws_bytes))) return rc;
   const int prof = profile_begin_call(st);
   if ((rc = queue_raw_score(pl, q_obs, k, v, ws, ws_bytes, st, prof))) return rc;
   rc = launch_refine(pl, at<float>(ws, pl.off_sraw), prior ? at<float>(ws, pl.off_nu) : nullptr, score_prev, score,
@@ -241,23 +241,14 @@ static ahakv_status score_impl(const ahakv_params* p, const int64_t* obs_pos, co
 ahakv_status ahakv_score(const ahakv_params* p, const void* q_obs, const void* k, const void* v,
                          const float* score_prev, float* score, void* ws, size_t ws_bytes,
                          ahakv_stream_t stream) {
-  return score_impl(p, nullptr, q_obs, k, v, score_prev, score, ws, ws_bytes, false, (cudaStream_t)stream);
+  return score_impl(p, nullptr, q_obs, k, v, score_prev, score, ws, ws_bytes, (cudaStream_t)stream);
 }
-
-}  // extern "C"
-
-ahakv_status ahakv::score_in_least_room(const ahakv_params* p, const void* q_obs, const void* k, const void* v, const float* score_prev,
-                                        float* score, void* ws, size_t ws_bytes, cudaStream_t st) {
-  return score_impl(p, nullptr, q_obs, k, v, score_prev, score, ws, ws_bytes, true, st);
-}
-
-extern "C" {
 
 ahakv_status ahakv_score_rows(const ahakv_params* p, const int64_t* obs_pos, const void* q_obs, const void* k,
                               const void* v, const float* score_prev, float* score, void* ws, size_t ws_bytes,
                               ahakv_stream_t stream) {
   if (!obs_pos) return AHAKV_ERR_INVALID_ARG;
-  return score_impl(p, obs_pos, q_obs, k, v, score_prev, score, ws, ws_bytes, false, (cudaStream_t)stream);
+  return score_impl(p, obs_pos, q_obs, k, v, score_prev, score, ws, ws_bytes, (cudaStream_t)stream);
 }
 
 ahakv_status ahakv_score_full_causal(const ahakv_params* p, const void* q_all, const void* k, const void* v,
@@ -405,7 +396,7 @@ ahakv_status ahakv_compact(const ahakv_params* p, const void* k, const void* v, 
 
 static ahakv_status evict_impl(const ahakv_params* p, const int32_t* budgets, const void* q_obs, const void* k,
                                const void* v, const float* score_prev, void* k_out, void* v_out, float* score_out,
-                               int32_t* kept_idx, void* ws, size_t ws_bytes, bool least, ahakv_stream_t stream) {
+                               int32_t* kept_idx, void* ws, size_t ws_bytes, ahakv_stream_t stream) {
   const Plan* plan;
   ahakv_status rc = plan_for(p, &plan);
   if (rc) return rc;
@@ -414,7 +405,7 @@ static ahakv_status evict_impl(const ahakv_params* p, const int32_t* budgets, co
   if (!aligned16(q_obs) || !aligned16(k) || !aligned16(v) || !aligned16(k_out) || !aligned16(v_out) ||
       ((uintptr_t)kept_idx & 3) || (score_prev && !aligned16(score_prev)))
     return AHAKV_ERR_INVALID_ARG;
-  if ((rc = check_ws(pl, ws, ws_bytes, least))) return rc;
+  if ((rc = check_ws(pl, ws, ws_bytes))) return rc;
   cudaStream_t st = (cudaStream_t)stream;
   TraceRange call("ahakv_evict");
   const int prof = profile_begin_call(st);
@@ -443,7 +434,7 @@ static ahakv_status evict_impl(const ahakv_params* p, const int32_t* budgets, co
 ahakv_status ahakv_evict(const ahakv_params* p, const void* q_obs, const void* k, const void* v,
                          const float* score_prev, void* k_out, void* v_out, float* score_out,
                          int32_t* kept_idx, void* ws, size_t ws_bytes, ahakv_stream_t stream) {
-  return evict_impl(p, nullptr, q_obs, k, v, score_prev, k_out, v_out, score_out, kept_idx, ws, ws_bytes, false, stream);
+  return evict_impl(p, nullptr, q_obs, k, v, score_prev, k_out, v_out, score_out, kept_idx, ws, ws_bytes, stream);
 }
 
 ahakv_status ahakv_evict_head_budgets(const ahakv_params* p, const int32_t* head_budget, const void* q_obs, const void* k,
@@ -451,7 +442,7 @@ ahakv_status ahakv_evict_head_budgets(const ahakv_params* p, const int32_t* head
                                       float* score_out, int32_t* kept_idx, void* ws, size_t ws_bytes,
                                       ahakv_stream_t stream) {
   if (!head_budget || ((uintptr_t)head_budget & 3)) return AHAKV_ERR_INVALID_ARG;
-  return evict_impl(p, head_budget, q_obs, k, v, score_prev, k_out, v_out, score_out, kept_idx, ws, ws_bytes, false, stream);
+  return evict_impl(p, head_budget, q_obs, k, v, score_prev, k_out, v_out, score_out, kept_idx, ws, ws_bytes, stream);
 }
 
 ahakv_status ahakv_evict_ragged(const ahakv_params* p, const ahakv_seq* seqs, const void* q_obs, const void* k,
@@ -482,7 +473,7 @@ ahakv_status ahakv_evict_ragged(const ahakv_params* p, const ahakv_seq* seqs, co
     const char* vb = (const char*)v + (size_t)b * outer.vs[0] * es;
     const size_t tok = (size_t)b * outer.Hkv * outer.n, kept = (size_t)b * outer.Hkv * keep_max;
     rc = evict_impl(&pb, nullptr, qb, kb, vb, score_prev ? score_prev + tok : nullptr, (char*)k_out + kept * row,
-                    (char*)v_out + kept * row, score_out ? score_out + kept : nullptr, kept_idx + kept, ws, ws_bytes, true, stream);
+                    (char*)v_out + kept * row, score_out ? score_out + kept : nullptr, kept_idx + kept, ws, ws_bytes, stream);
     if (rc) return rc;
   }
   return AHAKV_OK;

@@ -50,9 +50,8 @@ ahakv_status ahakv_score_static(const ahakv_params* p, const void* q_obs, const 
   void* ws = nullptr;
   rc = static_ws_address(&ws);
   if (rc != AHAKV_OK) return rc;
-  // Same kernels, same order as ahakv_score; it clears the words of the scratch that must start at
-  // zero (and marks the run partials "not published") itself, so what the last call left is harmless.
-  return ahakv::score_in_least_room(p, q_obs, k, v, score_prev, score, ws, (size_t)AHAKV_STATIC_WS_BYTES, (cudaStream_t)stream);
+  // ahakv_score resets what has to start clean in its scratch, so what the last call left is harmless.
+  return ahakv_score(p, q_obs, k, v, score_prev, score, ws, (size_t)AHAKV_STATIC_WS_BYTES, stream);
 }
 
 // The status word the kernels of the last ahakv_score_static call on this device left at the head of the

@@ -42,3 +42,26 @@ def test_scores_with_and_without_room_for_numerators_agree(n, r, Hq, Hkv, flags)
     ab.ahakv_score(p, q, k, v, None, a, ab.alloc_workspace(p))
     ab.ahakv_score_static(p, q, k, v, None, b)
     assert torch.allclose(a, b, rtol=1e-5, atol=0)
+
+
+@pytest.mark.parametrize("large,small", [
+    (dict(batch=24, n=3001), dict(batch=20, n=3001)),         # the smaller batch asks for room for its numerators, the larger does not
+    (dict(batch=1, n=66000), dict(batch=1, n=20000)),
+])
+def test_scratch_for_a_large_call_serves_the_smaller_ones(large, small):
+    from paper_2506_03762_b200 import binding as ab
+    params = lambda batch, n: ab.Params(batch, 8, 8, 64, n, 32, 4, 100, dtype=ab.F32)
+    p = params(**small)
+    ws = ab.alloc_workspace(params(**large))
+    assert ws.nbytes < ab.ahakv_workspace_bytes(p)
+    g = torch.Generator(device="cuda").manual_seed(5)
+    q = torch.randn((p.batch, 8, 32, 64), generator=g, device="cuda")
+    k, v = (torch.randn((p.batch, 8, p.n_ctx, 64), generator=g, device="cuda") for _ in range(2))
+    a, b = (torch.empty((p.batch, 8, p.n_ctx), device="cuda") for _ in range(2))
+    ab.ahakv_score(p, q, k, v, None, a, ws)
+    ab.ahakv_score(p, q, k, v, None, b, ab.alloc_workspace(p))
+    assert torch.allclose(a, b, rtol=1e-5, atol=0)
+    outs = ab.alloc_outputs(p), ab.alloc_outputs(p)
+    ab.ahakv_evict(p, q, k, v, None, *outs[0], ws)
+    ab.ahakv_evict(p, q, k, v, None, *outs[1], ab.alloc_workspace(p))
+    assert torch.allclose(outs[0][2], outs[1][2], rtol=1e-5, atol=0)
