@@ -77,7 +77,8 @@ typedef struct {
 
 /* Bytes of scratch the other entry points make use of for these parameters (0 if they are invalid).  Scratch sized for one
  * call serves every call of no larger batch, context, heads and rows too, also where this function asks for more there:
- * float32 calls use room for softmax numerators while that is moderate, and form the logits twice without it.
+ * float32 calls use room for softmax numerators while that is moderate, and form the logits twice without it (to the same
+ * bits).
  * The pointer handed in as `ws` must be 256-byte aligned.  The scratch holds no state between
  * calls, but two calls that overlap on the GPU must not share it. */
 size_t ahakv_workspace_bytes(const ahakv_params* p);

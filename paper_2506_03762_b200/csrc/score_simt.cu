@@ -11,11 +11,13 @@
 // Two kernels over 64-key tiles, one CTA a tile of a (sequence, KV head).
 //   simt_row_stats:   every observation row's softmax statistics (max and sum of 2^{c w}) per 128-key block, two CTAs (a
 //                     cluster) a block.
-//                     Leaves the numerators 2^{c w - m} (m the row's maximum over the tile) in the workspace if it has room.
+//                     Leaves the numerators 2^{c w - m} in the workspace if it has room; m is the row's maximum over a
+//                     warp's sixteen keys, rounded up to a whole number.
 //   simt_weighted_sums: merges the blocks' statistics and adds the kept numerators, weighted, into the keys' scores (Eq. 1,
 //                     5, 9); squares the tile's value rows on the side.
-//   simt_column_sums: the same without kept numerators: merges the blocks' statistics, recomputes the logits and adds the normalised weights of all rows
-//                     into the keys' scores (Eq. 1, 5, 9); squares the tile's value rows on the side.
+//   simt_column_sums: the same without kept numerators: forms them again.
+// The two give the same bits, so that a score does not depend on how much scratch a call has been given: the same numerators,
+// weights 2^{m - M} / (G sum) of which the power is exact, and sums in the same order.
 // What bounds them: the FP64 units, 64 multiply-adds a cycle and SM, as long as their operands come ready-made and cheaply.
 // Converting FP32 to FP64 runs at a quarter of that rate, so keys and queries are converted once, into shared memory; and
 // shared memory keeps up because the products are mma.sync m8n8k4 in double (the same multiply-adds, one rounding each,
@@ -61,8 +63,7 @@ struct Tiles {
   A q[kRows][row_pitch<A, D>()];
   A row_c[kRows];
   int row_last[kRows];
-  __align__(16) float fin4[kRows][kKeyWarps];         // simt_row_stats: row maxima of the key warps
-  float2 fin[kRows];                                  // shift and 1 / (G sum) of a row
+  float2 fin[kRows];                                  // simt_column_sums: shift and 1 / (G sum) of a row
   float2 stat[kMaxRows][kKeyWarps];                   // simt_row_stats: per row and key warp; simt_column_sums: scratch
 };
 
@@ -198,6 +199,31 @@ __device__ __forceinline__ float2 merge_pair(float2 a, float2 b) {
   return make_float2(m, z);
 }
 
+// Shifts m of a row's logits over this warp's keys, and their numerators 2^{c w - m}: this thread's two rows and four keys.
+// A shift is a whole number, at least the largest visible logit (rounded to FP32) and less than 1 above it; -inf if none is.
+template <typename A>
+__device__ __forceinline__ void row_shifts(const A (&acc)[4][2], const A (&cc)[2], const int (&last)[2], const int (&key)[4], float (&m)[2]) {
+#pragma unroll
+  for (int y = 0; y < 2; ++y) {
+    float top = -INFINITY;
+#pragma unroll
+    for (int x = 0; x < 4; ++x)
+      if (key[x] <= last[y]) top = fmaxf(top, (float)(acc[x][y] * cc[y]));
+#pragma unroll
+    for (int o = 2; o; o >>= 1) top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, o));
+    m[y] = ceilf(top);
+  }
+}
+template <typename A>
+__device__ __forceinline__ float numerator(A w, A c, float m) {
+  return fast_exp2((float)fma(w, c, -(A)m));
+}
+// 2^{m - M} for whole numbers m <= M, exactly (0 below the smallest normal number and for m = -inf).
+__device__ __forceinline__ float pow2_diff(float m, float M) {
+  const float d = m - M;
+  return d >= -126.f ? __int_as_float(((int)d + 127) << 23) : d == d ? 0.f : d;
+}
+
 // Pass 1: per (unit, 128-key block, stacked row) the pair (max of c*w, sum of 2^{c*w - max}).
 template <typename T, int D, bool kKeep>
 __global__ void __launch_bounds__(kThreads, 2) __cluster_dims__(2, 1, 1)
@@ -229,54 +255,29 @@ simt_row_stats(const T* __restrict__ q, const T* __restrict__ k, float2* __restr
     __syncthreads();
     A acc[4][2];
     dot_16x16<D>(sm, 16 * kw, 16 * rw, acc);
-    float ms[2];
+    const A cc[2] = {sm.row_c[row], sm.row_c[row + 8]};
+    const int last[2] = {sm.row_last[row], sm.row_last[row + 8]}, keys[4] = {j0 + key(0), j0 + key(1), j0 + key(2), j0 + key(3)};
+    float m[2];
+    row_shifts(acc, cc, last, keys, m);
 #pragma unroll
     for (int y = 0; y < 2; ++y) {
-      const A cc = sm.row_c[row + 8 * y];
-      const int last = sm.row_last[row + 8 * y];
-      float m = -INFINITY;                                      // the shift is an FP32 number on either path
-#pragma unroll
-      for (int x = 0; x < 4; ++x) {
-        acc[x][y] *= cc;
-        if (j0 + key(x) <= last) m = fmaxf(m, (float)acc[x][y]);
-      }
-#pragma unroll
-      for (int o = 2; o; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-      ms[y] = m;
-    }
-    if (kKeep) {
-      // one shift for the tile's keys, so that its numerators need one number a row beside them
-#pragma unroll
-      for (int y = 0; y < 2; ++y)
-        if ((lane & 3) == 0) sm.fin4[row + 8 * y][kw] = ms[y];
-      __syncthreads();
-#pragma unroll
-      for (int y = 0; y < 2; ++y) {
-        const float4 f = *reinterpret_cast<const float4*>(sm.fin4[row + 8 * y]);
-        ms[y] = fmaxf(fmaxf(f.x, f.y), fmaxf(f.z, f.w));
-      }
-    }
-#pragma unroll
-    for (int y = 0; y < 2; ++y) {
-      const int last = sm.row_last[row + 8 * y];
-      const float m = ms[y];
       float e[4], z = 0.f;
 #pragma unroll
       for (int x = 0; x < 4; ++x) {
-        e[x] = j0 + key(x) <= last ? fast_exp2((float)(acc[x][y] - (A)m)) : 0.f;
+        e[x] = keys[x] <= last[y] ? numerator(acc[x][y], cc[y], m[y]) : 0.f;
         z += e[x];
       }
 #pragma unroll
       for (int o = 2; o; o >>= 1) z += __shfl_xor_sync(0xffffffffu, z, o);
       if (row + 8 * y < c.rows) {
         const int s = c.s0 + row + 8 * y;
-        if ((lane & 3) == 0) sm.stat[s][kw] = make_float2(m, z);
+        if ((lane & 3) == 0) sm.stat[s][kw] = make_float2(m[y], z);
         if (kKeep) {
-          float* to = numer + ((size_t)unit * pl.R + s) * pl.n + j0;
+          float* to = numer + ((size_t)unit * pl.R + s) * pl.n;
 #pragma unroll
           for (int x = 0; x < 4; ++x)
-            if (j0 + key(x) < pl.n) to[key(x)] = e[x];
-          if (lane % 4 == 0 && kw == 0) shift[((size_t)unit * 2 * pl.n_blk + blockIdx.x) * pl.R + s] = m;
+            if (keys[x] < pl.n) to[keys[x]] = e[x];
+          if ((lane & 3) == 0) shift[(((size_t)unit * 2 * pl.n_blk + blockIdx.x) * kKeyWarps + kw) * pl.R + s] = m[y];
         }
       }
     }
@@ -324,7 +325,8 @@ __device__ __forceinline__ void tile_norms(const T* __restrict__ v, float* __res
   }
 }
 
-// Pass 2: S_j = sum over the stacked rows of 2^{c w - max} / (G * sum).
+// Pass 2: S_j = sum over the stacked rows of 2^{c w - m} 2^{m - M} / (G * sum), m the shift of the numerators of the row and
+// the key's warp, M and the sum those of the row.
 template <typename T, int D>
 __global__ void __launch_bounds__(kThreads, 2)
 simt_column_sums(const T* __restrict__ q, const T* __restrict__ k, const T* __restrict__ v, const float2* partial,
@@ -356,6 +358,10 @@ simt_column_sums(const T* __restrict__ q, const T* __restrict__ k, const T* __re
     __syncthreads();
     A acc[4][2];
     dot_16x16<D>(sm, 16 * kw, 16 * rw, acc);
+    const A cc[2] = {sm.row_c[row], sm.row_c[row + 8]};
+    const int last[2] = {sm.row_last[row], sm.row_last[row + 8]}, keys[4] = {j0 + key(0), j0 + key(1), j0 + key(2), j0 + key(3)};
+    float m[2];
+    row_shifts(acc, cc, last, keys, m);
     if (ch == 0) {
       griddep_wait();
       griddep_launch();
@@ -380,12 +386,11 @@ simt_column_sums(const T* __restrict__ q, const T* __restrict__ k, const T* __re
     }
 #pragma unroll
     for (int y = 0; y < 2; ++y) {
-      const A cc = sm.row_c[row + 8 * y];
-      const int last = sm.row_last[row + 8 * y];
       const float2 st = sm.fin[row + 8 * y];
+      const float weight = pow2_diff(m[y], st.x) * st.y;
 #pragma unroll
       for (int x = 0; x < 4; ++x)
-        if (j0 + key(x) <= last) sum[x] = fmaf(fast_exp2((float)fma(acc[x][y], cc, -(A)st.x)), st.y, sum[x]);
+        if (keys[x] <= last[y]) sum[x] = fmaf(numerator(acc[x][y], cc[y], m[y]), weight, sum[x]);
     }
     if (c.head_done || ch + 1 == chunks) {
       // the eight row groups of the warp, then the two warps along the rows
@@ -405,14 +410,14 @@ simt_column_sums(const T* __restrict__ q, const T* __restrict__ k, const T* __re
   if (threadIdx.x < kTile && j0 + (int)threadIdx.x < pl.n) s_raw[(size_t)unit * pl.n + j0 + threadIdx.x] = best;
 }
 
-// Pass 2 from kept numerators: S_j = sum over the stacked rows of e_sj 2^{m - M} / (G * sum), m the shift of the tile's
-// numerators, M and the sum those of the row.
+// Pass 2 from kept numerators.  A thread has one key and a quarter of the rows, those that a thread of simt_column_sums has
+// and three of its neighbours', and adds them up in the order they do.
 template <typename T, int D>
 __global__ void __launch_bounds__(kThreads)
 simt_weighted_sums(const T* __restrict__ v, const float2* partial, const float* numer, const float* shift, float* __restrict__ s_raw,
                    float* __restrict__ nu, const __grid_constant__ Shape pl) {
   __shared__ float2 part[kThreads / 32][kRows];
-  __shared__ float weight[kMaxRows], sums[kThreads / kTile][kTile];
+  __shared__ float weight[kKeyWarps][kMaxRows], sums[kThreads / kTile][kTile];
   const int unit = blockIdx.y, b = unit / pl.Hkv, h = unit % pl.Hkv, j0 = blockIdx.x * kTile;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   griddep_wait();
@@ -429,11 +434,12 @@ simt_weighted_sums(const T* __restrict__ v, const float2* partial, const float* 
     }
     part[warp][lane] = p;
     __syncthreads();
-    if (warp == 0 && s < pl.R) {
+    if (warp < kKeyWarps && s < pl.R) {                // a warp for every sixteen keys
+      p = part[0][lane];
 #pragma unroll
       for (int w = 1; w < kThreads / 32; ++w) p = merge_pair(p, part[w][lane]);
-      const float m = shift[((size_t)unit * 2 * pl.n_blk + blockIdx.x) * pl.R + s];
-      weight[s] = (m > -INFINITY ? fast_exp2(m - p.x) : 0.f) / (p.y * (float)(pl.group_max ? 1 : pl.G));
+      const float m = shift[(((size_t)unit * 2 * pl.n_blk + blockIdx.x) * kKeyWarps + warp) * pl.R + s];
+      weight[warp][s] = pow2_diff(m, p.x) * (1.f / (p.y * (float)(pl.group_max ? 1 : pl.G)));
     }
     __syncthreads();
   }
@@ -442,11 +448,23 @@ simt_weighted_sums(const T* __restrict__ v, const float2* partial, const float* 
   float best = 0.f;
   for (int g = 0; g < heads; ++g) {
     const float* from = numer + ((size_t)unit * pl.R + g * rows) * pl.n + j;
-    float sum = 0.f;
+    const float* by = weight[jl / 16] + g * rows;
+    float acc[4] = {};
     if (j < pl.n) {
-#pragma unroll 8
-      for (int i = share; i < rows; i += kThreads / kTile) sum = fmaf(from[(size_t)i * pl.n], weight[g * rows + i], sum);
+      for (int i0 = 16 * (share >> 1) + 4 * (share & 1); i0 < rows; i0 += kRows) {
+        float e[2][4];
+#pragma unroll
+        for (int y = 0; y < 2; ++y)
+#pragma unroll
+          for (int t = 0; t < 4; ++t) e[y][t] = i0 + 8 * y + t < rows ? from[(size_t)(i0 + 8 * y + t) * pl.n] : 0.f;
+#pragma unroll
+        for (int y = 0; y < 2; ++y)
+#pragma unroll
+          for (int t = 0; t < 4; ++t)
+            if (i0 + 8 * y + t < rows) acc[t] = fmaf(e[y][t], by[i0 + 8 * y + t], acc[t]);
+      }
     }
+    const float sum = (acc[0] + acc[1]) + (acc[2] + acc[3]);
     if (g > 0) __syncthreads();
     sums[share][jl] = sum;
     __syncthreads();
@@ -500,8 +518,8 @@ ahakv_status run(const Plan& pl, const void* q, const void* k, const void* v, fl
 
 }  // namespace
 
-// Floats kept per call: the numerators [unit][R][n] and the tiles' shifts [unit][2 n_blk][R].
-size_t simt_kept_floats(const Plan& pl) { return (size_t)pl.B * pl.Hkv * pl.R * ((size_t)pl.n + 2 * pl.n_blk); }
+// Floats kept per call: the numerators [unit][R][n] and their shifts [unit][2 n_blk][kKeyWarps][R].
+size_t simt_kept_floats(const Plan& pl) { return (size_t)pl.B * pl.Hkv * pl.R * ((size_t)pl.n + 2 * kKeyWarps * pl.n_blk); }
 
 ahakv_status launch_score_simt(const Plan& pl, const void* q, const void* k, const void* v, float* s_raw, float* nu, float2* partial,
                                float* kept, int* status, cudaStream_t st) {

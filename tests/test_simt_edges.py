@@ -65,3 +65,27 @@ def test_scratch_for_a_large_call_serves_the_smaller_ones(large, small):
     ab.ahakv_evict(p, q, k, v, None, *outs[0], ws)
     ab.ahakv_evict(p, q, k, v, None, *outs[1], ab.alloc_workspace(p))
     assert torch.allclose(outs[0][2], outs[1][2], rtol=1e-5, atol=0)
+
+
+@pytest.mark.parametrize("Hq,Hkv,n,r,flags", [(8, 8, 3001, 32, 1), (12, 4, 3300, 20, 5), (6, 2, 6100, 33, 1), (4, 4, 6007, 64, 4), (8, 8, 4099, 1, 1)])
+def test_scores_do_not_depend_on_the_room_for_numerators(Hq, Hkv, n, r, flags):
+    """A sequence of a ragged batch, a call on the library's own scratch and a call on scratch of another size get exactly what
+    a call with all the room it asks for gets: bit for bit, whether numerators are kept or formed twice."""
+    from paper_2506_03762_b200 import binding as ab
+    p = ab.Params(1, Hq, Hkv, 128, n, r, 4, 300, dtype=ab.F32, flags=flags)
+    need = ab.ahakv_workspace_bytes(p)
+    kept = Hkv * (Hq // Hkv) * r * n * 4
+    assert need > kept, "the call keeps its numerators"
+    g = torch.Generator(device="cuda").manual_seed(n)
+    q = 3 * torch.randn((1, Hq, r, 128), generator=g, device="cuda")
+    k, v = (torch.randn((1, Hkv, n, 128), generator=g, device="cuda") for _ in range(2))
+    ws = ab.alloc_workspace(p)
+    a, b = (torch.empty((1, Hkv, n), device="cuda") for _ in range(2))
+    ab.ahakv_score(p, q, k, v, None, a, ws)
+    ab.ahakv_score(p, q, k, v, None, b, ws, ws_bytes=need - kept)
+    assert torch.equal(a, b)
+    outs = ab.alloc_outputs(p), ab.alloc_outputs(p)
+    ab.ahakv_evict(p, q, k, v, None, *outs[0], ws)
+    ab.ahakv_evict(p, q, k, v, None, *outs[1], ws, ws_bytes=need - kept)
+    for x, y in zip(*outs):
+        assert torch.equal(x, y)
