@@ -396,14 +396,14 @@ ahakv_status ahakv_compact(const ahakv_params* p, const void* k, const void* v, 
 
 static ahakv_status evict_impl(const ahakv_params* p, const int32_t* budgets, const void* q_obs, const void* k,
                                const void* v, const float* score_prev, void* k_out, void* v_out, float* score_out,
-                               int32_t* kept_idx, void* ws, size_t ws_bytes, ahakv_stream_t stream) {
+                               int32_t* kept_idx, void* ws, size_t ws_bytes, uintptr_t prev_align, ahakv_stream_t stream) {
   const Plan* plan;
   ahakv_status rc = plan_for(p, &plan);
   if (rc) return rc;
   const Plan& pl = *plan;
   if (!q_obs || !k || !v || !k_out || !v_out || !kept_idx) return AHAKV_ERR_INVALID_ARG;
   if (!aligned16(q_obs) || !aligned16(k) || !aligned16(v) || !aligned16(k_out) || !aligned16(v_out) ||
-      ((uintptr_t)kept_idx & 3) || (score_prev && !aligned16(score_prev)))
+      ((uintptr_t)kept_idx & 3) || (score_prev && ((uintptr_t)score_prev & (prev_align - 1))))
     return AHAKV_ERR_INVALID_ARG;
   if ((rc = check_ws(pl, ws, ws_bytes))) return rc;
   cudaStream_t st = (cudaStream_t)stream;
@@ -434,7 +434,7 @@ static ahakv_status evict_impl(const ahakv_params* p, const int32_t* budgets, co
 ahakv_status ahakv_evict(const ahakv_params* p, const void* q_obs, const void* k, const void* v,
                          const float* score_prev, void* k_out, void* v_out, float* score_out,
                          int32_t* kept_idx, void* ws, size_t ws_bytes, ahakv_stream_t stream) {
-  return evict_impl(p, nullptr, q_obs, k, v, score_prev, k_out, v_out, score_out, kept_idx, ws, ws_bytes, stream);
+  return evict_impl(p, nullptr, q_obs, k, v, score_prev, k_out, v_out, score_out, kept_idx, ws, ws_bytes, 16, stream);
 }
 
 ahakv_status ahakv_evict_head_budgets(const ahakv_params* p, const int32_t* head_budget, const void* q_obs, const void* k,
@@ -442,7 +442,7 @@ ahakv_status ahakv_evict_head_budgets(const ahakv_params* p, const int32_t* head
                                       float* score_out, int32_t* kept_idx, void* ws, size_t ws_bytes,
                                       ahakv_stream_t stream) {
   if (!head_budget || ((uintptr_t)head_budget & 3)) return AHAKV_ERR_INVALID_ARG;
-  return evict_impl(p, head_budget, q_obs, k, v, score_prev, k_out, v_out, score_out, kept_idx, ws, ws_bytes, stream);
+  return evict_impl(p, head_budget, q_obs, k, v, score_prev, k_out, v_out, score_out, kept_idx, ws, ws_bytes, 16, stream);
 }
 
 ahakv_status ahakv_evict_ragged(const ahakv_params* p, const ahakv_seq* seqs, const void* q_obs, const void* k,
@@ -451,9 +451,10 @@ ahakv_status ahakv_evict_ragged(const ahakv_params* p, const ahakv_seq* seqs, co
   Plan outer;
   ahakv_status rc = make_plan(p, &outer);        // p describes the allocation: n_ctx and budget are the largest of the batch
   if (rc) return rc;
-  if (!seqs) return AHAKV_ERR_INVALID_ARG;
+  if (!seqs || (score_prev && !aligned16(score_prev))) return AHAKV_ERR_INVALID_ARG;
   if ((rc = check_ws(outer, ws, ws_bytes))) return rc;
-  // every sequence is checked before anything is queued
+  // every sequence is checked before anything is queued (the pointers with the first: the others' are multiples of a row on,
+  // but for the carried scores, which may then start at any float)
   for (int b = 0; b < outer.B; ++b) {
     if (seqs[b].n_ctx < outer.r || seqs[b].n_ctx > p->n_ctx || seqs[b].budget < 1 || seqs[b].budget > p->budget ||
         seqs[b].budget < p->recent_window || seqs[b].n_total < seqs[b].n_ctx)
@@ -473,7 +474,7 @@ ahakv_status ahakv_evict_ragged(const ahakv_params* p, const ahakv_seq* seqs, co
     const char* vb = (const char*)v + (size_t)b * outer.vs[0] * es;
     const size_t tok = (size_t)b * outer.Hkv * outer.n, kept = (size_t)b * outer.Hkv * keep_max;
     rc = evict_impl(&pb, nullptr, qb, kb, vb, score_prev ? score_prev + tok : nullptr, (char*)k_out + kept * row,
-                    (char*)v_out + kept * row, score_out ? score_out + kept : nullptr, kept_idx + kept, ws, ws_bytes, stream);
+                    (char*)v_out + kept * row, score_out ? score_out + kept : nullptr, kept_idx + kept, ws, ws_bytes, 4, stream);
     if (rc) return rc;
   }
   return AHAKV_OK;

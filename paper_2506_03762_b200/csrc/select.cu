@@ -227,6 +227,7 @@ __global__ void __launch_bounds__(kThreads, 2) refine_select_kernel(const __grid
   constexpr int kStride = 32 * kV;
   const int j0 = base + warp * (32 * kPer) + lane * kV;
   const bool prior = a.nu != nullptr, vec = (n & 3) == 0;
+  const bool vec_prev = vec && (reinterpret_cast<uintptr_t>(a.prev) & 15) == 0;   // a ragged batch's rows start anywhere
   *reinterpret_cast<uint4*>(&hist[4 * tid]) = make_uint4(0, 0, 0, 0);
   if (tid == 0) list_n = 0;
   if (kCluster) cl.barrier_arrive();                   // waited for before the first store into another CTA
@@ -322,7 +323,7 @@ __global__ void __launch_bounds__(kThreads, 2) refine_select_kernel(const __grid
   if (a.prev) {
     float p[kPer];
 #pragma unroll
-    for (int q = 0; q < kPieces; ++q) load_piece<kV>(a.prev + (size_t)unit * n, j0 + q * kStride, end, vec, p + q * kV);
+    for (int q = 0; q < kPieces; ++q) load_piece<kV>(a.prev + (size_t)unit * n, j0 + q * kStride, end, vec_prev, p + q * kV);
 #pragma unroll
     for (int e = 0; e < kPer; ++e) {
       if (j0 + (e / kV) * kStride + e % kV < end) top = fmaxf(top, s[e] + p[e]);
@@ -363,7 +364,7 @@ __global__ void __launch_bounds__(kThreads, 2) refine_select_kernel(const __grid
     float p[kPer];
     if (kPer > 8) {
 #pragma unroll
-      for (int q = 0; q < kPieces; ++q) load_piece<kV>(a.prev + (size_t)unit * n, j0 + q * kStride, end, vec, p + q * kV);
+      for (int q = 0; q < kPieces; ++q) load_piece<kV>(a.prev + (size_t)unit * n, j0 + q * kStride, end, vec_prev, p + q * kV);
     }
 #pragma unroll
     for (int e = 0; e < kPer; ++e) s[e] = __fadd_rn(s[e], kPer <= 8 ? held[e % kHeld] : p[e]);

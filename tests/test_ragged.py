@@ -59,6 +59,38 @@ def test_ragged_batch_equals_one_call_per_sequence(dtype_name, Hq, Hkv, d):
     assert torch.equal(idx, before)
 
 
+@pytest.mark.parametrize("dtype_name,Hkv,n_max,lengths", [("F16", 1, 4097, (4097, 4096, 4000, 2)), ("F32", 1, 1023, (1023, 600, 1020, 1)),
+                                                          ("BF16", 3, 9001, (5000, 9000, 8999)), ("F16", 1, 140001, (300, 20000, 132000))])
+def test_carried_scores_of_a_ragged_batch_start_anywhere(dtype_name, Hkv, n_max, lengths):
+    """Sequence b's carried scores start b * Hkv * n_ctx floats into the array: for an odd product on no 16-byte boundary, whatever
+    its own length is a multiple of.  Every sequence still gets what ``ahakv_evict`` gives it alone."""
+    from paper_2506_03762_b200 import binding as ab
+    from tests import parity
+    dtype = getattr(ab, dtype_name)
+    dt = ab.CODE_DTYPE[dtype]
+    B, d, bud = len(lengths), 64, 100
+    g = torch.Generator(device="cuda").manual_seed(n_max)
+    r = min(16, min(lengths))
+    q = torch.randn((B, Hkv, r, d), generator=g, device="cuda").to(dt)
+    k, v = (torch.randn((B, Hkv, n_max, d), generator=g, device="cuda").to(dt) for _ in range(2))
+    prev = torch.rand((B, Hkv * n_max), generator=g, device="cuda")
+    seqs = [(n, bud, 150000) for n in lengths]
+    for flags in (0, ab.FLAG_VALUE_PRIOR):
+        p = ab.Params(B, Hkv, Hkv, d, n_max, r, 1, bud, dtype=dtype, n_total=150000, flags=flags)
+        ws = ab.alloc_workspace(p, "cuda")
+        k_out, v_out, s_out, idx = ab.alloc_outputs(p, "cuda")
+        ab.ahakv_evict_ragged(p, seqs, q, k, v, prev, k_out, v_out, s_out, idx, ws)
+        assert ab.ahakv_last_device_status(ws) == ab.OK
+        for b, n in enumerate(lengths):
+            keep = min(n, bud)
+            pb = ab.Params(1, Hkv, Hkv, d, n, r, 1, bud, dtype=dtype, n_total=150000, flags=flags)
+            alone = parity.run_evict(pb, q[b:b + 1], k[b:b + 1, :, :n].contiguous(), v[b:b + 1, :, :n].contiguous(),
+                                     prev[b, : Hkv * n].view(1, Hkv, n).clone())
+            assert torch.equal(alone[3].flatten(), idx[b].flatten()[: Hkv * keep]), f"sequence {b}"
+            assert torch.equal(alone[2].flatten(), s_out[b].flatten()[: Hkv * keep])
+            assert torch.equal(alone[0].flatten(), k_out[b].flatten()[: Hkv * keep * d])
+
+
 @pytest.mark.parametrize("dtype_name,Hq,Hkv,d,n", [("F16", 8, 4, 128, 1500), ("BF16", 2, 2, 64, 33000), ("F32", 4, 2, 64, 600)])
 def test_a_budget_per_head(dtype_name, Hq, Hkv, d, n):
     """Every (sequence, KV head) keeps its recent window and the best of the rest up to its own budget: what
