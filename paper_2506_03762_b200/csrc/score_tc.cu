@@ -134,6 +134,7 @@ struct Shared {
   unsigned long long stat_full[2], stat_empty[2];
   uint32_t tmem_slot;
   int seg_pub, seg_done[kGroups];           // segments published / retired by each group of softmax warps
+  int seg_read;                             // segments the delivery warp has read
   int mrg_pub, mrg_done;                    // pass-2 runs announced to / finished by the table warp
 };
 
@@ -247,8 +248,10 @@ __device__ __forceinline__ void sched_round(const TcArgs& a, Shared* sh, Schedul
   int ds = ld_volatile(&sh->seg_done[0]);
 #pragma unroll
   for (int g = 1; g < kGroups; ++g) ds = min(ds, ld_volatile(&sh->seg_done[g]));
-  // not too far ahead of the tiles being worked on, and room in the table ring for a whole round
-  if (sc.k - ds >= kSegAhead || sc.m - ld_volatile(&sh->mrg_done) > kMergeRing - 2) return;
+  // Not too far ahead of the tiles being worked on, and room in the rings for a whole round (two segments).  The copies and
+  // products of a segment are issued before its softmax is done, so those roles are never behind `ds`; the delivery warp may
+  // be: it merges a row block's partials while the softmax warps go on, and has to have read what is overwritten.
+  if (sc.k - ds >= kSegAhead || sc.k - ld_volatile(&sh->seg_read) > kSegRing - 2 || sc.m - ld_volatile(&sh->mrg_done) > kMergeRing - 2) return;
   // Pass 1 may run ahead of pass 2 by max_lead runs, no further: what lies between the two counters has to stay in L2.
   if (sc.p1_left && (sc.pend < 0 || ld_volatile(&a.ctr[0]) - ld_volatile(&a.ctr[1]) < a.max_lead)) {
     const int r = sc.p1_next >= 0 ? sc.p1_next : atomicAdd(&a.ctr[0], 1) + 1;            // the counters start at -1
@@ -515,7 +518,9 @@ __device__ __forceinline__ void delivery(const TcArgs& a, Shared* sh) {
   const int lane = threadIdx.x & 31;
   int sc = 0;
   bool ok = true;
-  for_each_segment<kTest>(a, sh, [&](const Seg& sg, int pass, int, int) {
+  for_each_segment<kTest>(a, sh, [&](const Seg& sg, int pass, int, int idx) {
+    __syncwarp();
+    if (lane == 0) *(volatile int*)&sh->seg_read = idx + 1;
     if (pass != 0 || !ok) return;
     const int slot = sc & 1;
     if (!(ok = mbar_wait(&sh->stat_full[slot], (sc >> 1) & 1, a.status, wait_limit<kTest>(a)))) return;
@@ -685,7 +690,7 @@ score_tc_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_constant_
       for (int g = 0; g < kGroups; ++g) mbar_init(&sh->acc_full[g][s], 1);
     }
     for (int g = 0; g < kGroups; ++g) sh->seg_done[g] = 0;
-    sh->seg_pub = 0; sh->mrg_pub = 0; sh->mrg_done = 0;
+    sh->seg_pub = 0; sh->seg_read = 0; sh->mrg_pub = 0; sh->mrg_done = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   for (int t = threadIdx.x; t < 256; t += kThreads) {

@@ -335,3 +335,19 @@ def test_the_eviction_call_replays_from_a_cuda_graph():
         assert ab.ahakv_last_device_status(ws) == ab.OK
         for a, c in zip(eager, outs):
             assert torch.equal(a, c)
+
+
+@pytest.mark.parametrize("H,n,r,d", [(1, 300000, 8, 64), (3, 131000, 100, 64), (2, 90001, 128, 128)])
+def test_row_blocks_of_many_runs(H, n, r, d):
+    """A few heads of a very long context: a row block is cut into a run for every CTA, and whoever completes it merges all their
+    statistics while the other warps of its CTA go on to the second pass of what is already merged.  Against float64."""
+    q, k, v = _rand_problem(1, H, H, d, n, r, ab.F16, seed=n)
+    p = ab.Params(1, H, H, d, n, r, 16, 1000, dtype=ab.F16, flags=0, scale_mode=ab.SCALE_FIXED, scale=0.2)
+    first = parity.run_score(p, q, k, v)
+    for h in range(H):
+        x = float(np.float32(0.2)) * (q[0, h].double() @ k[0, h].double().T)
+        seen = torch.arange(n, device=x.device) <= torch.arange(n - r, n, device=x.device).view(r, 1)
+        want = x.masked_fill(~seen, float("-inf")).softmax(-1).sum(0)
+        parity.assert_scores_close(p, first[0, h].cpu().numpy(), want.cpu().numpy())
+    for _ in range(3):
+        assert torch.equal(first, parity.run_score(p, q, k, v))
