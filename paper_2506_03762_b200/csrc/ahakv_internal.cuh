@@ -109,7 +109,13 @@ ahakv_status launch_compact(const Plan& pl, const void* k, const void* v, const 
 int profile_begin_call(cudaStream_t st);             // returns a slot, or -1
 void profile_mark(int slot, int boundary, cudaStream_t st);   // boundary b closes stage b-1, opens stage b
 
-inline ahakv_status cuda_ok(cudaError_t e) { return e == cudaSuccess ? AHAKV_OK : AHAKV_ERR_CUDA; }
+// An error is reported once: cudaLaunchKernelEx leaves it behind as the thread's last error too, where the next
+// cudaGetLastError() of a call that went well would find it.
+inline ahakv_status cuda_ok(cudaError_t e) {
+  if (e == cudaSuccess) return AHAKV_OK;
+  cudaGetLastError();
+  return AHAKV_ERR_CUDA;
+}
 
 // Launches `kernel` so that it may start its prologue while the kernel before it in the stream still runs (programmatic
 // dependent launch; the kernel calls griddep_wait() before it touches anything), as clusters of `cluster` CTAs.

@@ -351,3 +351,29 @@ def test_row_blocks_of_many_runs(H, n, r, d):
         parity.assert_scores_close(p, first[0, h].cpu().numpy(), want.cpu().numpy())
     for _ in range(3):
         assert torch.equal(first, parity.run_score(p, q, k, v))
+
+
+def test_a_launch_that_is_refused_does_not_fail_the_next_call():
+    """A launch into the legacy stream is refused while a blocking stream is being captured (and ends the capture).  The call says
+    so; the next one, which looks at the last error after a launch of its own, finds none."""
+    import ctypes
+    cu = ctypes.CDLL("libcuda.so.1")
+    p = ab.Params(1, 2, 2, 64, 300, 8, 4, 40, dtype=ab.F16)
+    q, k, v = _rand_problem(1, 2, 2, 64, 300, 300, ab.F16, seed=1)
+    score, idx = torch.rand((1, 2, 300), device=DEV), torch.zeros((1, 2, 40), dtype=torch.int32, device=DEV)
+    ws = ab.alloc_workspace(p, DEV)
+    ab.ahakv_score_full_causal(p, q, k, v, None, score, ws)
+    torch.cuda.synchronize()
+    stream, graph = ctypes.c_void_p(), ctypes.c_void_p()
+    assert cu.cuStreamCreate(ctypes.byref(stream), 0) == 0
+    try:
+        assert cu.cuStreamBeginCapture_v2(stream, 0) == 0
+        try:
+            assert ab.ahakv_select(p, score, idx, stream=0, check=False) == ab.ERR_CUDA
+        finally:
+            cu.cuStreamEndCapture(stream, ctypes.byref(graph))
+    finally:
+        cu.cuStreamDestroy_v2(stream)
+    again = torch.empty_like(score)
+    ab.ahakv_score_full_causal(p, q, k, v, None, again, ws)
+    assert torch.equal(again, score)
