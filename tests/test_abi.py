@@ -115,3 +115,43 @@ def test_status_strings_and_errors(lib):
     with pytest.raises(ab.AhakvError):
         ab.ahakv_score(_good(batch=0), 256, 256, 256, None, 256, 256, 1 << 40, stream=0)
     assert ab.ahakv_launch_count() == 0
+
+
+def test_a_call_takes_the_present_values_of_its_parameters(lib):
+    """However they were set, and whatever other threads do: the struct handed over is that of the fields as they are."""
+    import copy
+    import dataclasses
+    import pickle
+    import threading
+    p = _good()
+    need = ab.ahakv_workspace_bytes(p)
+    assert set(vars(p)) == {f.name for f in dataclasses.fields(p)}
+    assert ab.Params(**vars(p)) == p == copy.deepcopy(p) == pickle.loads(pickle.dumps(p)) == dataclasses.replace(p)
+    p.__dict__.update(n_ctx=5000)
+    assert ab.ahakv_workspace_bytes(p) == ab.ahakv_workspace_bytes(_good(n_ctx=5000)) > need
+    q = copy.copy(p)
+    q.n_ctx = 1000
+    assert ab.ahakv_workspace_bytes(q) == need and ab.ahakv_workspace_bytes(p) > need
+    strides = [128 * 2000 * 2, 128 * 2000, 128]
+    p = _good(k_stride=strides)
+    assert ab.ahakv_workspace_bytes(p) > 0
+    strides[2] = 1                                            # a list may change unseen
+    assert ab.ahakv_workspace_bytes(p) == 0
+    # a thread that is between building the struct and keeping it while another sets a field
+    p = _good()
+    build, inside, go = ab.Params.c, threading.Event(), threading.Event()
+
+    class Slow(ab.Params):
+        def c(self):
+            r = build(self)
+            inside.set()
+            go.wait(10)
+            return r
+    slow = Slow(**vars(p))
+    t = threading.Thread(target=slow.ref)
+    t.start()
+    assert inside.wait(10)
+    slow.n_ctx = 5000
+    go.set()
+    t.join(10)
+    assert ab.ahakv_workspace_bytes(slow) == ab.ahakv_workspace_bytes(_good(n_ctx=5000))
