@@ -293,8 +293,7 @@ ahakv_status ahakv_score_static(const ahakv_params* p, const void* q_obs, const 
  * production use. */
 void ahakv_test_set_wait(int32_t wait_ms, int32_t withhold_first_partial);
 
-/* Number of kernels the library has launched in this process since it was loaded (the fills of scratch words with ones or
- * zeros are not counted, whether a memset or a kernel does them). */
+/* Number of kernels the library has launched in this process since it was loaded. */
 int64_t ahakv_launch_count(void);
 
 const char* ahakv_status_string(ahakv_status s);

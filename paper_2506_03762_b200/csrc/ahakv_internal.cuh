@@ -87,7 +87,7 @@ bool causal_tc_fits(const Plan& pl, size_t pool_bytes);
 ahakv_status launch_causal_tc(const Plan& pl, int scale_mode, double fixed, long long first_cached, const void* q, const long long qs[3],
                               const void* k, float* pool, size_t pool_bytes, float* sums, const float** slots, int* n_slots,
                               int* status, cudaStream_t st);
-// All ones into `bytes` (a multiple of 16) from `to` (16-byte aligned) on (clear.cu); not counted as a launch.
+// All ones into `bytes` (a multiple of 16) from `to` (16-byte aligned) on (clear.cu).
 ahakv_status launch_clear(void* to, size_t bytes, cudaStream_t st);
 ahakv_status launch_vnorm(const Plan& pl, const void* v, float* nu, cudaStream_t st);
 // `slots` partial scores per head (row blocks, or query heads when pooling by maximum) are combined here.

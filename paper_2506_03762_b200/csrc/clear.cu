@@ -22,6 +22,7 @@ __global__ void __launch_bounds__(kThreads) clear_kernel(uint4* to, int count) {
 
 ahakv_status launch_clear(void* to, size_t bytes, cudaStream_t st) {
   const int count = (int)(bytes / sizeof(uint4));
+  count_launch();
   return cuda_ok(launch_chained(clear_kernel, dim3((count + kThreads - 1) / kThreads), dim3(kThreads), 1, 0, st, (uint4*)to, count));
 }
 
