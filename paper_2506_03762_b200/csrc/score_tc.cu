@@ -774,11 +774,11 @@ static int runs_per_row_block(long long units, int n_blk, int slots, long long k
   const int longest = key_bytes > (96LL << 20) ? 8 : 16;
   int best = n_blk;
   long long best_cost = -1;
-  for (int rpu = (n_blk + longest - 1) / longest; rpu <= n_blk; ++rpu) {
-    const int ch = (n_blk + rpu - 1) / rpu;
+  // the fewest runs of every length; more runs of the same length cost the same
+  for (int len = longest; len >= 1; --len) {
+    const int rpu = (n_blk + len - 1) / len, ch = (n_blk + rpu - 1) / rpu;
     const long long cost = (units * ((n_blk + ch - 1) / ch) + slots - 1) / slots * (ch + 1);
     if (best_cost < 0 || cost < best_cost) { best = rpu; best_cost = cost; }
-    if (ch == 1) break;
   }
   return best;
 }

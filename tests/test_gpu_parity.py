@@ -378,3 +378,27 @@ def test_a_launch_that_is_refused_does_not_fail_the_next_call():
     again = torch.empty_like(score)
     ab.ahakv_score_full_causal(p, q, k, v, None, again, ws)
     assert torch.equal(again, score)
+
+
+def test_queueing_a_call_does_not_take_longer_for_a_longer_context():
+    """Host time of a scoring call, which only queues kernels: a million tokens may not cost more of it than four thousand do.  (A
+    walk over every number of runs a million tokens can be cut into takes 40 us; 25 are allowed for everything that differs.)"""
+    import time
+
+    def host_us(n):
+        q, k = torch.zeros((1, 1, 8, 64), dtype=torch.float16, device=DEV), torch.zeros((1, 1, n, 64), dtype=torch.float16, device=DEV)
+        score = torch.empty((1, 1, n), device=DEV)
+        p = ab.Params(1, 1, 1, 64, n, 8, 4, 40, dtype=ab.F16, flags=0)
+        ws = ab.alloc_workspace(p, DEV)
+        times = []
+        for i in range(60):
+            if i % 10 == 0:
+                torch.cuda.synchronize()
+            t = time.perf_counter()
+            ab.ahakv_score(p, q, k, None, None, score, ws)
+            times.append(time.perf_counter() - t)
+        torch.cuda.synchronize()
+        return 1e6 * sorted(times)[len(times) // 2]
+
+    host_us(4096)
+    assert host_us(1 << 20) < host_us(4096) + 25
