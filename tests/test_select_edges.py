@@ -87,3 +87,44 @@ def test_rows_gathered_by_the_selecting_cta_are_the_kept_ones(d, Bud):
     ab.ahakv_evict(p, q, k, v, None, k_out, v_out, s_out, idx, ws)
     at = idx.long().unsqueeze(-1).expand(-1, -1, -1, d)
     assert torch.equal(k_out, k.gather(2, at)) and torch.equal(v_out, v.gather(2, at))
+
+
+@pytest.mark.parametrize("H,n", [(2, 700), (3, 4096), (2, 9001), (1, 70001)])
+@pytest.mark.parametrize("m", [1, 2, 63, 64, 65, 127, 129, 512, 513, 600])
+def test_threshold_among_m_close_scores(H, n, m):
+    """`m` distinct scores within one bin of the first histogram, the threshold in the middle of them; around the most that are
+    ranked from a list."""
+    from paper_2506_03762_b200 import binding as ab
+    g = torch.Generator().manual_seed(n + m)
+    s = torch.rand((1, H, n), generator=g) * 0.5
+    for h in range(H):
+        at = torch.randperm(n, generator=g)[:m]
+        s[0, h, at] = 1.0 + torch.randperm(m, generator=g).float() * 2.0 ** -20
+    keep = max(1, m // 2)
+    p = ab.Params(1, H, H, 64, n, 1, 0, keep, dtype=ab.F16, flags=0)
+    idx = torch.full((1, H, keep), -7, dtype=torch.int32, device="cuda")
+    ab.ahakv_select(p, s.cuda(), idx)
+    for h in range(H):
+        assert np.array_equal(idx[0, h].cpu().numpy(), _expected(s[0, h].numpy(), 0, keep))
+
+
+def test_time_of_a_selection_does_not_hang_on_the_distribution():
+    """2048 heads that drop one of 1000 tokens each: scores over many octaves, where half of a head's tokens lie below the first
+    histogram's range, may take a few passes more than uniform ones, not seven times as long as ranking them by pairs did."""
+    from paper_2506_03762_b200 import binding as ab
+    u = torch.rand((64, 32, 1000), generator=torch.Generator(device="cuda").manual_seed(2), device="cuda")
+    p = ab.Params(64, 32, 32, 64, 1000, 1, 0, 999, dtype=ab.F16, flags=0)
+    idx = torch.empty((64, 32, 999), dtype=torch.int32, device="cuda")
+
+    def us(s):
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        best = 1e9
+        for _ in range(5):
+            a.record()
+            for _ in range(10):
+                ab.ahakv_select(p, s, idx)
+            b.record()
+            b.synchronize()
+            best = min(best, a.elapsed_time(b))
+        return best
+    assert us(torch.exp(20 * u - 30)) < 3 * us(u)
