@@ -17,8 +17,8 @@
 // compact_inplace_kernel: a cluster of CTAs per (sequence, KV head).  kept_idx is ascending, so row t of the result comes
 //   from row kept_idx[t] >= t: rows before the first evicted index do not move at all, and the others move in rounds
 //   through registers (all loads of a round, a barrier over the cluster, all its stores), so no row is overwritten
-//   before it has been read.  128 heads x 2049 rows of 256 bytes, half of them moving: 31 us for 128 MB each way; one CTA a
-//   head with batches through shared memory took 75.
+//   before it has been read.  128 heads x 2049 rows of 256 bytes, half of them moving (67 MB each way): 26 us; one CTA a head
+//   with batches through shared memory took 62.
 #include <cooperative_groups.h>
 
 #include <type_traits>
@@ -431,12 +431,15 @@ ahakv_status launch_step(StepArgs a, const Shape& pl, cudaStream_t st) {
 // ---- in-place compaction ------------------------------------------------------------------------------------------
 constexpr int kMoveThreads = 256;
 constexpr int kMoveVecs = 8;                    // 16-byte pieces of K, and as many of V, a thread holds per round
-constexpr int kMoveCluster = 8;
+constexpr int kMovePieces = kMoveThreads * kMoveVecs;   // and a CTA
+constexpr int kMoveCluster = 8;                 // at most
 
+// Two CTAs an SM: the rows in flight take 64 registers, and with the 80 that three CTAs leave a thread 20 of them were spilled
+// (128 heads x 2049: 32 us against 26; 2048 heads x 513 by one CTA each: 114 against 98).
 template <int LANES>                            // 16-byte pieces of a row
-__global__ void __launch_bounds__(kMoveThreads, 3) compact_inplace_kernel(char* k, char* v, float* score, const int32_t* kept,
+__global__ void __launch_bounds__(kMoveThreads, 2) compact_inplace_kernel(char* k, char* v, float* score, const int32_t* kept,
                                                                           const __grid_constant__ Shape pl) {
-  constexpr int kRowsCta = kMoveThreads * kMoveVecs / LANES;   // rows a CTA holds per round
+  constexpr int kRowsCta = kMovePieces / LANES;                // rows a CTA holds per round
   cg::cluster_group cl = cg::this_cluster();
   const int C = (int)cl.num_blocks(), rank = (int)cl.block_rank();
   const int unit = blockIdx.x / C, n_keep = pl.n_keep, tid = threadIdx.x;
@@ -522,12 +525,20 @@ ahakv_status launch_step_slots(const Plan& pl, const void* q, const void* k_new,
 ahakv_status launch_compact_inplace(const Plan& pl, void* k, void* v, float* score, const int32_t* kept_idx,
                                     cudaStream_t st) {
   const Shape& shape = pl;
-  const dim3 grid(pl.B * pl.Hkv * kMoveCluster), block(kMoveThreads);
+  // CTAs a head: eight while that is little more than the GPU holds.  Otherwise a barrier of a cluster between loads and stores
+  // costs more than it spreads: no more CTAs than heads need to fill the GPU a few times over, nor than two rounds of rows
+  // need.  us with eight / by this rule, rows of 128 bytes: 2048 heads x 513 177 / 53, 256 heads that keep 512 rows 26 / 10,
+  // 1024 heads x 1025 105 / 55; 128 heads x 2049 16 / 15; 8 heads x 2049 5 either way, 14 with one.
+  const int lanes = pl.d * pl.es / 16;
+  const long long heads = (long long)pl.B * pl.Hkv;
+  int C = kMoveCluster;
+  while (C > 1 && (heads * C > 1024 || (heads * C > 2 * 148 && 2LL * C * (kMovePieces / lanes) > pl.n_keep))) C /= 2;
+  const dim3 grid((unsigned)(heads * C)), block(kMoveThreads);
   cudaError_t e;
-  switch (pl.d * pl.es / 16) {
-    case 8: e = launch_chained(compact_inplace_kernel<8>, grid, block, kMoveCluster, 0, st, (char*)k, (char*)v, score, kept_idx, shape); break;
-    case 16: e = launch_chained(compact_inplace_kernel<16>, grid, block, kMoveCluster, 0, st, (char*)k, (char*)v, score, kept_idx, shape); break;
-    default: e = launch_chained(compact_inplace_kernel<32>, grid, block, kMoveCluster, 0, st, (char*)k, (char*)v, score, kept_idx, shape);
+  switch (lanes) {
+    case 8: e = launch_chained(compact_inplace_kernel<8>, grid, block, C, 0, st, (char*)k, (char*)v, score, kept_idx, shape); break;
+    case 16: e = launch_chained(compact_inplace_kernel<16>, grid, block, C, 0, st, (char*)k, (char*)v, score, kept_idx, shape); break;
+    default: e = launch_chained(compact_inplace_kernel<32>, grid, block, C, 0, st, (char*)k, (char*)v, score, kept_idx, shape);
   }
   count_launch();
   return cuda_ok(e);

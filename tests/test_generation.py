@@ -367,3 +367,52 @@ def test_step_and_slots_agree_when_a_head_is_split_over_ctas(B, Hq, Hkv, d, Bud,
     want = k_ord.gather(2, idx.long().unsqueeze(-1).expand(-1, -1, -1, d)), f_ord.gather(2, idx.long())
     ab.ahakv_compact_inplace(p, k_ord, v_ord, f_ord, idx)
     assert torch.equal(k_ord[:, :, :Bud], want[0]) and torch.equal(f_ord[..., :Bud], want[1])
+
+
+@pytest.mark.parametrize("B,H,d,n,keep,dtype_name", [
+    (64, 32, 64, 129, 128, "F16"), (1, 2, 128, 300, 200, "F32"), (8, 32, 64, 700, 300, "BF16"), (8, 32, 128, 1100, 1000, "F16"),
+    (16, 8, 128, 2049, 2048, "F16"), (33, 16, 128, 600, 599, "F32"), (1, 3, 64, 5000, 4999, "F16"), (40, 8, 64, 4100, 4096, "F16"), (1, 1, 64, 9, 8, "F32")])
+def test_compaction_in_place_by_clusters_of_every_size(B, H, d, n, keep, dtype_name):
+    """Few heads are compacted by eight CTAs each, many by four, two or one, in one round or several: rows and scores are those a
+    gather gives, and what lies behind the kept rows is left alone."""
+    from paper_2506_03762_b200 import binding as ab
+    dt = ab.CODE_DTYPE[getattr(ab, dtype_name)]
+    g = torch.Generator(device="cuda").manual_seed(n + H)
+    k, v = (torch.randn((B, H, n, d), generator=g, device="cuda").to(dt) for _ in range(2))
+    score = torch.rand((B, H, n), generator=g, device="cuda")
+    u = torch.rand((B, H, n), generator=g, device="cuda")
+    u[:, ::2, : n // 3] = 2.0                                 # the first rows of every other head stay where they are
+    idx = u.topk(keep, -1).indices.sort(-1).values.int().contiguous()
+    p = ab.Params(B, H, H, d, n, 1, 0, keep, dtype=getattr(ab, dtype_name), flags=0)
+    rows = idx.long().unsqueeze(-1).expand(B, H, keep, d)
+    want = [torch.cat([t.gather(2, rows), t[:, :, keep:]], 2) for t in (k, v)] + [torch.cat([score.gather(2, idx.long()), score[..., keep:]], 2)]
+    ab.ahakv_compact_inplace(p, k, v, score, idx)
+    for a, b in zip((k, v, score), want):
+        assert torch.equal(a, b)
+
+
+def _best_us(f):
+    a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+    best = 1e9
+    for _ in range(6):
+        a.record()
+        for _ in range(5):
+            f()
+        b.record()
+        b.synchronize()
+        best = min(best, a.elapsed_time(b) * 200)
+    return best
+
+
+def test_time_of_compaction_in_place_of_many_heads():
+    """2048 heads that drop one of 513 rows: half of the rows move, which may not take longer than gathering all of them into
+    another cache (one round of a cluster of eight for so few rows took twice as long)."""
+    from paper_2506_03762_b200 import binding as ab
+    B, H, d, n = 64, 32, 64, 513
+    g = torch.Generator(device="cuda").manual_seed(1)
+    k, v = (torch.randn((B, H, n, d), generator=g, device="cuda").half() for _ in range(2))
+    idx = torch.rand((B, H, n), generator=g, device="cuda").topk(n - 1, -1).indices.sort(-1).values.int().contiguous()
+    p = ab.Params(B, H, H, d, n, 1, 0, n - 1, dtype=ab.F16, flags=0)
+    k_out, v_out, _, _ = ab.alloc_outputs(p)
+    apart = _best_us(lambda: ab.ahakv_compact(p, k, v, None, idx, k_out, v_out, None))
+    assert _best_us(lambda: ab.ahakv_compact_inplace(p, k, v, None, idx)) < apart
