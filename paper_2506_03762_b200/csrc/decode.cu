@@ -37,6 +37,7 @@ constexpr int kStepWarps = kStepThreads / 32;
 constexpr int kStepMaxG = 16;                  // query heads per KV head the step kernel takes
 constexpr size_t kStepMaxLogitBytes = 160 * 1024;   // 40960 logits
 constexpr int kStepMaxCluster = 8;
+constexpr int kStepHeldG = 5;                  // float32: heads whose queries are held in registers
 
 template <typename T> using Acc = typename std::conditional<std::is_same<T, float>::value, double, float>::type;
 
@@ -163,38 +164,77 @@ __device__ __forceinline__ void step_logits_simt(const StepArgs& a, const Shape&
   constexpr int V = Vec16<T>::N, LANES = D / V, KEYS_PER_WARP = 32 / LANES;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, sub = lane % LANES, which = lane / LANES;
   const A c = (A)a.c;
-  // this lane's slice of each of the group's queries
-  float qreg[kG][V];
+  // The group's queries in double, converted once (a conversion costs as much as four multiply-adds): this lane's slices in
+  // registers, or, for more than kStepHeldG heads, the rows in shared memory.
+  constexpr bool kHeld = kG <= kStepHeldG;
+  __shared__ __align__(16) A q_sm[kHeld ? 1 : kG][D];
+  A qreg[kHeld ? kG : 1][V];
+  const auto query = [&](int g, A (&to)[V]) {
+    float f[V];
+    Vec16<T>::widen(*reinterpret_cast<const uint4*>((const T*)a.q + (long long)b * pl.qs[0] + (long long)(h * pl.G + g) * pl.qs[1] + sub * V), f);
 #pragma unroll
-  for (int g = 0; g < kG; ++g) {
-    const T* row = (const T*)a.q + (long long)b * pl.qs[0] + (long long)(h * pl.G + g) * pl.qs[1];
-    Vec16<T>::widen(*reinterpret_cast<const uint4*>(row + sub * V), qreg[g]);
-  }
-  const T* kbase = (const T*)a.k + (long long)b * pl.ks[0] + (long long)h * pl.ks[1] + sub * V;
-  const T* fresh = (const T*)a.k_new + ((long long)b * pl.Hkv + h) * D + sub * V;
+    for (int e = 0; e < V; ++e) to[e] = (A)f[e];
+  };
+  const char* kbase = reinterpret_cast<const char*>((const T*)a.k + (long long)b * pl.ks[0] + (long long)h * pl.ks[1] + sub * V);
+  // where the new token's row lies, seen from there
+  const long long fresh = reinterpret_cast<intptr_t>((const T*)a.k_new + ((long long)b * pl.Hkv + h) * D + sub * V) - reinterpret_cast<intptr_t>(kbase);
   constexpr int kUnroll = 4;                                     // key rows in flight per lane
   const int stride = kStepWarps * KEYS_PER_WARP;
-  for (int j0 = k0 + warp * KEYS_PER_WARP + which; j0 - which < k1; j0 += stride * kUnroll) {
-    uint4 raw[kUnroll];
+  uint4 raw[kUnroll];
+  const auto load = [&](int j0) {
 #pragma unroll
     for (int u = 0; u < kUnroll; ++u) {
       const int j = j0 + u * stride;
-      raw[u] = j < k1 ? *reinterpret_cast<const uint4*>(j == slot ? fresh : kbase + (long long)j * pl.ks[2]) : make_uint4(0, 0, 0, 0);
+      raw[u] = make_uint4(0, 0, 0, 0);
+      if (j < k1) raw[u] = *reinterpret_cast<const uint4*>(kbase + (j == slot ? fresh : (long long)j * pl.ks[2] * (long long)sizeof(T)));
     }
+  };
+  load(k0 + warp * KEYS_PER_WARP + which);
+  if (kHeld) {
+#pragma unroll
+    for (int g = 0; g < kG; ++g) query(g, qreg[kHeld ? g : 0]);
+  } else {
+    for (int g = threadIdx.x / LANES; g < kG; g += kStepThreads / LANES) {
+      A x[V];
+      query(g, x);
+#pragma unroll
+      for (int e = 0; e < V; ++e) q_sm[kHeld ? 0 : g][sub * V + e] = x[e];
+    }
+    __syncthreads();
+  }
+  // The next rows are asked for before this round's are multiplied (the stores of the logits keep the compiler from doing so by
+  // itself), and the reductions of four keys run side by side.  Without either, 512 heads of four queries x 513 keys of 512
+  // bytes took 180 us, now 78; 128 x 1025 72, now 34.
+  for (int j0 = k0 + warp * KEYS_PER_WARP + which; j0 - which < k1; j0 += stride * kUnroll) {
+    A kv[kUnroll][V];
 #pragma unroll
     for (int u = 0; u < kUnroll; ++u) {
-      const int j = j0 + u * stride;
-      float kv[V];
-      Vec16<T>::widen(raw[u], kv);
+      float f[V];
+      Vec16<T>::widen(raw[u], f);
 #pragma unroll
-      for (int g = 0; g < kG; ++g) {
-        A acc = 0;
+      for (int e = 0; e < V; ++e) kv[u][e] = (A)f[e];
+    }
+    load(j0 + stride * kUnroll);
 #pragma unroll
-        for (int e = 0; e < V; ++e) acc = fma((A)qreg[g][e], (A)kv[e], acc);
+    for (int g = 0; g < kG; ++g) {
+      A acc[kUnroll];
 #pragma unroll
-        for (int o = LANES / 2; o; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-        if (sub == 0 && j < k1) logit[g * pitch + j - k0] = (float)(acc * c);    // log2 units
+      for (int u = 0; u < kUnroll; ++u) {
+        acc[u] = 0;
+#pragma unroll
+        for (int e = 0; e < V; ++e) acc[u] = fma(kHeld ? qreg[kHeld ? g : 0][e] : q_sm[kHeld ? 0 : g][sub * V + e], kv[u][e], acc[u]);
       }
+#pragma unroll
+      for (int o = LANES / 2; o; o >>= 1) {
+#pragma unroll
+        for (int u = 0; u < kUnroll; ++u) acc[u] += __shfl_xor_sync(0xffffffffu, acc[u], o);
+      }
+      // every lane has the sums of its four rows: lane u of a row stores that of key u
+      A mine = acc[0];
+#pragma unroll
+      for (int u = 1; u < kUnroll; ++u) mine = sub == u ? acc[u] : mine;
+      const int j = j0 + sub * stride;
+      if (sub < kUnroll && j < k1) logit[g * pitch + j - k0] = (float)(mine * c);    // log2 units
     }
   }
   __syncthreads();
@@ -238,7 +278,7 @@ __device__ __forceinline__ void reduce_stats(int count, F at, float (&M)[kG], fl
 }
 
 template <typename T, int D, int kG, bool kSlots, bool kCluster>
-__global__ void __launch_bounds__(kStepThreads) step_kernel(const __grid_constant__ StepArgs a, const __grid_constant__ Shape pl) {
+__global__ void __launch_bounds__(kStepThreads, std::is_same<T, float>::value && kG == 1 ? 2 : 1) step_kernel(const __grid_constant__ StepArgs a, const __grid_constant__ Shape pl) {
   extern __shared__ __align__(16) float logit[];                 // [kG][chunk]
   __shared__ float2 st[kG][kStepWarps], cta_st[kG];
   __shared__ unsigned long long best[kStepWarps], cta_best;
@@ -373,7 +413,7 @@ __global__ void __launch_bounds__(kStepThreads) step_kernel(const __grid_constan
 template <typename T, int D, int kG, bool kSlots, bool kCluster>
 ahakv_status launch_step_as(const StepArgs& a, const Shape& pl, int C, cudaStream_t st) {
   const size_t smem = (size_t)kG * a.chunk * sizeof(float);
-  if (smem > 40 * 1024) {
+  if (smem > 24 * 1024) {                                        // beside up to 18 KB of static shared memory
     constexpr int kMaxDevices = 64;
     static bool configured[kMaxDevices] = {};
     int dev = -1;

@@ -416,3 +416,54 @@ def test_time_of_compaction_in_place_of_many_heads():
     k_out, v_out, _, _ = ab.alloc_outputs(p)
     apart = _best_us(lambda: ab.ahakv_compact(p, k, v, None, idx, k_out, v_out, None))
     assert _best_us(lambda: ab.ahakv_compact_inplace(p, k, v, None, idx)) < apart
+
+
+@pytest.mark.parametrize("G,n,B,d", [(1, 1, 1, 64), (2, 63, 1, 128), (4, 65, 2, 64), (5, 513, 2, 128), (6, 130, 1, 64), (7, 300, 1, 128), (8, 2049, 1, 128),
+                                     (12, 700, 2, 64), (16, 2044, 1, 128), (4, 1025, 30, 64)])
+def test_float32_steps_at_every_group_size(G, n, B, d):
+    """The float32 one-row kernel, with the queries in registers and in shared memory, by one CTA a head and by several, for an ordered
+    cache and for slots, against float64: 1e-5 as for every float32 score."""
+    from paper_2506_03762_b200 import binding as ab
+    Hkv = 2
+    g = torch.Generator(device="cuda").manual_seed(n * G)
+    q = 2 * torch.randn((B, G * Hkv, 1, d), generator=g, device="cuda")
+    k, v = (torch.randn((B, Hkv, n, d), generator=g, device="cuda") for _ in range(2))
+    prev = torch.rand((B, Hkv, n), generator=g, device="cuda")
+    lam = 0.11
+    a = (float(np.float32(lam)) * (q.double().view(B, Hkv, G, d) @ k.double().transpose(-1, -2))).softmax(-1).mean(2)
+    p = ab.Params(B, G * Hkv, Hkv, d, n, 1, 0, max(1, n - 1), dtype=ab.F32, flags=0, scale_mode=ab.SCALE_FIXED, scale=lam, n_total=5000 + n)
+    score = torch.empty_like(prev)
+    ab.ahakv_score_step(p, q, k, prev, score)
+    assert torch.allclose(score.double(), a + prev.double(), rtol=1e-5, atol=1e-7)
+    if n < 3:
+        return
+    # the same cache as slots, the new token's row (row 1 of the cache above) still on its way in
+    slot = torch.full((B, Hkv), 1, dtype=torch.int32, device="cuda")
+    pos = torch.arange(5000, 5000 + n, dtype=torch.int32, device="cuda").expand(B, Hkv, n).contiguous()
+    pos[..., 1] = -1
+    k_t, v_t = k[:, :, 1:2].clone().contiguous(), v[:, :, 1:2].clone().contiguous()
+    want_k = k.clone()
+    k[:, :, 1] = float("nan")
+    f = prev.clone()
+    ab.ahakv_step_slots(p, q, k_t, v_t, k, v, f, pos, slot)
+    want = a + prev.double()
+    want[..., 1] = a[..., 1]
+    assert torch.allclose(f.double(), want, rtol=1e-5, atol=1e-7)
+    assert torch.equal(k, want_k)
+    assert torch.equal(slot.long(), f.argmin(-1))
+
+
+def test_time_of_a_float32_step():
+    """512 heads of four queries against 513 float32 keys: twice the bytes of 16-bit ones, and FP64 multiply-adds with their
+    reductions.  Three times as long is expected; seven times is what it took while every round of loads was waited for."""
+    from paper_2506_03762_b200 import binding as ab
+    B, Hkv, G, d, n = 64, 8, 4, 128, 513
+    us = {}
+    for dt, code in ((torch.float16, ab.F16), (torch.float32, ab.F32)):
+        g = torch.Generator(device="cuda").manual_seed(1)
+        q = torch.randn((B, G * Hkv, 1, d), generator=g, device="cuda").to(dt)
+        k = torch.randn((B, Hkv, n, d), generator=g, device="cuda").to(dt)
+        score = torch.empty((B, Hkv, n), device="cuda")
+        p = ab.Params(B, G * Hkv, Hkv, d, n, 1, 16, n - 1, dtype=code, flags=0)
+        us[code] = _best_us(lambda: ab.ahakv_score_step(p, q, k, None, score))
+    assert us[ab.F32] < 4 * us[ab.F16], us
