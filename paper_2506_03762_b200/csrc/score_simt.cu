@@ -423,6 +423,18 @@ simt_weighted_sums(const T* __restrict__ v, const float2* partial, const float* 
   griddep_wait();
   griddep_launch();
   if (nu) tile_norms<T, D>(v, nu, pl, b, h, unit, j0);
+  const int jl = threadIdx.x % kTile, share = threadIdx.x / kTile, j = j0 + jl;
+  const int heads = pl.group_max ? pl.G : 1, rows = pl.R / heads, first = 16 * (share >> 1) + 4 * (share & 1);
+  // numerators of eight of this thread's rows: i0 .. i0 + 3 and eight on
+  float e[2][4];
+  const auto load = [&](int g, int i0) {
+    const float* from = numer + ((size_t)unit * pl.R + g * rows) * pl.n + j;
+#pragma unroll
+    for (int y = 0; y < 2; ++y)
+#pragma unroll
+      for (int t = 0; t < 4; ++t) e[y][t] = j < pl.n && i0 + 8 * y + t < rows ? from[(size_t)(i0 + 8 * y + t) * pl.n] : 0.f;
+  };
+  load(0, first);                                      // on their way while the weights are formed
   for (int s0 = 0; s0 < pl.R; s0 += kRows) {
     // eight threads a row, each every eighth block in order, then the eight in order
     float2 p = make_float2(-INFINITY, 0.f);
@@ -443,26 +455,17 @@ simt_weighted_sums(const T* __restrict__ v, const float2* partial, const float* 
     }
     __syncthreads();
   }
-  const int jl = threadIdx.x % kTile, share = threadIdx.x / kTile, j = j0 + jl;
-  const int heads = pl.group_max ? pl.G : 1, rows = pl.R / heads;
   float best = 0.f;
   for (int g = 0; g < heads; ++g) {
-    const float* from = numer + ((size_t)unit * pl.R + g * rows) * pl.n + j;
     const float* by = weight[jl / 16] + g * rows;
     float acc[4] = {};
-    if (j < pl.n) {
-      for (int i0 = 16 * (share >> 1) + 4 * (share & 1); i0 < rows; i0 += kRows) {
-        float e[2][4];
+    for (int i0 = first; i0 < rows; i0 += kRows) {
+      if (g > 0 || i0 > first) load(g, i0);
 #pragma unroll
-        for (int y = 0; y < 2; ++y)
+      for (int y = 0; y < 2; ++y)
 #pragma unroll
-          for (int t = 0; t < 4; ++t) e[y][t] = i0 + 8 * y + t < rows ? from[(size_t)(i0 + 8 * y + t) * pl.n] : 0.f;
-#pragma unroll
-        for (int y = 0; y < 2; ++y)
-#pragma unroll
-          for (int t = 0; t < 4; ++t)
-            if (i0 + 8 * y + t < rows) acc[t] = fmaf(e[y][t], by[i0 + 8 * y + t], acc[t]);
-      }
+        for (int t = 0; t < 4; ++t)
+          if (i0 + 8 * y + t < rows) acc[t] = fmaf(e[y][t], by[i0 + 8 * y + t], acc[t]);
     }
     const float sum = (acc[0] + acc[1]) + (acc[2] + acc[3]);
     if (g > 0) __syncthreads();
