@@ -19,6 +19,8 @@
 // output, most of 8000 more.
 #include <cooperative_groups.h>
 
+#include <atomic>
+
 #include "ahakv_internal.cuh"
 #include "select_common.cuh"
 
@@ -746,32 +748,59 @@ __global__ void __launch_bounds__(kWideThreads) select_kernel(const float* __res
 
 template <int kPer, bool kCluster>
 cudaError_t launch_as(const SelectArgs& a, const Shape& pl, int C, cudaStream_t st) {
-  if (C > 8) {
-    // leave to use clusters beyond the portable size, asked for once per device
-    constexpr int kMaxDevices = 64;
-    static bool configured[kMaxDevices] = {};
-    int dev = -1;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess || dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
-    if (!configured[dev]) {
-      e = cudaFuncSetAttribute(refine_select_kernel<kPer, kCluster>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-      if (e != cudaSuccess) return e;
-      configured[dev] = true;
+  return launch_chained(refine_select_kernel<kPer, kCluster>, dim3(pl.B * pl.Hkv * C), dim3(kThreads), kCluster ? C : 1, 0, st, a, pl);
+}
+
+// The most CTAs a cluster may have on the current device: sixteen where it has room for one such cluster, beyond the portable eight
+// (a process that is given part of a GPU may not).  Asked once per device.
+cudaError_t cluster_limit(int* limit) {
+  constexpr int kMaxDevices = 64;
+  static std::atomic<int> known[kMaxDevices] = {};
+  int dev = -1;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess || dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
+  *limit = known[dev].load(std::memory_order_relaxed);
+  if (*limit != 0) return cudaSuccess;
+  const void* kernels[] = {(const void*)refine_select_kernel<4, true>, (const void*)refine_select_kernel<8, true>,
+                           (const void*)refine_select_kernel<kMaxPer, true>};
+  *limit = kMaxCluster;
+  for (const void* kernel : kernels) {
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e != cudaSuccess) return e;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(kMaxCluster);
+    cfg.blockDim = dim3(kThreads);
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = kMaxCluster;
+    attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    int fit = 0;
+    if (cudaOccupancyMaxActiveClusters(&fit, kernel, &cfg) != cudaSuccess || fit < 1) {
+      cudaGetLastError();
+      *limit = 8;
     }
   }
-  return launch_chained(refine_select_kernel<kPer, kCluster>, dim3(pl.B * pl.Hkv * C), dim3(kThreads), kCluster ? C : 1, 0, st, a, pl);
+  known[dev].store(*limit, std::memory_order_relaxed);
+  return cudaSuccess;
 }
 
 // One cluster per head.  False: no cluster holds a head.
 bool launch_clustered(SelectArgs a, const Shape& pl, cudaStream_t st, cudaError_t* err) {
-  if (pl.n > kMaxCluster * kThreads * kMaxPer) return false;   // 131072 tokens
+  int most = 8;
+  if (pl.n > most * kThreads * 8) {                    // more than eight CTAs would be wanted
+    *err = cluster_limit(&most);
+    if (*err != cudaSuccess) return true;
+  }
+  if (pl.n > most * kThreads * kMaxPer) return false;  // 131072 tokens
   // Eight tokens a thread while all heads' clusters fit on the GPU at once, two CTAs an SM; beyond that sixteen, with whose
   // smaller clusters fewer CTAs go through the same steps (256 heads of 32768 tokens: 72 us against 94, and 106 with one
   // such CTA an SM; 32 heads of 32768: 19 against 15; 4 of 70001: 21, before 26).
   const long long ctas8 = (long long)pl.B * pl.Hkv * ((pl.n + kThreads * 8 - 1) / (kThreads * 8));
   const int per_cta = kThreads * (ctas8 > 2 * 148 ? 16 : 8);
   int C = (pl.n + per_cta - 1) / per_cta;
-  if (C > kMaxCluster) C = kMaxCluster;
+  if (C > most) C = most;
   a.chunk = ((pl.n + C - 1) / C + kMaxPer - 1) / kMaxPer * kMaxPer;
   const int per = (a.chunk + kThreads - 1) / kThreads;
   if (C == 1) {
