@@ -44,7 +44,7 @@ struct Plan : Shape {
   size_t ws_wanted;          // ws_total and room for the softmax numerators of the FP32-pipe kernels at off ws_total
 };
 
-// plan.cu
+// api.cu
 // `obs_pos` (nullable, host, r ascending logical positions) places the observation rows; by default they are the
 // last r positions.
 ahakv_status make_plan(const ahakv_params* p, Plan* plan, const int64_t* obs_pos = nullptr);
@@ -82,8 +82,8 @@ ahakv_status launch_entropy(const Plan& pl, const void* q, const void* k, void* 
 size_t entropy_tc_scratch_bytes(const Plan& pl);
 ahakv_status launch_entropy_tc(const Plan& pl, const void* q, const void* k, void* scratch, float* out, cudaStream_t st);
 // Accumulation over every causal row on the tensor cores (score_stream.cu; plans with use_tc).  Leaves *n_slots partial sums
-// per head in *slots (`sums` if there is one: [B * Hkv][n]); `pool` is scratch, 256-byte aligned.
-bool causal_tc_fits(const Plan& pl, size_t pool_bytes);
+// per head in *slots (`sums` if there is one: [B * Hkv][n]); `pool` is scratch, 256-byte aligned: the room a plan with use_tc has
+// for raw scores and partials, over 2 n_rb floats for every row of the 128-row tiles of each head, always suffices.
 ahakv_status launch_causal_tc(const Plan& pl, int scale_mode, double fixed, long long first_cached, const void* q, const long long qs[3],
                               const void* k, float* pool, size_t pool_bytes, float* sums, const float** slots, int* n_slots,
                               int* status, cudaStream_t st);

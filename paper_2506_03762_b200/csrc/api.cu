@@ -279,7 +279,7 @@ ahakv_status ahakv_score_full_causal(const ahakv_params* p, const void* q_all, c
     if ((rc = launch_vnorm(full, v, nu, st))) return rc;
   }
   const size_t pool = full.off_nu - full.off_final;            // room for row statistics
-  if (full.use_tc && causal_tc_fits(full, pool)) {
+  if (full.use_tc) {
     long long qs[3];
     if (!resolve_strides(pc.q_stride, qs, full.Hq, full.n, full.d, full.es)) return AHAKV_ERR_INVALID_ARG;
     const double fixed = p->scale_mode == AHAKV_SCALE_FIXED ? (double)p->scale : eq12((double)p->n_total, (double)p->budget, p->head_dim);

@@ -738,11 +738,6 @@ ahakv_status launch_entropy_tc(const Plan& pl, const void* q, const void* k, voi
 
 // The room: row scales, -L per row of the query heads of a pass, the parts of their statistics, and the column sums of
 // every split.  `pool` is what the workspace has for them.  As many query heads of each group a pass as fit.
-bool causal_tc_fits(const Plan& pl, size_t pool_bytes) {
-  const size_t n_pad = (size_t)pl.n_blk * kKeyTile;
-  return pool_bytes >= sizeof(float) * (n_pad + (size_t)pl.B * pl.Hkv * n_pad);
-}
-
 ahakv_status launch_causal_tc(const Plan& pl, int scale_mode, double fixed, long long first_cached, const void* q, const long long qs[3],
                               const void* k, float* pool, size_t pool_bytes, float* sums, const float** slots_out, int* n_slots,
                               int* status, cudaStream_t st) {

@@ -1,6 +1,6 @@
-// Pieces shared by the refinement / selection kernels (select.cu, finish.cu): the mean filter of Eq. 13 and
-// the order-preserving integer image of a score.  Both files must produce bit-identical refined scores, so the
-// order of the additions below is part of the contract.
+// Pieces shared by the refinement / selection kernels (select.cu) and the one-row kernels (decode.cu): the mean filter of
+// Eq. 13 and the order-preserving integer image of a score.  The kernels for contexts of any length must produce bit-identical
+// refined scores, so the order of the additions below is part of the contract.
 #pragma once
 
 #include "ahakv_internal.cuh"

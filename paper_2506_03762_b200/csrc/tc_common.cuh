@@ -91,18 +91,6 @@ __device__ __forceinline__ void tc_commit(void* bar) {
                : "memory");
 }
 
-// Shared-memory operand descriptor (fields as described at umma_desc_lo below) of a K-major tile of 32-byte
-// rows (16 elements, one k-step), 32-byte swizzle, 8-row groups 256 bytes apart.
-__device__ __forceinline__ uint64_t umma_desc_ext(uint32_t smem_addr) {
-  uint64_t d = 0;
-  d |= (uint64_t)((smem_addr & 0x3ffff) >> 4);
-  d |= (uint64_t)1 << 16;
-  d |= (uint64_t)(256 >> 4) << 32;
-  d |= (uint64_t)1 << 46;
-  d |= (uint64_t)6 << 61;                               // SWIZZLE_32B
-  return d;
-}
-
 // Instruction descriptor for kind::f16: FP32 accumulate, A and B both K-major and of one type.
 __device__ __forceinline__ uint32_t umma_idesc(int M, int N, int bf16) {
   uint32_t d = 0;
@@ -139,37 +127,10 @@ __device__ __forceinline__ void tmem_ld_wait(uint32_t* r) {
                : "memory");
 }
 
-// 16 consecutive FP32 columns of this thread's TMEM lane: issue now, use after tmem_ld_wait16(r).
-__device__ __forceinline__ void tmem_ld16_issue(uint32_t taddr, uint32_t* r) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
-      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-      : "r"(taddr)
-      : "memory");
-}
-__device__ __forceinline__ void tmem_ld_wait16(uint32_t* r) {
-  asm volatile("tcgen05.wait::ld.sync.aligned;"
-               : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),
-                 "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15])
-               :
-               : "memory");
-}
-
-__device__ __forceinline__ void group_sync(int id, int threads) {
-  asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
-}
-
 // One partial, straight from L2 (other CTAs write it while this one polls).
 __device__ __forceinline__ float2 ld_partial2(const float2* p) {   // two adjacent rows
   float2 v;
   asm volatile("ld.relaxed.gpu.global.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p) : "memory");
-  return v;
-}
-__device__ __forceinline__ float ld_partial(const float* p) {
-  float v;
-  asm volatile("ld.relaxed.gpu.global.f32 %0, [%1];" : "=f"(v) : "l"(p) : "memory");
   return v;
 }
 __device__ __forceinline__ void st_partial(float* p, float v) {
