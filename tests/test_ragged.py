@@ -95,8 +95,8 @@ def test_carried_scores_of_a_ragged_batch_start_anywhere(dtype_name, Hkv, n_max,
 def test_a_budget_per_head(dtype_name, Hq, Hkv, d, n):
     """Every (sequence, KV head) keeps its recent window and the best of the rest up to its own budget: what
     ``ahakv_evict`` gives that head when the whole batch has that budget, bit for bit, and what the oracle says;
-    entries past a head's own count are -1 and the output rows there are not touched.  (33000 tokens take the separate selection
-    kernel, the others the fused one.)"""
+    entries past a head's own count are -1 and the output rows there are not touched.  (33000 tokens are selected by a cluster of
+    CTAs a head, the others by one.)"""
     from paper_2506_03762_b200 import binding as ab
     from tests import parity
     dtype = getattr(ab, dtype_name)
