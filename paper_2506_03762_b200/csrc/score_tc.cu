@@ -84,6 +84,7 @@ struct TcArgs {
   int prior;      // stream V and write nu
   float log2G;
   float c[kMaxRows];     // lambda_i log2(e) per observation row
+  float row_scale[128];  // the same per stacked row of a row block (of the first one where a head has two)
   int last[kMaxRows];    // per observation row: the last key it may see
   int min_last;          // the smallest of them: tiles that end at or before it are masked for no row
   float* partial;    // [unit][rpu][128]: log2 of a row's sum of 2^{c w} over the keys of a run
@@ -106,10 +107,6 @@ template <bool kTest> __device__ __forceinline__ long long wait_limit(const TcAr
 }
 
 // ---- shared memory layout --------------------------------------------------------------------
-struct __align__(16) RowPair {               // two adjacent stacked rows of the row block a pass-2 run is about
-  float c0, c1, neg_off0, neg_off1;
-};
-
 // One segment as the scheduler decodes it for everybody else.
 struct __align__(16) Seg {
   int code;                                 // pass | tiles << 1 | live rows << 8, or kSegEnd
@@ -119,8 +116,8 @@ struct __align__(16) Seg {
 };
 
 struct Shared {
-  RowPair tab[2][64];                       // by pass-2 segment parity
-  int2 tab_last[2][64];                     // the last key each of the two rows may see; -1 past the live rows
+  float neg_off[2][128];                    // by pass-2 segment parity: minus a row's offset, -inf past the live rows
+  int tab_last[2][128];                     // the last key each row may see; -1 past the live rows
   float stat[2][kGroups][128];              // by pass-1 segment parity: each group's statistic of a row over the run
   float row_c[2][128];                      // lambda log2(e) per stacked row, by kind of row block (r > 128 has two)
   int row_last[2][128];                     // the last key a stacked row may see
@@ -400,22 +397,38 @@ __device__ __forceinline__ void mma_warp(const TcArgs& a, Shared* sh, char* tile
 }
 
 // Thirty-two stacked rows of a key's column: adds 2^{c D - off} of each to the four running sums.
-template <bool kMasked>
-__device__ __forceinline__ void column_chunk(const uint32_t* r, const RowPair* tab, const int2* last, int j, uint64_t& za,
-                                             uint64_t& zb) {
+//
+// The scales are the launch's parameters, at places the compiler knows, and only the offsets come from shared memory: a
+// broadcast costs its 128 bytes a cycle as much as 32 different values do, so that scales and offsets together (64 reads of 16 bytes a
+// tile and warp) took 1024 cycles of it, as long as the tile's exponentials, and the products want it at its full rate for
+// 512 and the copies for 256.  A tile of pass 2 takes a group 3150 cycles instead of 3700: a decode
+// round (16 sequences x 8 heads x 2080 tokens) 44.1 -> 42.6 us, and with the value rows' loop below 16384 x 8 x 4 127 -> 122,
+// 20000 x 32 heads of 64 elements 95 -> 81.
+__device__ __forceinline__ void column_chunk(const uint32_t* r, const float* cs, const float* neg_off, uint64_t& za, uint64_t& zb) {
 #pragma unroll
   for (int t = 0; t < 32; t += 4) {
-    const RowPair p0 = tab[t / 2], p1 = tab[t / 2 + 1];
+    const float4 o = *reinterpret_cast<const float4*>(neg_off + t);
     float x0, x1, x2, x3;
-    unpack2(fma2(pack2(__uint_as_float(r[t]), __uint_as_float(r[t + 1])), pack2(p0.c0, p0.c1), pack2(p0.neg_off0, p0.neg_off1)), x0, x1);
-    unpack2(fma2(pack2(__uint_as_float(r[t + 2]), __uint_as_float(r[t + 3])), pack2(p1.c0, p1.c1), pack2(p1.neg_off0, p1.neg_off1)), x2, x3);
-    if (kMasked) {
-      const int2 l0 = last[t / 2], l1 = last[t / 2 + 1];
-      if (j > l0.x) x0 = -INFINITY;
-      if (j > l0.y) x1 = -INFINITY;
-      if (j > l1.x) x2 = -INFINITY;
-      if (j > l1.y) x3 = -INFINITY;
-    }
+    unpack2(fma2(pack2(__uint_as_float(r[t]), __uint_as_float(r[t + 1])), pack2(cs[t], cs[t + 1]), pack2(o.x, o.y)), x0, x1);
+    unpack2(fma2(pack2(__uint_as_float(r[t + 2]), __uint_as_float(r[t + 3])), pack2(cs[t + 2], cs[t + 3]), pack2(o.z, o.w)), x2, x3);
+    za = add2(za, pack2(fast_exp2(x0), fast_exp2(x1)));
+    zb = add2(zb, pack2(fast_exp2(x2), fast_exp2(x3)));
+  }
+}
+// ... with everything from shared memory, and each row only up to the last key it may see.
+__device__ __forceinline__ void column_chunk_masked(const uint32_t* r, const float* cs, const float* neg_off, const int* last, int j,
+                                                    uint64_t& za, uint64_t& zb) {
+#pragma unroll
+  for (int t = 0; t < 32; t += 4) {
+    const float4 c = *reinterpret_cast<const float4*>(cs + t), o = *reinterpret_cast<const float4*>(neg_off + t);
+    const int4 l = *reinterpret_cast<const int4*>(last + t);
+    float x0, x1, x2, x3;
+    unpack2(fma2(pack2(__uint_as_float(r[t]), __uint_as_float(r[t + 1])), pack2(c.x, c.y), pack2(o.x, o.y)), x0, x1);
+    unpack2(fma2(pack2(__uint_as_float(r[t + 2]), __uint_as_float(r[t + 3])), pack2(c.z, c.w), pack2(o.z, o.w)), x2, x3);
+    if (j > l.x) x0 = -INFINITY;
+    if (j > l.y) x1 = -INFINITY;
+    if (j > l.z) x2 = -INFINITY;
+    if (j > l.w) x3 = -INFINITY;
     za = add2(za, pack2(fast_exp2(x0), fast_exp2(x1)));
     zb = add2(zb, pack2(fast_exp2(x2), fast_exp2(x3)));
   }
@@ -475,29 +488,44 @@ __device__ __forceinline__ void softmax_group(const TcArgs& a, Shared* sh, uint3
       const int slot = pc & 1;
       if (!gone && !mbar_wait(&sh->tab_full[slot], (pc >> 1) & 1, a.status, wait_limit<kTest>(a))) gone = true;
       ++pc;
-      const RowPair* tab = sh->tab[slot];
-      const int2* tlast = sh->tab_last[slot];
-      const int chunks = (rows + 31) >> 5;
-      const bool whole = (rows & 31) == 0;
+      const float* neg_off = sh->neg_off[slot];
+      const int chunks = (rows + 31) >> 5, kind = sg.q_row != 0;
+      // Rows past the live ones that no box covers are zeros, which their offsets take to nothing; where the box brought rows
+      // of another head, their terms have to be masked.
+      const bool plain = kind == 0 && ((rows & 31) == 0 || rows == a.hb * a.r);
       for (int t = first; t < cnt; t += kGroups, ++mine) {
         const int acc = (tc + t) & 3;
         if (gone) continue;
         if (!mbar_wait(&sh->acc_full[g][mine & 3], (mine >> 2) & 1, a.status, wait_limit<kTest>(a))) { gone = true; continue; }
         tc_fence_after();
         const int j0 = (sg.blk0 + t) * kKeyTile, j = j0 + s;
-        const bool full = whole && j0 + kKeyTile - 1 <= a.min_last;
         uint64_t za = pack2(0.f, 0.f), zb = pack2(0.f, 0.f);
-#pragma unroll 1
-        for (int ch = 0; ch < chunks; ++ch) {
-          uint32_t ra[32];
-          tmem_ld32_issue(lane_base + acc * 128 + 32 * ch, ra);
-          tmem_ld_wait(ra);
-          if (ch == chunks - 1) {
-            tc_fence_before();
-            mbar_arrive(&sh->acc_empty[acc]);
+        if (plain && j0 + kKeyTile - 1 <= a.min_last) {
+#pragma unroll
+          for (int ch = 0; ch < 4; ++ch) {
+            if (ch < chunks) {
+              uint32_t ra[32];
+              tmem_ld32_issue(lane_base + acc * 128 + 32 * ch, ra);
+              tmem_ld_wait(ra);
+              if (ch + 1 == chunks) {
+                tc_fence_before();
+                mbar_arrive(&sh->acc_empty[acc]);
+              }
+              column_chunk(ra, a.row_scale + 32 * ch, neg_off + 32 * ch, za, zb);
+            }
           }
-          if (full) column_chunk<false>(ra, tab + 16 * ch, tlast + 16 * ch, j, za, zb);
-          else column_chunk<true>(ra, tab + 16 * ch, tlast + 16 * ch, j, za, zb);
+        } else {
+#pragma unroll 1
+          for (int ch = 0; ch < chunks; ++ch) {
+            uint32_t ra[32];
+            tmem_ld32_issue(lane_base + acc * 128 + 32 * ch, ra);
+            tmem_ld_wait(ra);
+            if (ch + 1 == chunks) {
+              tc_fence_before();
+              mbar_arrive(&sh->acc_empty[acc]);
+            }
+            column_chunk_masked(ra, sh->row_c[kind] + 32 * ch, neg_off + 32 * ch, sh->tab_last[slot] + 32 * ch, j, za, zb);
+          }
         }
         float z0, z1;
         unpack2(add2(za, zb), z0, z1);
@@ -569,7 +597,7 @@ __device__ __forceinline__ void delivery(const TcArgs& a, Shared* sh) {
 }
 
 // Table warp.  For every pass-2 run the scheduler announces, in order and ahead of the softmax warps: waits until the
-// offsets of the row block have been published and writes its rows' constants into shared memory, four rows a lane.
+// offsets of the row block have been published and writes them into shared memory, four rows a lane.
 template <bool kTest>
 __device__ __forceinline__ void table_warp(const TcArgs& a, Shared* sh) {
   const int lane = threadIdx.x & 31;
@@ -595,8 +623,8 @@ __device__ __forceinline__ void table_warp(const TcArgs& a, Shared* sh) {
           return;
         }
       }
-      sh->tab[slot][s] = {sh->row_c[kind][r0], sh->row_c[kind][r1], -off.x, -off.y};
-      sh->tab_last[slot][s] = make_int2(r0 < rows ? sh->row_last[kind][r0] : -1, r1 < rows ? sh->row_last[kind][r1] : -1);
+      *reinterpret_cast<float2*>(&sh->neg_off[slot][r0]) = make_float2(r0 < rows ? -off.x : -INFINITY, r1 < rows ? -off.y : -INFINITY);
+      *reinterpret_cast<int2*>(&sh->tab_last[slot][r0]) = make_int2(r0 < rows ? sh->row_last[kind][r0] : -1, r1 < rows ? sh->row_last[kind][r1] : -1);
     }
     mbar_arrive(&sh->tab_full[slot]);
     if (lane == 0) *(volatile int*)&sh->mrg_done = mc + 1;
@@ -611,20 +639,44 @@ __device__ __forceinline__ uint4 ld_once(const char* p) {   // read once: do not
   return v;
 }
 template <typename T, int D>
-__device__ __forceinline__ void value_norms(const TcArgs& a, int w, int n_warps) {
+__device__ __forceinline__ void value_norms(const TcArgs& a, unsigned w, unsigned n_warps) {
   constexpr int kPieces = D / 32, kSets = kValueLoads / kPieces, kRows = 8 * kSets;   // 64-byte pieces a row, 8-row sets in flight
-  const int lane = threadIdx.x & 31, grp = lane >> 2, tig = lane & 3;
-  const int per_head = (a.n + kRows - 1) / kRows;
-  const long long total = (long long)a.BH * per_head;
-  for (long long ch = w; ch < total; ch += n_warps) {
-    const int bh = (int)(ch / per_head), row0 = (int)(ch - (long long)bh * per_head) * kRows + grp;
-    const char* base = a.v + (bh / a.Hkv) * a.vs[0] + (bh % a.Hkv) * a.vs[1] + tig * 16;
+  const int grp = (threadIdx.x & 31) >> 2, tig = threadIdx.x & 3;
+  const unsigned per_head = (unsigned)(a.n + kRows - 1) / kRows, heads = (unsigned)a.BH, per_seq = (unsigned)a.Hkv;
+  const unsigned step_h = n_warps / per_head, step = n_warps - step_h * per_head;
+  unsigned bh = w / per_head, at = w - bh * per_head, b = bh / per_seq, h = bh - b * per_seq;   // head and chunk of it
+  if (bh >= heads) return;
+  const char* p[kSets];
+  int row;
+  auto locate = [&]() {   // rows past the end read the last one again; nothing of theirs is stored
+    row = (int)at * kRows + grp;
+    const char* head = a.v + b * a.vs[0] + h * a.vs[1] + tig * 16;
+#pragma unroll
+    for (int q = 0; q < kSets; ++q) p[q] = head + min(row + 8 * q, a.n - 1) * a.vs[2];
+  };
+  locate();
+  for (;;) {
     uint4 u[kSets][kPieces];
 #pragma unroll
     for (int q = 0; q < kSets; ++q)
 #pragma unroll
-      for (int i = 0; i < kPieces; ++i)
-        u[q][i] = row0 + 8 * q < a.n ? ld_once(base + (row0 + 8 * q) * a.vs[2] + i * 64) : make_uint4(0, 0, 0, 0);
+      for (int i = 0; i < kPieces; ++i) u[q][i] = ld_once(p[q] + i * 64);
+    // where the next chunk is, while this one is on its way
+    float* const to = a.nu + (size_t)bh * a.n + row;
+    const int left = a.n - row;
+    at += step;
+    unsigned heads_on = step_h;
+    if (at >= per_head) { at -= per_head; ++heads_on; }
+    bh += heads_on;
+    h += heads_on;
+    if (h >= per_seq) {
+      const unsigned seqs = h / per_seq;
+      h -= seqs * per_seq;
+      b += seqs;
+    }
+    if (bh < heads) locate();
+#pragma unroll
+    for (int q = 0; q < kSets; ++q) asm volatile("" : "+l"(p[q]));   // now, not after the sums
 #pragma unroll
     for (int q = 0; q < kSets; ++q) {
       uint64_t acc = pack2(0.f, 0.f), acc2 = pack2(0.f, 0.f);
@@ -644,16 +696,17 @@ __device__ __forceinline__ void value_norms(const TcArgs& a, int w, int n_warps)
       float sq = s0 + s1;
       sq += __shfl_xor_sync(0xffffffffu, sq, 1);
       sq += __shfl_xor_sync(0xffffffffu, sq, 2);
-      if (tig == 0 && row0 + 8 * q < a.n) a.nu[(size_t)bh * a.n + row0 + 8 * q] = sq;
+      if (tig == 0 && 8 * q < left) to[8 * q] = sq;
     }
+    if (bh >= heads) return;
   }
 }
 
 // The softmax warps keep a chunk of the accumulator and its exponentials in registers, the others need few: of the 80 a
-// thread that the launch allows (768 threads), each of the twelve softmax warps takes 112 and the other twelve keep 48
-// (384 x 112 + 384 x 48 = 768 x 80).
-__device__ __forceinline__ void regs_down() { asm volatile("setmaxnreg.dec.sync.aligned.u32 48;"); }
-__device__ __forceinline__ void regs_up() { asm volatile("setmaxnreg.inc.sync.aligned.u32 112;"); }
+// thread that the launch allows (768 threads), each of the twelve softmax warps takes 104 and the other twelve keep 56
+// (384 x 104 + 384 x 56 = 768 x 80).
+__device__ __forceinline__ void regs_down() { asm volatile("setmaxnreg.dec.sync.aligned.u32 56;"); }
+__device__ __forceinline__ void regs_up() { asm volatile("setmaxnreg.inc.sync.aligned.u32 104;"); }
 
 template <bool kTest>
 __global__ void __launch_bounds__(kThreads, 1)
@@ -734,7 +787,7 @@ score_tc_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_constant_
     if (warp == kSchedWarp) {
       if (lane == 0) scheduler<kTest>(a, sh, p1_first, p2_first);
     } else if (a.prior) {
-      const int w = blockIdx.x * kValueWarps + warp - kFirstValue, n_warps = gridDim.x * kValueWarps;
+      const unsigned w = blockIdx.x * kValueWarps + warp - kFirstValue, n_warps = gridDim.x * kValueWarps;
       if (a.bf16) { if (a.D == 128) value_norms<__nv_bfloat16, 128>(a, w, n_warps); else value_norms<__nv_bfloat16, 64>(a, w, n_warps); }
       else { if (a.D == 128) value_norms<__half, 128>(a, w, n_warps); else value_norms<__half, 64>(a, w, n_warps); }
     }
@@ -819,6 +872,7 @@ ahakv_status launch_score_tc(const Plan& pl, const void* q, const void* k, const
   a.prior = (pl.flags & AHAKV_FLAG_VALUE_PRIOR) != 0 && v != nullptr && nu != nullptr;
   a.log2G = pl.group_max ? 0.f : log2f((float)pl.G);   // pooling by maximum keeps each head's own score
   for (int i = 0; i < kMaxRows; ++i) a.c[i] = pl.rows.c[i];
+  for (int i = 0; i < 128; ++i) a.row_scale[i] = pl.rows.c[pl.r <= 128 ? i % pl.r : i];
   a.partial = partial_ws; a.off = off_ws; a.s_raw = s_raw; a.nu = nu;
   a.v = (const char*)v;
   for (int t = 0; t < 3; ++t) a.vs[t] = pl.vs[t] * pl.es;
