@@ -30,12 +30,13 @@
 //
 // Schedule.  A run is a few consecutive key tiles of one row block.  Runs are handed out to the CTAs (one per SM)
 // as they come free, from two global counters: one for pass 1, one for pass 2.  The scheduler warp of
-// every CTA takes one run of each per round (pass 2 only once every pass-1 run of that row block, and half a grid round
-// more, have been taken by somebody) and publishes the CTA's sequence of segments, P1(a), P2(b), P1(a'), P2(b'), ..., in
-// a ring in shared memory that all other roles read in order; the pass-2 run of a round is announced to the
-// table warp a round early.  Pass 2 trails pass 1 by about one round of the whole grid: long enough for every CTA to
-// have delivered its share of a row block's statistics, short enough for the keys to be still in L2, so that HBM sees K
-// (nearly) once.  SMs that fall behind simply take fewer runs.
+// every CTA takes one run of each per round and publishes the CTA's sequence of segments, P1(a), P1(a'), P2(b), P1(a''),
+// P2(b'), ..., in a ring in shared memory that all other roles read in order; the pass-2 run of a round is announced to the
+// table warp a round early.  Where a CTA does enough runs, pass 2 trails pass 1 by a round of the whole grid in that sequence:
+// long enough for every CTA to have delivered its share of a row block's statistics, short enough for the keys to be still in
+// L2, so that HBM sees K (nearly) once.  (What counts is the order in which a CTA does its runs.  By the counters alone, which
+// run ahead of the work by the segments published, a row block's pass 2 came right behind its own pass 1, and every group of softmax
+// warps stood still for the merge: 11 % of the time at 32768 tokens x 64 heads, now 3.)  SMs that fall behind simply take fewer runs.
 //
 // Between the passes: the delivery warp stores every run's row statistics as a partial and counts the run on its row
 // block's counter; whoever completes the count merges the partials of the whole row block, always in the order of the
@@ -61,7 +62,7 @@ namespace {
 
 using namespace tc;
 
-constexpr int kKStages = 4;                // K-tile ring depth
+constexpr int kKStages = 3;                // K-tile ring depth (four: 119 us for 115 at 16384 tokens x 8 heads x 4; two: 49 for 47 at 8192 x 32)
 constexpr int kGroups = 3;                 // groups of four softmax warps
 constexpr int kSubTileBytes = 128 * 128;   // 128 rows x 64 16-bit elements, 128-byte swizzled
 constexpr int kSegRing = 16;               // published segments a role may lag behind the scheduler
@@ -78,7 +79,7 @@ struct TcArgs {
   int CH;         // key tiles per run
   int rpu;        // runs per row block = ceil(n_blk / CH)
   int n_runs;     // row blocks * rpu
-  int gap;        // pass-1 runs that have to be taken after a row block's last before pass 2 turns to it
+  int gap;        // how far behind a row block's last run the pass-1 run lies that a CTA does before pass 2 turns to the block
   int max_lead;   // runs that pass 1 may be ahead of pass 2
   int bf16;       // operand type of the products
   int prior;      // stream V and write nu
@@ -220,6 +221,7 @@ __device__ __forceinline__ int2 mrg_get(Shared* sh, int idx, int* status, long l
 struct Scheduler {
   int k, m, pend;
   int p1_next, p2_next;                 // runs already asked of the counters, or -1
+  int own;                              // the last pass-1 run of this CTA
   bool p1_left, p2_left, done;
 };
 __device__ __forceinline__ void sched_publish(Shared* sh, Scheduler& sc, const Seg& entry) {
@@ -250,16 +252,26 @@ __device__ __forceinline__ void sched_round(const TcArgs& a, Shared* sh, Schedul
   // be: it merges a row block's partials while the softmax warps go on, and has to have read what is overwritten.
   if (sc.k - ds >= kSegAhead || sc.k - ld_volatile(&sh->seg_read) > kSegRing - 2 || sc.m - ld_volatile(&sh->mrg_done) > kMergeRing - 2) return;
   // Pass 1 may run ahead of pass 2 by max_lead runs, no further: what lies between the two counters has to stay in L2.
-  if (sc.p1_left && (sc.pend < 0 || ld_volatile(&a.ctr[0]) - ld_volatile(&a.ctr[1]) < a.max_lead)) {
+  const bool room = sc.pend < 0 || ld_volatile(&a.ctr[0]) - ld_volatile(&a.ctr[1]) < a.max_lead;
+  if (sc.p1_left && room) {
     const int r = sc.p1_next >= 0 ? sc.p1_next : atomicAdd(&a.ctr[0], 1) + 1;            // the counters start at -1
     sc.p1_next = -1;
-    if (r < a.n_runs) sched_publish(sh, sc, decode(a, r, 0));
-    else sc.p1_left = false;
+    if (r < a.n_runs) {
+      sched_publish(sh, sc, decode(a, r, 0));
+      sc.own = r;
+    } else {
+      sc.p1_left = false;
+    }
   }
   if (sc.pend >= 0) {
-    // the pass-2 run in hand joins the sequence once all pass-1 runs of its row block, and `gap` more, have been taken
-    const int need = min((sc.pend / a.rpu + 1) * a.rpu + a.gap, a.n_runs);
-    if (ld_volatile(&a.ctr[0]) + 1 >= need) { sched_publish(sh, sc, decode(a, sc.pend, 1)); sc.pend = -1; }
+    // The pass-2 run in hand joins the sequence behind a pass-1 run of this CTA that lies `gap` runs beyond its row block: when
+    // its turn comes the other CTAs are about as far, and have delivered theirs.  Where the counters are too far apart for
+    // another pass-1 run, all runs of its row block have been taken long ago.
+    const int end = (sc.pend / a.rpu + 1) * a.rpu;
+    if (!sc.p1_left || sc.own >= end + a.gap || (!room && ld_volatile(&a.ctr[0]) + 1 >= end)) {
+      sched_publish(sh, sc, decode(a, sc.pend, 1));
+      sc.pend = -1;
+    }
   }
   if (sc.pend < 0 && sc.p2_left) {
     const int b = sc.p2_next >= 0 ? sc.p2_next : atomicAdd(&a.ctr[1], 1) + 1;
@@ -282,7 +294,7 @@ __device__ __forceinline__ void sched_round(const TcArgs& a, Shared* sh, Schedul
 // Scheduler: one thread keeps the CTA's sequence of segments filled.
 template <bool kTest>
 __device__ __forceinline__ void scheduler(const TcArgs& a, Shared* sh, int p1_first, int p2_first) {
-  Scheduler sched = {0, 0, -1, p1_first, p2_first, true, true, false};
+  Scheduler sched = {0, 0, -1, p1_first, p2_first, -1, true, true, false};
   long long t0 = now_ns();
   int last_k = 0, last_ds = 0;
   for (int spins = 0; !sched.done; ++spins) {
@@ -819,16 +831,15 @@ TestHooks test_hooks() { return {g_test_wait_ns.load(), g_test_withhold.load()};
 
 // How many runs a row block's key tiles are cut into.  A run boundary costs about as much as a tile visit (a Q tile to
 // load, statistics to hand over, constants to pick up), and the runs of all row blocks are dealt to the CTAs in rounds:
-// the number that makes rounds x (tiles of a run + 1) smallest.  Runs have at most 8 tiles where the keys do not stay in
-// L2 (126 MB) as a whole: what lies between the two passes of a run, about two grid rounds, has to.  Where they do (96 MB,
-// with room for what else passes through) they have up to 16: one long request of 70001 tokens x 4 heads 138 -> 88 us a
-// call against 8, a decode round 94 -> 92.5; 12 and 24 are slower or no better.
-static int runs_per_row_block(long long units, int n_blk, int slots, long long key_bytes) {
-  const int longest = key_bytes > (96LL << 20) ? 8 : 16;
+// the number that makes rounds x (tiles of a run + 1) smallest, with runs of at most 16 tiles.  Two grid rounds of those are
+// 155 MB of keys where each row block has its own, more than L2, and yet shorter ones are slower: at most 8 tiles a run 1125
+// us for 1054 at 32768 tokens x 256 heads, 80.5 for 77.6 at 16384 x 32; at most 24 no better, and slower where one long request has few heads.
+static int runs_per_row_block(long long units, int n_blk, int slots) {
+  constexpr int kLongest = 16;
   int best = n_blk;
   long long best_cost = -1;
   // the fewest runs of every length; more runs of the same length cost the same
-  for (int len = longest; len >= 1; --len) {
+  for (int len = kLongest; len >= 1; --len) {
     const int rpu = (n_blk + len - 1) / len, ch = (n_blk + rpu - 1) / rpu;
     const long long cost = (units * ((n_blk + ch - 1) / ch) + slots - 1) / slots * (ch + 1);
     if (best_cost < 0 || cost < best_cost) { best = rpu; best_cost = cost; }
@@ -859,14 +870,16 @@ ahakv_status launch_score_tc(const Plan& pl, const void* q, const void* k, const
   a.D = pl.d;
   for (int i = 0; i < kMaxRows; ++i) a.last[i] = pl.last[i];
   a.min_last = pl.last[0];
-  a.rpu = runs_per_row_block(units, a.n_blk, slots, (long long)pl.B * pl.Hkv * a.n_blk * kKeyTile * pl.d * pl.es);
+  a.rpu = runs_per_row_block(units, a.n_blk, slots);
   a.CH = (a.n_blk + a.rpu - 1) / a.rpu;
   a.rpu = (a.n_blk + a.CH - 1) / a.CH;
   a.n_runs = units * a.rpu;
   const int grid = a.n_runs < slots ? a.n_runs : slots;
-  // Half a grid round: most CTAs have then finished and delivered the runs they held.  At 32768 tokens x 256 heads a gap of
-  // none, half and one round measured 1.43, 1.41 and 1.44 ms a step under sustained load.
-  a.gap = grid / 2;
+  // A grid round, where each CTA does three runs or more.  With fewer the wait for a row block's statistics costs less than a
+  // round in which only one of the passes runs: 70001 tokens x 4 heads of 7 queries (1.9 rounds) 66 us with no gap, 73 with a
+  // round; 32768 x 8 heads of 4 (1.7) 69 and 72.  16384 x 32 (3.5) 87 and 81, and 84 with half a round; 16384 x 8 x 4 119 and 115; 32768 x 64
+  // 278 and 262.  One and a half are no better anywhere.
+  a.gap = a.n_runs >= 3 * grid ? grid : 0;
   a.max_lead = 3 * grid + a.rpu;
   a.bf16 = pl.dtype == AHAKV_BF16;
   a.prior = (pl.flags & AHAKV_FLAG_VALUE_PRIOR) != 0 && v != nullptr && nu != nullptr;
