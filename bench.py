@@ -81,7 +81,7 @@ def kernel_source_digest():
     """sha1 of the scoring kernel's sources: DRAM counters taken from an older kernel are not reported."""
     import hashlib
     h = hashlib.sha1()
-    for name in ("score_tc.cu", "tc_common.cuh"):
+    for name in ("score_tc.cu", "score_common.cuh", "tc_common.cuh"):
         with open(os.path.join(ROOT, "paper_2506_03762_b200", "csrc", name), "rb") as f:
             h.update(f.read())
     return h.hexdigest()

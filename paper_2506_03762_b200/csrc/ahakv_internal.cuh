@@ -57,7 +57,7 @@ size_t simt_kept_floats(const Plan& pl);
 ahakv_status launch_score_simt(const Plan& pl, const void* q, const void* k, const void* v, float* s_raw, float* nu, float2* partial,
                                float* kept, int* status, cudaStream_t st);
 ahakv_status launch_score_tc(const Plan& pl, const void* q, const void* k, const void* v, float* s_raw, float* nu,
-                             float* partial, float* off, int* counters, int* status, cudaStream_t st);
+                             float* partial, float* off, int* counters, int* status, void* ones, size_t ones_bytes, cudaStream_t st);
 bool score_tc_available();
 // See ahakv_test_set_wait: the limit of the tensor-core kernels' bounded waits (0: their own), and whether a fault is planted.
 struct TestHooks {

@@ -183,9 +183,8 @@ static ahakv_status queue_raw_score(const Plan& pl, const void* q, const void* k
   if (pl.use_tc) {
     // the kernel skips the tiles that no observation row sees: their raw score is zero
     if (pl.n_eff != pl.n && cudaMemsetAsync(s_raw, 0, pl.off_partial - pl.off_sraw, st) != cudaSuccess) return AHAKV_ERR_CUDA;
-    if ((rc = launch_clear(at<char>(ws, pl.off_status), pl.off_sraw - pl.off_status, st))) return rc;
     rc = launch_score_tc(pl, q, k, prior ? v : nullptr, s_raw, nu, at<float>(ws, pl.off_partial), final_off,
-                         at<int>(ws, pl.off_sync), at<int>(ws, pl.off_status), st);
+                         at<int>(ws, pl.off_sync), at<int>(ws, pl.off_status), at<char>(ws, pl.off_status), pl.off_sraw - pl.off_status, st);
     profile_mark(prof, 1, st);
   } else {
     float* kept = pl.ws_wanted > pl.ws_total && ws_bytes >= pl.ws_wanted ? at<float>(ws, pl.ws_total) : nullptr;

@@ -1,0 +1,469 @@
+// Tensor-core scoring for calls that fit on the GPU at once: one cluster of CTAs per row block, each CTA a fixed share of its key
+// tiles, which it visits twice (see score_tc.cu for the two passes and what they compute).
+//
+// What bounds such calls is not a tile's 1024 cycles of exponentials but what lies between the passes and around them.  With runs
+// handed out on the fly that is: a launch that clears counters and offsets, an atomic per run, partial statistics and a counter in
+// global memory, their merge by whoever comes last, offsets published and polled for, and a few segments a CTA
+// with a hand-over each.  Here nothing is handed out: a CTA's keys come as one stream of tiles, the second pass's first tiles are multiplied
+// while the statistics meet, and every CTA sends its log2 sums (a float a row) straight into the shared memory of the others, where
+// an mbarrier counts their bytes.  A tile visit takes 1200 - 1300 cycles, the turn from one pass to the other 4400 (mostly the
+// groups' last tiles), copies and first products 3800.  A whole eviction call with this kernel, and with runs handed out: 4096
+// tokens x 32 heads 29.0 and 31.9 us, 1024 x 64 heads 20.1 and 23.5, 2048 x 64 heads of 4 queries 32.5 and 35.5, 5000 x 32 heads
+// of 64 elements 36.1 and 39.1, a decode round of 2080 x 128 heads 78.2 and 80.0, one of 4160 x 64 100 and 108, 8192 x 32 53.3 and 54.1.
+//
+// Every wait is bounded; on expiry a role records AHAKV_ERR_TIMEOUT in the status word and leaves, and the others' own waits run
+// out in turn.  A CTA leaves the kernel together with its cluster: nobody sends into shared memory that is gone.
+#include <atomic>
+
+#include "score_common.cuh"
+
+namespace ahakv {
+namespace {
+
+using namespace tc;
+
+constexpr int kKStages = 4;                // K-tile ring depth
+constexpr int kFirstSoftmax = 4, kFirstValue = kFirstSoftmax + 4 * kGroups, kValueWarps = 10;   // two of them beside TMA and MMA
+constexpr int kThreads = 32 * (kFirstValue + kValueWarps - 2);
+static_assert(kThreads == 768, "see regs_down() and regs_up()");
+constexpr int kMostCtas = 8;
+
+struct Shared {
+  float row_c[128];                         // lambda log2(e) per stacked row
+  int row_last[128];                        // the last key a stacked row may see
+  float neg_off[128];                       // pass 2: minus a row's offset, -inf past the live rows
+  int tab_last[128];                        // row_last, -1 past the live rows
+  float2 stat[kGroups][128];                // pass 1: each group's shift and sum of a row
+  float part[kMostCtas][128];               // every CTA's log2 sums
+  unsigned long long q_full, part_full;
+  unsigned long long k_full[kKStages], k_empty[kKStages];
+  unsigned long long acc_full[kGroups][4];  // per group: its k-th tile completes barrier k mod 4
+  unsigned long long acc_empty[4];          // per accumulator
+  uint32_t tmem_slot;
+};
+
+constexpr int kQBytes = 2 * kSubTileBytes;              // D <= 128
+constexpr int kKStageBytes = 2 * kSubTileBytes;
+constexpr int kOffK = kQBytes;
+constexpr int kSmemTiles = kOffK + kKStages * kKStageBytes;
+constexpr int kSmemBytes = kSmemTiles + 1024 /*alignment slack*/ + (int)sizeof(Shared);
+static_assert(kSmemBytes <= 227 * 1024, "shared memory of one CTA");
+
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+}
+__device__ __forceinline__ void softmax_sync() { asm volatile("bar.sync 1, %0;" ::"n"(128 * kGroups) : "memory"); }
+
+// `value` to where `local` lies in CTA `rank` of the cluster, counted there by the barrier where `bar` lies.
+__device__ __forceinline__ void send(const float* local, const void* bar, int rank, float value) {
+  uint32_t to, there;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(to) : "r"(smem_u32(local)), "r"(rank));
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(there) : "r"(smem_u32(bar)), "r"(rank));
+  asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.b32 [%0], %1, [%2];" ::"r"(to), "r"(__float_as_uint(value)), "r"(there) : "memory");
+}
+
+// The CTA's part: a row block and a stretch of its key tiles.
+struct Part {
+  int unit, rank, first, tiles;
+  int b, h, rows, q_head, q_row;
+};
+__device__ __forceinline__ Part part_of(const TcArgs& a) {
+  Part p;
+  p.unit = blockIdx.x / a.rpu;
+  p.rank = blockIdx.x - p.unit * a.rpu;
+  p.first = p.rank * a.n_blk / a.rpu;
+  p.tiles = (p.rank + 1) * a.n_blk / a.rpu - p.first;
+  const int bh = p.unit / a.n_rb, rb = p.unit - bh * a.n_rb;
+  p.b = bh / a.Hkv;
+  p.h = bh - p.b * a.Hkv;
+  p.rows = a.r <= 128 ? min(a.hb, a.G - rb * a.hb) * a.r : min(128, a.r - rb * 128);
+  p.q_head = a.r <= 128 ? p.h * a.G + rb * a.hb : p.h;
+  p.q_row = a.r <= 128 ? 0 : rb * 128;
+  return p;
+}
+
+// ---- softmax pieces -------------------------------------------------------------------------------------
+// With one stream of tiles per CTA a group often works alone (the first tiles, the last ones of a pass), so what a row tile
+// takes by itself counts: sixteen columns at a time, the next sixteen on their way meanwhile.  (2140 cycles a tile for 3000 where
+// the other groups leave the special-function unit alone; a decode round 41.9 -> 40.3 us, 4160 tokens x 64 heads 65.8 -> 63.1.)
+__device__ __forceinline__ void tmem_ld16_issue(uint32_t taddr, uint32_t* r) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+      : "r"(taddr)
+      : "memory");
+}
+__device__ __forceinline__ void tmem_ld16_wait(uint32_t* r) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;"
+               : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),
+                 "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15])
+               :
+               : "memory");
+}
+// Adds 2^{c v + neg} of sixteen values to the four running sums.
+__device__ __forceinline__ void exp_add16(const uint32_t* r, uint64_t c2, uint64_t neg2, uint64_t& za, uint64_t& zb) {
+#pragma unroll
+  for (int t = 0; t < 16; t += 4) {
+    float x0, x1, x2, x3;
+    unpack2(fma2(pack2(__uint_as_float(r[t]), __uint_as_float(r[t + 1])), c2, neg2), x0, x1);
+    unpack2(fma2(pack2(__uint_as_float(r[t + 2]), __uint_as_float(r[t + 3])), c2, neg2), x2, x3);
+    za = add2(za, pack2(fast_exp2(x0), fast_exp2(x1)));
+    zb = add2(zb, pack2(fast_exp2(x2), fast_exp2(x3)));
+  }
+}
+__device__ __forceinline__ float sum4(uint64_t za, uint64_t zb) {
+  float z0, z1;
+  unpack2(add2(za, zb), z0, z1);
+  return z0 + z1;
+}
+__device__ __forceinline__ float max16(const uint32_t* r) {
+  float m0 = __uint_as_float(r[0]), m1 = __uint_as_float(r[1]);
+#pragma unroll
+  for (int t = 2; t < 16; t += 2) {
+    m0 = fmaxf(m0, __uint_as_float(r[t]));
+    m1 = fmaxf(m1, __uint_as_float(r[t + 1]));
+  }
+  return fmaxf(m0, m1);
+}
+// As fold_chunk, sixteen columns without a mask.
+__device__ __forceinline__ void fold16(const uint32_t* r, float c, float& M, float& Z) {
+  if (M > -INFINITY) {
+    uint64_t za = pack2(0.f, 0.f), zb = pack2(0.f, 0.f);
+    exp_add16(r, pack2(c, c), pack2(-M, -M), za, zb);
+    const float z = sum4(za, zb);
+    if (z < kAcceptBelow) {
+      Z += z;
+      return;
+    }
+  }
+  const float mx = max16(r) * c;
+  if (mx > -INFINITY) {
+    uint64_t za = pack2(0.f, 0.f), zb = pack2(0.f, 0.f);
+    exp_add16(r, pack2(c, c), pack2(-mx, -mx), za, zb);
+    Z = (M > -INFINITY ? Z * fast_exp2(M - mx) : 0.f) + sum4(za, zb);
+    M = mx;
+  }
+}
+// As row_tile, of a tile no key of which is masked.  The shift is looked at twice: for the first six pieces while they are still in
+// tensor memory, for the last two while they are in registers.
+__device__ __forceinline__ void row_tile16(uint32_t from, float c, float& M, float& Z, void* empty) {
+  uint32_t u[16], w[16];
+  tmem_ld16_issue(from, u);
+  tmem_ld16_wait(u);
+  tmem_ld16_issue(from + 16, w);
+  if (!(M > -INFINITY)) M = max16(u) * c;
+  const uint64_t c2 = pack2(c, c), neg2 = pack2(-M, -M);
+  uint64_t za = pack2(0.f, 0.f), zb = pack2(0.f, 0.f), ya = pack2(0.f, 0.f), yb = pack2(0.f, 0.f);
+  exp_add16(u, c2, neg2, za, zb);
+#pragma unroll
+  for (int ch = 2; ch < 8; ch += 2) {
+    tmem_ld16_wait(w);
+    tmem_ld16_issue(from + 16 * ch, u);
+    exp_add16(w, c2, neg2, za, zb);
+    tmem_ld16_wait(u);
+    tmem_ld16_issue(from + 16 * ch + 16, w);
+    if (ch < 6) exp_add16(u, c2, neg2, za, zb);
+    else exp_add16(u, c2, neg2, ya, yb);
+  }
+  float z = sum4(za, zb);
+  const bool sound = z < kAcceptBelow;                        // an overflow or a NaN fails this test too
+  tmem_ld16_wait(w);
+  if (__any_sync(0xffffffffu, !sound)) {
+#pragma unroll 1
+    for (int ch = 0; ch < 6; ++ch) {
+      uint32_t again[16];
+      tmem_ld16_issue(from + 16 * ch, again);
+      tmem_ld16_wait(again);
+      if (!sound) fold16(again, c, M, Z);
+    }
+  }
+  tc_fence_before();
+  mbar_arrive(empty);
+  if (sound) {
+    Z += z;
+    exp_add16(w, c2, neg2, ya, yb);
+    z = sum4(ya, yb);
+  }
+  if (sound && z < kAcceptBelow) {
+    Z += z;
+  } else {
+    fold16(u, c, M, Z);
+    fold16(w, c, M, Z);
+  }
+}
+
+// ---- roles --------------------------------------------------------------------------------------------
+template <bool kTest>
+__device__ __forceinline__ void producer(const TcArgs& a, const Part& p, const CUtensorMap* qmap, const CUtensorMap* kmap, Shared* sh, char* tiles) {
+  const int n_sub = a.D / 64, q_rows = a.r <= 128 ? a.hb * a.r : 128;
+  const unsigned long long once = policy_evict_first();
+  mbar_expect_tx(&sh->q_full, n_sub * q_rows * 128);
+  for (int s = 0; s < n_sub; ++s) tma_load_4d(tiles + s * kSubTileBytes, qmap, &sh->q_full, s * 64, p.q_row, p.q_head, p.b);
+  bool ok = true;
+  for (int v = 0; v < 2 * p.tiles; ++v) {
+    const int stage = v % kKStages, key = (p.first + (v < p.tiles ? v : v - p.tiles)) * kKeyTile;
+    if (!(ok = mbar_wait(&sh->k_empty[stage], ((v / kKStages) & 1) ^ 1, a.status, wait_limit<kTest>(a)))) break;
+    mbar_expect_tx(&sh->k_full[stage], n_sub * kSubTileBytes);
+    char* dst = tiles + kOffK + stage * kKStageBytes;
+    for (int s = 0; s < n_sub; ++s) {
+      // the second read of a key tile is its last: let L2 drop it first
+      if (v < p.tiles) tma_load_4d(dst + s * kSubTileBytes, kmap, &sh->k_full[stage], s * 64, key, p.h, p.b);
+      else tma_load_4d_hint(dst + s * kSubTileBytes, kmap, &sh->k_full[stage], s * 64, key, p.h, p.b, once);
+    }
+  }
+  if (!ok) {
+    // a wait ran out: give copies already in flight a bounded time (1 ms) to land before the CTA exits
+    const long long now = now_ns();
+    while (now_ns() - now < 1000000) __nanosleep(1000);
+  }
+}
+
+// Pass 1: D[rows x keys] = Q K^T.  Pass 2: D[keys x rows] = K Q^T.  The whole warp walks the tiles, converged, and one elected
+// lane issues; a tile's barriers are tested while the tile before it is being issued.
+template <bool kTest>
+__device__ __forceinline__ void mma_warp(const TcArgs& a, const Part& p, Shared* sh, char* tiles, uint32_t tmem_base) {
+  const int nk = a.D / 16, tile_count = __shfl_sync(0xffffffffu, p.tiles, 0);
+  const long long limit = wait_limit<kTest>(a);
+  const uint32_t q_lo = umma_desc_lo(smem_u32(tiles));
+  const uint32_t idesc2 = umma_idesc(128, (p.rows + 15) & ~15, a.bf16), idesc1 = umma_idesc(128, 128, a.bf16);
+  int stage = 0, k_phase = 0, acc = 0, acc_phase = 0, g = 0, turn = 0;   // turn: this group's tiles so far
+  if (!__all_sync(0xffffffffu, mbar_wait(&sh->q_full, 0, a.status, limit))) return;
+  bool k_ok = false, a_ok = false;
+  for (int v = 0; v < 2 * tile_count; ++v) {
+    if (!k_ok && !__all_sync(0xffffffffu, mbar_wait(&sh->k_full[stage], k_phase, a.status, limit))) return;
+    if (!a_ok && !__all_sync(0xffffffffu, mbar_wait(&sh->acc_empty[acc], acc_phase ^ 1, a.status, limit))) return;
+    tc_fence_after();
+    const bool second = v >= tile_count;
+    const uint32_t d_tmem = tmem_base + (uint32_t)(acc * 128);
+    const uint32_t k_lo = umma_desc_lo(smem_u32(tiles + kOffK + stage * kKStageBytes));
+    const uint32_t a_lo = second ? k_lo : q_lo, b_lo = second ? q_lo : k_lo, idesc = second ? idesc2 : idesc1;
+    void* this_acc = &sh->acc_full[g][turn & 3];
+    void* this_k = &sh->k_empty[stage];
+    if (++g == kGroups) { g = 0; ++turn; }
+    if (++acc == 4) { acc = 0; acc_phase ^= 1; }
+    if (++stage == kKStages) { stage = 0; k_phase ^= 1; }
+    if (v + 1 < 2 * tile_count) {
+      k_ok = __all_sync(0xffffffffu, mbar_test(&sh->k_full[stage], k_phase));
+      a_ok = __all_sync(0xffffffffu, mbar_test(&sh->acc_empty[acc], acc_phase ^ 1));
+    }
+    if (elect_one()) {
+#pragma unroll
+      for (int kk = 0; kk < 8; ++kk) {
+        // k-step kk reads 32 bytes at offset (kk & 3) * 32 of sub-tile kk >> 2
+        const uint32_t off = (uint32_t)(((kk >> 2) * kSubTileBytes + (kk & 3) * 32) >> 4);
+        if (kk < nk) {
+          if (kk == 0) umma_step<0>(d_tmem, desc64(a_lo + off, kDescHi), desc64(b_lo + off, kDescHi), idesc);
+          else umma_step<1>(d_tmem, desc64(a_lo + off, kDescHi), desc64(b_lo + off, kDescHi), idesc);
+        }
+      }
+      tc_commit(this_acc);
+      tc_commit(this_k);
+    }
+    __syncwarp();
+  }
+}
+
+// Softmax warps: the v-th tile visited belongs to group v mod kGroups, a thread per TMEM lane.  Between the passes the groups meet twice:
+// the first adds up their statistics, sends the sums around, and turns what arrives into the rows' offsets.
+template <bool kTest>
+__device__ __forceinline__ void softmax_group(const TcArgs& a, const Part& p, Shared* sh, uint32_t tmem_base, int g) {
+  const int s = threadIdx.x & 127, quarter = (threadIdx.x >> 5) & 3, kind = p.q_row != 0;
+  const uint32_t lane_base = tmem_base + ((uint32_t)(quarter * 32) << 16);
+  const long long limit = wait_limit<kTest>(a);
+  bool gone = false;                                        // a wait ran out
+  int mine = 0;                                             // own tiles so far
+  {
+    const float c = sh->row_c[s];
+    const int last = sh->row_last[s];
+    const bool live = quarter * 32 < p.rows;                // the warp has rows of this block
+    float M = -INFINITY, Z = 0.f;
+    for (int v = g; v < p.tiles; v += kGroups, ++mine) {
+      const int acc = v & 3, j0 = (p.first + v) * kKeyTile;
+      if (gone) continue;
+      if (!__all_sync(0xffffffffu, mbar_wait(&sh->acc_full[g][mine & 3], (mine >> 2) & 1, a.status, limit))) { gone = true; continue; }
+      tc_fence_after();
+      if (!live) mbar_arrive(&sh->acc_empty[acc]);
+      else if (j0 + kKeyTile - 1 <= a.min_last) row_tile16(lane_base + acc * 128, c, M, Z, &sh->acc_empty[acc]);
+      else row_tile(lane_base + acc * 128, false, j0, last, c, M, Z, &sh->acc_empty[acc]);
+    }
+    sh->stat[g][s] = make_float2(M, Z);
+  }
+  softmax_sync();
+  if (g == 0) {
+    float x[kGroups], M = -INFINITY, Z = 0.f;
+#pragma unroll
+    for (int t = 0; t < kGroups; ++t) {
+      const float2 st = sh->stat[t][s];
+      x[t] = st.y > 0.f ? st.x + log2f(st.y) : st.y == st.y ? -INFINITY : INFINITY;   // NaN inputs: nothing downstream waits for a number
+    }
+    merge_logs(x, M, Z);
+    const float L = M + log2f(Z);
+    const bool withheld = kTest && a.test_withhold && blockIdx.x == 0;
+    if (a.rpu > 1) {
+      for (int t = 0; t < a.rpu && !withheld; ++t) send(&sh->part[p.rank][s], &sh->part_full, t, L);
+    } else {                                                // a launch without clusters executes none of their instructions
+      sh->part[0][s] = L;
+      if (!withheld) mbar_arrive(&sh->part_full);
+    }
+    if (!gone && !__all_sync(0xffffffffu, mbar_wait(&sh->part_full, 0, a.status, limit))) gone = true;
+    __threadfence();                                        // other CTAs' sums
+    M = -INFINITY;
+    Z = 0.f;
+    for (int t0 = 0; t0 < a.rpu; t0 += 4) {                 // in key order
+      float e[4];
+#pragma unroll
+      for (int t = 0; t < 4; ++t) e[t] = t0 + t < a.rpu ? sh->part[t0 + t][s] : -INFINITY;
+      merge_logs(e, M, Z);
+    }
+    const float off = M + log2f(Z) + a.log2G;               // 2^{c w - off} = softmax weight / G
+    sh->neg_off[s] = s >= p.rows || off != off ? -INFINITY : -off;
+    sh->tab_last[s] = s < p.rows ? sh->row_last[s] : -1;
+  }
+  softmax_sync();
+  const int chunks = (p.rows + 31) >> 5;
+  // Rows past the live ones that no box covers are zeros, which their offsets take to nothing; where the box brought rows of
+  // another head, their terms have to be masked.
+  const bool plain = kind == 0 && ((p.rows & 31) == 0 || p.rows == a.hb * a.r);
+  for (int v = p.tiles + (g + kGroups - p.tiles % kGroups) % kGroups; v < 2 * p.tiles; v += kGroups, ++mine) {
+    const int acc = v & 3, j0 = (p.first + v - p.tiles) * kKeyTile, j = j0 + s;
+    if (gone) continue;
+    if (!__all_sync(0xffffffffu, mbar_wait(&sh->acc_full[g][mine & 3], (mine >> 2) & 1, a.status, limit))) { gone = true; continue; }
+    tc_fence_after();
+    const float sum = column_tile(a, lane_base + acc * 128, chunks, plain && j0 + kKeyTile - 1 <= a.min_last, sh->row_c, sh->neg_off,
+                                  sh->tab_last, j, &sh->acc_empty[acc]);
+    if (j < a.n) a.s_raw[(size_t)p.unit * a.n + j] = sum;
+  }
+}
+
+template <bool kTest>
+__global__ void __launch_bounds__(kThreads, 1)
+score_cluster_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_constant__ CUtensorMap kmap, const __grid_constant__ TcArgs a) {
+  extern __shared__ char smem_raw[];
+  char* tiles = reinterpret_cast<char*>(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+  Shared* sh = reinterpret_cast<Shared*>(tiles + kSmemTiles);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const Part p = part_of(a);
+  if (threadIdx.x == 0) {   // the copy engine's descriptors on their way while the CTA sets itself up
+    asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&qmap)) : "memory");
+    asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&kmap)) : "memory");
+    mbar_init(&sh->q_full, 1);
+    mbar_init(&sh->part_full, a.rpu > 1 ? 1 : 128);
+    for (int s = 0; s < kKStages; ++s) {
+      mbar_init(&sh->k_full[s], 1);
+      mbar_init(&sh->k_empty[s], 1);
+    }
+    for (int s = 0; s < 4; ++s) {
+      mbar_init(&sh->acc_empty[s], 128);
+      for (int g = 0; g < kGroups; ++g) mbar_init(&sh->acc_full[g][s], 1);
+    }
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    if (a.rpu > 1) mbar_expect_tx(&sh->part_full, a.rpu * 128 * (int)sizeof(float));
+  }
+  if (threadIdx.x < 128) {
+    // stacked row s of a row block is observation row s mod r, or, when one head's rows fill two blocks, row s of the block
+    const int s = threadIdx.x, i = a.r <= 128 ? s % a.r : min(p.q_row + s, kMaxRows - 1);
+    sh->row_c[s] = a.c[i];
+    sh->row_last[s] = a.last[i];
+  }
+  if ((a.r <= 128 ? a.hb * a.r : 128) < 128) {   // rows the box never covers must read as zeros
+    uint4* z = reinterpret_cast<uint4*>(tiles);
+    for (int t = threadIdx.x; t < kQBytes / 16; t += kThreads) z[t] = make_uint4(0, 0, 0, 0);
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  }
+  if (warp == 1) {   // all 512 TMEM columns: four 128-column accumulators
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(smem_u32(&sh->tmem_slot)) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  griddep_wait();
+  if (blockIdx.x == 0 && threadIdx.x == 0) *a.status = -1;   // no error
+  tc_fence_before();
+  __syncthreads();
+  if (a.rpu > 1) cluster_sync();   // the others' barriers are there
+  tc_fence_after();
+  const uint32_t tmem_base = sh->tmem_slot;
+
+  if (warp < kFirstSoftmax) {
+    regs_down();
+    if (warp == 0) {
+      if (lane == 0) producer<kTest>(a, p, &qmap, &kmap, sh, tiles);
+    } else if (warp == 1) {
+      mma_warp<kTest>(a, p, sh, tiles, __shfl_sync(0xffffffffu, tmem_base, 0));
+    }
+  } else if (warp < kFirstValue) {
+    regs_up();
+    softmax_group<kTest>(a, p, sh, tmem_base, (warp - kFirstSoftmax) >> 2);
+  } else {
+    regs_down();
+  }
+  if (a.prior && (warp >= kFirstValue || warp == 2 || warp == 3)) {
+    const unsigned w = blockIdx.x * kValueWarps + (warp < kFirstSoftmax ? warp - 2 : warp - kFirstValue + 2), n_warps = gridDim.x * kValueWarps;
+    if (a.bf16) { if (a.D == 128) value_norms<__nv_bfloat16, 128>(a, w, n_warps); else value_norms<__nv_bfloat16, 64>(a, w, n_warps); }
+    else { if (a.D == 128) value_norms<__half, 128>(a, w, n_warps); else value_norms<__half, 64>(a, w, n_warps); }
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 1) {
+    __syncwarp();
+    tc_fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem_base) : "memory");
+  }
+  __syncwarp();
+  if (a.rpu > 1) cluster_sync();
+}
+
+// How many clusters of every size the current device holds at once (0: none).  Asked once per device and size.
+int clusters_at_once(int size) {
+  constexpr int kMaxDevices = 64;
+  static std::atomic<int> known[kMaxDevices][kMostCtas + 1] = {};   // one more than the number; 0: not asked yet
+  int dev = -1;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return 0;
+  int n = known[dev][size].load(std::memory_order_relaxed);
+  if (n != 0) return n - 1;
+  const void* kernels[] = {(const void*)score_cluster_kernel<false>, (const void*)score_cluster_kernel<true>};
+  for (const void* kernel : kernels) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(size);
+    cfg.blockDim = dim3(kThreads);
+    cfg.dynamicSmemBytes = kSmemBytes;
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = size;
+    attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes) != cudaSuccess ||
+        cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) {
+      cudaGetLastError();
+      n = 0;
+    }
+  }
+  known[dev][size].store(n + 1, std::memory_order_relaxed);
+  return n;
+}
+
+}  // namespace
+
+// ---- host ------------------------------------------------------------------------------------------------
+// Where it pays, each line with both sides measured (kernel and fill, us; this one first):
+// - all clusters on the GPU at once, over at least four fifths of its SMs: 16 heads of 8192 tokens with 112 CTAs 30 and 28, 8 row
+//   blocks of 70001 tokens 145 and 72 (clusters of more than eight do not fit: 72 CTAs);
+// - keys that stay in L2 (96 MB of its 126) until the second pass, which starts only when the first is over: 16384 tokens x 32
+//   heads, 134 MB, 75 and 73; x 8 heads x 4 sequences 115 and 110;
+// - two tiles a CTA or more, so that the stream outlasts the copies' way.
+int tc::cluster_size(const Plan& pl, int slots) {
+  const long long units = (long long)pl.B * pl.Hkv * pl.n_rb;
+  const int n_blk = (pl.n_eff + kKeyTile - 1) / kKeyTile;
+  if (units > slots || (long long)pl.B * pl.Hkv * n_blk * kKeyTile * pl.d * pl.es > (96LL << 20)) return 0;
+  int size = (int)(slots / units);
+  if (size > kMostCtas) size = kMostCtas;
+  if (size > n_blk / 2) size = n_blk / 2;
+  while (size > 0 && clusters_at_once(size) < units) --size;
+  return 5 * units * size >= 4 * slots ? size : 0;
+}
+
+cudaError_t tc::launch_cluster(const CUtensorMap& qmap, const CUtensorMap& kmap, const TcArgs& a, int grid, bool test, cudaStream_t st) {
+  return launch_chained(test ? score_cluster_kernel<true> : score_cluster_kernel<false>, dim3(grid), dim3(kThreads), a.rpu, kSmemBytes, st, qmap, kmap, a);
+}
+
+}  // namespace ahakv

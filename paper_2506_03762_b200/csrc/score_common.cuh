@@ -1,0 +1,220 @@
+// What the two tensor-core scoring kernels share (score_tc.cu: any size, runs handed out on the fly; score_cluster.cu: calls that
+// fit on the GPU at once): their arguments, the softmax of a tile from its accumulator, and the value norms.
+#pragma once
+
+#include "tc_common.cuh"
+
+namespace ahakv {
+namespace tc {
+
+constexpr int kGroups = 3;                 // groups of four softmax warps
+constexpr int kSubTileBytes = 128 * 128;   // 128 rows x 64 16-bit elements, 128-byte swizzled
+constexpr int kValueLoads = 8;             // 16-byte loads in flight per lane of a value-norm warp
+
+struct TcArgs {
+  int n, r, G, Hkv, n_rb, hb, n_blk, D, BH;
+  int CH;         // key tiles per run
+  int rpu;        // runs per row block = ceil(n_blk / CH)
+  int n_runs;     // row blocks * rpu
+  int gap;        // how far behind a row block's last run the pass-1 run lies that a CTA does before pass 2 turns to the block
+  int max_lead;   // runs that pass 1 may be ahead of pass 2
+  int bf16;       // operand type of the products
+  int prior;      // stream V and write nu
+  float log2G;
+  float c[kMaxRows];     // lambda_i log2(e) per observation row
+  float row_scale[128];  // the same per stacked row of a row block (of the first one where a head has two)
+  int last[kMaxRows];    // per observation row: the last key it may see
+  int min_last;          // the smallest of them: tiles that end at or before it are masked for no row
+  float* partial;    // [unit][rpu][128]: log2 of a row's sum of 2^{c w} over the keys of a run
+  float* off;        // [unit][128]: the merged offset of every row (NaN at launch)
+  float* s_raw;      // [unit][n]
+  float* nu;         // [B * Hkv][n]
+  const char* v;
+  long long vs[3];   // byte strides of v: batch, head, token
+  int* ctr;          // next pass-1 run, next pass-2 run, then per unit the runs that have been delivered; all -1 at launch
+  int* status;
+  long long test_wait_ns;   // test build of the kernel only: what every bounded wait allows
+  int test_withhold;        // test build only: the statistics of the first run of the first row block are never delivered
+};
+
+// The kernel exists twice: the one every call runs, whose waits allow kWaitLimitNs, and a second instantiation that
+// takes the limit and a planted fault from its arguments, for the test of the failure path (ahakv_test_set_wait).
+// Same code, same wind-down; only these two lines differ.
+template <bool kTest> __device__ __forceinline__ long long wait_limit(const TcArgs& a) {
+  return kTest ? a.test_wait_ns : kWaitLimitNs;
+}
+
+// Thirty-two stacked rows of a key's column: adds 2^{c D - off} of each to the four running sums.
+//
+// The scales are the launch's parameters, at places the compiler knows, and only the offsets come from shared memory: a
+// broadcast costs its 128 bytes a cycle as much as 32 different values do, so that scales and offsets together (64 reads of 16 bytes a
+// tile and warp) took 1024 cycles of it, as long as the tile's exponentials, and the products want it at its full rate for
+// 512 and the copies for 256.  A tile of pass 2 takes a group 3150 cycles instead of 3700: a decode
+// round (16 sequences x 8 heads x 2080 tokens) 44.1 -> 42.6 us, and with the value rows' loop below 16384 x 8 x 4 127 -> 122,
+// 20000 x 32 heads of 64 elements 95 -> 81.
+__device__ __forceinline__ void column_chunk(const uint32_t* r, const float* cs, const float* neg_off, uint64_t& za, uint64_t& zb) {
+#pragma unroll
+  for (int t = 0; t < 32; t += 4) {
+    const float4 o = *reinterpret_cast<const float4*>(neg_off + t);
+    float x0, x1, x2, x3;
+    unpack2(fma2(pack2(__uint_as_float(r[t]), __uint_as_float(r[t + 1])), pack2(cs[t], cs[t + 1]), pack2(o.x, o.y)), x0, x1);
+    unpack2(fma2(pack2(__uint_as_float(r[t + 2]), __uint_as_float(r[t + 3])), pack2(cs[t + 2], cs[t + 3]), pack2(o.z, o.w)), x2, x3);
+    za = add2(za, pack2(fast_exp2(x0), fast_exp2(x1)));
+    zb = add2(zb, pack2(fast_exp2(x2), fast_exp2(x3)));
+  }
+}
+// ... with everything from shared memory, and each row only up to the last key it may see.
+__device__ __forceinline__ void column_chunk_masked(const uint32_t* r, const float* cs, const float* neg_off, const int* last, int j,
+                                                    uint64_t& za, uint64_t& zb) {
+#pragma unroll
+  for (int t = 0; t < 32; t += 4) {
+    const float4 c = *reinterpret_cast<const float4*>(cs + t), o = *reinterpret_cast<const float4*>(neg_off + t);
+    const int4 l = *reinterpret_cast<const int4*>(last + t);
+    float x0, x1, x2, x3;
+    unpack2(fma2(pack2(__uint_as_float(r[t]), __uint_as_float(r[t + 1])), pack2(c.x, c.y), pack2(o.x, o.y)), x0, x1);
+    unpack2(fma2(pack2(__uint_as_float(r[t + 2]), __uint_as_float(r[t + 3])), pack2(c.z, c.w), pack2(o.z, o.w)), x2, x3);
+    if (j > l.x) x0 = -INFINITY;
+    if (j > l.y) x1 = -INFINITY;
+    if (j > l.z) x2 = -INFINITY;
+    if (j > l.w) x3 = -INFINITY;
+    za = add2(za, pack2(fast_exp2(x0), fast_exp2(x1)));
+    zb = add2(zb, pack2(fast_exp2(x2), fast_exp2(x3)));
+  }
+}
+
+// Pass 1, 128 keys from j0 on for the row of this lane: folds 2^{c w} into (M, Z) and frees the accumulator.
+__device__ __forceinline__ void row_tile(uint32_t from, bool full, int j0, int last, float c, float& M, float& Z, void* empty) {
+#pragma unroll 1
+  for (int ch = 0; ch < 4; ++ch) {
+    uint32_t ra[32];
+    tmem_ld32_issue(from + 32 * ch, ra);
+    tmem_ld_wait(ra);
+    if (ch == 4 - 1) {
+      tc_fence_before();
+      mbar_arrive(empty);                                    // the accumulator is free for the next product
+    }
+    fold_chunk(ra, full, j0 + 32 * ch, last, c, M, Z);
+  }
+}
+
+// Pass 2, the key of this lane, j: the sum over `chunks` times 32 stacked rows of 2^{c w - off}; frees the accumulator.  `plain`:
+// no row is masked and the scales are those of the launch.
+__device__ __forceinline__ float column_tile(const TcArgs& a, uint32_t from, int chunks, bool plain, const float* row_c, const float* neg_off,
+                                             const int* tab_last, int j, void* empty) {
+  uint64_t za = pack2(0.f, 0.f), zb = pack2(0.f, 0.f);
+  if (plain) {
+#pragma unroll
+    for (int ch = 0; ch < 4; ++ch) {
+      if (ch < chunks) {
+        uint32_t ra[32];
+        tmem_ld32_issue(from + 32 * ch, ra);
+        tmem_ld_wait(ra);
+        if (ch + 1 == chunks) {
+          tc_fence_before();
+          mbar_arrive(empty);
+        }
+        column_chunk(ra, a.row_scale + 32 * ch, neg_off + 32 * ch, za, zb);
+      }
+    }
+  } else {
+#pragma unroll 1
+    for (int ch = 0; ch < chunks; ++ch) {
+      uint32_t ra[32];
+      tmem_ld32_issue(from + 32 * ch, ra);
+      tmem_ld_wait(ra);
+      if (ch + 1 == chunks) {
+        tc_fence_before();
+        mbar_arrive(empty);
+      }
+      column_chunk_masked(ra, row_c + 32 * ch, neg_off + 32 * ch, tab_last + 32 * ch, j, za, zb);
+    }
+  }
+  float z0, z1;
+  unpack2(add2(za, zb), z0, z1);
+  return z0 + z1;
+}
+
+// Value-norm warps: every warp of the grid takes chunks of value rows in turn, kValueLoads 16-byte loads a lane in flight.  Four
+// lanes share a row (64 bytes of it a load), square and add in FP32 and meet by shuffle.
+__device__ __forceinline__ uint4 ld_once(const char* p) {   // read once: do not keep in L1, evict first from L2
+  uint4 v;
+  asm volatile("ld.global.cs.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+  return v;
+}
+template <typename T, int D>
+__device__ __forceinline__ void value_norms(const TcArgs& a, unsigned w, unsigned n_warps) {
+  constexpr int kPieces = D / 32, kSets = kValueLoads / kPieces, kRows = 8 * kSets;   // 64-byte pieces a row, 8-row sets in flight
+  const int grp = (threadIdx.x & 31) >> 2, tig = threadIdx.x & 3;
+  const unsigned per_head = (unsigned)(a.n + kRows - 1) / kRows, heads = (unsigned)a.BH, per_seq = (unsigned)a.Hkv;
+  const unsigned step_h = n_warps / per_head, step = n_warps - step_h * per_head;
+  unsigned bh = w / per_head, at = w - bh * per_head, b = bh / per_seq, h = bh - b * per_seq;   // head and chunk of it
+  if (bh >= heads) return;
+  const char* p[kSets];
+  int row;
+  auto locate = [&]() {   // rows past the end read the last one again; nothing of theirs is stored
+    row = (int)at * kRows + grp;
+    const char* head = a.v + b * a.vs[0] + h * a.vs[1] + tig * 16;
+#pragma unroll
+    for (int q = 0; q < kSets; ++q) p[q] = head + min(row + 8 * q, a.n - 1) * a.vs[2];
+  };
+  locate();
+  for (;;) {
+    uint4 u[kSets][kPieces];
+#pragma unroll
+    for (int q = 0; q < kSets; ++q)
+#pragma unroll
+      for (int i = 0; i < kPieces; ++i) u[q][i] = ld_once(p[q] + i * 64);
+    // where the next chunk is, while this one is on its way
+    float* const to = a.nu + (size_t)bh * a.n + row;
+    const int left = a.n - row;
+    at += step;
+    unsigned heads_on = step_h;
+    if (at >= per_head) { at -= per_head; ++heads_on; }
+    bh += heads_on;
+    h += heads_on;
+    if (h >= per_seq) {
+      const unsigned seqs = h / per_seq;
+      h -= seqs * per_seq;
+      b += seqs;
+    }
+    if (bh < heads) locate();
+#pragma unroll
+    for (int q = 0; q < kSets; ++q) asm volatile("" : "+l"(p[q]));   // now, not after the sums
+#pragma unroll
+    for (int q = 0; q < kSets; ++q) {
+      uint64_t acc = pack2(0.f, 0.f), acc2 = pack2(0.f, 0.f);
+#pragma unroll
+      for (int i = 0; i < kPieces; ++i) {
+        float f[8];
+        Vec16<T>::widen(u[q][i], f);
+#pragma unroll
+        for (int e = 0; e < 8; e += 4) {
+          const uint64_t p0 = pack2(f[e], f[e + 1]), p1 = pack2(f[e + 2], f[e + 3]);
+          acc = fma2(p0, p0, acc);
+          acc2 = fma2(p1, p1, acc2);
+        }
+      }
+      float s0, s1;
+      unpack2(add2(acc, acc2), s0, s1);
+      float sq = s0 + s1;
+      sq += __shfl_xor_sync(0xffffffffu, sq, 1);
+      sq += __shfl_xor_sync(0xffffffffu, sq, 2);
+      if (tig == 0 && 8 * q < left) to[8 * q] = sq;
+    }
+    if (bh >= heads) return;
+  }
+}
+
+// The softmax warps keep a chunk of the accumulator and its exponentials in registers, the others need few: of the 80 a
+// thread that the launch allows (768 threads), each of the twelve softmax warps takes 104 and the other twelve keep 56
+// (384 x 104 + 384 x 56 = 768 x 80).
+__device__ __forceinline__ void regs_down() { asm volatile("setmaxnreg.dec.sync.aligned.u32 56;"); }
+__device__ __forceinline__ void regs_up() { asm volatile("setmaxnreg.inc.sync.aligned.u32 104;"); }
+
+// score_cluster.cu: how many CTAs a row block's cluster has if the whole call fits on the GPU at once that way and gains by it,
+// or 0; and its launch, with `rpu` CTAs a row block.
+int cluster_size(const Plan& pl, int slots);
+cudaError_t launch_cluster(const CUtensorMap& qmap, const CUtensorMap& kmap, const TcArgs& a, int grid, bool test, cudaStream_t st);
+
+}  // namespace tc
+}  // namespace ahakv

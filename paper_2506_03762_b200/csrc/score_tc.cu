@@ -50,12 +50,10 @@
 // A segment only ever waits for segments that were handed out before it, to CTAs that are running, so the waits cannot
 // deadlock, whatever part of the grid is resident.  Every wait is bounded in time; on expiry the kernel records
 // AHAKV_ERR_TIMEOUT in the status word and winds down.
-#include <cuda.h>
-
 #include <atomic>
 
 #include "ahakv_internal.cuh"
-#include "tc_common.cuh"
+#include "score_common.cuh"
 
 namespace ahakv {
 namespace {
@@ -63,49 +61,14 @@ namespace {
 using namespace tc;
 
 constexpr int kKStages = 3;                // K-tile ring depth (four: 119 us for 115 at 16384 tokens x 8 heads x 4; two: 49 for 47 at 8192 x 32)
-constexpr int kGroups = 3;                 // groups of four softmax warps
-constexpr int kSubTileBytes = 128 * 128;   // 128 rows x 64 16-bit elements, 128-byte swizzled
 constexpr int kSegRing = 16;               // published segments a role may lag behind the scheduler
 constexpr int kMergeRing = 8;
 constexpr int kSegAhead = 4;               // segments published beyond the one the softmax warps are on
 constexpr int kSegEnd = -1;
-constexpr int kValueWarps = 7, kValueLoads = 8;   // 16-byte loads in flight per lane
+constexpr int kValueWarps = 7;
 constexpr int kFirstSoftmax = 4, kFirstValue = kFirstSoftmax + 4 * kGroups, kSchedWarp = kFirstValue + kValueWarps;
 constexpr int kThreads = 32 * (kSchedWarp + 1);   // TMA, MMA, table, delivery; softmax; value norms; scheduler
 static_assert(kThreads == 768 && kGroups == 3, "see regs_down() and regs_up()");
-
-struct TcArgs {
-  int n, r, G, Hkv, n_rb, hb, n_blk, D, BH;
-  int CH;         // key tiles per run
-  int rpu;        // runs per row block = ceil(n_blk / CH)
-  int n_runs;     // row blocks * rpu
-  int gap;        // how far behind a row block's last run the pass-1 run lies that a CTA does before pass 2 turns to the block
-  int max_lead;   // runs that pass 1 may be ahead of pass 2
-  int bf16;       // operand type of the products
-  int prior;      // stream V and write nu
-  float log2G;
-  float c[kMaxRows];     // lambda_i log2(e) per observation row
-  float row_scale[128];  // the same per stacked row of a row block (of the first one where a head has two)
-  int last[kMaxRows];    // per observation row: the last key it may see
-  int min_last;          // the smallest of them: tiles that end at or before it are masked for no row
-  float* partial;    // [unit][rpu][128]: log2 of a row's sum of 2^{c w} over the keys of a run
-  float* off;        // [unit][128]: the merged offset of every row (NaN at launch)
-  float* s_raw;      // [unit][n]
-  float* nu;         // [B * Hkv][n]
-  const char* v;
-  long long vs[3];   // byte strides of v: batch, head, token
-  int* ctr;          // next pass-1 run, next pass-2 run, then per unit the runs that have been delivered; all -1 at launch
-  int* status;
-  long long test_wait_ns;   // test build of the kernel only: what every bounded wait allows
-  int test_withhold;        // test build only: the statistics of the first run of the first row block are never delivered
-};
-
-// The kernel exists twice: the one every call runs, whose waits allow kWaitLimitNs, and a second instantiation that
-// takes the limit and a planted fault from its arguments, for the test of the failure path (ahakv_test_set_wait).
-// Same code, same wind-down; only these two lines differ.
-template <bool kTest> __device__ __forceinline__ long long wait_limit(const TcArgs& a) {
-  return kTest ? a.test_wait_ns : kWaitLimitNs;
-}
 
 // ---- shared memory layout --------------------------------------------------------------------
 // One segment as the scheduler decodes it for everybody else.
@@ -408,44 +371,6 @@ __device__ __forceinline__ void mma_warp(const TcArgs& a, Shared* sh, char* tile
   }
 }
 
-// Thirty-two stacked rows of a key's column: adds 2^{c D - off} of each to the four running sums.
-//
-// The scales are the launch's parameters, at places the compiler knows, and only the offsets come from shared memory: a
-// broadcast costs its 128 bytes a cycle as much as 32 different values do, so that scales and offsets together (64 reads of 16 bytes a
-// tile and warp) took 1024 cycles of it, as long as the tile's exponentials, and the products want it at its full rate for
-// 512 and the copies for 256.  A tile of pass 2 takes a group 3150 cycles instead of 3700: a decode
-// round (16 sequences x 8 heads x 2080 tokens) 44.1 -> 42.6 us, and with the value rows' loop below 16384 x 8 x 4 127 -> 122,
-// 20000 x 32 heads of 64 elements 95 -> 81.
-__device__ __forceinline__ void column_chunk(const uint32_t* r, const float* cs, const float* neg_off, uint64_t& za, uint64_t& zb) {
-#pragma unroll
-  for (int t = 0; t < 32; t += 4) {
-    const float4 o = *reinterpret_cast<const float4*>(neg_off + t);
-    float x0, x1, x2, x3;
-    unpack2(fma2(pack2(__uint_as_float(r[t]), __uint_as_float(r[t + 1])), pack2(cs[t], cs[t + 1]), pack2(o.x, o.y)), x0, x1);
-    unpack2(fma2(pack2(__uint_as_float(r[t + 2]), __uint_as_float(r[t + 3])), pack2(cs[t + 2], cs[t + 3]), pack2(o.z, o.w)), x2, x3);
-    za = add2(za, pack2(fast_exp2(x0), fast_exp2(x1)));
-    zb = add2(zb, pack2(fast_exp2(x2), fast_exp2(x3)));
-  }
-}
-// ... with everything from shared memory, and each row only up to the last key it may see.
-__device__ __forceinline__ void column_chunk_masked(const uint32_t* r, const float* cs, const float* neg_off, const int* last, int j,
-                                                    uint64_t& za, uint64_t& zb) {
-#pragma unroll
-  for (int t = 0; t < 32; t += 4) {
-    const float4 c = *reinterpret_cast<const float4*>(cs + t), o = *reinterpret_cast<const float4*>(neg_off + t);
-    const int4 l = *reinterpret_cast<const int4*>(last + t);
-    float x0, x1, x2, x3;
-    unpack2(fma2(pack2(__uint_as_float(r[t]), __uint_as_float(r[t + 1])), pack2(c.x, c.y), pack2(o.x, o.y)), x0, x1);
-    unpack2(fma2(pack2(__uint_as_float(r[t + 2]), __uint_as_float(r[t + 3])), pack2(c.z, c.w), pack2(o.z, o.w)), x2, x3);
-    if (j > l.x) x0 = -INFINITY;
-    if (j > l.y) x1 = -INFINITY;
-    if (j > l.z) x2 = -INFINITY;
-    if (j > l.w) x3 = -INFINITY;
-    za = add2(za, pack2(fast_exp2(x0), fast_exp2(x1)));
-    zb = add2(zb, pack2(fast_exp2(x2), fast_exp2(x3)));
-  }
-}
-
 // Softmax warps: groups of four warps; a key tile of a unit belongs to group (tile index mod kGroups).
 //   pass 1: thread `s` of a group owns stacked row s; at the end of the run the group leaves the row's statistic,
 //           log2 of the sum over its tiles, in shared memory for the delivery warp.
@@ -473,17 +398,7 @@ __device__ __forceinline__ void softmax_group(const TcArgs& a, Shared* sh, uint3
         const int j0 = (sg.blk0 + t) * kKeyTile;
         const bool full = j0 + kKeyTile - 1 <= a.min_last;   // no key of the tile is masked
         if (live) {
-#pragma unroll 1
-          for (int ch = 0; ch < 4; ++ch) {
-            uint32_t ra[32];
-            tmem_ld32_issue(lane_base + acc * 128 + 32 * ch, ra);
-            tmem_ld_wait(ra);
-            if (ch == 4 - 1) {
-              tc_fence_before();
-              mbar_arrive(&sh->acc_empty[acc]);              // the accumulator is free for the next product
-            }
-            fold_chunk(ra, full, j0 + 32 * ch, last, c, M, Z);
-          }
+          row_tile(lane_base + acc * 128, full, j0, last, c, M, Z, &sh->acc_empty[acc]);
         } else {
           mbar_arrive(&sh->acc_empty[acc]);
         }
@@ -511,37 +426,9 @@ __device__ __forceinline__ void softmax_group(const TcArgs& a, Shared* sh, uint3
         if (!mbar_wait(&sh->acc_full[g][mine & 3], (mine >> 2) & 1, a.status, wait_limit<kTest>(a))) { gone = true; continue; }
         tc_fence_after();
         const int j0 = (sg.blk0 + t) * kKeyTile, j = j0 + s;
-        uint64_t za = pack2(0.f, 0.f), zb = pack2(0.f, 0.f);
-        if (plain && j0 + kKeyTile - 1 <= a.min_last) {
-#pragma unroll
-          for (int ch = 0; ch < 4; ++ch) {
-            if (ch < chunks) {
-              uint32_t ra[32];
-              tmem_ld32_issue(lane_base + acc * 128 + 32 * ch, ra);
-              tmem_ld_wait(ra);
-              if (ch + 1 == chunks) {
-                tc_fence_before();
-                mbar_arrive(&sh->acc_empty[acc]);
-              }
-              column_chunk(ra, a.row_scale + 32 * ch, neg_off + 32 * ch, za, zb);
-            }
-          }
-        } else {
-#pragma unroll 1
-          for (int ch = 0; ch < chunks; ++ch) {
-            uint32_t ra[32];
-            tmem_ld32_issue(lane_base + acc * 128 + 32 * ch, ra);
-            tmem_ld_wait(ra);
-            if (ch + 1 == chunks) {
-              tc_fence_before();
-              mbar_arrive(&sh->acc_empty[acc]);
-            }
-            column_chunk_masked(ra, sh->row_c[kind] + 32 * ch, neg_off + 32 * ch, sh->tab_last[slot] + 32 * ch, j, za, zb);
-          }
-        }
-        float z0, z1;
-        unpack2(add2(za, zb), z0, z1);
-        if (j < a.n) a.s_raw[(size_t)sg.unit * a.n + j] = z0 + z1;
+        const float sum = column_tile(a, lane_base + acc * 128, chunks, plain && j0 + kKeyTile - 1 <= a.min_last, sh->row_c[kind], neg_off,
+                                      sh->tab_last[slot], j, &sh->acc_empty[acc]);
+        if (j < a.n) a.s_raw[(size_t)sg.unit * a.n + j] = sum;
       }
       mbar_arrive(&sh->tab_empty[slot]);
     }
@@ -643,83 +530,6 @@ __device__ __forceinline__ void table_warp(const TcArgs& a, Shared* sh) {
   }
 }
 
-// Value-norm warps: every warp of the grid takes chunks of value rows in turn, kValueLoads 16-byte loads a lane in flight.  Four
-// lanes share a row (64 bytes of it a load), square and add in FP32 and meet by shuffle.
-__device__ __forceinline__ uint4 ld_once(const char* p) {   // read once: do not keep in L1, evict first from L2
-  uint4 v;
-  asm volatile("ld.global.cs.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
-  return v;
-}
-template <typename T, int D>
-__device__ __forceinline__ void value_norms(const TcArgs& a, unsigned w, unsigned n_warps) {
-  constexpr int kPieces = D / 32, kSets = kValueLoads / kPieces, kRows = 8 * kSets;   // 64-byte pieces a row, 8-row sets in flight
-  const int grp = (threadIdx.x & 31) >> 2, tig = threadIdx.x & 3;
-  const unsigned per_head = (unsigned)(a.n + kRows - 1) / kRows, heads = (unsigned)a.BH, per_seq = (unsigned)a.Hkv;
-  const unsigned step_h = n_warps / per_head, step = n_warps - step_h * per_head;
-  unsigned bh = w / per_head, at = w - bh * per_head, b = bh / per_seq, h = bh - b * per_seq;   // head and chunk of it
-  if (bh >= heads) return;
-  const char* p[kSets];
-  int row;
-  auto locate = [&]() {   // rows past the end read the last one again; nothing of theirs is stored
-    row = (int)at * kRows + grp;
-    const char* head = a.v + b * a.vs[0] + h * a.vs[1] + tig * 16;
-#pragma unroll
-    for (int q = 0; q < kSets; ++q) p[q] = head + min(row + 8 * q, a.n - 1) * a.vs[2];
-  };
-  locate();
-  for (;;) {
-    uint4 u[kSets][kPieces];
-#pragma unroll
-    for (int q = 0; q < kSets; ++q)
-#pragma unroll
-      for (int i = 0; i < kPieces; ++i) u[q][i] = ld_once(p[q] + i * 64);
-    // where the next chunk is, while this one is on its way
-    float* const to = a.nu + (size_t)bh * a.n + row;
-    const int left = a.n - row;
-    at += step;
-    unsigned heads_on = step_h;
-    if (at >= per_head) { at -= per_head; ++heads_on; }
-    bh += heads_on;
-    h += heads_on;
-    if (h >= per_seq) {
-      const unsigned seqs = h / per_seq;
-      h -= seqs * per_seq;
-      b += seqs;
-    }
-    if (bh < heads) locate();
-#pragma unroll
-    for (int q = 0; q < kSets; ++q) asm volatile("" : "+l"(p[q]));   // now, not after the sums
-#pragma unroll
-    for (int q = 0; q < kSets; ++q) {
-      uint64_t acc = pack2(0.f, 0.f), acc2 = pack2(0.f, 0.f);
-#pragma unroll
-      for (int i = 0; i < kPieces; ++i) {
-        float f[8];
-        Vec16<T>::widen(u[q][i], f);
-#pragma unroll
-        for (int e = 0; e < 8; e += 4) {
-          const uint64_t p0 = pack2(f[e], f[e + 1]), p1 = pack2(f[e + 2], f[e + 3]);
-          acc = fma2(p0, p0, acc);
-          acc2 = fma2(p1, p1, acc2);
-        }
-      }
-      float s0, s1;
-      unpack2(add2(acc, acc2), s0, s1);
-      float sq = s0 + s1;
-      sq += __shfl_xor_sync(0xffffffffu, sq, 1);
-      sq += __shfl_xor_sync(0xffffffffu, sq, 2);
-      if (tig == 0 && 8 * q < left) to[8 * q] = sq;
-    }
-    if (bh >= heads) return;
-  }
-}
-
-// The softmax warps keep a chunk of the accumulator and its exponentials in registers, the others need few: of the 80 a
-// thread that the launch allows (768 threads), each of the twelve softmax warps takes 104 and the other twelve keep 56
-// (384 x 104 + 384 x 56 = 768 x 80).
-__device__ __forceinline__ void regs_down() { asm volatile("setmaxnreg.dec.sync.aligned.u32 56;"); }
-__device__ __forceinline__ void regs_up() { asm volatile("setmaxnreg.inc.sync.aligned.u32 104;"); }
-
 template <bool kTest>
 __global__ void __launch_bounds__(kThreads, 1)
 score_tc_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_constant__ CUtensorMap kmap,
@@ -814,8 +624,9 @@ score_tc_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_constant_
   }
 }
 
-// ---- host ------------------------------------------------------------------------------------------------
 }  // namespace
+
+// ---- host ------------------------------------------------------------------------------------------------
 
 bool score_tc_available() { return encode_fn() != nullptr; }
 
@@ -848,7 +659,7 @@ static int runs_per_row_block(long long units, int n_blk, int slots) {
 }
 
 ahakv_status launch_score_tc(const Plan& pl, const void* q, const void* k, const void* v, float* s_raw, float* nu,
-                             float* partial_ws, float* off_ws, int* counters, int* status, cudaStream_t st) {
+                             float* partial_ws, float* off_ws, int* counters, int* status, void* ones, size_t ones_bytes, cudaStream_t st) {
   // once per device: its SM count, and leave to use more than 48 KB of dynamic shared memory
   constexpr int kMaxDevices = 64;
   static int sm_count[kMaxDevices] = {};
@@ -870,11 +681,12 @@ ahakv_status launch_score_tc(const Plan& pl, const void* q, const void* k, const
   a.D = pl.d;
   for (int i = 0; i < kMaxRows; ++i) a.last[i] = pl.last[i];
   a.min_last = pl.last[0];
-  a.rpu = runs_per_row_block(units, a.n_blk, slots);
+  const int cluster = cluster_size(pl, slots);
+  a.rpu = cluster ? cluster : runs_per_row_block(units, a.n_blk, slots);
   a.CH = (a.n_blk + a.rpu - 1) / a.rpu;
-  a.rpu = (a.n_blk + a.CH - 1) / a.CH;
+  if (!cluster) a.rpu = (a.n_blk + a.CH - 1) / a.CH;
   a.n_runs = units * a.rpu;
-  const int grid = a.n_runs < slots ? a.n_runs : slots;
+  const int grid = cluster || a.n_runs < slots ? a.n_runs : slots;
   // A grid round, where each CTA does three runs or more.  With fewer the wait for a row block's statistics costs less than a
   // round in which only one of the passes runs: 70001 tokens x 4 heads of 7 queries (1.9 rounds) 66 us with no gap, 73 with a
   // round; 32768 x 8 heads of 4 (1.7) 69 and 72.  16384 x 32 (3.5) 87 and 81, and 84 with half a round; 16384 x 8 x 4 119 and 115; 32768 x 64
@@ -902,6 +714,12 @@ ahakv_status launch_score_tc(const Plan& pl, const void* q, const void* k, const
       !make_map(&kmap, k, a.bf16, pl.d, pl.n, pl.Hkv, pl.B, pl.ks, pl.es, kKeyTile, 1))
     return AHAKV_ERR_CUDA;
 
+  if (cluster) {
+    count_launch();
+    return cuda_ok(launch_cluster(qmap, kmap, a, grid, test, st));
+  }
+  const ahakv_status rc = launch_clear(ones, ones_bytes, st);
+  if (rc) return rc;
   const cudaError_t e = launch_chained(test ? score_tc_kernel<true> : score_tc_kernel<false>, dim3(grid), dim3(kThreads), 1, kSmemBytes, st,
                                        qmap, kmap, a);
   count_launch();

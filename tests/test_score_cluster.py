@@ -1,0 +1,89 @@
+"""The scoring kernel for calls that fit on the GPU at once (a cluster of CTAs per row block): sizes at which its shares, groups
+and row blocks come out uneven, against the oracle.  An eviction call that takes it is three launches; one more, the fill of
+the counters, is the kernel that hands its work out."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import ahakv_oracle as orc
+from paper_2506_03762_b200 import synth
+
+pytestmark = pytest.mark.gpu
+
+
+def _inputs(B, Hq, Hkv, d, n, r, dtype, seed):
+    g = torch.Generator(device="cuda").manual_seed(seed)
+    q, k, v = (torch.randn(s, generator=g, device="cuda").to(dtype) for s in ((B, Hq, r, d), (B, Hkv, n, d), (B, Hkv, n, d)))
+    k[:, :, 0] *= 4.0                                    # an attention sink: a row's shift may fall behind
+    return q, k, v
+
+
+@pytest.mark.parametrize("dtype_name,B,Hq,Hkv,d,n,r,flags", [
+    ("F16", 1, 32, 32, 128, 1061, 64, 1),     # clusters of four, shares of two and three tiles
+    ("F16", 1, 32, 32, 128, 1025, 64, 1),     # a last tile of one key
+    ("BF16", 1, 40, 40, 128, 2000, 100, 1),   # of three; rows that no box covers
+    ("BF16", 8, 32, 8, 64, 1000, 16, 0),      # of two; no value prior
+    ("F16", 4, 56, 8, 128, 1100, 24, 1),      # of two; a last row block with rows of another head in it
+    ("BF16", 8, 56, 8, 128, 700, 32, 1),      # one CTA a row block; a last row block of three heads
+    ("F16", 4, 32, 32, 64, 257, 8, 1),        # one CTA, three tiles: a tile for every group of warps
+    ("F16", 4, 32, 32, 128, 256, 128, 0),     # one CTA, two tiles: a group without one; every tile masked
+    ("F16", 1, 16, 16, 128, 1500, 200, 1),    # more than 128 rows: two row blocks a head
+])
+def test_calls_that_fit_at_once_match_the_oracle(dtype_name, B, Hq, Hkv, d, n, r, flags):
+    from paper_2506_03762_b200 import binding as ab
+    from tests import parity
+    dtype = getattr(ab, dtype_name)
+    q, k, v = _inputs(B, Hq, Hkv, d, n, r, ab.CODE_DTYPE[dtype], n + r)
+    p = ab.Params(B, Hq, Hkv, d, n, r, 16, max(32, n // 4), dtype=dtype, flags=flags)
+    before = ab.ahakv_launch_count()
+    parity.run_evict(p, q, k, v)
+    launches = ab.ahakv_launch_count() - before
+    assert launches == (2 if n <= 4096 and 2 * p.n_keep * d * 2 <= 128 * 1024 else 3)   # few rows are gathered by the selection
+    parity.check_units(p, q, k, v, [(0, 0), (B - 1, Hkv - 1), (B // 2, Hkv // 2)])
+    a, b = parity.run_score(p, q, k, v), parity.run_score(p, q, k, v)
+    assert torch.equal(a, b)
+
+
+def test_tiles_beyond_the_last_row_are_left_out():
+    from paper_2506_03762_b200 import binding as ab
+    from tests import parity
+    B, H, d, n, r = 1, 32, 128, 1500, 40
+    q, k, v = _inputs(B, H, H, d, n, r, torch.float16, 5)
+    rows = np.sort(np.random.default_rng(1).choice(900, size=r, replace=False))
+    p = ab.Params(B, H, H, d, n, r, 16, 300, dtype=ab.F16)
+    ws = ab.alloc_workspace(p, "cuda")
+    score = torch.empty((B, H, n), device="cuda")
+    ab.ahakv_score_rows(p, rows.tolist(), q, k, v, None, score, ws)
+    assert ab.ahakv_last_device_status(ws) == ab.OK
+    pick = [0, 31]
+    op = parity.oracle_params(ab.Params(B, 2, 2, d, n, r, 16, 300, dtype=ab.F16))
+    op.obs_pos = rows.tolist()
+    ref = orc.score(op, *(synth.to_numpy(t[:, pick]) for t in (q, k, v)), None)
+    parity.assert_scores_close(p, score[:, pick].cpu().numpy(), ref, "score_rows")
+
+
+@pytest.mark.parametrize("B,H,n", [(1, 32, 2048), (4, 32, 600)])     # a cluster's statistics withheld; a CTA's own
+def test_a_wait_that_runs_out_is_reported_and_the_next_call_is_clean(B, H, n):
+    from paper_2506_03762_b200 import binding as ab
+    q, k, v = _inputs(B, H, H, 128, n, 32, torch.bfloat16, 3)
+    p = ab.Params(B, H, H, 128, n, 32, 16, 200, dtype=ab.BF16)
+    ws = ab.alloc_workspace(p, "cuda")
+    outs = ab.alloc_outputs(p, "cuda")
+    ab.ahakv_evict(p, q, k, v, None, *outs, ws)
+    assert ab.ahakv_last_device_status(ws) == ab.OK
+    clean = [t.clone() for t in outs]
+    try:
+        ab.ahakv_test_set_wait(20, True)
+        t0, t1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        t0.record()
+        assert ab.ahakv_evict(p, q, k, v, None, *outs, ws, check=False) == ab.OK      # the fault is on the device
+        t1.record()
+        assert ab.ahakv_last_device_status(ws) == ab.ERR_TIMEOUT
+        assert t0.elapsed_time(t1) < 2000.0                                           # a few wait limits, not a hang
+        ab.ahakv_test_set_wait(50, False)                                             # a short limit alone changes nothing
+        ab.ahakv_evict(p, q, k, v, None, *outs, ws)
+        assert ab.ahakv_last_device_status(ws) == ab.OK
+    finally:
+        ab.ahakv_test_set_wait(0, False)
+    for a, b in zip(outs, clean):
+        assert torch.equal(a, b)
