@@ -82,117 +82,6 @@ __device__ __forceinline__ Part part_of(const TcArgs& a) {
   return p;
 }
 
-// ---- softmax pieces -------------------------------------------------------------------------------------
-// With one stream of tiles per CTA a group often works alone (the first tiles, the last ones of a pass), so what a row tile
-// takes by itself counts: sixteen columns at a time, the next sixteen on their way meanwhile.  (2140 cycles a tile for 3000 where
-// the other groups leave the special-function unit alone; a decode round 41.9 -> 40.3 us, 4160 tokens x 64 heads 65.8 -> 63.1.)
-__device__ __forceinline__ void tmem_ld16_issue(uint32_t taddr, uint32_t* r) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-      : "r"(taddr)
-      : "memory");
-}
-__device__ __forceinline__ void tmem_ld16_wait(uint32_t* r) {
-  asm volatile("tcgen05.wait::ld.sync.aligned;"
-               : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),
-                 "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15])
-               :
-               : "memory");
-}
-// Adds 2^{c v + neg} of sixteen values to the four running sums.
-__device__ __forceinline__ void exp_add16(const uint32_t* r, uint64_t c2, uint64_t neg2, uint64_t& za, uint64_t& zb) {
-#pragma unroll
-  for (int t = 0; t < 16; t += 4) {
-    float x0, x1, x2, x3;
-    unpack2(fma2(pack2(__uint_as_float(r[t]), __uint_as_float(r[t + 1])), c2, neg2), x0, x1);
-    unpack2(fma2(pack2(__uint_as_float(r[t + 2]), __uint_as_float(r[t + 3])), c2, neg2), x2, x3);
-    za = add2(za, pack2(fast_exp2(x0), fast_exp2(x1)));
-    zb = add2(zb, pack2(fast_exp2(x2), fast_exp2(x3)));
-  }
-}
-__device__ __forceinline__ float sum4(uint64_t za, uint64_t zb) {
-  float z0, z1;
-  unpack2(add2(za, zb), z0, z1);
-  return z0 + z1;
-}
-__device__ __forceinline__ float max16(const uint32_t* r) {
-  float m0 = __uint_as_float(r[0]), m1 = __uint_as_float(r[1]);
-#pragma unroll
-  for (int t = 2; t < 16; t += 2) {
-    m0 = fmaxf(m0, __uint_as_float(r[t]));
-    m1 = fmaxf(m1, __uint_as_float(r[t + 1]));
-  }
-  return fmaxf(m0, m1);
-}
-// As fold_chunk, sixteen columns without a mask.
-__device__ __forceinline__ void fold16(const uint32_t* r, float c, float& M, float& Z) {
-  if (M > -INFINITY) {
-    uint64_t za = pack2(0.f, 0.f), zb = pack2(0.f, 0.f);
-    exp_add16(r, pack2(c, c), pack2(-M, -M), za, zb);
-    const float z = sum4(za, zb);
-    if (z < kAcceptBelow) {
-      Z += z;
-      return;
-    }
-  }
-  const float mx = max16(r) * c;
-  if (mx > -INFINITY) {
-    uint64_t za = pack2(0.f, 0.f), zb = pack2(0.f, 0.f);
-    exp_add16(r, pack2(c, c), pack2(-mx, -mx), za, zb);
-    Z = (M > -INFINITY ? Z * fast_exp2(M - mx) : 0.f) + sum4(za, zb);
-    M = mx;
-  }
-}
-// As row_tile, of a tile no key of which is masked.  The shift is looked at twice: for the first six pieces while they are still in
-// tensor memory, for the last two while they are in registers.
-__device__ __forceinline__ void row_tile16(uint32_t from, float c, float& M, float& Z, void* empty) {
-  uint32_t u[16], w[16];
-  tmem_ld16_issue(from, u);
-  tmem_ld16_wait(u);
-  tmem_ld16_issue(from + 16, w);
-  if (!(M > -INFINITY)) M = max16(u) * c;
-  const uint64_t c2 = pack2(c, c), neg2 = pack2(-M, -M);
-  uint64_t za = pack2(0.f, 0.f), zb = pack2(0.f, 0.f), ya = pack2(0.f, 0.f), yb = pack2(0.f, 0.f);
-  exp_add16(u, c2, neg2, za, zb);
-#pragma unroll
-  for (int ch = 2; ch < 8; ch += 2) {
-    tmem_ld16_wait(w);
-    tmem_ld16_issue(from + 16 * ch, u);
-    exp_add16(w, c2, neg2, za, zb);
-    tmem_ld16_wait(u);
-    tmem_ld16_issue(from + 16 * ch + 16, w);
-    if (ch < 6) exp_add16(u, c2, neg2, za, zb);
-    else exp_add16(u, c2, neg2, ya, yb);
-  }
-  float z = sum4(za, zb);
-  const bool sound = z < kAcceptBelow;                        // an overflow or a NaN fails this test too
-  tmem_ld16_wait(w);
-  if (__any_sync(0xffffffffu, !sound)) {
-#pragma unroll 1
-    for (int ch = 0; ch < 6; ++ch) {
-      uint32_t again[16];
-      tmem_ld16_issue(from + 16 * ch, again);
-      tmem_ld16_wait(again);
-      if (!sound) fold16(again, c, M, Z);
-    }
-  }
-  tc_fence_before();
-  mbar_arrive(empty);
-  if (sound) {
-    Z += z;
-    exp_add16(w, c2, neg2, ya, yb);
-    z = sum4(ya, yb);
-  }
-  if (sound && z < kAcceptBelow) {
-    Z += z;
-  } else {
-    fold16(u, c, M, Z);
-    fold16(w, c, M, Z);
-  }
-}
-
 // ---- roles --------------------------------------------------------------------------------------------
 template <bool kTest>
 __device__ __forceinline__ void producer(const TcArgs& a, const Part& p, const CUtensorMap* qmap, const CUtensorMap* kmap, Shared* sh, char* tiles) {
@@ -284,8 +173,8 @@ __device__ __forceinline__ void softmax_group(const TcArgs& a, const Part& p, Sh
       if (!__all_sync(0xffffffffu, mbar_wait(&sh->acc_full[g][mine & 3], (mine >> 2) & 1, a.status, limit))) { gone = true; continue; }
       tc_fence_after();
       if (!live) mbar_arrive(&sh->acc_empty[acc]);
-      else if (j0 + kKeyTile - 1 <= a.min_last) row_tile16(lane_base + acc * 128, c, M, Z, &sh->acc_empty[acc]);
-      else row_tile(lane_base + acc * 128, false, j0, last, c, M, Z, &sh->acc_empty[acc]);
+      else if (j0 + kKeyTile - 1 <= a.min_last) row_tile(lane_base + acc * 128, c, M, Z, &sh->acc_empty[acc]);
+      else row_tile_masked(lane_base + acc * 128, j0, last, c, M, Z, &sh->acc_empty[acc]);
     }
     sh->stat[g][s] = make_float2(M, Z);
   }
@@ -450,7 +339,9 @@ int clusters_at_once(int size) {
 //   blocks of 70001 tokens 145 and 72 (clusters of more than eight do not fit: 72 CTAs);
 // - keys that stay in L2 (96 MB of its 126) until the second pass, which starts only when the first is over: 16384 tokens x 32
 //   heads, 134 MB, 75 and 73; x 8 heads x 4 sequences 115 and 110;
-// - two tiles a CTA or more, so that the stream outlasts the copies' way.
+// - two tiles a CTA or more, so that the stream outlasts the copies' way, and with value rows beside it at most twenty: with sixteen
+//   (8192 x 32 heads) a call takes 53.3 for 54.1, with 39 (20000 x 32 of 64 elements) 84.1 for 80.5.  Without them one of 4160 x 128
+//   row blocks with 33 takes 100 for 107.
 int tc::cluster_size(const Plan& pl, int slots) {
   const long long units = (long long)pl.B * pl.Hkv * pl.n_rb;
   const int n_blk = (pl.n_eff + kKeyTile - 1) / kKeyTile;
@@ -459,7 +350,8 @@ int tc::cluster_size(const Plan& pl, int slots) {
   if (size > kMostCtas) size = kMostCtas;
   if (size > n_blk / 2) size = n_blk / 2;
   while (size > 0 && clusters_at_once(size) < units) --size;
-  return 5 * units * size >= 4 * slots ? size : 0;
+  const bool short_enough = (pl.flags & AHAKV_FLAG_VALUE_PRIOR) == 0 || n_blk <= 20 * size;
+  return 5 * units * size >= 4 * slots && short_enough ? size : 0;
 }
 
 cudaError_t tc::launch_cluster(const CUtensorMap& qmap, const CUtensorMap& kmap, const TcArgs& a, int grid, bool test, cudaStream_t st) {
