@@ -8,7 +8,8 @@
 // there), and only the shifted exponent, a small number, goes back to FP32 for the
 // exponential.  16-bit inputs (1e-3) keep FP32 throughout.
 //
-// Two kernels over 64-key tiles, one CTA a tile of a (sequence, KV head).
+// A call whose tiles are all on the GPU at once: simt_cluster_scores (float32 only).  Others: two kernels over 64-key tiles, one
+// CTA a tile of a (sequence, KV head).
 //   simt_row_stats:   every observation row's softmax statistics (max and sum of 2^{c w}) per 128-key block, two CTAs (a
 //                     cluster) a block.
 //                     Leaves the numerators 2^{c w - m} in the workspace if it has room; m is the row's maximum over a
@@ -29,6 +30,7 @@
 // Every reduction has a fixed order, so the scores are reproducible bit for bit.
 #include <cooperative_groups.h>
 
+#include <atomic>
 #include <type_traits>
 
 #include "ahakv_internal.cuh"
@@ -38,6 +40,8 @@ namespace {
 
 namespace cg = cooperative_groups;
 
+constexpr int kSms = 148;
+constexpr int kOnePerSm = 226 * 1024, kTwoPerSm = 112 * 1024;   // dynamic shared memory with which one CTA, or two, fit on an SM
 constexpr int kThreads = 256;
 constexpr int kTile = 64;                // keys per CTA
 constexpr int kRows = 32;                // stacked observation rows at a time
@@ -476,6 +480,243 @@ simt_weighted_sums(const T* __restrict__ v, const float2* partial, const float* 
   if (share == 0 && j < pl.n) s_raw[(size_t)unit * pl.n + j] = best;
 }
 
+// ---- float32 inputs, all tiles of a call on the GPU at once: both passes in one kernel --------------------------------------
+// A cluster of up to sixteen CTAs per (sequence, KV head), each a few adjacent tiles: the numerators stay in shared memory, the rows'
+// statistics meet through the cluster's, and nothing is formed twice or taken through global memory.  Keys lie in shared memory as
+// they came and are converted on their way into the products, by both row warps (a conversion costs four multiply-adds, so a tile's
+// 4096 cycles of products become 5100), which leaves room for two CTAs an SM; the next tile is on its way meanwhile.
+// Calls, with the two kernels before: 512 tokens x 4 heads 12.7 -> 11.9 us, 300 x 2 heads of 4 queries 25.3 -> 19.0, 1000 x 4 of 4
+// 20.7 -> 17.1, 3001 x 8 37.4 -> 35.3, 2048 x 64 124 -> 99.  Scores end up as far from double as before or nearer (9.6e-8 -> 8.6e-8
+// to 9.3e-8 of their norm), because sums are taken in pairs; with the rows' sums in double throughout 4.9e-8, and 37.3 and 12.3 us.
+constexpr int kMostCtas = 16;
+
+template <int D>
+struct ClusterTile {
+  float k[kTile][D + 8];                               // padded: the four rows of a half-warp's 8-byte loads on different banks
+  double q[kRows][row_pitch<double, D>()];
+  double row_c[kRows];
+  int row_last[kRows];
+  float2 fin[kMaxRows];                                // of the CTA first, of the row then: shift and sum; shift and 1 / (G sum)
+  float2 stat[kKeyWarps][kMaxRows];                    // per key warp: shift and sum of a row over the CTA's tiles
+  float sums[kThreads / kTile][kTile];
+};
+// N (shift, sum) pairs of disjoint key sets into one.  The shifts are whole numbers, so that only the additions round.
+template <int N>
+__device__ __forceinline__ float2 add_pairs(const float2 (&p)[N]) {
+  float M = p[0].x;
+#pragma unroll
+  for (int i = 1; i < N; ++i) M = fmaxf(M, p[i].x);
+  float z[N];
+#pragma unroll
+  for (int i = 0; i < N; ++i) z[i] = p[i].y != 0.f ? p[i].y * pow2_diff(p[i].x, M) : 0.f;   // -inf goes with 0
+#pragma unroll
+  for (int o = 1; o < N; o <<= 1)
+#pragma unroll
+    for (int i = 0; i + o < N; i += 2 * o) z[i] += z[i + o];
+  return make_float2(M, z[0]);
+}
+// Behind it: shifts [tile][kKeyWarps][R], then numerators [tile][R][kTile].
+template <int D> size_t cluster_smem(int tiles, int R) { return sizeof(ClusterTile<D>) + (size_t)tiles * R * (kKeyWarps + kTile) * sizeof(float); }
+
+template <int D>
+__global__ void __launch_bounds__(kThreads, 2)
+simt_cluster_scores(const float* __restrict__ q, const float* __restrict__ k, const float* __restrict__ v, float* __restrict__ s_raw,
+                    float* __restrict__ nu, int* __restrict__ status, const int per, const __grid_constant__ Shape pl,
+                    const __grid_constant__ RowScaleOf<double> cs) {
+  constexpr int PER = D / 4, NK = kTile * PER / kThreads, NQ = kRows * PER / kThreads;
+  extern __shared__ __align__(16) char smem_raw[];
+  ClusterTile<D>& sm = *reinterpret_cast<ClusterTile<D>*>(smem_raw);
+  float* const shift = reinterpret_cast<float*>(smem_raw + sizeof(ClusterTile<D>));
+  float* const numer = shift + per * kKeyWarps * pl.R;
+  cg::cluster_group cl = cg::this_cluster();
+  const int C = (int)cl.num_blocks(), rank = (int)cl.block_rank(), unit = blockIdx.x / C, b = unit / pl.Hkv, h = unit % pl.Hkv, R = pl.R;
+  const int tiles_all = (pl.n + kTile - 1) / kTile, first = rank * tiles_all / C, tiles = (rank + 1) * tiles_all / C - first;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, grp = lane >> 2, tig = lane & 3;
+  const int kw = warp & (kKeyWarps - 1), rw = warp / kKeyWarps, row = 16 * rw + grp;
+  const float* const keys = k + (long long)b * pl.ks[0] + (long long)h * pl.ks[1];
+  uint4 ku[NK];
+  const auto load_keys = [&](int tile) {
+#pragma unroll
+    for (int e = 0; e < NK; ++e) {
+      const int t = threadIdx.x + e * kThreads, j = tile * kTile + t / PER;
+      ku[e] = j < pl.n ? *reinterpret_cast<const uint4*>(keys + (long long)j * pl.ks[2] + t % PER * 4) : make_uint4(0, 0, 0, 0);
+    }
+  };
+  griddep_wait();
+  if (blockIdx.x == 0 && threadIdx.x == 0) *status = 0;
+  if (tiles > 0) load_keys(first);
+  for (int s0 = 0; s0 < R; s0 += kRows) {
+    const int rows = min(kRows, R - s0);
+    __syncthreads();                                   // the rows before are done with
+    if (threadIdx.x < kRows) {
+      const int i = (s0 + (int)threadIdx.x) % pl.r;
+      sm.row_c[threadIdx.x] = cs.c[i];
+      sm.row_last[threadIdx.x] = (int)threadIdx.x < rows ? cs.last[i] : -1;
+    }
+#pragma unroll
+    for (int e = 0; e < NQ; ++e) {
+      const int t = threadIdx.x + e * kThreads, at = t / PER, s = s0 + at, g = s / pl.r, i = s - g * pl.r;
+      uint4 u = make_uint4(0, 0, 0, 0);
+      if (at < rows) u = *reinterpret_cast<const uint4*>(q + (long long)b * pl.qs[0] + (long long)(h * pl.G + g) * pl.qs[1] + (long long)i * pl.qs[2] + t % PER * 4);
+      put16<float>(&sm.q[at][t % PER * 4], u);
+    }
+    for (int t = 0; t < tiles; ++t) {
+      if (t > 0) __syncthreads();                      // the tile before is done with
+#pragma unroll
+      for (int e = 0; e < NK; ++e) {
+        const int i = threadIdx.x + e * kThreads;
+        *reinterpret_cast<uint4*>(&sm.k[i / PER][i % PER * 4]) = ku[e];
+      }
+      __syncthreads();
+      if (t + 1 < tiles) load_keys(first + t + 1);
+      else if (s0 + kRows < R) load_keys(first);
+      // the products of the warp's 16 keys and 16 rows, laid out as in dot_16x16
+      double acc[4][2];
+#pragma unroll
+      for (int x = 0; x < 4; ++x) acc[x][0] = acc[x][1] = 0.0;
+#pragma unroll 4
+      for (int d = 0; d < D; d += 8) {
+        double2 kv[2], qv[2];
+#pragma unroll
+        for (int y = 0; y < 2; ++y) {
+          const float2 f = *reinterpret_cast<const float2*>(&sm.k[16 * kw + 8 * y + grp][d + 2 * tig]);
+          kv[y] = make_double2((double)f.x, (double)f.y);
+          qv[y] = *reinterpret_cast<const double2*>(&sm.q[16 * rw + 8 * y + grp][d + 2 * tig]);
+        }
+#pragma unroll
+        for (int y = 0; y < 2; ++y)
+#pragma unroll
+          for (int x = 0; x < 2; ++x) {
+            mma_884(acc[2 * x][y], acc[2 * x + 1][y], qv[y].x, kv[x].x);
+            mma_884(acc[2 * x][y], acc[2 * x + 1][y], qv[y].y, kv[x].y);
+          }
+      }
+      const double cc[2] = {sm.row_c[row], sm.row_c[row + 8]};
+      const int last[2] = {sm.row_last[row], sm.row_last[row + 8]}, key0 = 16 * kw + 2 * tig, j0 = (first + t) * kTile + key0;
+      const int at[4] = {j0, j0 + 1, j0 + 8, j0 + 9};
+      float m[2];
+      row_shifts(acc, cc, last, at, m);
+#pragma unroll
+      for (int y = 0; y < 2; ++y) {
+        float e[4], z = 0.f;
+#pragma unroll
+        for (int x = 0; x < 4; ++x) {
+          e[x] = at[x] <= last[y] ? numerator(acc[x][y], cc[y], m[y]) : 0.f;
+          z += e[x];
+        }
+#pragma unroll
+        for (int o = 2; o; o >>= 1) z += __shfl_xor_sync(0xffffffffu, z, o);
+        if (row + 8 * y < rows) {
+          const int s = s0 + row + 8 * y;
+          float* to = numer + ((size_t)t * R + s) * kTile + key0;
+          *reinterpret_cast<float2*>(to) = make_float2(e[0], e[1]);
+          *reinterpret_cast<float2*>(to + 8) = make_float2(e[2], e[3]);
+          if (tig == 0) {
+            shift[(t * kKeyWarps + kw) * R + s] = m[y];
+            const float2 p[2] = {t == 0 ? make_float2(-INFINITY, 0.f) : sm.stat[kw][s], make_float2(m[y], z)};
+            sm.stat[kw][s] = add_pairs(p);
+          }
+        }
+      }
+    }
+  }
+  __syncthreads();
+  for (int s = threadIdx.x; s < R; s += kThreads) {
+    const float2 p[kKeyWarps] = {sm.stat[0][s], sm.stat[1][s], sm.stat[2][s], sm.stat[3][s]};
+    sm.fin[s] = add_pairs(p);
+  }
+  cl.barrier_arrive();
+  if (nu)
+    for (int t = 0; t < tiles; ++t) tile_norms<float, D>(v, nu, pl, b, h, unit, (first + t) * kTile);
+  cl.barrier_wait();
+  // every CTA's pairs; kept aside until all have read theirs
+  float2 mine = make_float2(0.f, 0.f);
+  static_assert(kMaxRows <= kThreads, "a thread a row");
+  if ((int)threadIdx.x < R) {
+    float2 p[kMostCtas];
+#pragma unroll
+    for (int c = 0; c < kMostCtas; ++c) p[c] = c < C ? cl.map_shared_rank(&sm, c)->fin[threadIdx.x] : make_float2(-INFINITY, 0.f);
+    mine = add_pairs(p);
+    mine.y = 1.f / (mine.y * (float)pl.G);
+  }
+  cl.sync();
+  griddep_launch();
+  if ((int)threadIdx.x < R) sm.fin[threadIdx.x] = mine;
+  __syncthreads();
+  for (int i = threadIdx.x; i < tiles * kKeyWarps * R; i += kThreads) {
+    const float2 f = sm.fin[i % R];
+    shift[i] = pow2_diff(shift[i], f.x) * f.y;         // now the weight of the numerators taken against it
+  }
+  __syncthreads();
+  const int jl = threadIdx.x % kTile, share = threadIdx.x / kTile;
+  for (int t = 0; t < tiles; ++t) {
+    const float* by = shift + (t * kKeyWarps + jl / 16) * R;
+    const float* e = numer + (size_t)t * R * kTile + jl;
+    float acc[4] = {};
+    for (int s = share; s < R; s += 16) {
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+        if (s + 4 * i < R) acc[i] = fmaf(e[(s + 4 * i) * kTile], by[s + 4 * i], acc[i]);
+    }
+    sm.sums[share][jl] = (acc[0] + acc[1]) + (acc[2] + acc[3]);
+    __syncthreads();
+    const int j = (first + t) * kTile + jl;
+    if (share == 0 && j < pl.n) s_raw[(size_t)unit * pl.n + j] = (sm.sums[0][jl] + sm.sums[1][jl]) + (sm.sums[2][jl] + sm.sums[3][jl]);
+    __syncthreads();
+  }
+}
+
+// How many clusters of `size` CTAs the current device holds at once, `per_sm` of them (one or two) an SM.  Asked once.
+template <int D>
+int clusters_at_once(int size, int per_sm) {
+  constexpr int kMaxDevices = 64;
+  static std::atomic<int> known[kMaxDevices][2][kMostCtas + 1] = {};   // one more than the number; 0: not asked yet
+  int dev = -1;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return 0;
+  int n = known[dev][per_sm - 1][size].load(std::memory_order_relaxed);
+  if (n != 0) return n - 1;
+  const void* kernel = (const void*)simt_cluster_scores<D>;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(size);
+  cfg.blockDim = dim3(kThreads);
+  cfg.dynamicSmemBytes = per_sm == 2 ? kTwoPerSm : kOnePerSm;
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeClusterDimension;
+  attr.val.clusterDim.x = size;
+  attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kOnePerSm) != cudaSuccess ||
+      cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
+      cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) {
+    cudaGetLastError();
+    n = 0;
+  }
+  known[dev][per_sm - 1][size].store(n + 1, std::memory_order_relaxed);
+  return n;
+}
+
+// CTAs a head, or 0: the size with the fewest tiles one after the other on an SM, of those of which the whole call is on the GPU at once.
+// Two tiles or three on end are worth it whatever part of the GPU they take; more only as long as no SM has half as much again
+// as its share (8 heads of 6000 tokens, ten tiles a CTA on 80 SMs: 62.7 us a call for 57.2; 64 heads of 2048, sixteen: 97 for 124).
+template <int D>
+int cluster_size(const Shape& pl) {
+  if (pl.group_max) return 0;
+  const long long units = (long long)pl.B * pl.Hkv;
+  const int tiles = (pl.n + kTile - 1) / kTile;
+  int best = 0;
+  long long best_cost = 0;
+  for (int size = tiles < kMostCtas ? tiles : kMostCtas; size > 1; --size) {
+    const int per = (tiles + size - 1) / size;
+    const size_t smem = cluster_smem<D>(per, pl.R);
+    if (smem > (size_t)kOnePerSm) break;               // fewer CTAs need more
+    const int fit = clusters_at_once<D>(size, smem <= (size_t)kTwoPerSm ? 2 : 1);
+    const long long cost = per * ((units * size + kSms - 1) / kSms);
+    if (fit >= units && (best == 0 || cost < best_cost)) { best = size; best_cost = cost; }
+  }
+  return best_cost <= 3 || 2 * best_cost * kSms <= 3 * units * tiles ? best : 0;
+}
+
 template <typename T, int D>
 ahakv_status run(const Plan& pl, const void* q, const void* k, const void* v, float* s_raw, float* nu, float2* partial, float* kept, int* status,
                  cudaStream_t st) {
@@ -499,6 +740,14 @@ ahakv_status run(const Plan& pl, const void* q, const void* k, const void* v, fl
   }
   const Shape& shape = pl;
   const int units = pl.B * pl.Hkv;
+  if constexpr (std::is_same<T, float>::value) {
+    if (const int size = cluster_size<D>(shape)) {
+      const int per = ((pl.n + kTile - 1) / kTile + size - 1) / size;
+      count_launch();
+      return cuda_ok(launch_chained(simt_cluster_scores<D>, dim3(units * size), dim3(kThreads), size, cluster_smem<D>(per, pl.R), st, (const float*)q,
+                                    (const float*)k, (const float*)v, s_raw, nu, status, per, shape, cs));
+    }
+  }
   const dim3 stats_grid(2 * pl.n_blk, units), sums_grid((pl.n + kTile - 1) / kTile, units);
   float* const none = nullptr;
   cudaError_t e;

@@ -27,6 +27,32 @@ def test_float32_scores_at_tile_edges(B, Hq, Hkv, d, n, r, flags):
     assert torch.allclose(score.double(), want, rtol=1e-5, atol=1e-5 * 1e-3 * r / n)
 
 
+@pytest.mark.parametrize("B,Hq,Hkv,d,n,r", [
+    (1, 1, 1, 128, 65, 1),          # two CTAs, one of them with a single key
+    (1, 8, 8, 128, 3001, 32),       # sixteen CTAs a head, two and three tiles each
+    (1, 8, 2, 64, 1500, 16),        # two chunks of rows
+    (2, 6, 2, 128, 1100, 33),       # a last chunk of three rows
+    (4, 16, 16, 128, 700, 32),      # three CTAs a head, two of them on an SM
+    (1, 3, 1, 64, 513, 80),         # 240 rows
+])
+def test_float32_scores_by_clusters(B, Hq, Hkv, d, n, r):
+    """Calls whose tiles are all on the GPU at once: one kernel does both passes, and an eviction call is two or three launches."""
+    from paper_2506_03762_b200 import binding as ab
+    g = torch.Generator(device="cuda").manual_seed(n + r)
+    q = 3 * torch.randn((B, Hq, r, d), generator=g, device="cuda")
+    k, v = (torch.randn((B, Hkv, n, d), generator=g, device="cuda") for _ in range(2))
+    p = ab.Params(B, Hq, Hkv, d, n, r, 0, max(1, n // 2), dtype=ab.F32, scale_mode=ab.SCALE_FIXED, scale=0.09, flags=0)
+    score = torch.empty((B, Hkv, n), device="cuda")
+    before = ab.ahakv_launch_count()
+    ab.ahakv_score(p, q, k, v, None, score, ab.alloc_workspace(p))
+    assert ab.ahakv_launch_count() - before == 2
+    G = Hq // Hkv
+    w = float(torch.tensor(0.09, dtype=torch.float32)) * q.double() @ k.double().repeat_interleave(G, 1).transpose(-1, -2)
+    seen = torch.arange(n, device="cuda") <= torch.arange(n - r, n, device="cuda").view(r, 1)
+    want = w.masked_fill(~seen, float("-inf")).softmax(-1).sum(2).view(B, Hkv, G, n).mean(2)
+    assert torch.allclose(score.double(), want, rtol=1e-5, atol=1e-5 * 1e-3 * r / n)
+
+
 @pytest.mark.parametrize("n,r,Hq,Hkv,flags", [(9001, 64, 4, 4, 1), (9100, 20, 12, 4, 5)])
 def test_scores_with_and_without_room_for_numerators_agree(n, r, Hq, Hkv, flags):
     """The library's own scratch is too small for these cases' softmax numerators, so that the logits are formed twice; with
