@@ -40,6 +40,12 @@ def test_selection_equals_a_stable_sort(H, n, Br, Bud, kind):
         assert np.array_equal(got[0, h], _expected(sn[0, h], Br, Bud))
 
 
+@pytest.mark.parametrize("H,n", [(1, 65552), (1, 98304), (1, 98305), (200, 12288), (200, 12290)])     # nine to thirteen tokens a thread
+@pytest.mark.parametrize("kind", ["spread", "one_bin"])
+def test_selection_around_twelve_tokens_a_thread(H, n, kind):
+    test_selection_equals_a_stable_sort(H, n, 5, n // 3, kind)
+
+
 @pytest.mark.parametrize("n", [130, 1027, 4100, 9001, 33001])
 @pytest.mark.parametrize("pool,flags", [(1, 1), (3, 1), (7, 1), (7, 3), (31, 1)])
 def test_refinement_in_the_eviction_call_equals_the_definition(n, pool, flags):
