@@ -28,6 +28,9 @@ def _inputs(B, Hq, Hkv, d, n, r, dtype, seed):
     ("F16", 4, 32, 32, 64, 257, 8, 1),        # one CTA, three tiles: a tile for every group of warps
     ("F16", 4, 32, 32, 128, 256, 128, 0),     # one CTA, two tiles: a group without one; every tile masked
     ("F16", 1, 16, 16, 128, 1500, 200, 1),    # more than 128 rows: two row blocks a head
+    ("BF16", 1, 1, 1, 64, 256, 16, 1),        # one head, one CTA
+    ("F16", 1, 8, 1, 128, 4992, 16, 1),       # one head, eight CTAs of five tiles, less one
+    ("BF16", 1, 20, 5, 128, 1400, 32, 1),     # clusters of five
 ])
 def test_calls_that_fit_at_once_match_the_oracle(dtype_name, B, Hq, Hkv, d, n, r, flags):
     from paper_2506_03762_b200 import binding as ab
