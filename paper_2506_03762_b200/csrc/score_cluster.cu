@@ -5,7 +5,7 @@
 // handed out on the fly that is: a launch that clears counters and offsets, an atomic per run, partial statistics and a counter in
 // global memory, their merge by whoever comes last, offsets published and polled for, and a few segments a CTA
 // with a hand-over each.  Here nothing is handed out: a CTA's keys come as one stream of tiles, the second pass's first tiles are multiplied
-// while the statistics meet, and every CTA sends its log2 sums (a float a row) straight into the shared memory of the others, where
+// while the statistics meet, and every CTA sends its rows' shifts and sums straight into the shared memory of the others, where
 // an mbarrier counts their bytes.  A tile visit takes 1200 - 1300 cycles, the turn from one pass to the other 4400 (mostly the
 // groups' last tiles), copies and first products 3800.  A whole eviction call with this kernel, and with runs handed out: 4096
 // tokens x 32 heads 29.0 and 31.9 us, 1024 x 64 heads 20.1 and 23.5, 2048 x 64 heads of 4 queries 32.5 and 35.5, 5000 x 32 heads
@@ -34,7 +34,7 @@ struct Shared {
   float neg_off[128];                       // pass 2: minus a row's offset, -inf past the live rows
   int tab_last[128];                        // row_last, -1 past the live rows
   float2 stat[kGroups][128];                // pass 1: each group's shift and sum of a row
-  float part[kMostCtas][128];               // every CTA's log2 sums
+  float2 part[kMostCtas][128];              // every CTA's shifts and sums
   unsigned long long q_full, part_full;
   unsigned long long k_full[kKStages], k_empty[kKStages];
   unsigned long long acc_full[kGroups][4];  // per group: its k-th tile completes barrier k mod 4
@@ -55,11 +55,24 @@ __device__ __forceinline__ void cluster_sync() {
 __device__ __forceinline__ void softmax_sync() { asm volatile("bar.sync 1, %0;" ::"n"(128 * kGroups) : "memory"); }
 
 // `value` to where `local` lies in CTA `rank` of the cluster, counted there by the barrier where `bar` lies.
-__device__ __forceinline__ void send(const float* local, const void* bar, int rank, float value) {
+__device__ __forceinline__ void send(const float2* local, const void* bar, int rank, float2 value) {
   uint32_t to, there;
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(to) : "r"(smem_u32(local)), "r"(rank));
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(there) : "r"(smem_u32(bar)), "r"(rank));
-  asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.b32 [%0], %1, [%2];" ::"r"(to), "r"(__float_as_uint(value)), "r"(there) : "memory");
+  asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.b64 [%0], %1, [%2];" ::"r"(to), "l"(pack2(value.x, value.y)), "r"(there) : "memory");
+}
+
+// (shift, sum) pairs of disjoint key sets into one.  A NaN stays.
+template <int N>
+__device__ __forceinline__ void add_pairs(const float2 (&p)[N], float& M, float& Z) {
+  float m = M;
+#pragma unroll
+  for (int t = 0; t < N; ++t) m = fmaxf(m, p[t].x);
+  float z = Z != 0.f ? Z * fast_exp2(M - m) : 0.f;
+#pragma unroll
+  for (int t = 0; t < N; ++t) z += p[t].y != 0.f ? p[t].y * fast_exp2(p[t].x - m) : 0.f;
+  M = m;
+  Z = z;
 }
 
 // The CTA's part: a row block and a stretch of its key tiles.
@@ -180,19 +193,14 @@ __device__ __forceinline__ void softmax_group(const TcArgs& a, const Part& p, Sh
   }
   softmax_sync();
   if (g == 0) {
-    float x[kGroups], M = -INFINITY, Z = 0.f;
-#pragma unroll
-    for (int t = 0; t < kGroups; ++t) {
-      const float2 st = sh->stat[t][s];
-      x[t] = st.y > 0.f ? st.x + log2f(st.y) : st.y == st.y ? -INFINITY : INFINITY;   // NaN inputs: nothing downstream waits for a number
-    }
-    merge_logs(x, M, Z);
-    const float L = M + log2f(Z);
+    float M = -INFINITY, Z = 0.f;
+    const float2 groups[kGroups] = {sh->stat[0][s], sh->stat[1][s], sh->stat[2][s]};
+    add_pairs(groups, M, Z);
     const bool withheld = kTest && a.test_withhold && blockIdx.x == 0;
     if (a.rpu > 1) {
-      for (int t = 0; t < a.rpu && !withheld; ++t) send(&sh->part[p.rank][s], &sh->part_full, t, L);
+      for (int t = 0; t < a.rpu && !withheld; ++t) send(&sh->part[p.rank][s], &sh->part_full, t, make_float2(M, Z));
     } else {                                                // a launch without clusters executes none of their instructions
-      sh->part[0][s] = L;
+      sh->part[0][s] = make_float2(M, Z);
       if (!withheld) mbar_arrive(&sh->part_full);
     }
     if (!gone && !__all_sync(0xffffffffu, mbar_wait(&sh->part_full, 0, a.status, limit))) gone = true;
@@ -200,10 +208,10 @@ __device__ __forceinline__ void softmax_group(const TcArgs& a, const Part& p, Sh
     M = -INFINITY;
     Z = 0.f;
     for (int t0 = 0; t0 < a.rpu; t0 += 4) {                 // in key order
-      float e[4];
+      float2 e[4];
 #pragma unroll
-      for (int t = 0; t < 4; ++t) e[t] = t0 + t < a.rpu ? sh->part[t0 + t][s] : -INFINITY;
-      merge_logs(e, M, Z);
+      for (int t = 0; t < 4; ++t) e[t] = t0 + t < a.rpu ? sh->part[t0 + t][s] : make_float2(-INFINITY, 0.f);
+      add_pairs(e, M, Z);
     }
     const float off = M + log2f(Z) + a.log2G;               // 2^{c w - off} = softmax weight / G
     sh->neg_off[s] = s >= p.rows || off != off ? -INFINITY : -off;
@@ -247,7 +255,7 @@ score_cluster_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_cons
       for (int g = 0; g < kGroups; ++g) mbar_init(&sh->acc_full[g][s], 1);
     }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    if (a.rpu > 1) mbar_expect_tx(&sh->part_full, a.rpu * 128 * (int)sizeof(float));
+    if (a.rpu > 1) mbar_expect_tx(&sh->part_full, a.rpu * 128 * (int)sizeof(float2));
   }
   if (threadIdx.x < 128) {
     // stacked row s of a row block is observation row s mod r, or, when one head's rows fill two blocks, row s of the block
