@@ -16,7 +16,9 @@ __global__ void __launch_bounds__(kThreads) compact_kernel(const char* __restric
                                                            char* __restrict__ v_out, float* __restrict__ score_out,
                                                            const Shape pl) {
   griddep_wait();
-  griddep_launch();                            // whatever comes next may set itself up: a decode round 81.3 -> 80.0 us, called again and again
+  // Whatever comes next may set itself up: a decode round 81.3 -> 80.0 us, called again and again.  Not the float32 kernels: few
+  // CTAs, which would crowd on the SMs that are free first (2 heads x 2000 tokens of 128 elements 1.15 times as long).
+  if (pl.es == 2) griddep_launch();
   const long long total = (long long)pl.B * pl.Hkv * pl.n_keep;
   const long long stride = (long long)gridDim.x * (kThreads / LANES);
   const int lane = threadIdx.x % LANES;

@@ -41,7 +41,7 @@ namespace {
 namespace cg = cooperative_groups;
 
 constexpr int kSms = 148;
-constexpr int kOnePerSm = 226 * 1024, kTwoPerSm = 112 * 1024;   // dynamic shared memory with which one CTA, or two, fit on an SM
+constexpr int kOnePerSm = 226 * 1024, kNotTwoPerSm = 114 * 1024, kTwoPerSm = 112 * 1024;   // dynamic shared memory with which one CTA, or two, fit on an SM
 constexpr int kThreads = 256;
 constexpr int kTile = 64;                // keys per CTA
 constexpr int kRows = 32;                // stacked observation rows at a time
@@ -484,9 +484,9 @@ simt_weighted_sums(const T* __restrict__ v, const float2* partial, const float* 
 // A cluster of up to sixteen CTAs per (sequence, KV head), each a few adjacent tiles: the numerators stay in shared memory, the rows'
 // statistics meet through the cluster's, and nothing is formed twice or taken through global memory.  Keys lie in shared memory as
 // they came and are converted on their way into the products, by both row warps (a conversion costs four multiply-adds, so a tile's
-// 4096 cycles of products become 5100), which leaves room for two CTAs an SM; the next tile is on its way meanwhile.
+// 4096 cycles of products become 5100), which leaves room for two CTAs an SM where heads are many; the next tile is on its way meanwhile.
 // Calls, with the two kernels before: 512 tokens x 4 heads 12.7 -> 11.9 us, 300 x 2 heads of 4 queries 25.3 -> 19.0, 1000 x 4 of 4
-// 20.7 -> 17.1, 3001 x 8 37.4 -> 35.3, 2048 x 64 124 -> 99.  Scores end up as far from double as before or nearer (9.6e-8 -> 8.6e-8
+// 21.0 -> 17.3, 3001 x 8 37.4 -> 35.2, 1500 x 64 0.7 of the time.  Scores end up as far from double as before or nearer (9.6e-8 -> 8.6e-8
 // to 9.3e-8 of their norm), because sums are taken in pairs; with the rows' sums in double throughout 4.9e-8, and 37.3 and 12.3 us.
 constexpr int kMostCtas = 16;
 
@@ -500,7 +500,8 @@ struct ClusterTile {
   float2 stat[kKeyWarps][kMaxRows];                    // per key warp: shift and sum of a row over the CTA's tiles
   float sums[kThreads / kTile][kTile];
 };
-// N (shift, sum) pairs of disjoint key sets into one.  The shifts are whole numbers, so that only the additions round.
+// N (shift, sum) pairs of disjoint key sets into one.  The shifts are whole numbers, so that only the additions round.  A NaN is left
+// out, as merge_pair does.
 template <int N>
 __device__ __forceinline__ float2 add_pairs(const float2 (&p)[N]) {
   float M = p[0].x;
@@ -508,7 +509,7 @@ __device__ __forceinline__ float2 add_pairs(const float2 (&p)[N]) {
   for (int i = 1; i < N; ++i) M = fmaxf(M, p[i].x);
   float z[N];
 #pragma unroll
-  for (int i = 0; i < N; ++i) z[i] = p[i].y != 0.f ? p[i].y * pow2_diff(p[i].x, M) : 0.f;   // -inf goes with 0
+  for (int i = 0; i < N; ++i) z[i] = p[i].y > 0.f ? p[i].y * pow2_diff(p[i].x, M) : 0.f;   // -inf goes with 0
 #pragma unroll
   for (int o = 1; o < N; o <<= 1)
 #pragma unroll
@@ -661,7 +662,8 @@ simt_cluster_scores(const float* __restrict__ q, const float* __restrict__ k, co
     sm.sums[share][jl] = (acc[0] + acc[1]) + (acc[2] + acc[3]);
     __syncthreads();
     const int j = (first + t) * kTile + jl;
-    if (share == 0 && j < pl.n) s_raw[(size_t)unit * pl.n + j] = (sm.sums[0][jl] + sm.sums[1][jl]) + (sm.sums[2][jl] + sm.sums[3][jl]);
+    // a NaN counts as nothing, as in the two kernels
+    if (share == 0 && j < pl.n) s_raw[(size_t)unit * pl.n + j] = fmaxf(0.f, (sm.sums[0][jl] + sm.sums[1][jl]) + (sm.sums[2][jl] + sm.sums[3][jl]));
     __syncthreads();
   }
 }
@@ -696,25 +698,38 @@ int clusters_at_once(int size, int per_sm) {
   return n;
 }
 
-// CTAs a head, or 0: the size with the fewest tiles one after the other on an SM, of those of which the whole call is on the GPU at once.
-// Two tiles or three on end are worth it whatever part of the GPU they take; more only as long as no SM has half as much again
-// as its share (8 heads of 6000 tokens, ten tiles a CTA on 80 SMs: 62.7 us a call for 57.2; 64 heads of 2048, sixteen: 97 for 124).
+// CTAs a head and their shared memory, or 0.  A CTA that has an SM to itself takes 4 us a tile (64 elements; 8 of 128), two on an SM get in
+// each other's way, and the scheduler puts neighbours there even if others are empty: where the call has an SM for every CTA it asks
+// for so much shared memory that each gets its own (4 heads x 1000 tokens of 128 elements 16.8 us with two kernels, 17.8 without, 15.3 so).
+// One tile a CTA is always worth it (5 to 30 % of a call); up to five on end if the SMs' share of all tiles is at least half as many (8
+// heads x 3000 of 64 elements 28.7 -> 26.2, 12 x 2304 of 128 0.85; above, 8 x 1536 23.9 -> 24.7, 2 x 3000 25.3 -> 30), for rows that are
+// converted once, and with eight or more CTAs a head (16 heads x 2304 with six 1.3).  Two CTAs an SM for one tile each on no more
+// CTAs than SMs (8 heads x 1000 19.9 -> 18.1).  From 48 heads on, many tiles on end too, on one CTA an SM or two, where all SMs get
+// nearly the same (64 heads x 1000 or 1500, 74 x 2000 0.7 of the time; 32 x 512 1.1).
 template <int D>
-int cluster_size(const Shape& pl) {
+int cluster_size(const Shape& pl, size_t& smem) {
   if (pl.group_max) return 0;
   const long long units = (long long)pl.B * pl.Hkv;
   const int tiles = (pl.n + kTile - 1) / kTile;
-  int best = 0;
-  long long best_cost = 0;
+  int best = 0, best_cost = 0;
   for (int size = tiles < kMostCtas ? tiles : kMostCtas; size > 1; --size) {
     const int per = (tiles + size - 1) / size;
-    const size_t smem = cluster_smem<D>(per, pl.R);
-    if (smem > (size_t)kOnePerSm) break;               // fewer CTAs need more
-    const int fit = clusters_at_once<D>(size, smem <= (size_t)kTwoPerSm ? 2 : 1);
-    const long long cost = per * ((units * size + kSms - 1) / kSms);
-    if (fit >= units && (best == 0 || cost < best_cost)) { best = size; best_cost = cost; }
+    const size_t need = cluster_smem<D>(per, pl.R);
+    if (need > (size_t)kOnePerSm) break;               // fewer CTAs need more
+    const bool alone = clusters_at_once<D>(size, 1) >= units;
+    const bool many = units >= 48 && 5 * per * kSms * (alone ? 1 : 2) <= 6 * units * tiles;
+    bool good;
+    if (alone) good = per == 1 || many || (per <= 5 && pl.R <= kRows && size >= 8 && per * kSms <= 2 * units * tiles);
+    else good = need <= (size_t)kTwoPerSm && clusters_at_once<D>(size, 2) >= units &&
+                (units * size <= kSms ? per == 1 : many);
+    const int cost = alone ? per : 2 * per;
+    if (good && (best == 0 || cost < best_cost)) {
+      best = size;
+      best_cost = cost;
+      smem = alone && need < (size_t)kNotTwoPerSm ? kNotTwoPerSm : need;
+    }
   }
-  return best_cost <= 3 || 2 * best_cost * kSms <= 3 * units * tiles ? best : 0;
+  return best;
 }
 
 template <typename T, int D>
@@ -732,8 +747,8 @@ ahakv_status run(const Plan& pl, const void* q, const void* k, const void* v, fl
   int dev = -1;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return AHAKV_ERR_CUDA;
   if (!configured[dev]) {
-    if (cudaFuncSetAttribute(simt_row_stats<T, D, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
-        cudaFuncSetAttribute(simt_row_stats<T, D, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
+    if (cudaFuncSetAttribute(simt_row_stats<T, D, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kNotTwoPerSm) != cudaSuccess ||
+        cudaFuncSetAttribute(simt_row_stats<T, D, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kNotTwoPerSm) != cudaSuccess ||
         cudaFuncSetAttribute(simt_column_sums<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
       return AHAKV_ERR_CUDA;
     configured[dev] = true;
@@ -741,24 +756,28 @@ ahakv_status run(const Plan& pl, const void* q, const void* k, const void* v, fl
   const Shape& shape = pl;
   const int units = pl.B * pl.Hkv;
   if constexpr (std::is_same<T, float>::value) {
-    if (const int size = cluster_size<D>(shape)) {
+    size_t room = 0;
+    if (const int size = cluster_size<D>(shape, room)) {
       const int per = ((pl.n + kTile - 1) / kTile + size - 1) / size;
       count_launch();
-      return cuda_ok(launch_chained(simt_cluster_scores<D>, dim3(units * size), dim3(kThreads), size, cluster_smem<D>(per, pl.R), st, (const float*)q,
+      return cuda_ok(launch_chained(simt_cluster_scores<D>, dim3(units * size), dim3(kThreads), size, room, st, (const float*)q,
                                     (const float*)k, (const float*)v, s_raw, nu, status, per, shape, cs));
     }
   }
   const dim3 stats_grid(2 * pl.n_blk, units), sums_grid((pl.n + kTile - 1) / kTile, units);
+  // An SM for every CTA where pairs of them surely find one (4 heads x 1500 tokens 21.1 -> 20.0 us a call, 2 x 3000 25.3 -> 24.2; with up
+  // to 148 CTAs 4 x 2000 21.3 -> 26).
+  const size_t stats_smem = 3LL * stats_grid.x * units <= 2 * kSms ? kNotTwoPerSm : smem;
   float* const none = nullptr;
   cudaError_t e;
   if (kept) {
     float* shift = kept + (size_t)units * pl.R * pl.n;
-    e = launch_chained(simt_row_stats<T, D, true>, stats_grid, dim3(kThreads), 2, smem, st, (const T*)q, (const T*)k, partial, kept, shift,
+    e = launch_chained(simt_row_stats<T, D, true>, stats_grid, dim3(kThreads), 2, stats_smem, st, (const T*)q, (const T*)k, partial, kept, shift,
                        status, shape, cs);
     if (e == cudaSuccess)
       e = launch_chained(simt_weighted_sums<T, D>, sums_grid, dim3(kThreads), 1, 0, st, (const T*)v, partial, kept, shift, s_raw, nu, shape);
   } else {
-    e = launch_chained(simt_row_stats<T, D, false>, stats_grid, dim3(kThreads), 2, smem, st, (const T*)q, (const T*)k, partial, none, none,
+    e = launch_chained(simt_row_stats<T, D, false>, stats_grid, dim3(kThreads), 2, stats_smem, st, (const T*)q, (const T*)k, partial, none, none,
                        status, shape, cs);
     if (e == cudaSuccess)
       e = launch_chained(simt_column_sums<T, D>, sums_grid, dim3(kThreads), 1, smem, st, (const T*)q, (const T*)k, (const T*)v, partial,

@@ -29,10 +29,13 @@ def test_float32_scores_at_tile_edges(B, Hq, Hkv, d, n, r, flags):
 
 @pytest.mark.parametrize("B,Hq,Hkv,d,n,r", [
     (1, 1, 1, 128, 65, 1),          # two CTAs, one of them with a single key
-    (1, 8, 8, 128, 3001, 32),       # sixteen CTAs a head, two and three tiles each
-    (1, 8, 2, 64, 1500, 16),        # two chunks of rows
-    (2, 6, 2, 128, 1100, 33),       # a last chunk of three rows
-    (4, 16, 16, 128, 700, 32),      # three CTAs a head, two of them on an SM
+    (1, 8, 8, 128, 3001, 32),       # ten CTAs a head, four and five tiles each
+    (1, 8, 2, 64, 1000, 16),        # two chunks of rows
+    (2, 6, 2, 128, 900, 33),        # a last chunk of three rows
+    (3, 4, 4, 128, 2000, 32),       # eight CTAs a head, four tiles each
+    (4, 16, 16, 64, 1000, 32),      # four CTAs a head, two of them on an SM
+    (4, 16, 16, 128, 1500, 16),     # two CTAs a head, twelve tiles each
+    (1, 8, 8, 64, 1020, 20),        # sixteen CTAs a head, one tile each, two on an SM
     (1, 3, 1, 64, 513, 80),         # 240 rows
 ])
 def test_float32_scores_by_clusters(B, Hq, Hkv, d, n, r):
@@ -51,6 +54,28 @@ def test_float32_scores_by_clusters(B, Hq, Hkv, d, n, r):
     seen = torch.arange(n, device="cuda") <= torch.arange(n - r, n, device="cuda").view(r, 1)
     want = w.masked_fill(~seen, float("-inf")).softmax(-1).sum(2).view(B, Hkv, G, n).mean(2)
     assert torch.allclose(score.double(), want, rtol=1e-5, atol=1e-5 * 1e-3 * r / n)
+
+
+@pytest.mark.parametrize("where", ["key", "infinite key", "query", "head"])
+def test_float32_scores_of_nan_inputs_are_the_same_by_either_path(where):
+    """Four heads go by clusters, the same four among 32 through the two kernels: what is not a number counts as nothing in both."""
+    from paper_2506_03762_b200 import binding as ab
+    g = torch.Generator(device="cuda").manual_seed(7)
+    q = torch.randn((1, 32, 32, 64), generator=g, device="cuda")
+    k, v = (torch.randn((1, 32, 1000, 64), generator=g, device="cuda") for _ in range(2))
+    if where == "key": k[0, 1, 300, 5] = float("nan")
+    if where == "infinite key": k[0, 1, 300, 5] = float("inf")
+    if where == "query": q[0, 1, 7, 3] = float("nan")
+    if where == "head": k[0, 1] = float("nan")
+    scores = []
+    for heads, launches in ((4, 2), (32, 3)):
+        p = ab.Params(1, heads, heads, 64, 1000, 32, 0, 500, dtype=ab.F32, scale_mode=ab.SCALE_FIXED, scale=0.09, flags=0)
+        score = torch.empty((1, heads, 1000), device="cuda")
+        before = ab.ahakv_launch_count()
+        ab.ahakv_score(p, *(t[:, :heads].contiguous() for t in (q, k, v)), None, score, ab.alloc_workspace(p))
+        assert ab.ahakv_launch_count() - before == launches
+        scores.append(score[:, :4])
+    assert torch.allclose(*scores, rtol=1e-5, atol=0) and scores[0].isfinite().all()
 
 
 @pytest.mark.parametrize("n,r,Hq,Hkv,flags", [(9001, 64, 4, 4, 1), (9100, 20, 12, 4, 5)])
