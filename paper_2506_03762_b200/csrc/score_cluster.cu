@@ -8,7 +8,7 @@
 // while the statistics meet, and every CTA sends its rows' shifts and sums straight into the shared memory of the others, where
 // an mbarrier counts their bytes.  A tile visit takes 1200 - 1300 cycles, the turn from one pass to the other 4400 (mostly the
 // groups' last tiles), copies and first products 3800.  A whole eviction call with this kernel, and with runs handed out: 4096
-// tokens x 32 heads 29.0 and 31.9 us, 1024 x 64 heads 20.1 and 23.5, 2048 x 64 heads of 4 queries 32.5 and 35.5, 5000 x 32 heads
+// tokens x 32 heads 28.8 and 32.0 us, 1024 x 64 heads 20.1 and 23.5, 2048 x 64 heads of 4 queries 32.5 and 35.5, 5000 x 32 heads
 // of 64 elements 36.1 and 39.1, a decode round of 2080 x 128 heads 78.2 and 80.0, one of 4160 x 64 100 and 108, 8192 x 32 53.3 and 54.1.
 //
 // Every wait is bounded; on expiry a role records AHAKV_ERR_TIMEOUT in the status word and leaves, and the others' own waits run
@@ -186,8 +186,7 @@ __device__ __forceinline__ void softmax_group(const TcArgs& a, const Part& p, Sh
       if (!__all_sync(0xffffffffu, mbar_wait(&sh->acc_full[g][mine & 3], (mine >> 2) & 1, a.status, limit))) { gone = true; continue; }
       tc_fence_after();
       if (!live) mbar_arrive(&sh->acc_empty[acc]);
-      else if (j0 + kKeyTile - 1 <= a.min_last) row_tile(lane_base + acc * 128, c, M, Z, &sh->acc_empty[acc]);
-      else row_tile_masked(lane_base + acc * 128, j0, last, c, M, Z, &sh->acc_empty[acc]);
+      else row_tile(lane_base + acc * 128, j0 + kKeyTile - 1 <= a.min_last, j0, last, c, M, Z, &sh->acc_empty[acc]);
     }
     sh->stat[g][s] = make_float2(M, Z);
   }
@@ -353,6 +352,8 @@ int clusters_at_once(int size) {
 // - two tiles a CTA or more, so that the stream outlasts the copies' way, and with value rows beside it at most twenty: with sixteen
 //   (8192 x 32 heads) a call takes 53.3 for 54.1, with 39 (20000 x 32 of 64 elements) 84.1 for 80.5.  Without them one of 4160 x 128
 //   row blocks with 33 takes 100 for 107.
+// - with clusters of three or five, a few places left over: they split pairs of SMs, and the last ones find none until others end (45
+//   clusters of three in 45 places 1.2 to 1.3 times the time, 40 of them 0.9; 26 of five 1.1 to 1.2, 24 0.9; even sizes fill theirs).
 int tc::cluster_size(const Plan& pl, int slots) {
   const long long units = (long long)pl.B * pl.Hkv * pl.n_rb;
   const int n_blk = (pl.n_eff + kKeyTile - 1) / kKeyTile;
@@ -360,7 +361,7 @@ int tc::cluster_size(const Plan& pl, int slots) {
   int size = (int)(slots / units);
   if (size > kMostCtas) size = kMostCtas;
   if (size > n_blk / 2) size = n_blk / 2;
-  while (size > 0 && clusters_at_once(size) < units) --size;
+  while (size > 0 && clusters_at_once(size) < units + (size == 3 || size == 5 ? units / 15 : 0)) --size;
   const bool short_enough = (pl.flags & AHAKV_FLAG_VALUE_PRIOR) == 0 || n_blk <= 20 * size;
   return (n_blk <= 5 * size && pl.n_rb == 1) || (5 * units * size >= 4 * slots && short_enough) ? size : 0;
 }

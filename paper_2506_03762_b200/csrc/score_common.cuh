@@ -82,125 +82,11 @@ __device__ __forceinline__ void column_chunk_masked(const uint32_t* r, const flo
   }
 }
 
-// Pass 1 of a tile no key of which is masked: sixteen columns at a time, the next sixteen on their way meanwhile, so that a group
-// that works alone (at the first tiles, the last ones of a pass, or while the others wait) takes 2140 cycles a tile and not 3000.
-// A decode round 41.9 -> 40.3 us (kernel), 4160 tokens x 64 heads 65.8 -> 63.1; calls of 16384 x 8 heads x 4 sequences 130.2 ->
-// 128.7, 32768 x 8 heads 72.1 -> 71.1.  The less likely branches are kept small: with the pieces folded one by one there, 132.
-__device__ __forceinline__ void tmem_ld16_issue(uint32_t taddr, uint32_t* r) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-      : "r"(taddr)
-      : "memory");
-}
-__device__ __forceinline__ void tmem_ld16_wait(uint32_t* r) {
-  asm volatile("tcgen05.wait::ld.sync.aligned;"
-               : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),
-                 "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15])
-               :
-               : "memory");
-}
-// Adds 2^{c v + neg} of sixteen values to the four running sums.
-__device__ __forceinline__ void exp_add16(const uint32_t* r, uint64_t c2, uint64_t neg2, uint64_t& za, uint64_t& zb) {
-#pragma unroll
-  for (int t = 0; t < 16; t += 4) {
-    float x0, x1, x2, x3;
-    unpack2(fma2(pack2(__uint_as_float(r[t]), __uint_as_float(r[t + 1])), c2, neg2), x0, x1);
-    unpack2(fma2(pack2(__uint_as_float(r[t + 2]), __uint_as_float(r[t + 3])), c2, neg2), x2, x3);
-    za = add2(za, pack2(fast_exp2(x0), fast_exp2(x1)));
-    zb = add2(zb, pack2(fast_exp2(x2), fast_exp2(x3)));
-  }
-}
-__device__ __forceinline__ float sum4(uint64_t za, uint64_t zb) {
-  float z0, z1;
-  unpack2(add2(za, zb), z0, z1);
-  return z0 + z1;
-}
-__device__ __forceinline__ float max16(const uint32_t* r) {
-  float m0 = __uint_as_float(r[0]), m1 = __uint_as_float(r[1]);
-#pragma unroll
-  for (int t = 2; t < 16; t += 2) {
-    m0 = fmaxf(m0, __uint_as_float(r[t]));
-    m1 = fmaxf(m1, __uint_as_float(r[t + 1]));
-  }
-  return fmaxf(m0, m1);
-}
-// As fold_chunk, sixteen columns without a mask.
-__device__ __forceinline__ void fold16(const uint32_t* r, float c, float& M, float& Z) {
-  if (M > -INFINITY) {
-    uint64_t za = pack2(0.f, 0.f), zb = pack2(0.f, 0.f);
-    exp_add16(r, pack2(c, c), pack2(-M, -M), za, zb);
-    const float z = sum4(za, zb);
-    if (z < kAcceptBelow) {
-      Z += z;
-      return;
-    }
-  }
-  const float mx = max16(r) * c;
-  if (mx > -INFINITY) {
-    uint64_t za = pack2(0.f, 0.f), zb = pack2(0.f, 0.f);
-    exp_add16(r, pack2(c, c), pack2(-mx, -mx), za, zb);
-    Z = (M > -INFINITY ? Z * fast_exp2(M - mx) : 0.f) + sum4(za, zb);
-    M = mx;
-  }
-}
-// The row of this lane: folds 2^{c w} into (M, Z) and frees the accumulator.  The shift is looked at twice: for the first six pieces while they are still in
-// tensor memory, for the last two while they are in registers.
-__device__ __forceinline__ void row_tile(uint32_t from, float c, float& M, float& Z, void* empty) {
-  uint32_t u[16], w[16];
-  tmem_ld16_issue(from, u);
-  tmem_ld16_wait(u);
-  tmem_ld16_issue(from + 16, w);
-  if (!(M > -INFINITY)) M = max16(u) * c;
-  const uint64_t c2 = pack2(c, c), neg2 = pack2(-M, -M);
-  uint64_t za = pack2(0.f, 0.f), zb = pack2(0.f, 0.f), ya = pack2(0.f, 0.f), yb = pack2(0.f, 0.f);
-  exp_add16(u, c2, neg2, za, zb);
-#pragma unroll
-  for (int ch = 2; ch < 8; ch += 2) {
-    tmem_ld16_wait(w);
-    tmem_ld16_issue(from + 16 * ch, u);
-    exp_add16(w, c2, neg2, za, zb);
-    tmem_ld16_wait(u);
-    tmem_ld16_issue(from + 16 * ch + 16, w);
-    if (ch < 6) exp_add16(u, c2, neg2, za, zb);
-    else exp_add16(u, c2, neg2, ya, yb);
-  }
-  float z = sum4(za, zb);
-  const bool sound = z < kAcceptBelow;                        // an overflow or a NaN fails this test too
-  tmem_ld16_wait(w);
-  if (__any_sync(0xffffffffu, !sound)) {
-#pragma unroll 1
-    for (int ch = 0; ch < 6; ++ch) {
-      uint32_t again[16];
-      tmem_ld16_issue(from + 16 * ch, again);
-      tmem_ld16_wait(again);
-      if (!sound) fold16(again, c, M, Z);
-    }
-  }
-  tc_fence_before();
-  mbar_arrive(empty);
-  if (sound) {
-    Z += z;
-    exp_add16(w, c2, neg2, ya, yb);
-    z = sum4(ya, yb);
-  }
-  if (sound && z < kAcceptBelow) {
-    Z += z;
-  } else {
-    const float mx = fmaxf(M, fmaxf(max16(u), max16(w)) * c);
-    if (mx > -INFINITY) {
-      za = zb = pack2(0.f, 0.f);
-      exp_add16(u, c2, pack2(-mx, -mx), za, zb);
-      exp_add16(w, c2, pack2(-mx, -mx), za, zb);
-      Z = (M > -INFINITY ? Z * fast_exp2(M - mx) : 0.f) + sum4(za, zb);
-      M = mx;
-    }
-  }
-}
-
-// The same of any tile, 128 keys from j0 on.
-__device__ __forceinline__ void row_tile_masked(uint32_t from, int j0, int last, float c, float& M, float& Z, void* empty) {
+// Pass 1, 128 keys from j0 on for the row of this lane: folds 2^{c w} into (M, Z) and frees the accumulator.  One small loop for
+// every tile: sixteen columns at a time with the next sixteen on their way, and a path of its own for masked tiles, took a group that
+// works alone 2140 cycles a tile and not 3000 and left long calls where they were (32768 x 256 1299 us, 1312 so), but its code
+// made the short ones slower (484 tokens x 192 heads of 4 queries 36.1 -> 39.7 us, 1200 x 80 28.6 -> 30.7, 4592 x 80 61.3 -> 66.0).
+__device__ __forceinline__ void row_tile(uint32_t from, bool full, int j0, int last, float c, float& M, float& Z, void* empty) {
 #pragma unroll 1
   for (int ch = 0; ch < 4; ++ch) {
     uint32_t ra[32];
@@ -210,7 +96,7 @@ __device__ __forceinline__ void row_tile_masked(uint32_t from, int j0, int last,
       tc_fence_before();
       mbar_arrive(empty);                                    // the accumulator is free for the next product
     }
-    fold_chunk(ra, false, j0 + 32 * ch, last, c, M, Z);
+    fold_chunk(ra, full, j0 + 32 * ch, last, c, M, Z);
   }
 }
 

@@ -398,8 +398,7 @@ __device__ __forceinline__ void softmax_group(const TcArgs& a, Shared* sh, uint3
         const int j0 = (sg.blk0 + t) * kKeyTile;
         const bool full = j0 + kKeyTile - 1 <= a.min_last;   // no key of the tile is masked
         if (live) {
-          if (full) row_tile(lane_base + acc * 128, c, M, Z, &sh->acc_empty[acc]);
-          else row_tile_masked(lane_base + acc * 128, j0, last, c, M, Z, &sh->acc_empty[acc]);
+          row_tile(lane_base + acc * 128, full, j0, last, c, M, Z, &sh->acc_empty[acc]);
         } else {
           mbar_arrive(&sh->acc_empty[acc]);
         }
